@@ -112,9 +112,10 @@ struct LvPtrs {
 };
 
 struct InstCtl {
-  int outer_done, inner_done, solving, rounds, status, pad;
+  int outer_done, inner_done, solving, rounds, status;
+  int round_iters;  // CG iterations of the current round
   long long iters;
-  double res, res0, alpha, beta, gamma;
+  double res, alpha, beta, gamma;
 };
 
 struct BatchCtl {
@@ -540,7 +541,7 @@ __global__ void __launch_bounds__(kBlock) kb_outer(const InstDev *__restrict__ i
                                                    const double *__restrict__ part, InstCtl *c, BatchCtl *b,
                                                    double tol, int maxit, int nfam, const int *__restrict__ fam_cnt,
                                                    int *__restrict__ fam_pref, cudaGraphConditionalHandle hout,
-                                                   cudaGraphConditionalHandle hin, int use_cond, int set_hin) {
+                                                   cudaGraphConditionalHandle hin, int use_cond) {
   const int ii = blockIdx.x;
   if (!c[ii].outer_done) {
     const InstDev &I = inst[ii];
@@ -552,7 +553,7 @@ __global__ void __launch_bounds__(kBlock) kb_outer(const InstDev *__restrict__ i
       const double prev = C.res;
       C.res = m;
       int done = 0;
-      if (m <= tol) done = 1;
+      if (m <= tol || C.status) done = 1;  // converged, or the round's CG failed
       else if (!(m == m) || m > 1e300) { done = 1; C.status = LBE_ERR_NONFINITE; }
       // out of rounds or iterations, or a round that did not halve the
       // residual (the tolerance is below what the arithmetic resolves)
@@ -563,6 +564,7 @@ __global__ void __launch_bounds__(kBlock) kb_outer(const InstDev *__restrict__ i
       C.outer_done = done;
       C.inner_done = done;
       C.solving = !done;
+      C.round_iters = 0;
       C.rounds += 1;
     }
   } else if (threadIdx.x == 0) {
@@ -575,7 +577,7 @@ __global__ void __launch_bounds__(kBlock) kb_outer(const InstDev *__restrict__ i
     int any = 0;
     for (int i = 0; i < n; ++i) any |= !__ldcg(&c[i].outer_done);
     set_cond(hout, use_cond, any ? 1u : 0u);
-    if (!any && set_hin) set_cond(hin, use_cond, 0u);
+    set_cond(hin, use_cond, any ? 1u : 0u);
     b->any_outer = any;
     if (!any) b->any_inner = 0;
   }
@@ -618,48 +620,65 @@ __global__ void __launch_bounds__(kBlock) kb_cg_b(const InstDev *__restrict__ in
   }
 }
 
-// per-instance scalar recurrence (one block per instance); the last block
-// sets the CG loop's condition (any instance still iterating) and rebuilds
-// the active-tile lists
-__global__ void __launch_bounds__(kBlock) kb_scal(const InstDev *__restrict__ inst, int n, int T,
+// per-instance scalar recurrence (one block per instance): the step lengths
+// of the update that follows.  A breakdown (the correction is converged to
+// rounding, or a zero residual) ends the instance's inner solve without an
+// update.
+__global__ void __launch_bounds__(kBlock) kb_scal(const InstDev *__restrict__ inst, int T,
+                                                  const double *__restrict__ part, InstCtl *c) {
+  const int ii = blockIdx.x;
+  if (c[ii].inner_done) return;
+  const InstDev &I = inst[ii];
+  double g = 0.0, d = 0.0;
+  for (int k = threadIdx.x; k < I.ntiles; k += kBlock) {
+    g += __ldcg(part + I.tile0 + k);
+    d += __ldcg(part + (long long)T + I.tile0 + k);
+  }
+  g = breduce<false>(g);
+  d = breduce<false>(d);
+  if (threadIdx.x == 0) {
+    InstCtl &C = c[ii];
+    if (C.round_iters == 0) {
+      C.beta = 0.0;
+      C.alpha = g / d;
+      C.gamma = g;
+      if (!(d > 0.0) || !(g > 0.0)) C.inner_done = 1;
+    } else if (!(d == d)) {
+      C.inner_done = 1;
+      C.status = LBE_ERR_NONFINITE;
+    } else {
+      const double beta = g / C.gamma;
+      const double den = d - beta * g / C.alpha;
+      if (!(den > 0.0) || !(g > 0.0)) C.inner_done = 1;
+      else { C.beta = beta; C.alpha = g / den; C.gamma = g; }
+    }
+  }
+}
+
+// per-instance stopping test on the updated residual (one block per
+// instance); the last block sets the CG loop's condition (any instance still
+// iterating) and rebuilds the active-tile lists.  The loop ends here, before
+// the V-cycle and the stencil that the next update would need.
+__global__ void __launch_bounds__(kBlock) kb_test(const InstDev *__restrict__ inst, int n, int T,
                                                   const double *__restrict__ part, InstCtl *c, BatchCtl *b,
-                                                  double eta, double tol_abs, int maxit, int init, int nfam,
+                                                  double eta, double tol_abs, int maxit, int nfam,
                                                   const int *__restrict__ fam_cnt, int *__restrict__ fam_pref,
                                                   cudaGraphConditionalHandle hin, int use_cond) {
   const int ii = blockIdx.x;
   if (!c[ii].inner_done) {
     const InstDev &I = inst[ii];
-    double g = 0.0, d = 0.0, m = 0.0;
-    for (int k = threadIdx.x; k < I.ntiles; k += kBlock) {
-      g += __ldcg(part + I.tile0 + k);
-      d += __ldcg(part + (long long)T + I.tile0 + k);
-      if (!init) m = fmax(m, __ldcg(part + 2LL * T + I.tile0 + k));
-    }
-    g = breduce<false>(g);
-    d = breduce<false>(d);
+    double m = 0.0;
+    for (int k = threadIdx.x; k < I.ntiles; k += kBlock) m = fmax(m, __ldcg(part + 2LL * T + I.tile0 + k));
     m = breduce<true>(m);
     if (threadIdx.x == 0) {
       InstCtl &C = c[ii];
+      C.round_iters += 1;
+      C.iters += 1;
+      atomicAdd((unsigned long long *)&b->total_iters, 1ULL);
       int done = 0;
-      if (init) {
-        C.res0 = C.res;
-        C.beta = 0.0;
-        C.alpha = g / d;
-        C.gamma = g;
-        if (!(d > 0.0) || !(g > 0.0)) done = 1;  // zero residual: nothing to solve
-      } else {
-        C.iters += 1;
-        atomicAdd((unsigned long long *)&b->total_iters, 1ULL);
-        if (m <= fmax(eta * C.res0, tol_abs)) done = 1;
-        else if (!(m == m) || m > 1e300 || !(d == d)) { done = 1; C.status = LBE_ERR_NONFINITE; C.outer_done = 1; }
-        else if (C.iters >= maxit) done = 1;
-        else {
-          const double beta = g / C.gamma;
-          const double den = d - beta * g / C.alpha;
-          if (!(den > 0.0) || !(g > 0.0)) done = 1;  // breakdown: converged to rounding
-          else { C.beta = beta; C.alpha = g / den; C.gamma = g; }
-        }
-      }
+      if (m <= fmax(eta * C.res, tol_abs)) done = 1;
+      else if (!(m == m) || m > 1e300) { done = 1; C.status = LBE_ERR_NONFINITE; }
+      else if (C.iters >= maxit) done = 1;
       C.inner_done = done;
     }
   }
@@ -688,6 +707,7 @@ __global__ void __launch_bounds__(kBlock) kb_cg_a(const InstDev *__restrict__ in
   const int Tact = pref[n];
   for (int tp = blockIdx.x; tp < Tact; tp += gridDim.x) {
     const int ii = find_inst(pref, n, tp);
+    if (c[ii].inner_done) continue;  // a breakdown in this iteration (block-uniform)
     const InstDev &I = inst[ii];
     const int j = tp - pref[ii];
     const float alpha = (float)c[ii].alpha, beta = (float)c[ii].beta;
@@ -1360,7 +1380,7 @@ int vcycle_kernels(const lbe_batch *b) { return b->mg_nlev >= 2 ? 2 * (b->mg_nle
 struct SolveArgs {
   const lbe::InstDev *inst;
   const int *tile_inst, *pref0, *fam_cnt;
-  int T, Ntot, n, maxit, nfam, use = 1, init1 = 1, init0 = 0, set_hist, hin_no = 0, hin_yes = 1;
+  int T, Ntot, n, maxit, nfam, use = 1, set_hist;
   const uint32_t *mask;
   const float *fin;
   float *fout;
@@ -1447,17 +1467,12 @@ cudaError_t build_graph(lbe_batch *b, bool step, const float *fin, float *fout, 
   void *a_ext[] = {&A.inst, &A.tile_inst, &A.T, &A.Ntot, &A.mask, &A.phifx, &A.phi_prev, &A.phi32, &A.hist};
   void *a_reset[] = {&A.n, &A.c, &A.bc, &A.hist, &A.set_hist};
   void *a_res[] = {&A.inst, &A.tile_inst, &A.T, &A.Ntot, &A.mask, &A.qsolve, &A.phifx, &A.v, &A.part, &A.c};
-  // the test before the round loop must not touch the inner loop's
-  // condition (it belongs to the loop body); the one closing a round does
-  void *a_out0[] = {&A.inst, &A.n,    &A.T,       &A.part,     &A.c,    &A.bc,  &A.tol,
-                    &A.maxit, &A.nfam, &A.fam_cnt, &A.fam_pref, &A.hout, &A.hin, &A.use, &A.hin_no};
   void *a_out[] = {&A.inst, &A.n,    &A.T,       &A.part,     &A.c,    &A.bc,  &A.tol,
-                   &A.maxit, &A.nfam, &A.fam_cnt, &A.fam_pref, &A.hout, &A.hin, &A.use, &A.hin_yes};
+                   &A.maxit, &A.nfam, &A.fam_cnt, &A.fam_pref, &A.hout, &A.hin, &A.use};
   void *a_b[] = {&A.inst, &A.n, &A.pref0, &A.T, &A.mask, &A.vr, &A.vu, &A.vw, &A.part};
-  void *a_si[] = {&A.inst, &A.n,     &A.T,    &A.part,    &A.c,        &A.bc,  &A.eta, &A.tol_abs,
-                  &A.maxit, &A.init1, &A.nfam, &A.fam_cnt, &A.fam_pref, &A.hin, &A.use};
-  void *a_st[] = {&A.inst, &A.n,     &A.T,    &A.part,    &A.c,        &A.bc,  &A.eta, &A.tol_abs,
-                  &A.maxit, &A.init0, &A.nfam, &A.fam_cnt, &A.fam_pref, &A.hin, &A.use};
+  void *a_sc[] = {&A.inst, &A.T, &A.part, &A.c};
+  void *a_te[] = {&A.inst, &A.n,    &A.T,       &A.part,     &A.c,   &A.bc, &A.eta, &A.tol_abs,
+                  &A.maxit, &A.nfam, &A.fam_cnt, &A.fam_pref, &A.hin, &A.use};
   void *a_a[] = {&A.inst, &A.n, &A.pref0, &A.T, &A.mask, &A.v, &A.part, &A.c};
   void *a_cor[] = {&A.inst, &A.tile_inst, &A.T, &A.mask, &A.vx, &A.phifx, &A.phi32, &A.flag, &A.c};
   if (step) {
@@ -1472,24 +1487,21 @@ cudaError_t build_graph(lbe_batch *b, bool step, const float *fin, float *fout, 
     if (e == cudaSuccess && !b->flow) e = add_node(g, &last, (void *)kb_extrapolate, Gext, B, a_ext);
   }
   if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&A.hout, g, 1, cudaGraphCondAssignDefault);
-  // reset -> residual test -> while (any instance unconverged) { V-cycle ->
-  // CG -> correct -> residual test }
+  // reset -> while (any instance unconverged) { residual test -> while (any
+  // instance iterating) { V-cycle -> stencil and dot products -> step lengths
+  // -> update -> test } -> correct }
   if (e == cudaSuccess) e = add_node(g, &last, (void *)kb_solve_reset, rb, dim3(256), a_reset);
-  if (e == cudaSuccess) e = add_node(g, &last, (void *)kb_res, Gres, B, a_res);
-  if (e == cudaSuccess) e = add_node(g, &last, (void *)kb_outer, NB, B, a_out0);
   if (e == cudaSuccess) e = add_while(g, &last, A.hout, &bo);
   if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&A.hin, bo, 0, 0);
-  if (e == cudaSuccess) e = add_vcycle(b, bo, &lo);
-  if (e == cudaSuccess) e = add_node(bo, &lo, (void *)kb_cg_b, Gb, B, a_b);
-  if (e == cudaSuccess) e = add_node(bo, &lo, (void *)kb_scal, NB, B, a_si);
-  if (e == cudaSuccess) e = add_while(bo, &lo, A.hin, &bi);
-  if (e == cudaSuccess) e = add_node(bi, &li, (void *)kb_cg_a, Ga, B, a_a);
-  if (e == cudaSuccess) e = add_vcycle(b, bi, &li);
-  if (e == cudaSuccess) e = add_node(bi, &li, (void *)kb_cg_b, Gb, B, a_b);
-  if (e == cudaSuccess) e = add_node(bi, &li, (void *)kb_scal, NB, B, a_st);
-  if (e == cudaSuccess) e = add_node(bo, &lo, (void *)kb_correct, Gcor, B, a_cor);
   if (e == cudaSuccess) e = add_node(bo, &lo, (void *)kb_res, Gres, B, a_res);
   if (e == cudaSuccess) e = add_node(bo, &lo, (void *)kb_outer, NB, B, a_out);
+  if (e == cudaSuccess) e = add_while(bo, &lo, A.hin, &bi);
+  if (e == cudaSuccess) e = add_vcycle(b, bi, &li);
+  if (e == cudaSuccess) e = add_node(bi, &li, (void *)kb_cg_b, Gb, B, a_b);
+  if (e == cudaSuccess) e = add_node(bi, &li, (void *)kb_scal, NB, B, a_sc);
+  if (e == cudaSuccess) e = add_node(bi, &li, (void *)kb_cg_a, Ga, B, a_a);
+  if (e == cudaSuccess) e = add_node(bi, &li, (void *)kb_test, NB, B, a_te);
+  if (e == cudaSuccess) e = add_node(bo, &lo, (void *)kb_correct, Gcor, B, a_cor);
   if (e == cudaSuccess && prof) e = add_event(g, &last, b->ev[3]);
   if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);
   cudaGraphDestroy(g);
@@ -1560,24 +1572,19 @@ int run_polled(lbe_batch *b, bool step, const float *fin, float *fout, int64_t *
   while (any_outer && err == cudaSuccess) {
     kb_res<<<Gres, kBlock, 0, st>>>(A.inst, A.tile_inst, A.T, A.Ntot, A.mask, A.qsolve, A.phifx, A.v, A.part, A.c);
     kb_outer<<<n, kBlock, 0, st>>>(A.inst, n, A.T, A.part, A.c, A.bc, A.tol, A.maxit, A.nfam, A.fam_cnt, A.fam_pref,
-                                   h0, h0, 0, 0);
+                                   h0, h0, 0);
     nl += 2;
     flags(&any_outer, nullptr);
     if (!any_outer) break;
-    if (vc && err == cudaSuccess) err = cudaGraphLaunch(vc, st), nl += vck;
-    kb_cg_b<<<Gb, kBlock, 0, st>>>(A.inst, n, A.pref0, A.T, A.mask, A.vr, A.vu, A.vw, A.part);
-    kb_scal<<<n, kBlock, 0, st>>>(A.inst, n, A.T, A.part, A.c, A.bc, A.eta, A.tol_abs, A.maxit, 1, A.nfam, A.fam_cnt,
-                                  A.fam_pref, h0, 0);
-    nl += 2;
-    int any_inner = 0;
-    flags(nullptr, &any_inner);
+    int any_inner = 1;
     while (any_inner && err == cudaSuccess) {
-      kb_cg_a<<<Ga, kBlock, 0, st>>>(A.inst, n, A.pref0, A.T, A.mask, A.v, A.part, A.c);
       if (vc) err = cudaGraphLaunch(vc, st), nl += vck;
       kb_cg_b<<<Gb, kBlock, 0, st>>>(A.inst, n, A.pref0, A.T, A.mask, A.vr, A.vu, A.vw, A.part);
-      kb_scal<<<n, kBlock, 0, st>>>(A.inst, n, A.T, A.part, A.c, A.bc, A.eta, A.tol_abs, A.maxit, 0, A.nfam,
-                                    A.fam_cnt, A.fam_pref, h0, 0);
-      nl += 3;
+      kb_scal<<<n, kBlock, 0, st>>>(A.inst, A.T, A.part, A.c);
+      kb_cg_a<<<Ga, kBlock, 0, st>>>(A.inst, n, A.pref0, A.T, A.mask, A.v, A.part, A.c);
+      kb_test<<<n, kBlock, 0, st>>>(A.inst, n, A.T, A.part, A.c, A.bc, A.eta, A.tol_abs, A.maxit, A.nfam, A.fam_cnt,
+                                    A.fam_pref, h0, 0);
+      nl += 4;
       flags(nullptr, &any_inner);
     }
     kb_correct<<<Gcor, kBlock, 0, st>>>(A.inst, A.tile_inst, A.T, A.mask, A.vx, A.phifx, A.phi32, A.flag, A.c);

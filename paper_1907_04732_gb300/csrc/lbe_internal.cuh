@@ -204,8 +204,10 @@ constexpr int kBlock = 256;
 // Control block of the Poisson solves (device memory; see poisson.cu).
 struct PoissonCtl {
   int outer_done, inner_done, rounds, status, sticky_status, arrive;
+  int round_iters;  // CG iterations of the current round
+  unsigned long long max_bits;  // max |r|/diag of an update, as the bits of a double
   long long solve_iters, total_iters, total_rounds, solves, max_solve_iters;
-  double res, res0, alpha, beta, gamma;
+  double res, alpha, beta, gamma;
   double ref;  // linear solves: max |rhs|/diag, the scale of the relative test
 };
 

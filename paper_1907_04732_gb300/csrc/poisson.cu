@@ -20,9 +20,9 @@
 // Each step starts from the extrapolation in time of the previous solutions
 // (fp32::extrapolate_node, fp32::extrapolate_fx).  The CG is the Chronopoulos-Gear variant: both
 // inner products of an iteration come from one reduction phase, so an
-// iteration is the vector update (k_cg_a), the preconditioner, and the
-// stencil with the dot products (k_cg_b, whose last block runs the scalar
-// recurrence).  The whole solve is one CUDA graph: a device-side `while`
+// iteration is the preconditioner, the stencil with the dot products (k_cg_b,
+// whose last block runs the scalar recurrence) and the vector update with the
+// stopping test (k_cg_a).  The whole solve is one CUDA graph: a device-side `while`
 // over refinement rounds containing a `while` over CG iterations; kernels set
 // the loop conditions, bounded by the round limit and poisson_max_iter.
 // Where conditional graph nodes are not available the same kernels run from
@@ -43,7 +43,6 @@ constexpr int kMaxOuter = 24;  // refinement rounds per solve
 constexpr int kChunk = 16;     // fallback: iterations between host polls
 
 enum { S_RU = 0, S_WU = 1, S_MAX = 2 };
-enum { C_INIT = 0, C_ITER = 1 };
 
 __host__ __device__ constexpr uint32_t nn_bits() {
   uint32_t b = 0;
@@ -65,6 +64,25 @@ __device__ __forceinline__ T diag_t(uint32_t m, uint32_t selfmask) {
   const int nn = __popc(kNN & nself), nns = dbl * __popc(kNN & nself & ~m);
   const int mm = __popc(kNNN & nself), mms = dbl * __popc(kNNN & nself & ~m);
   return (T)(2 * (nn + nns) + (mm + mms)) * (T)(1.0 / 6.0);
+}
+
+// 1/diag.  A double division takes a dozen instructions on the narrow FP64
+// pipe; the diagonal is an integer over 6, so its inverses are a table.
+struct InvDiag {
+  double v[49];
+  constexpr InvDiag() : v() {
+    for (int k = 1; k < 49; ++k) v[k] = 1.0 / ((double)k * (1.0 / 6.0));
+  }
+};
+__constant__ InvDiag kInvDiag = InvDiag();
+template <typename T>
+__device__ __forceinline__ T inv_diag(uint32_t m, uint32_t selfmask) {
+  if (sizeof(T) == 4) return (T)1 / diag_t<T>(m, selfmask);
+  const uint32_t nself = ~selfmask;
+  const int dbl = (selfmask & kPlainLaplacian) ? 0 : 1;
+  const int nn = __popc(kNN & nself), nns = dbl * __popc(kNN & nself & ~m);
+  const int mm = __popc(kNNN & nself), mms = dbl * __popc(kNNN & nself & ~m);
+  return (T)kInvDiag.v[2 * (nn + nns) + (mm + mms)];
 }
 
 // lap_mod(v)(r) at a fluid node, FP64.  With the link weights scaled by 6
@@ -129,44 +147,39 @@ __device__ __forceinline__ bool last_block(PoissonCtl *c, int nblk) {
   return last;
 }
 
-// two sums and a max over the block in one pass (the order of block_reduce
-// for each value, with one pair of barriers); results valid in thread 0
-__device__ __forceinline__ void block_reduce3(double &a, double &b, double &m) {
-  __shared__ double sh[3][kBlock / 32];
+// two sums over the block in one pass (the order of block_reduce for each
+// value, with one pair of barriers); results valid in thread 0
+__device__ __forceinline__ void block_reduce2(double &a, double &b) {
+  __shared__ double sh[2][kBlock / 32];
   const int t = flat_tid(), lane = t & 31, wid = t >> 5;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const double ua = __shfl_down_sync(0xffffffffu, a, o), ub = __shfl_down_sync(0xffffffffu, b, o),
-                 um = __shfl_down_sync(0xffffffffu, m, o);
+    const double ua = __shfl_down_sync(0xffffffffu, a, o), ub = __shfl_down_sync(0xffffffffu, b, o);
     a += ua;
     b += ub;
-    m = fmax(m, um);
   }
   __syncthreads();
   if (lane == 0) {
     sh[0][wid] = a;
     sh[1][wid] = b;
-    sh[2][wid] = m;
   }
   __syncthreads();
   if (t == 0) {
     a = sh[0][0];
     b = sh[1][0];
-    m = sh[2][0];
     for (int w = 1; w < kBlock / 32; ++w) {
       a += sh[0][w];
       b += sh[1][w];
-      m = fmax(m, sh[2][w]);
     }
   }
 }
 
-// sums/max of the partials in block order (every thread of the block calls).
+// sums of the partials in block order (every thread of the block calls).
 // All of a thread's partials are loaded before any is added (one L2 latency
 // instead of one per stride of the block), then summed in the same order.
-__device__ __forceinline__ void reduce_partials(const double *part, int nblk, double *ru, double *wu, double *mx) {
+__device__ __forceinline__ void reduce_partials(const double *part, int nblk, double *ru, double *wu) {
   constexpr int kPer = (kSolveBlocks + kBlock - 1) / kBlock;  // the solve launches at most kSolveBlocks blocks
-  double pa[kPer], pb[kPer], pm[kPer];
+  double pa[kPer], pb[kPer];
   const int t = flat_tid();
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
@@ -174,26 +187,22 @@ __device__ __forceinline__ void reduce_partials(const double *part, int nblk, do
     const bool in = i < nblk;
     pa[k] = in ? __ldcg(part + S_RU * nblk + i) : 0.0;
     pb[k] = in ? __ldcg(part + S_WU * nblk + i) : 0.0;
-    pm[k] = in ? __ldcg(part + S_MAX * nblk + i) : 0.0;
   }
-  double a = 0.0, b = 0.0, m = 0.0;
+  double a = 0.0, b = 0.0;
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     if (t + k * kBlock < nblk) {
       a += pa[k];
       b += pb[k];
-      m = fmax(m, pm[k]);
     }
   }
   for (int i = t + kPer * kBlock; i < nblk; i += kBlock) {  // a larger launch (not used by the solve)
     a += __ldcg(part + S_RU * nblk + i);
     b += __ldcg(part + S_WU * nblk + i);
-    m = fmax(m, __ldcg(part + S_MAX * nblk + i));
   }
-  block_reduce3(a, b, m);
+  block_reduce2(a, b);
   *ru = a;
   *wu = b;
-  *mx = m;
 }
 
 // outer test of a refinement round (thread 0 of the last block of k_res):
@@ -202,11 +211,11 @@ __device__ __forceinline__ void reduce_partials(const double *part, int nblk, do
 // resolves: the solve stops there (LBE_ERR_NOCONVERGE) instead of repeating
 // rounds that cannot help.
 __device__ void outer_check(PoissonCtl *c, double m, double tol, int maxit, cudaGraphConditionalHandle hout,
-                            cudaGraphConditionalHandle hin, int use_cond, int set_hin) {
+                            cudaGraphConditionalHandle hin, int use_cond) {
   const double prev = c->res;
   c->res = m;
   int done = 0;
-  if (m <= tol) {
+  if (m <= tol || c->status) {  // converged, or the round's CG failed
     done = 1;
   } else if (!(m == m) || m > 1e300) {
     done = 1;
@@ -217,46 +226,59 @@ __device__ void outer_check(PoissonCtl *c, double m, double tol, int maxit, cuda
   }
   c->outer_done = done;
   c->inner_done = done;  // nothing more of the round runs once converged
+  c->round_iters = 0;
   c->rounds += 1;
   c->total_rounds += 1;
   set_cond(hout, use_cond, done ? 0u : 1u);
-  if (done && set_hin) set_cond(hin, use_cond, 0u);
+  set_cond(hin, use_cond, done ? 0u : 1u);
 }
 
-// scalar recurrence of the Chronopoulos-Gear CG and the inner stopping test
-// (relative reduction eta of the round's starting residual); thread 0 of the
-// last block of k_cg_b
-__device__ void cg_scalars(PoissonCtl *c, double gam, double del, double mx, double eta, double tol_abs, int maxit,
-                           int mode, cudaGraphConditionalHandle hin, int use_cond) {
+// scalar recurrence of the Chronopoulos-Gear CG (thread 0 of the last block
+// of k_cg_b): step lengths of the update that follows.  A breakdown (the
+// correction is converged to rounding, or a zero residual) ends the inner
+// solve without an update.
+__device__ void cg_scalars(PoissonCtl *c, double gam, double del, cudaGraphConditionalHandle hin, int use_cond) {
   int done = 0;
-  if (mode == C_INIT) {
-    c->res0 = c->res;
+  if (c->round_iters == 0) {
     c->beta = 0.0;
     c->alpha = gam / del;
     c->gamma = gam;
-    if (!(del > 0.0) || !(gam > 0.0)) done = 1;  // zero residual: nothing to solve
+    if (!(del > 0.0) || !(gam > 0.0)) done = 1;
+  } else if (!(del == del)) {
+    done = 1;
+    c->status = LBE_ERR_NONFINITE;
   } else {
-    c->solve_iters += 1;
-    c->total_iters += 1;
-    if (mx <= fmax(eta * c->res0, tol_abs)) {
-      done = 1;
-    } else if (!(mx == mx) || mx > 1e300 || !(del == del)) {
-      done = 1;
-      c->status = LBE_ERR_NONFINITE;
-      c->outer_done = 1;
-    } else if (c->solve_iters >= maxit) {
+    const double beta = gam / c->gamma;
+    const double den = del - beta * gam / c->alpha;
+    if (!(den > 0.0) || !(gam > 0.0)) {
       done = 1;
     } else {
-      const double beta = gam / c->gamma;
-      const double den = del - beta * gam / c->alpha;
-      if (!(den > 0.0) || !(gam > 0.0)) {
-        done = 1;  // breakdown: the correction is converged to rounding
-      } else {
-        c->beta = beta;
-        c->alpha = gam / den;
-        c->gamma = gam;
-      }
+      c->beta = beta;
+      c->alpha = gam / den;
+      c->gamma = gam;
     }
+  }
+  if (done) {
+    c->inner_done = 1;
+    set_cond(hin, use_cond, 0u);
+  }
+}
+
+// inner stopping test (relative reduction eta of the round's starting
+// residual) on the updated residual; thread 0 of the last block of k_cg_a
+__device__ void cg_test(PoissonCtl *c, double mx, double eta, double tol_abs, int maxit,
+                        cudaGraphConditionalHandle hin, int use_cond) {
+  int done = 0;
+  c->round_iters += 1;
+  c->solve_iters += 1;
+  c->total_iters += 1;
+  if (mx <= fmax(eta * c->res, tol_abs)) {
+    done = 1;
+  } else if (!(mx == mx) || mx > 1e300) {
+    done = 1;
+    c->status = LBE_ERR_NONFINITE;
+  } else if (c->solve_iters >= maxit) {
+    done = 1;
   }
   c->inner_done = done;
   set_cond(hin, use_cond, done ? 0u : 1u);
@@ -299,7 +321,7 @@ __global__ void __launch_bounds__(kBlock) k_res(const Geo g, int zpt, const Phys
                                                 T *__restrict__ s, double *__restrict__ part, int nblk,
                                                 PoissonCtl *c, double tol, double tol_rel, int maxit,
                                                 cudaGraphConditionalHandle hout, cudaGraphConditionalHandle hin,
-                                                int use_cond, int set_hin) {
+                                                int use_cond) {
   constexpr bool RHS = MODE == R_RHS || MODE == R_RHS_FF;
   float mx = 0.f, mb = 0.f;
   for (int kz = 0; kz < zpt; ++kz) {
@@ -390,7 +412,7 @@ __global__ void __launch_bounds__(kBlock) k_res(const Geo g, int zpt, const Phys
   if (flat_tid() == 0) {
     c->arrive = 0;
     if (RHS) c->ref = ref;
-    outer_check(c, m, RHS ? fmax(tol, tol_rel * ref) : tol, maxit, hout, hin, use_cond, set_hin);
+    outer_check(c, m, RHS ? fmax(tol, tol_rel * ref) : tol, maxit, hout, hin, use_cond);
   }
 }
 
@@ -400,8 +422,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock) k_cg_b(const Geo g, int zpt, uint32_t selfmask,
                                                  const uint32_t *__restrict__ mask, const T *__restrict__ u,
                                                  const T *__restrict__ r, T *__restrict__ w,
-                                                 double *__restrict__ part, int nblk, PoissonCtl *c, double eta,
-                                                 double tol_abs, int maxit, int mode,
+                                                 double *__restrict__ part, int nblk, PoissonCtl *c,
                                                  cudaGraphConditionalHandle hin, int use_cond) {
   if (c->inner_done) return;
   T ru = 0, wu = 0;
@@ -438,22 +459,27 @@ __global__ void __launch_bounds__(kBlock) k_cg_b(const Geo g, int zpt, uint32_t 
     part[S_WU * nblk + flat_bid()] = (double)b;
   }
   if (!last_block(c, nblk)) return;
-  double gam, del, mx;
-  reduce_partials(part, nblk, &gam, &del, &mx);
+  double gam, del;
+  reduce_partials(part, nblk, &gam, &del);
   if (flat_tid() == 0) {
     c->arrive = 0;
-    cg_scalars(c, gam, del, mx, eta, tol_abs, maxit, mode, hin, use_cond);
+    cg_scalars(c, gam, del, hin, use_cond);
   }
 }
 
 // vector update: p = u + beta p, s = w + beta s, x += alpha p,
-// r -= alpha s, u = r/diag; partial max |r|/diag
+// r -= alpha s, u = r/diag; the last block runs the stopping test on
+// max |r|/diag, so that the loop ends here.  (With the test in the stencil
+// kernel, the round's last V-cycle and stencil served only to carry it: on
+// the 64x64x256 electro-osmosis lattice, tolerance 1e-13, the solve took
+// 388 us per step instead of 333.)
 template <typename T>
 __global__ void __launch_bounds__(kBlock) k_cg_a(const Geo g, int zpt, uint32_t selfmask,
                                                  const uint32_t *__restrict__ mask, T *__restrict__ x,
                                                  T *__restrict__ r, T *__restrict__ u, const T *__restrict__ w,
-                                                 T *__restrict__ p, T *__restrict__ s, double *__restrict__ part,
-                                                 int nblk, const PoissonCtl *c) {
+                                                 T *__restrict__ p, T *__restrict__ s, int nblk, PoissonCtl *c,
+                                                 double eta, double tol_abs, int maxit,
+                                                 cudaGraphConditionalHandle hin, int use_cond) {
   if (c->inner_done) return;
   const T alpha = (T)c->alpha, beta = (T)c->beta;
   T mx = 0;
@@ -470,12 +496,23 @@ __global__ void __launch_bounds__(kBlock) k_cg_a(const Geo g, int zpt, uint32_t 
     x[i] += alpha * pv;
     const T rv = r[i] - alpha * sv;
     r[i] = rv;
-    const T dinv = (T)1 / diag_t<T>(m, selfmask);
+    const T dinv = inv_diag<T>(m, selfmask);
     u[i] = rv * dinv;
     mx = fmax(mx, finite_or_inf(fabs(rv) * dinv));
   }
+  // a maximum does not depend on the order: the blocks combine theirs in one
+  // word (the bits of a non-negative double order as an integer), and the
+  // last ticket's thread has no partials to read
   const T v = block_reduce<true, T>(mx);
-  if (flat_tid() == 0) part[S_MAX * nblk + flat_bid()] = (double)v;
+  if (flat_tid() == 0) {
+    atomicMax(&c->max_bits, (unsigned long long)__double_as_longlong((double)v));
+    __threadfence();
+    if (atomicAdd(&c->arrive, 1) == nblk - 1) {
+      const double m = __longlong_as_double((long long)atomicExch(&c->max_bits, 0ULL));
+      c->arrive = 0;
+      cg_test(c, m, eta, tol_abs, maxit, hin, use_cond);
+    }
+  }
 }
 
 // warm start of a step's solve on fluid nodes (fp32::extrapolate_node); the
@@ -495,7 +532,9 @@ __global__ void k_extrapolate(const Geo g, int zpt, const uint32_t *__restrict__
 // unit) on fluid nodes and its float copy; |phi| reaching kPhiMax raises
 // range flag 4
 __global__ void k_correct_fx(const Geo g, int zpt, const uint32_t *__restrict__ mask, const float *__restrict__ e,
-                             int64_t *__restrict__ phifx, float *__restrict__ phi32, int *__restrict__ flag) {
+                             int64_t *__restrict__ phifx, float *__restrict__ phi32, int *__restrict__ flag,
+                             const PoissonCtl *__restrict__ c) {
+  if (c->outer_done) return;  // the round's test had already converged
   constexpr float kMaxFx = (float)(kPhiMax * 281474976710656.0);  // kPhiMax 2^kPhiFixBits
   bool over = false;
   for (int kz = 0; kz < zpt; ++kz) {
@@ -532,7 +571,9 @@ __global__ void k_extrapolate_fx(const Geo g, int zpt, const uint32_t *__restric
 // (the FP64 form, and the linear solves' FP64 iterates)
 template <typename T>
 __global__ void k_correct(const Geo g, int zpt, const uint32_t *__restrict__ mask, const T *__restrict__ e,
-                          double *__restrict__ phi, float *__restrict__ phi32, float *__restrict__ phi_lo) {
+                          double *__restrict__ phi, float *__restrict__ phi32, float *__restrict__ phi_lo,
+                          const PoissonCtl *__restrict__ c) {
+  if (c && c->outer_done) return;  // the round's test had already converged
   for (int kz = 0; kz < zpt; ++kz) {
     int X, Y, Z;
     long long i;
@@ -554,7 +595,7 @@ __global__ void k_correct(const Geo g, int zpt, const uint32_t *__restrict__ mas
 // kernel argument storage for graph nodes (values are copied at node creation)
 struct Args {
   Geo g;
-  int zpt, nblk, maxit, use_cond = 1, mode_init = C_INIT, mode_iter = C_ITER, hin_no = 0, hin_yes = 1;
+  int zpt, nblk, maxit, use_cond = 1;
   Phys P;
   P32 P3;
   uint32_t selfmask;
@@ -663,42 +704,32 @@ cudaError_t build_graph(lbe_handle *h, Args &A, cudaGraphExec_t *exec) {
   cudaGraphNode_t last = nullptr, lo = nullptr, li = nullptr;
   cudaGraph_t body_out = nullptr, body_in = nullptr;
   void *a_reset[] = {&A.c};
-  // the residual before the round loop must not touch the inner loop's
-  // condition (it belongs to the loop body); the one closing a round does
-  void *a_res0[] = {&A.g,     &A.zpt,   &A.P,      &A.P3,    &A.mask,    &A.n64,   &A.nq, &A.rhs,
-                    &A.phi,   &A.phi32, &A.phi_lo, &A.phifx, &A.c6_hi,   &A.c6_lo, &A.r,  &A.u,
-                    &A.x,     &A.p,     &A.s,      &A.part,  &A.nblk,    &A.c,     &A.tol, &A.tol_rel,
-                    &A.maxit, &A.hout,  &A.hin,    &A.use_cond, &A.hin_no};
   void *a_res[] = {&A.g,     &A.zpt,   &A.P,      &A.P3,    &A.mask,    &A.n64,   &A.nq, &A.rhs,
                    &A.phi,   &A.phi32, &A.phi_lo, &A.phifx, &A.c6_hi,   &A.c6_lo, &A.r,  &A.u,
                    &A.x,     &A.p,     &A.s,      &A.part,  &A.nblk,    &A.c,     &A.tol, &A.tol_rel,
-                   &A.maxit, &A.hout,  &A.hin,    &A.use_cond, &A.hin_yes};
-  void *a_bi[] = {&A.g, &A.zpt, &A.selfmask, &A.mask, &A.u, &A.r, &A.w, &A.part, &A.nblk, &A.c,
-                  &A.eta, &A.tol_inner, &A.maxit, &A.mode_init, &A.hin, &A.use_cond};
-  void *a_bt[] = {&A.g, &A.zpt, &A.selfmask, &A.mask, &A.u, &A.r, &A.w, &A.part, &A.nblk, &A.c,
-                  &A.eta, &A.tol_inner, &A.maxit, &A.mode_iter, &A.hin, &A.use_cond};
-  void *a_a[] = {&A.g, &A.zpt, &A.selfmask, &A.mask, &A.x, &A.r, &A.u, &A.w, &A.p, &A.s, &A.part, &A.nblk, &A.c};
-  void *a_cor[] = {&A.g, &A.zpt, &A.mask, &A.x, &A.phi, &A.phi32, &A.phi_lo};
-  void *a_corfx[] = {&A.g, &A.zpt, &A.mask, &A.x, &A.phifx, &A.phi32, &A.flag};
-  // reset -> residual test -> while (not converged) { V-cycle -> CG -> correct
-  // -> residual test }: a converged test ends the solve without running the
-  // rest of a round
+                   &A.maxit, &A.hout,  &A.hin,    &A.use_cond};
+  void *a_b[] = {&A.g, &A.zpt, &A.selfmask, &A.mask, &A.u, &A.r, &A.w, &A.part, &A.nblk, &A.c, &A.hin, &A.use_cond};
+  void *a_a[] = {&A.g, &A.zpt,  &A.selfmask, &A.mask, &A.x,   &A.r,         &A.u,     &A.w,   &A.p,
+                 &A.s, &A.nblk, &A.c,        &A.eta,  &A.tol_inner, &A.maxit, &A.hin, &A.use_cond};
+  void *a_cor[] = {&A.g, &A.zpt, &A.mask, &A.x, &A.phi, &A.phi32, &A.phi_lo, &A.c};
+  void *a_corfx[] = {&A.g, &A.zpt, &A.mask, &A.x, &A.phifx, &A.phi32, &A.flag, &A.c};
+  // reset -> while (not converged) { residual test -> while (CG) { V-cycle ->
+  // stencil and dot products -> update and test } -> correct }.  The residual
+  // test sets both conditions; in the pass where it converges the CG loop is
+  // not entered and the correction returns at once.
   e = cudaGraphConditionalHandleCreate(&A.hout, G, 1, cudaGraphCondAssignDefault);
   if (e == cudaSuccess) e = add_kernel(G, &last, (void *)k_solve_reset, one, one, a_reset);
-  if (e == cudaSuccess) e = add_kernel(G, &last, f_res, L.grid, L.block, a_res0);
   if (e == cudaSuccess) e = add_while(G, &last, A.hout, &body_out);
   if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&A.hin, body_out, 0, 0);
   const bool mg = sizeof(T) == 4 && h->mg.nlev >= 2;
-  if (e == cudaSuccess && mg) e = mg_vcycle(h, (const float *)A.r, (float *)A.u, A.c, body_out, &lo, nullptr);
-  if (e == cudaSuccess) e = add_kernel(body_out, &lo, (void *)k_cg_b<T>, L.grid, L.block, a_bi);
+  if (e == cudaSuccess) e = add_kernel(body_out, &lo, f_res, L.grid, L.block, a_res);
   if (e == cudaSuccess) e = add_while(body_out, &lo, A.hin, &body_in);
-  if (e == cudaSuccess) e = add_kernel(body_in, &li, (void *)k_cg_a<T>, L.grid, L.block, a_a);
   if (e == cudaSuccess && mg) e = mg_vcycle(h, (const float *)A.r, (float *)A.u, A.c, body_in, &li, nullptr);
-  if (e == cudaSuccess) e = add_kernel(body_in, &li, (void *)k_cg_b<T>, L.grid, L.block, a_bt);
+  if (e == cudaSuccess) e = add_kernel(body_in, &li, (void *)k_cg_b<T>, L.grid, L.block, a_b);
+  if (e == cudaSuccess) e = add_kernel(body_in, &li, (void *)k_cg_a<T>, L.grid, L.block, a_a);
   if (e == cudaSuccess)
     e = corr_fx ? add_kernel(body_out, &lo, (void *)k_correct_fx, L.grid, L.block, a_corfx)
                 : add_kernel(body_out, &lo, (void *)k_correct<T>, L.grid, L.block, a_cor);
-  if (e == cudaSuccess) e = add_kernel(body_out, &lo, f_res, L.grid, L.block, a_res);
   if (e == cudaSuccess) e = cudaGraphInstantiate(exec, G, 0);
   cudaGraphDestroy(G);
   return e;
@@ -714,45 +745,41 @@ int solve_polled(lbe_handle *h, Args &A) {
   A.use_cond = 0;
   k_solve_reset<<<1, 1, 0, st>>>(A.c);
   h->launches += 1;
-  for (int round = 0; round <= kMaxOuter; ++round) {
-    {
-      auto kres = A.rhs ? (A.phi32 && A.phi_lo ? k_res<T, R_RHS_FF> : k_res<T, R_RHS>)
-                        : (fixed ? (h->p32.salt11 ? k_res<T, R_FX> : k_res<T, R_FXG>) : k_res<T, R_N64>);
-      kres<<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.P, A.P3, A.mask, A.n64, A.nq, A.rhs, A.phi, A.phi32, A.phi_lo,
-                                        A.phifx, A.c6_hi, A.c6_lo, (T *)A.r, (T *)A.u, (T *)A.x, (T *)A.p,
-                                        (T *)A.s, A.part, A.nblk, A.c, A.tol, A.tol_rel, A.maxit, 0, 0, 0, 0);
-    }
-    const bool mg = sizeof(T) == 4 && h->mg.nlev >= 2;
-    if (mg && mg_vcycle(h, (const float *)A.r, (float *)A.u, A.c, nullptr, nullptr, st) != cudaSuccess)
-      return LBE_ERR_CUDA;
-    k_cg_b<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.selfmask, A.mask, (T *)A.u, (T *)A.r, (T *)A.w, A.part,
-                                           A.nblk, A.c, A.eta, A.tol_inner, A.maxit, C_INIT, 0, 0);
-    h->launches += 2;
+  const bool mg = sizeof(T) == 4 && h->mg.nlev >= 2;
+  auto kres = A.rhs ? (A.phi32 && A.phi_lo ? k_res<T, R_RHS_FF> : k_res<T, R_RHS>)
+                    : (fixed ? (h->p32.salt11 ? k_res<T, R_FX> : k_res<T, R_FXG>) : k_res<T, R_N64>);
+  auto poll = [&]() {
+    cudaError_t e = cudaMemcpyAsync(w.ctl_host, w.ctl, sizeof(PoissonCtl), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) h->err = std::string("poisson: ") + cudaGetErrorString(e);
+    return e;
+  };
+  for (int round = 0; round <= kMaxOuter + 1; ++round) {
+    kres<<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.P, A.P3, A.mask, A.n64, A.nq, A.rhs, A.phi, A.phi32, A.phi_lo,
+                                     A.phifx, A.c6_hi, A.c6_lo, (T *)A.r, (T *)A.u, (T *)A.x, (T *)A.p, (T *)A.s,
+                                     A.part, A.nblk, A.c, A.tol, A.tol_rel, A.maxit, 0, 0, 0);
+    h->launches += 1;
+    if (poll() != cudaSuccess) return LBE_ERR_CUDA;
+    if (w.ctl_host->outer_done) break;
     const long long max_chunks = (long long)A.maxit / kChunk + 2;
-    for (long long ch = 0;; ++ch) {
-      cudaError_t e = cudaMemcpyAsync(w.ctl_host, w.ctl, sizeof(PoissonCtl), cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) {
-        h->err = std::string("poisson: ") + cudaGetErrorString(e);
-        return LBE_ERR_CUDA;
-      }
-      if (w.ctl_host->inner_done || ch >= max_chunks) break;
+    for (long long ch = 0; ch <= max_chunks && !w.ctl_host->inner_done; ++ch) {
       for (int k = 0; k < kChunk; ++k) {
-        k_cg_a<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.selfmask, A.mask, (T *)A.x, (T *)A.r, (T *)A.u,
-                                               (T *)A.w, (T *)A.p, (T *)A.s, A.part, A.nblk, A.c);
         if (mg && mg_vcycle(h, (const float *)A.r, (float *)A.u, A.c, nullptr, nullptr, st) != cudaSuccess)
           return LBE_ERR_CUDA;
-        k_cg_b<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.selfmask, A.mask, (T *)A.u, (T *)A.r, (T *)A.w,
-                                               A.part, A.nblk, A.c, A.eta, A.tol_inner, A.maxit, C_ITER, 0, 0);
+        k_cg_b<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.selfmask, A.mask, (T *)A.u, (T *)A.r, (T *)A.w, A.part,
+                                               A.nblk, A.c, 0, 0);
+        k_cg_a<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.selfmask, A.mask, (T *)A.x, (T *)A.r, (T *)A.u,
+                                               (T *)A.w, (T *)A.p, (T *)A.s, A.nblk, A.c, A.eta,
+                                               A.tol_inner, A.maxit, 0, 0);
       }
       h->launches += 2 * kChunk;
+      if (poll() != cudaSuccess) return LBE_ERR_CUDA;
     }
     if (fixed && !A.rhs)
-      k_correct_fx<<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.mask, (const float *)A.x, A.phifx, A.phi32, A.flag);
+      k_correct_fx<<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.mask, (const float *)A.x, A.phifx, A.phi32, A.flag, A.c);
     else
-      k_correct<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.mask, (const T *)A.x, A.phi, A.phi32, A.phi_lo);
+      k_correct<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.mask, (const T *)A.x, A.phi, A.phi32, A.phi_lo, A.c);
     h->launches += 1;
-    if (w.ctl_host->outer_done) break;
   }
   return cudaGetLastError() == cudaSuccess ? LBE_OK : LBE_ERR_CUDA;
 }
@@ -854,7 +881,7 @@ int poisson_solve_linear(lbe_handle *h, const double *rhs, double *x, double tol
   A.phi32 = x_hi;
   A.phi_lo = x_lo;
   if (x_hi && x_lo) {  // the split of the starting x; the corrections keep it current
-    k_correct<float><<<w.L.grid, w.L.block, 0, h->stream>>>(h->geo, w.L.zpt, h->mask, nullptr, x, x_hi, x_lo);
+    k_correct<float><<<w.L.grid, w.L.block, 0, h->stream>>>(h->geo, w.L.zpt, h->mask, nullptr, x, x_hi, x_lo, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LBE_ERR_CUDA;
   }
   A.tol = tol_abs;
@@ -920,14 +947,12 @@ int poisson_status(lbe_handle *h, lbe_stats *st, long long *kernels) {
     st->poisson_max_iters = (int)(c.solve_iters > c.max_solve_iters ? c.solve_iters : c.max_solve_iters);
     st->poisson_residual = c.res;
   }
-  // kernels of the graph path: reset + per round (residual, stencil,
-  // correct) + per iteration (update, stencil)
   if (kernels && w.graph_ok) {
-    // per solve: reset and the residual tests; per round that ran (every
-    // test but the last of a solve): V-cycle, CG stencil, correction; per
-    // iteration: update, V-cycle, stencil (a V-cycle only with multigrid)
+    // kernels of the graph path: per solve the reset; per residual test the
+    // test and the correction; per iteration V-cycle (with multigrid),
+    // stencil and update
     const long long vc = h->prm.precision == LBE_FP32 ? mg_kernels_per_cycle(h) : 0;
-    *kernels = c.solves + c.total_rounds + (2 + vc) * (c.total_rounds - c.solves) + (2 + vc) * c.total_iters;
+    *kernels = c.solves + 2 * c.total_rounds + (2 + vc) * c.total_iters;
   }
   if (c.sticky_status == LBE_ERR_NOCONVERGE || c.status == LBE_ERR_NOCONVERGE) {
     h->err = "poisson: no convergence within poisson_max_iter";
