@@ -29,41 +29,12 @@
 #include <vector>
 
 #include "fp32_device.cuh"
+#include "march.cuh"
 #include "mg_device.cuh"
 
 constexpr int kBE = LBE_BATCH_MAX_ELECTRODES;  // electrodes per instance
 
 namespace lbe {
-
-// Division of unsigned 32-bit integers by a run-time invariant divisor d >= 1
-// by a multiplication and shifts (Granlund and Montgomery, "Division by
-// invariant integers using multiplication", PLDI 1994, Sec. 4): with
-// l = ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1,
-// q = (t + ((n - t) >> min(l,1))) >> max(l-1,0), t = high word of m n.
-struct FastDiv {
-  uint32_t d, m;
-  int sh1, sh2;
-};
-
-inline FastDiv make_fastdiv(uint32_t d) {
-  int l = 0;
-  while ((1ull << l) < d) ++l;
-  FastDiv f;
-  f.d = d;
-  f.m = (uint32_t)(((((uint64_t)1 << l) - d) << 32) / d + 1);
-  f.sh1 = l < 1 ? l : 1;
-  f.sh2 = l > 1 ? l - 1 : 0;
-  return f;
-}
-
-__host__ __device__ __forceinline__ uint32_t fdiv(const FastDiv &f, uint32_t n) {
-#ifdef __CUDA_ARCH__
-  const uint32_t t = __umulhi(f.m, n);
-#else
-  const uint32_t t = (uint32_t)(((uint64_t)f.m * n) >> 32);
-#endif
-  return (t + ((n - t) >> f.sh1)) >> f.sh2;
-}
 
 // host check of a divisor on the values around every multiple boundary that
 // matters for indices below nmax, and a spread of others

@@ -12,6 +12,7 @@
 //                   paper's Sec. "Lattice Boltzmann Electrokinetics")
 //  * k_charge       induced electrode charge, Eq. Qelec
 #include "lbe_internal.cuh"
+#include "march.cuh"
 
 namespace lbe {
 
@@ -39,6 +40,24 @@ __global__ void k_build_mask(const Geo g, const uint8_t *__restrict__ id, uint32
         if (r2 >= 0 && id[r2] == 0) m |= 1u << corner_bit(sx, sy, sz);
       }
   mask[r] = m;
+}
+
+// Node codes: 6 x the diagonal of -lap_mod (2 per nearest and 1 per
+// next-nearest link, doubled towards solid except under the first-order rule,
+// links of a node to itself left out), bit 7 for a node with a link to solid
+__global__ void k_build_code(const Geo g, uint32_t selfmask, const uint32_t *__restrict__ mask,
+                             uint8_t *__restrict__ code) {
+  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= g.N) return;
+  const uint32_t m = mask[r];
+  const int dbl = (selfmask & kPlainLaplacian) ? 1 : 2;
+  int d = 0;
+#pragma unroll
+  for (int i = 1; i < kQ; ++i) {
+    const uint32_t b = 1u << (i - 1);
+    if (!(selfmask & b)) d += (c2_of(i) == 1 ? 2 : 1) * ((m & b) ? 1 : dbl);
+  }
+  code[r] = !(m & kFluidBit) ? 0 : (uint8_t)(d | ((m & kLinkBits) == kLinkBits ? 0 : kCodeWall));
 }
 
 __global__ void k_init(const Geo g, int ns, const uint8_t *__restrict__ id,
@@ -341,6 +360,11 @@ inline unsigned grid_for(long long N) { return (unsigned)((N + kBlock - 1) / kBl
 
 cudaError_t launch_build_mask(const Geo &g, const uint8_t *id, uint32_t *mask, cudaStream_t s) {
   k_build_mask<<<grid_for(g.N), kBlock, 0, s>>>(g, id, mask);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_build_code(const Geo &g, uint32_t selfmask, const uint32_t *mask, uint8_t *code, cudaStream_t s) {
+  k_build_code<<<grid_for(g.N), kBlock, 0, s>>>(g, selfmask, mask, code);
   return cudaGetLastError();
 }
 

@@ -41,7 +41,7 @@ struct StreamGuard {
 bool fp32(const lbe_handle *h) { return h->prm.precision == LBE_FP32; }
 
 void free_all(lbe_handle *h) {
-  void *ptrs[] = {h->id, h->mask, h->f[0], h->f[1], h->n, h->nstar, h->phi, h->u, h->qpart, h->qout, h->psi_dev,
+  void *ptrs[] = {h->id, h->mask, h->code, h->f[0], h->f[1], h->n, h->nstar, h->phi, h->u, h->qpart, h->qout, h->psi_dev,
                   h->f32[0], h->f32[1], h->q, h->qstar, h->phifx, h->phi32, h->u32, h->flag, h->lf};
   for (void *p : ptrs) cudaFree(p);
   if (h->qhost) cudaFreeHost(h->qhost);
@@ -202,6 +202,7 @@ int lbe_create(const lbe_params *p, void *cuda_stream, lbe_handle **out) {
   const size_t nd = sizeof(double) * (size_t)N, nf = sizeof(float) * (size_t)N;
   alloc((void **)&h->id, (size_t)N);
   alloc((void **)&h->mask, sizeof(uint32_t) * (size_t)N);
+  alloc((void **)&h->code, (size_t)N);
   alloc((void **)&h->phi, nd);
   alloc((void **)&h->psi_dev, sizeof(double) * (LBE_MAX_ELECTRODES + 1));
   if (fp32(h)) {
@@ -275,6 +276,7 @@ int lbe_set_geometry(lbe_handle *h, const uint8_t *node_id, int n_electrodes, in
   }
   LBE_CK(h, cudaMemcpyAsync(h->id, ids.data(), (size_t)g.N, cudaMemcpyHostToDevice, h->stream));
   LBE_CK(h, lbe::launch_build_mask(g, h->id, h->mask, h->stream));
+  LBE_CK(h, lbe::launch_build_code(g, h->phys.selfmask, h->mask, h->code, h->stream));
   if (fp32(h)) LBE_CK(h, lbe::mg_setup(h));  // multigrid preconditioner of the FP32 Poisson solve
   lbe::poisson_drop_graphs(h);               // graphs capture the hierarchy
   LBE_CK(h, cudaStreamSynchronize(h->stream));  // ids is a host vector

@@ -205,7 +205,8 @@ constexpr int kBlock = 256;
 struct PoissonCtl {
   int outer_done, inner_done, rounds, status, sticky_status, arrive;
   int round_iters;  // CG iterations of the current round
-  unsigned long long max_bits;  // max |r|/diag of an update, as the bits of a double
+  unsigned long long max_bits;  // max |r|/diag of a residual or an update, as the bits of a double
+  unsigned long long ref_bits;  // linear solves: max |rhs|/diag likewise
   long long solve_iters, total_iters, total_rounds, solves, max_solve_iters;
   double res, alpha, beta, gamma;
   double ref;  // linear solves: max |rhs|/diag, the scale of the relative test
@@ -250,21 +251,22 @@ static_assert(kHist >= 1 && kHist <= 3, "extrapolation order 1..3");
 #endif
 constexpr int kSolveBlocks = LBE_SOLVE_BLOCKS;
 
-// Multigrid hierarchy of the FP32 Poisson preconditioner (mg.cu); level 0 is
+// Multigrid hierarchy of the Poisson preconditioner (mg.cu); level 0 is
 // the lattice itself.
 constexpr int kMaxLevels = 10;
 struct MGLevel {
   int nx = 0, ny = 0, nz = 0, sx = 0, sy = 0, sz = 0;
   long long N = 0;
-  float *A = nullptr;  // 27-point Galerkin operator [27][N]
-  float *r = nullptr, *e = nullptr, *t = nullptr;
-  float *z = nullptr;  // pre-smoothed iterate omega r/diag
+  // arrays of the form's type (float or double)
+  void *A = nullptr;               // 27-point Galerkin operator [27][N]
+  void *r = nullptr, *e = nullptr;
+  void *z = nullptr;               // pre-smoothed iterate omega r/diag
 };
 struct MGWork {
   MGLevel lv[kMaxLevels];
-  int nlev = 0;        // 0: no hierarchy (Jacobi preconditioning)
-  float *t0 = nullptr;  // fine-level scratch
-  float *cinv = nullptr;  // inverse of the coarsest operator [N][N] (null: Jacobi sweeps)
+  int nlev = 0;          // 0: no hierarchy (Jacobi preconditioning)
+  void *t0 = nullptr;    // the Jacobi vector r/diag of the finest level
+  void *cinv = nullptr;  // inverse of the coarsest operator [N][N] (null: Jacobi sweeps)
 };
 
 struct AdjWork;  // adjoint.cu
@@ -288,6 +290,7 @@ struct lbe_handle {
   // device state
   uint8_t *id = nullptr;
   uint32_t *mask = nullptr;
+  uint8_t *code = nullptr;            // node codes of the solve's kernels (march.cuh)
   double *f[2] = {nullptr, nullptr};  // post-collision populations, [i][r]
   int cur = 0;                        // f[cur] holds the latest populations
   double *n = nullptr;                // [k][r]
@@ -333,6 +336,8 @@ struct lbe_handle {
 namespace lbe {
 // kernels_fp64.cu
 cudaError_t launch_build_mask(const Geo &g, const uint8_t *id, uint32_t *mask, cudaStream_t s);
+// node codes of the solve's kernels (march.cuh) from the link mask
+cudaError_t launch_build_code(const Geo &g, uint32_t selfmask, const uint32_t *mask, uint8_t *code, cudaStream_t s);
 cudaError_t launch_init_state(lbe_handle *h);
 cudaError_t launch_init_phi(lbe_handle *h);
 cudaError_t launch_set_solid_phi(lbe_handle *h);
@@ -383,7 +388,9 @@ void adjoint_free(lbe_handle *h);
 // mg.cu
 cudaError_t mg_setup(lbe_handle *h);
 void mg_free(lbe_handle *h);
-cudaError_t mg_vcycle(lbe_handle *h, const float *r0, float *u0, const PoissonCtl *c, cudaGraph_t gr,
+// u0 = M r0 (vectors of the form's type; uj = r0/diag).  c: skip the work when
+// its inner_done is set (null in a graph, whose loop has ended by then)
+cudaError_t mg_vcycle(lbe_handle *h, const void *r0, const void *uj, void *u0, const PoissonCtl *c, cudaGraph_t gr,
                       cudaGraphNode_t *last, cudaStream_t st);
 int mg_kernels_per_cycle(const lbe_handle *h);
 // FP32 form: the FP64 potential (set by the API) -> the fixed-point master

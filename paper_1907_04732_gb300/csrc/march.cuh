@@ -1,0 +1,176 @@
+// Column-marching launch of the single lattice's finest-level stencil kernels.
+//
+// A thread owns one (x, y) column position of the lattice and walks a chunk
+// of consecutive z planes.  The 19-point Laplacian's link weights are 2
+// (axis) and 1 (diagonal) over 6, so with, per plane, c the value at the
+// column, s the sum of its four in-plane axis neighbours and d that of its
+// four in-plane diagonal ones, the weighted neighbour sum of plane z is
+//   6 sum_l w_l v_l = 2 s(z) + d(z) + T(z-1) + T(z+1),   T = 2 c + s.
+// T(z-1) is carried from plane to plane and plane z+1 becomes the next centre:
+// nine loads and ten additions per node instead of eighteen neighbours, each
+// with its own address and weight.  Every neighbour is read unconditionally:
+// the solve's correction vectors hold zeros on solid nodes (Dirichlet), so no
+// link needs its mask bit, and no load waits for another one.  Measured
+// with the other changes that came with it on the 64x64x256 lattice: see
+// k_cg_b, k_res, k_restrict0 and k_post0.
+//
+// Column positions are flattened (p = x + nx y): a block covers 256
+// consecutive positions, or all positions of a smaller plane for several z
+// chunks, so that a ragged nx leaves no thread idle (a launch tiled over x
+// rounds nx up to a power of two).
+#pragma once
+
+#include "lbe_internal.cuh"
+
+namespace lbe {
+
+// Division of unsigned 32-bit integers by a run-time invariant divisor d >= 1
+// by a multiplication and shifts (Granlund and Montgomery, "Division by
+// invariant integers using multiplication", PLDI 1994, Sec. 4): with
+// l = ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1,
+// q = (t + ((n - t) >> min(l,1))) >> max(l-1,0), t = high word of m n.
+struct FastDiv {
+  uint32_t d, m;
+  int sh1, sh2;
+};
+
+inline FastDiv make_fastdiv(uint32_t d) {
+  int l = 0;
+  while ((1ull << l) < d) ++l;
+  FastDiv f;
+  f.d = d;
+  f.m = (uint32_t)(((((uint64_t)1 << l) - d) << 32) / d + 1);
+  f.sh1 = l < 1 ? l : 1;
+  f.sh2 = l > 1 ? l - 1 : 0;
+  return f;
+}
+
+__host__ __device__ __forceinline__ uint32_t fdiv(const FastDiv &f, uint32_t n) {
+#ifdef __CUDA_ARCH__
+  const uint32_t t = __umulhi(f.m, n);
+#else
+  const uint32_t t = (uint32_t)(((uint64_t)f.m * n) >> 32);
+#endif
+  return (t + ((n - t) >> f.sh1)) >> f.sh2;
+}
+
+// Node codes of the solve's kernels (one byte per node): 6 x the diagonal of
+// -lap_mod at a fluid node (6..48; links of a node to itself left out), bit 7
+// set when one of its 18 links joins a solid node; 0 on solid nodes.
+constexpr int kCodeDiag = 0x7f, kCodeWall = 0x80;
+
+// A lattice cut into columns of K planes
+struct Cols {
+  int nx, ny, nz, plane;  // plane = nx ny
+  int K;                  // planes per thread
+  int selfw;              // 6 x the weights of the links that join a node to itself
+  FastDiv fnx;
+};
+struct ColLaunch {
+  Cols c{};
+  dim3 grid, block;
+  long long nblk() const { return (long long)grid.x * grid.y; }
+};
+
+inline ColLaunch make_cols(const Geo &g, uint32_t selfmask, long long max_blocks) {
+  ColLaunch L;
+  L.c.nx = g.nx;
+  L.c.ny = g.ny;
+  L.c.nz = g.nz;
+  L.c.plane = g.nx * g.ny;
+  L.c.fnx = make_fastdiv((uint32_t)g.nx);
+  L.c.selfw = 0;
+  for (int i = 1; i < kQ; ++i)
+    if (selfmask & (1u << (i - 1))) L.c.selfw += c2_of(i) == 1 ? 2 : 1;
+  const int cb = L.c.plane < 256 ? pow2_at_least(L.c.plane) : 256, zb = 256 / cb;
+  const long long gx = ((long long)L.c.plane + cb - 1) / cb;
+  long long K = 1;
+  auto gy = [&](long long k) { return (g.nz + k * zb - 1) / (k * zb); };
+  while (gx * gy(K) > max_blocks && K < g.nz) ++K;
+  L.c.K = (int)K;
+  L.block = dim3((unsigned)cb, (unsigned)zb);
+  L.grid = dim3((unsigned)gx, (unsigned)gy(K));
+  return L;
+}
+
+// in-plane neighbour offsets of a column, periodic wrap included
+struct PlaneOffs {
+  int xm, xp, ym, yp;
+};
+__device__ __forceinline__ PlaneOffs plane_offs(int nx, int ny, int x, int y) {
+  PlaneOffs o;
+  o.xm = x == 0 ? nx - 1 : -1;
+  o.xp = x == nx - 1 ? 1 - nx : 1;
+  o.ym = y == 0 ? (ny - 1) * nx : -nx;
+  o.yp = y == ny - 1 ? (1 - ny) * nx : nx;
+  return o;
+}
+
+// this thread's column and chunk [z0, z1); false when it has none
+struct Column {
+  int p, x, y, z0, z1;
+  PlaneOffs o;
+};
+__device__ __forceinline__ bool column_of(const Cols &C, Column &c) {
+  c.p = blockIdx.x * blockDim.x + threadIdx.x;
+  c.z0 = (int)(blockIdx.y * blockDim.y + threadIdx.y) * C.K;
+  if (c.p >= C.plane || c.z0 >= C.nz) return false;
+  c.z1 = min(c.z0 + C.K, C.nz);
+  c.y = (int)fdiv(C.fnx, (uint32_t)c.p);
+  c.x = c.p - c.y * C.nx;
+  c.o = plane_offs(C.nx, C.ny, c.x, c.y);
+  return true;
+}
+
+// neighbour offsets of node (column, z) for the per-link forms
+__device__ __forceinline__ Offs col_offs(const PlaneOffs &o, int plane, int nz, int z) {
+  Offs f;
+  f.xm = o.xm;
+  f.xp = o.xp;
+  f.ym = o.ym;
+  f.yp = o.yp;
+  f.zm = z == 0 ? (nz - 1) * plane : -plane;
+  f.zp = z == nz - 1 ? (1 - nz) * plane : plane;
+  return f;
+}
+
+template <typename V>
+__device__ __forceinline__ void plane_sums(const V *v, const PlaneOffs &o, int j, bool diag, V &c, V &s, V &d) {
+  const V *q = v + j;
+  c = q[0];
+  s = (q[o.xm] + q[o.xp]) + (q[o.ym] + q[o.yp]);
+  d = diag ? (q[o.xm + o.ym] + q[o.xp + o.ym]) + (q[o.xm + o.yp] + q[o.xp + o.yp]) : (V)0;
+}
+
+// one column's march over the planes of v
+template <typename V>
+struct ZMarch {
+  V c, s, d, below;  // of the current plane; T of the plane below it
+  int j;             // its node
+  __device__ __forceinline__ void begin(const V *v, const PlaneOffs &o, int p, int plane, int nz, int z) {
+    V c0, s0, d0;
+    j = p + plane * z;
+    plane_sums(v, o, z == 0 ? p + plane * (nz - 1) : j - plane, false, c0, s0, d0);
+    below = 2 * c0 + s0;
+    plane_sums(v, o, j, true, c, s, d);
+  }
+  // 6 sum_l w_l v_l of plane z, then plane z + 1 becomes the current one
+  // (its diagonal sums are read only when it will be a centre: more)
+  __device__ __forceinline__ V step(const V *v, const PlaneOffs &o, int p, int plane, int nz, int z, bool more,
+                                    V &centre, int &at) {
+    const int k = z + 1 == nz ? p : j + plane;
+    V c1, s1, d1;
+    plane_sums(v, o, k, more, c1, s1, d1);
+    const V sum = (2 * s + d) + (below + (2 * c1 + s1));
+    centre = c;
+    at = j;
+    below = 2 * c + s;
+    c = c1;
+    s = s1;
+    d = d1;
+    j = k;
+    return sum;
+  }
+};
+
+}  // namespace lbe

@@ -8,8 +8,8 @@
 //
 // Kernels per V-cycle: the pre-smoothing sweep from zero (e = omega r/diag)
 // is evaluated on the fly where it is needed (restriction, prolongation), so
-// a cycle over levels 0..L is L restrictions, the coarsest solve, L-1 fused
-// prolongation+post-smoothing kernels and two on the finest level.  The
+// a cycle over levels 0..L is L restrictions, the coarsest solve and L fused
+// prolongation+post-smoothing kernels.  The
 // coarsest level is solved exactly (its inverse, formed once on the host)
 // where its operator is positive definite: a weak coarse solve costs CG
 // iterations (on the 64x64x256 electro-osmosis lattice 3.2 per step with 32
@@ -22,6 +22,7 @@
 #include <cmath>
 #include <vector>
 
+#include "march.cuh"
 #include "mg_device.cuh"
 
 namespace lbe {
@@ -41,150 +42,213 @@ __device__ __forceinline__ bool lnode(const MgLevel &L, int &x, int &y, int &z, 
 
 // --- set-up: level-0 inverse diagonal, Galerkin coarse operators -------------
 // level 1 from the fine lattice (mask-defined operator)
+template <typename T>
 __global__ void k_galerkin0(const Geo g, uint32_t selfmask, const uint32_t *__restrict__ mask, const MgLevel C,
-                            float *__restrict__ A) {
+                            T *__restrict__ A) {
   int X, Y, Z, I;
   if (!lnode(C, X, Y, Z, I)) return;
-  float a[27];
+  T a[27];
   galerkin0_row(g, selfmask, mask, C, X, Y, Z, a);
 #pragma unroll
   for (int d = 0; d < 27; ++d) A[d * C.S + I] = a[d];
 }
 
 // level l+1 from level l (27-point)
-__global__ void k_galerkin(const MgLevel F, const float *__restrict__ AF, const MgLevel C, float *__restrict__ A) {
+template <typename T>
+__global__ void k_galerkin(const MgLevel F, const T *__restrict__ AF, const MgLevel C, T *__restrict__ A) {
   int X, Y, Z, I;
   if (!lnode(C, X, Y, Z, I)) return;
-  float a[27];
+  T a[27];
   galerkin_row(F, AF, C, X, Y, Z, a);
 #pragma unroll
   for (int d = 0; d < 27; ++d) A[d * C.S + I] = a[d];
 }
 
 // --- V-cycle kernels ---------------------------------------------------------
-// Restriction with 8 threads per coarse node (one per child) and a fixed-order
-// shuffle sum of the children's pre-smoothed residuals (store_coarse in
-// mg_device.cuh).
-
-// level 1: a fluid child's pre-smoothed residual is r - omega A u, u = r/diag
-// being the Jacobi vector the CG formed.  A block covers a tile of 32 coarse
-// nodes (2^txl along X, the rest along Y; lanes 8k..8k+7 the children of one
-// coarse node, child index = lane % 8 as in child_of) on zpb consecutive
-// coarse planes: coordinates come from the block and lane indices, with no
-// division, and every lane runs the same iterations (the shuffle sum).
-__global__ void __launch_bounds__(256) k_restrict0(const Geo g, uint32_t selfmask, const uint32_t *__restrict__ mask,
-                                                   const float *__restrict__ r, const float *__restrict__ u,
-                                                   const MgLevel C, const float *__restrict__ AC,
-                                                   float *__restrict__ rc, float *__restrict__ zc, int txl, int zpb,
-                                                   const PoissonCtl *c) {
-  if (c->inner_done) return;
-  const int ch = threadIdx.x & 7, j = threadIdx.x >> 3;
-  const int X = (blockIdx.x << txl) + (j & ((1 << txl) - 1));
-  const int Y = blockIdx.y * (32 >> txl) + (j >> txl);
-  for (int kz = 0; kz < zpb; ++kz) {
-    const int Z = blockIdx.z * zpb + kz;
-    const bool own = X < C.nx && Y < C.ny && Z < C.nz;
-    int x, y, z;
-    float v = 0.f;
-    if (own && child_of(C, X, Y, Z, ch, g.nx, g.ny, g.nz, x, y, z)) {
-      const int i = x + g.nx * (y + g.ny * z);
-      const uint32_t m = mask[i];
-      if (m & kFluidBit) {
-        const float s6 = nbsum6(m, selfmask, offsets_of(g, x, y, z), i, u);
-        v = r[i] - kOmega * ((float)diag6(m, selfmask) * u[i] - s6) * (1.f / 6.f);
+// Level 1: a fluid child's pre-smoothed residual is r - omega A u, u = r/diag
+// being the Jacobi vector the CG formed.  A thread marches (march.cuh) a fine
+// column over the planes of Kc coarse ones; a warp covers 2^xl x 2^yl columns
+// (aligned pairs along every halved axis) of 2^zl chunks, so that the
+// children of a coarse node meet in the thread (z) and in two shuffles (x, y),
+// a fixed order.
+struct RestrictMap {
+  int xl, yl, zl;  // lanes 2^xl x 2^yl x 2^zl
+  int wy;          // warps of a block along y (the rest along z)
+  int Kc;          // coarse planes per thread
+};
+template <typename T>
+__global__ void __launch_bounds__(256) k_restrict0(const Cols F, const uint8_t *__restrict__ code,
+                                                   const T *__restrict__ r, const T *__restrict__ u, const MgLevel C,
+                                                   const T *__restrict__ AC, T *__restrict__ rc, T *__restrict__ zc,
+                                                   const RestrictMap M, const PoissonCtl *c) {
+  if (c && c->inner_done) return;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lx = lane & ((1 << M.xl) - 1), ly = (lane >> M.xl) & ((1 << M.yl) - 1), lz = lane >> (M.xl + M.yl);
+  const int x = (blockIdx.x << M.xl) + lx;
+  const int y = ((blockIdx.y * M.wy + w % M.wy) << M.yl) + ly;
+  const int Z0 = ((((blockIdx.z * (8 / M.wy) + w / M.wy) << M.zl) + lz)) * M.Kc;
+  const bool own = x < F.nx && y < F.ny && Z0 < C.nz;
+  const int p = x + F.nx * y;
+  const PlaneOffs o = plane_offs(F.nx, F.ny, x, y);
+  ZMarch<T> m;
+  int z = Z0 << C.sz;
+  const int zend = min((Z0 + M.Kc) << C.sz, F.nz);
+  if (own) m.begin(u, o, p, F.plane, F.nz, z);
+  for (int k = 0; k < M.Kc; ++k) {  // every lane runs the same iterations (the shuffles)
+    const int Z = Z0 + k;
+    T v = 0;
+    if (own && Z < C.nz) {
+      for (int h = 0; h <= C.sz && z < F.nz; ++h, ++z) {
+        T u0;
+        int i;
+        const T nsum = m.step(u, o, p, F.plane, F.nz, z, z + 1 < zend, u0, i);
+        const int cd = code[i];
+        const T res = r[i] - (T)kOmega * ((T)((cd & kCodeDiag) + F.selfw) * u0 - nsum) * (T)(1.0 / 6.0);
+        v += cd ? res : (T)0;
       }
     }
-    v = sum8(v);
-    if (ch == 0 && own) store_coarse(C, X + C.nx * (Y + C.ny * Z), v, AC, rc, zc);
+    if (C.sx) v += __shfl_xor_sync(0xffffffffu, v, 1);
+    if (C.sy) v += __shfl_xor_sync(0xffffffffu, v, 1 << M.xl);
+    if (own && Z < C.nz && !(C.sx & lx & 1) && !(C.sy & ly & 1))
+      store_coarse(C, (x >> C.sx) + C.nx * ((y >> C.sy) + C.ny * Z), v, AC, rc, zc);
   }
 }
 
-__global__ void __launch_bounds__(256) k_restrict(const MgLevel F, const float *__restrict__ AF,
-                                                  const float *__restrict__ r, const float *__restrict__ zf,
-                                                  const MgLevel C, const float *__restrict__ AC,
-                                                  float *__restrict__ rc, float *__restrict__ zc, int txl,
+// Restriction between coarse levels with 8 threads per coarse node (one per
+// child) and a fixed-order shuffle sum of the children's pre-smoothed
+// residuals (store_coarse in mg_device.cuh).  A block covers a tile of 32
+// coarse nodes (2^txl along X, the rest along Y; lanes 8k..8k+7 the children
+// of one coarse node, child index = lane % 8 as in child_of) of one plane:
+// coordinates come from the block and lane indices, with no division.
+template <typename T>
+__global__ void __launch_bounds__(256) k_restrict(const MgLevel F, const T *__restrict__ AF,
+                                                  const T *__restrict__ r, const T *__restrict__ zf,
+                                                  const MgLevel C, const T *__restrict__ AC,
+                                                  T *__restrict__ rc, T *__restrict__ zc, int txl,
                                                   const PoissonCtl *c) {
-  if (c->inner_done) return;
-  // the tile mapping of k_restrict0, one coarse plane per block
+  if (c && c->inner_done) return;
   const int ch = threadIdx.x & 7, j = threadIdx.x >> 3;
   const int X = (blockIdx.x << txl) + (j & ((1 << txl) - 1));
   const int Y = blockIdx.y * (32 >> txl) + (j >> txl), Z = blockIdx.z;
   const bool own = X < C.nx && Y < C.ny;
   int x, y, z;
-  float v = 0.f;
+  T v = 0;
   if (own && child_of(C, X, Y, Z, ch, F.nx, F.ny, F.nz, x, y, z)) v = presmoothed_res_z(F, AF, r, zf, x, y, z);
   v = sum8(v);
   if (ch == 0 && own) store_coarse(C, X + C.nx * (Y + C.ny * Z), v, AC, rc, zc);
 }
 
 // fused prolongation + post-smoothing on a 27-point level
-__global__ void k_post(const MgLevel L, const float *__restrict__ A, const float *__restrict__ r,
-                       const float *__restrict__ z, const MgLevel C, const float *__restrict__ ec,
-                       float *__restrict__ out, const PoissonCtl *c) {
-  if (c->inner_done) return;
+template <typename T>
+__global__ void k_post(const MgLevel L, const T *__restrict__ A, const T *__restrict__ r,
+                       const T *__restrict__ z, const MgLevel C, const T *__restrict__ ec,
+                       T *__restrict__ out, const PoissonCtl *c) {
+  if (c && c->inner_done) return;
   int X, Y, Z, I;
   if (!lnode(L, X, Y, Z, I)) return;
   out[I] = post_value_z(L, A, r, z, C, ec, X, Y, Z);
 }
 
-// level 0: t = omega u + alpha P e_1 (fluid nodes), then
-// u = t + omega (r - A t)/diag
-__global__ void k_prolong0(const Geo g, int zpt, const uint32_t *__restrict__ mask, const float *__restrict__ u,
-                           const MgLevel C, const float *__restrict__ ec, float *__restrict__ t,
-                           const PoissonCtl *c) {
-  if (c->inner_done) return;
-  for (int kz = 0; kz < zpt; ++kz) {
-    int x, y, z;
-    long long il;
-    if (!node_of(g, zpt, kz, x, y, z, il)) continue;
-    const int i = (int)il;
-    t[i] = (mask[i] & kFluidBit) ? fmaf(kAlpha, ec[agg_index(C, x, y, z)], kOmega * u[i]) : 0.f;
+// fused prolongation + post-smoothing on the finest level:
+// t = omega u + alpha P e_1 (fluid nodes), out = t + omega (r - A t)/diag.
+// The neighbour sum of u is marched; that of P e_1 likewise, with the coarse
+// array's offsets (a column's neighbours lie in its own aggregate or the next
+// one) and each coarse plane's sums kept while the fine planes stay in it.
+// Next to a wall, P e_1 is nonzero on the solid neighbours too and the links
+// are taken one by one.
+template <typename T>
+__global__ void __launch_bounds__(256) k_post0(const Cols F, const uint8_t *__restrict__ code,
+                                               const uint32_t *__restrict__ mask, const T *__restrict__ r,
+                                               const T *__restrict__ u, const MgLevel C, const T *__restrict__ ec,
+                                               T *__restrict__ out, const PoissonCtl *c) {
+  if (c && c->inner_done) return;
+  Column col;
+  if (!column_of(F, col)) return;
+  const int X = col.x >> C.sx, Y = col.y >> C.sy, cplane = C.nx * C.ny;
+  PlaneOffs q;  // coarse offsets of the in-plane neighbours' aggregates
+  q.xm = ((col.x + col.o.xm) >> C.sx) - X;
+  q.xp = ((col.x + col.o.xp) >> C.sx) - X;
+  q.ym = C.nx * (((col.y == 0 ? F.ny - 1 : col.y - 1) >> C.sy) - Y);
+  q.yp = C.nx * (((col.y == F.ny - 1 ? 0 : col.y + 1) >> C.sy) - Y);
+  const int P = X + C.nx * Y;
+  const T om = (T)kOmega, al = (T)kAlpha;
+  ZMarch<T> m;
+  m.begin(u, col.o, col.p, F.plane, F.nz, col.z0);
+  int Z = col.z0 >> C.sz;
+  T c0, s0, d0, c1, s1, d1, below;
+  {
+    T cb, sb, db;
+    const int Zb = (col.z0 == 0 ? F.nz - 1 : col.z0 - 1) >> C.sz;
+    plane_sums(ec, q, P + cplane * Zb, false, cb, sb, db);
+    below = 2 * cb + sb;
   }
-}
-
-__global__ void k_post0(const Geo g, int zpt, uint32_t selfmask, const uint32_t *__restrict__ mask,
-                        const float *__restrict__ r, const float *__restrict__ t, float *__restrict__ u,
-                        const PoissonCtl *c) {
-  if (c->inner_done) return;
-  for (int kz = 0; kz < zpt; ++kz) {
-    int x, y, z;
-    long long il;
-    if (!node_of(g, zpt, kz, x, y, z, il)) continue;
-    const int i = (int)il;
-    const uint32_t m = mask[i];
-    if (!(m & kFluidBit)) {
-      u[i] = 0.f;
-      continue;
+  plane_sums(ec, q, P + cplane * Z, true, c0, s0, d0);
+  for (int z = col.z0; z < col.z1; ++z) {
+    T u0;
+    int i;
+    const int Zn = (z + 1 == F.nz ? 0 : z + 1) >> C.sz;
+    if (Zn != Z) {
+      plane_sums(ec, q, P + cplane * Zn, true, c1, s1, d1);
+    } else {
+      c1 = c0;
+      s1 = s0;
+      d1 = d0;
     }
-    const float d6 = (float)diag6(m, selfmask);
-    const float s6 = nbsum6(m, selfmask, offsets_of(g, x, y, z), i, t);
-    const float ti = t[i];
-    u[i] = ti + kOmega * __fdividef(6.f * r[i] - (d6 * ti - s6), d6);
+    const T nu = m.step(u, col.o, col.p, F.plane, F.nz, z, z + 1 < col.z1, u0, i);
+    T ne = (2 * s0 + d0) + (below + (2 * c1 + s1));
+    const int cd = code[i];
+    T v = 0;
+    if (cd) {
+      if (cd & kCodeWall) {
+        const uint32_t mk = mask[i];
+        const int Zm = (z == 0 ? F.nz - 1 : z - 1) >> C.sz;
+        ne = 0;
+#pragma unroll
+        for (int l = 1; l < kQ; ++l) {
+          const int dx = cx_of(l), dy = cy_of(l), dz = cz_of(l);
+          const int a = P + (dx < 0 ? q.xm : (dx > 0 ? q.xp : 0)) + (dy < 0 ? q.ym : (dy > 0 ? q.yp : 0)) +
+                        cplane * (dz < 0 ? Zm : (dz > 0 ? Zn : Z));
+          if (mk & (1u << (l - 1))) ne += (T)(c2_of(l) == 1 ? 2 : 1) * ec[a];
+        }
+      }
+      const T d6 = (T)(cd & kCodeDiag);
+      const T t = om * u0 + al * c0;
+      const T s6 = om * nu + al * ne - (T)F.selfw * t;
+      const T res6 = (T)6 * r[i] - (d6 * t - s6);
+      v = t + om * (sizeof(T) == 4 ? (T)__fdividef((float)res6, (float)d6) : res6 / d6);
+    }
+    out[i] = v;
+    below = 2 * c0 + s0;
+    c0 = c1;
+    s0 = s1;
+    d0 = d1;
+    Z = Zn;
   }
 }
 
 // coarsest level solved exactly: e = A^-1 r with the inverse formed at
 // set-up, one warp per row (a fixed summation order)
-__global__ void __launch_bounds__(256) k_coarse_direct(int N, const float *__restrict__ Ainv,
-                                                       const float *__restrict__ r, float *__restrict__ e,
-                                                       const PoissonCtl *c) {
-  if (c->inner_done) return;
+template <typename T>
+__global__ void __launch_bounds__(256) k_coarse_direct(int N, const T *__restrict__ Ainv, const T *__restrict__ r,
+                                                       T *__restrict__ e, const PoissonCtl *c) {
+  if (c && c->inner_done) return;
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= N) return;
-  const float *a = Ainv + (size_t)row * N;
-  float s = 0.f;
-  for (int j = lane; j < N; j += 32) s = fmaf(a[j], r[j], s);
+  const T *a = Ainv + (size_t)row * N;
+  T s = 0;
+  for (int j = lane; j < N; j += 32) s = fma(a[j], r[j], s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) e[row] = s;
 }
 
 // coarsest level in one block
-__global__ void __launch_bounds__(kCoarseMax) k_coarsest(const MgLevel L, const float *__restrict__ A,
-                                                         const float *__restrict__ r, float *__restrict__ e,
+template <typename T>
+__global__ void __launch_bounds__(kCoarseMax) k_coarsest(const MgLevel L, const T *__restrict__ A,
+                                                         const T *__restrict__ r, T *__restrict__ e,
                                                          const PoissonCtl *c) {
-  if (c->inner_done) return;
-  __shared__ float buf[2][kCoarseMax];
+  if (c && c->inner_done) return;
+  __shared__ T buf[2][kCoarseMax];
   coarsest_solve(L, A, r, e, buf);
 }
 
@@ -200,7 +264,6 @@ MgLevel level_dev(const MGLevel &L) { return MgLevel{L.nx, L.ny, L.nz, L.sx, L.s
 
 }  // namespace
 
-// build the hierarchy for the current geometry (after the link mask)
 // Inverse of the coarsest level's operator from its 27-point rows (host,
 // FP64): the operator restricted to the nodes with a non-zero diagonal
 // (aggregates holding fluid) is assembled densely, factored A = L L^T
@@ -208,25 +271,26 @@ MgLevel level_dev(const MGLevel &L) { return MgLevel{L.nx, L.ny, L.nz, L.sx, L.s
 // as the Jacobi sweeps leave them.  False when the operator is not
 // symmetric positive definite to working accuracy (e.g. a periodic lattice
 // without electrodes, whose operator is singular): the sweeps are used then.
-bool mgd::coarse_inverse(const MgLevel &L, const std::vector<float> &A27, std::vector<float> &inv) {
+template <typename T>
+static bool coarse_inverse_t(const mgd::MgLevel &L, const std::vector<T> &A27, std::vector<T> &inv) {
   const int N = L.N;
   std::vector<int> act;  // active node -> level index
   std::vector<int> pos(N, -1);
   for (int i = 0; i < N; ++i)
-    if (A27[13 * (size_t)N + i] != 0.f) {
+    if (A27[13 * (size_t)N + i] != (T)0) {
       pos[i] = (int)act.size();
       act.push_back(i);
     }
   const int n = (int)act.size();
-  inv.assign((size_t)N * N, 0.f);
+  inv.assign((size_t)N * N, (T)0);
   if (n == 0) return true;
   std::vector<double> M((size_t)n * n, 0.0);
   for (int a = 0; a < n; ++a) {
     const int I = act[a];
     const int X = I % L.nx, Y = (I / L.nx) % L.ny, Z = I / (L.nx * L.ny);
     for (int q = 0; q < 27; ++q) {
-      const float v = A27[(size_t)q * N + I];
-      if (v == 0.f) continue;
+      const T v = A27[(size_t)q * N + I];
+      if (v == (T)0) continue;
       auto wr = [](int c, int m) { return c < 0 ? c + m : (c >= m ? c - m : c); };
       const int J = wr(X + q % 3 - 1, L.nx) + L.nx * (wr(Y + (q / 3) % 3 - 1, L.ny) + L.ny * wr(Z + q / 9 - 1, L.nz));
       if (pos[J] < 0) continue;  // a zero of the correction
@@ -269,12 +333,17 @@ bool mgd::coarse_inverse(const MgLevel &L, const std::vector<float> &A27, std::v
       for (int k = i + 1; k < n; ++k) s -= M[(size_t)k * n + i] * x[k];
       x[i] = s / M[(size_t)i * n + i];
     }
-    for (int i = 0; i < n; ++i) inv[(size_t)act[i] * N + act[cidx]] = (float)x[i];
+    for (int i = 0; i < n; ++i) inv[(size_t)act[i] * N + act[cidx]] = (T)x[i];
   }
   return true;
 }
+bool mgd::coarse_inverse(const MgLevel &L, const std::vector<float> &A27, std::vector<float> &inv) {
+  return coarse_inverse_t(L, A27, inv);
+}
 
-cudaError_t mg_setup(lbe_handle *h) {
+// build the hierarchy for the current geometry (after the link mask)
+template <typename T>
+static cudaError_t mg_setup_t(lbe_handle *h) {
   MGWork &mg = h->mg;
   mg_free(h);
   const Geo &g = h->geo;
@@ -291,13 +360,13 @@ cudaError_t mg_setup(lbe_handle *h) {
     L.sz = shp[l].sz;
     L.N = shp[l].N;
   }
-  cudaError_t e = cudaMalloc(&mg.t0, sizeof(float) * g.N);
+  cudaError_t e = cudaMalloc(&mg.t0, sizeof(T) * g.N);
   for (int l = 1; l < mg.nlev && e == cudaSuccess; ++l) {
     MGLevel &L = mg.lv[l];
-    e = cudaMalloc(&L.A, sizeof(float) * 27 * L.N);
-    if (e == cudaSuccess) e = cudaMalloc(&L.r, sizeof(float) * L.N);
-    if (e == cudaSuccess) e = cudaMalloc(&L.e, sizeof(float) * L.N);
-    if (e == cudaSuccess) e = cudaMalloc(&L.z, sizeof(float) * L.N);
+    e = cudaMalloc(&L.A, sizeof(T) * 27 * L.N);
+    if (e == cudaSuccess) e = cudaMalloc(&L.r, sizeof(T) * L.N);
+    if (e == cudaSuccess) e = cudaMalloc(&L.e, sizeof(T) * L.N);
+    if (e == cudaSuccess) e = cudaMalloc(&L.z, sizeof(T) * L.N);
   }
   if (e != cudaSuccess) {
     mg_free(h);
@@ -308,9 +377,10 @@ cudaError_t mg_setup(lbe_handle *h) {
     dim3 blk;
     const dim3 grd = lgrid(C, blk);
     if (l == 1)
-      k_galerkin0<<<grd, blk, 0, h->stream>>>(g, h->phys.selfmask, h->mask, C, mg.lv[1].A);
+      k_galerkin0<T><<<grd, blk, 0, h->stream>>>(g, h->phys.selfmask, h->mask, C, (T *)mg.lv[1].A);
     else
-      k_galerkin<<<grd, blk, 0, h->stream>>>(level_dev(mg.lv[l - 1]), mg.lv[l - 1].A, C, mg.lv[l].A);
+      k_galerkin<T><<<grd, blk, 0, h->stream>>>(level_dev(mg.lv[l - 1]), (const T *)mg.lv[l - 1].A, C,
+                                                (T *)mg.lv[l].A);
   }
   cudaError_t le = cudaGetLastError();
   if (le != cudaSuccess) return le;
@@ -319,20 +389,21 @@ cudaError_t mg_setup(lbe_handle *h) {
   const char *denv = getenv("LBE_MG_DIRECT");
   if (!(denv && denv[0] == '0')) {
     const MGLevel &Lc = mg.lv[mg.nlev - 1];
-    std::vector<float> a27((size_t)27 * Lc.N), inv;
-    le = cudaMemcpyAsync(a27.data(), Lc.A, sizeof(float) * a27.size(), cudaMemcpyDeviceToHost, h->stream);
+    std::vector<T> a27((size_t)27 * Lc.N), inv;
+    le = cudaMemcpyAsync(a27.data(), Lc.A, sizeof(T) * a27.size(), cudaMemcpyDeviceToHost, h->stream);
     if (le == cudaSuccess) le = cudaStreamSynchronize(h->stream);
     if (le != cudaSuccess) return le;
-    if (coarse_inverse(level_dev(Lc), a27, inv)) {
-      le = cudaMalloc(&mg.cinv, sizeof(float) * inv.size());
+    if (coarse_inverse_t(level_dev(Lc), a27, inv)) {
+      le = cudaMalloc(&mg.cinv, sizeof(T) * inv.size());
       if (le == cudaSuccess)
-        le = cudaMemcpyAsync(mg.cinv, inv.data(), sizeof(float) * inv.size(), cudaMemcpyHostToDevice, h->stream);
+        le = cudaMemcpyAsync(mg.cinv, inv.data(), sizeof(T) * inv.size(), cudaMemcpyHostToDevice, h->stream);
       if (le == cudaSuccess) le = cudaStreamSynchronize(h->stream);  // inv is released on return
       if (le != cudaSuccess) return le;
     }
   }
   return cudaSuccess;
 }
+cudaError_t mg_setup(lbe_handle *h) { return mg_setup_t<float>(h); }
 
 void mg_free(lbe_handle *h) {
   MGWork &mg = h->mg;
@@ -340,7 +411,6 @@ void mg_free(lbe_handle *h) {
     cudaFree(mg.lv[l].A);
     cudaFree(mg.lv[l].r);
     cudaFree(mg.lv[l].e);
-    cudaFree(mg.lv[l].t);
     cudaFree(mg.lv[l].z);
   }
   cudaFree(mg.t0);
@@ -350,15 +420,13 @@ void mg_free(lbe_handle *h) {
 
 // u = M r as a sequence of kernels, either launched on the stream or added to
 // a graph (gr != nullptr) after *last
-cudaError_t mg_vcycle(lbe_handle *h, const float *r0, float *u0, const PoissonCtl *c, cudaGraph_t gr,
-                      cudaGraphNode_t *last, cudaStream_t st) {
+template <typename T>
+static cudaError_t mg_vcycle_t(lbe_handle *h, const void *r0, const void *uj, void *u0, const PoissonCtl *c,
+                               cudaGraph_t gr, cudaGraphNode_t *last, cudaStream_t st) {
   MGWork &mg = h->mg;
   const int nl = mg.nlev;
-  const Geo g = h->geo;
-  // finest-level kernels: the solve's launch (zpt nodes along z per thread)
-  const Launch L0 = h->pw.L;
-  int zpt0 = L0.zpt;
-  const uint32_t sm = h->phys.selfmask;
+  // finest-level kernels: the solve's launch
+  ColLaunch L0 = make_cols(h->geo, h->phys.selfmask, kSolveBlocks);
   // kernel arguments live in these arrays until the nodes are created or the
   // kernels launched
   struct Node {
@@ -375,49 +443,59 @@ cudaError_t mg_vcycle(lbe_handle *h, const float *r0, float *u0, const PoissonCt
     return &ptr.back();
   };
   for (int l = 1; l < nl; ++l) lv[l] = level_dev(mg.lv[l]);
-  const void *pg = &g, *psm = &sm;
   // down: restrictions (pre-smoothing on the fly)
-  // restrictions: tiles of 32 coarse nodes per block, 2^txl along X (at
-  // most 32) and the rest along Y; level 1 with zpb coarse planes per block
-  // (at most kSolveBlocks blocks), the others one plane per block
-  int txl[kMaxLevels];
-  dim3 rgrid[kMaxLevels];
-  for (int l = 1; l < nl; ++l) {
-    txl[l] = 0;
-    while ((1 << txl[l]) < mg.lv[l].nx && txl[l] < 5) ++txl[l];
-    rgrid[l] = dim3((unsigned)((mg.lv[l].nx + (1 << txl[l]) - 1) >> txl[l]),
-                    (unsigned)((mg.lv[l].ny + (32 >> txl[l]) - 1) / (32 >> txl[l])), (unsigned)mg.lv[l].nz);
+  // level 1: lanes along x, a pair of rows, the rest along z; at most
+  // kSolveBlocks blocks (Kc coarse planes per thread)
+  RestrictMap M;
+  {
+    const int nx = h->geo.nx, ny = h->geo.ny;
+    M.yl = lv[1].sy;
+    M.xl = 0;
+    while ((1 << M.xl) < nx && M.xl < 5 - M.yl) ++M.xl;
+    M.zl = 5 - M.xl - M.yl;
   }
-  int zpb = (int)(((long long)rgrid[1].x * rgrid[1].y * mg.lv[1].nz + kSolveBlocks - 1) / kSolveBlocks);
-  rgrid[1].z = (unsigned)((mg.lv[1].nz + zpb - 1) / zpb);
-  nodes.push_back(Node{(void *)k_restrict0, rgrid[1], dim3(256),
-                       {(void *)pg, (void *)psm, P(h->mask), P(r0), P(u0), &lv[1], P(mg.lv[1].A), P(mg.lv[1].r),
-                        P(mg.lv[1].z), &txl[1], &zpb, P(c)}});
-  for (int l = 1; l < nl - 1; ++l)
-    nodes.push_back(Node{(void *)k_restrict, rgrid[l + 1], dim3(256),
-                         {&lv[l], P(mg.lv[l].A), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1], P(mg.lv[l + 1].A),
-                          P(mg.lv[l + 1].r), P(mg.lv[l + 1].z), &txl[l + 1], P(c)}});
+  const int xt = (h->geo.nx + (1 << M.xl) - 1) >> M.xl, yt = (h->geo.ny + (1 << M.yl) - 1) >> M.yl;
+  M.wy = yt < 8 ? pow2_at_least(yt) : 8;
+  dim3 rg0;
+  for (M.Kc = 1;; ++M.Kc) {
+    const int per = (8 / M.wy) * (M.Kc << M.zl);  // coarse planes per block
+    rg0 = dim3((unsigned)xt, (unsigned)((yt + M.wy - 1) / M.wy), (unsigned)((lv[1].nz + per - 1) / per));
+    if ((long long)rg0.x * rg0.y * rg0.z <= kSolveBlocks || M.Kc >= lv[1].nz) break;
+  }
+  nodes.push_back(Node{(void *)k_restrict0<T>, rg0, dim3(256),
+                       {&L0.c, P(h->code), P(r0), P(uj), &lv[1], P(mg.lv[1].A), P(mg.lv[1].r), P(mg.lv[1].z), &M,
+                        P(c)}});
+  // the others: tiles of 32 coarse nodes per block, 2^txl along X (at most
+  // 32) and the rest along Y, one plane per block
+  int txl[kMaxLevels];
+  for (int l = 1; l < nl - 1; ++l) {
+    const MGLevel &Lc = mg.lv[l + 1];
+    txl[l] = 0;
+    while ((1 << txl[l]) < Lc.nx && txl[l] < 5) ++txl[l];
+    const dim3 rg((unsigned)((Lc.nx + (1 << txl[l]) - 1) >> txl[l]),
+                  (unsigned)((Lc.ny + (32 >> txl[l]) - 1) / (32 >> txl[l])), (unsigned)Lc.nz);
+    nodes.push_back(Node{(void *)k_restrict<T>, rg, dim3(256),
+                         {&lv[l], P(mg.lv[l].A), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1], P(Lc.A), P(Lc.r), P(Lc.z),
+                          &txl[l], P(c)}});
+  }
   // coarsest: exact (inverse) or Jacobi sweeps
   int ncoarse = (int)mg.lv[nl - 1].N;
   if (mg.cinv)
-    nodes.push_back(Node{(void *)k_coarse_direct, dim3((unsigned)((ncoarse + 7) / 8)), dim3(256),
+    nodes.push_back(Node{(void *)k_coarse_direct<T>, dim3((unsigned)((ncoarse + 7) / 8)), dim3(256),
                          {&ncoarse, P(mg.cinv), P(mg.lv[nl - 1].r), P(mg.lv[nl - 1].e), P(c)}});
   else
-    nodes.push_back(Node{(void *)k_coarsest, dim3(1), dim3(kCoarseMax),
+    nodes.push_back(Node{(void *)k_coarsest<T>, dim3(1), dim3(kCoarseMax),
                          {&lv[nl - 1], P(mg.lv[nl - 1].A), P(mg.lv[nl - 1].r), P(mg.lv[nl - 1].e), P(c)}});
-  // up: fused prolongation + post-smoothing on the coarse levels
+  // up: fused prolongation + post-smoothing
   for (int l = nl - 2; l >= 1; --l) {
     dim3 blk;
     const dim3 grd = lgrid(lv[l], blk);
-    nodes.push_back(Node{(void *)k_post, grd, blk,
+    nodes.push_back(Node{(void *)k_post<T>, grd, blk,
                          {&lv[l], P(mg.lv[l].A), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1], P(mg.lv[l + 1].e),
                           P(mg.lv[l].e), P(c)}});
   }
-  // finest level
-  nodes.push_back(Node{(void *)k_prolong0, L0.grid, L0.block,
-                       {(void *)pg, &zpt0, P(h->mask), P(u0), &lv[1], P(mg.lv[1].e), P(mg.t0), P(c)}});
-  nodes.push_back(Node{(void *)k_post0, L0.grid, L0.block,
-                       {(void *)pg, &zpt0, (void *)psm, P(h->mask), P(r0), P(mg.t0), P(u0), P(c)}});
+  nodes.push_back(Node{(void *)k_post0<T>, L0.grid, L0.block,
+                       {&L0.c, P(h->code), P(h->mask), P(r0), P(uj), &lv[1], P(mg.lv[1].e), P(u0), P(c)}});
   cudaError_t e = cudaSuccess;
   for (Node &n : nodes) {
     if (gr) {
@@ -439,8 +517,12 @@ cudaError_t mg_vcycle(lbe_handle *h, const float *r0, float *u0, const PoissonCt
   }
   return e;
 }
+cudaError_t mg_vcycle(lbe_handle *h, const void *r0, const void *uj, void *u0, const PoissonCtl *c, cudaGraph_t gr,
+                      cudaGraphNode_t *last, cudaStream_t st) {
+  return mg_vcycle_t<float>(h, r0, uj, u0, c, gr, last, st);
+}
 
 // kernels of one V-cycle (launch accounting of the graph path)
-int mg_kernels_per_cycle(const lbe_handle *h) { return h->mg.nlev >= 2 ? 2 * (h->mg.nlev - 1) + 2 : 0; }
+int mg_kernels_per_cycle(const lbe_handle *h) { return h->mg.nlev >= 2 ? 2 * (h->mg.nlev - 1) + 1 : 0; }
 
 }  // namespace lbe

@@ -122,23 +122,24 @@ __device__ __forceinline__ bool child_of(const MgLevel &C, int X, int Y, int Z, 
 // --- set-up ------------------------------------------------------------------
 // Galerkin row of coarse node (X,Y,Z) of level 1 from the fine lattice
 // (mask-defined operator); mask points at the lattice's node 0
+template <typename T>
 __device__ __forceinline__ void galerkin0_row(const Geo &g, uint32_t selfmask, const uint32_t *__restrict__ mask,
-                                              const MgLevel &C, int X, int Y, int Z, float a[27]) {
+                                              const MgLevel &C, int X, int Y, int Z, T a[27]) {
 #pragma unroll
-  for (int d = 0; d < 27; ++d) a[d] = 0.f;
+  for (int d = 0; d < 27; ++d) a[d] = 0;
   for (int c = 0; c < 8; ++c) {
     int x, y, z;
     if (!child_of(C, X, Y, Z, c, g.nx, g.ny, g.nz, x, y, z)) continue;
     const int i = x + g.nx * (y + g.ny * z);
     const uint32_t m = mask[i];
     if (!(m & kFluidBit)) continue;
-    float diag = 0.f;
+    T diag = 0;
     for (int l = 1; l < kQ; ++l) {
       const uint32_t b = 1u << (l - 1);
       if (selfmask & b) continue;
-      const float w = (float)lapc_of(l);
-      if (!(m & b)) {  // link to solid: doubled, Dirichlet
-        diag += 2.f * w;
+      const T w = (T)lapc_of(l);
+      if (!(m & b)) {  // link to solid: doubled (not under the first-order rule), Dirichlet
+        diag += (selfmask & kPlainLaplacian) ? w : 2 * w;
         continue;
       }
       diag += w;
@@ -151,18 +152,19 @@ __device__ __forceinline__ void galerkin0_row(const Geo &g, uint32_t selfmask, c
 }
 
 // Galerkin row of coarse node (X,Y,Z) of level l+1 from level l (27-point)
-__device__ __forceinline__ void galerkin_row(const MgLevel &F, const float *__restrict__ AF, const MgLevel &C, int X,
-                                             int Y, int Z, float a[27]) {
+template <typename T>
+__device__ __forceinline__ void galerkin_row(const MgLevel &F, const T *__restrict__ AF, const MgLevel &C, int X,
+                                             int Y, int Z, T a[27]) {
 #pragma unroll
-  for (int d = 0; d < 27; ++d) a[d] = 0.f;
+  for (int d = 0; d < 27; ++d) a[d] = 0;
   for (int c = 0; c < 8; ++c) {
     int x, y, z;
     if (!child_of(C, X, Y, Z, c, F.nx, F.ny, F.nz, x, y, z)) continue;
     const int i = x + F.nx * (y + F.ny * z);
-    if (AF[13 * F.S + i] == 0.f) continue;  // inactive node
+    if (AF[13 * F.S + i] == (T)0) continue;  // inactive node
     for (int d = 0; d < 27; ++d) {
-      const float v = AF[d * F.S + i];
-      if (v == 0.f) continue;
+      const T v = AF[d * F.S + i];
+      if (v == (T)0) continue;
       const int jx = wrap(x + d % 3 - 1, F.nx), jy = wrap(y + (d / 3) % 3 - 1, F.ny), jz = wrap(z + d / 9 - 1, F.nz);
       const int dx = rel(jx >> C.sx, X, C.nx), dy = rel(jy >> C.sy, Y, C.ny), dz = rel(jz >> C.sz, Z, C.nz);
       a[d27(dx, dy, dz)] += v;
@@ -171,7 +173,8 @@ __device__ __forceinline__ void galerkin_row(const MgLevel &F, const float *__re
 }
 
 // --- V-cycle -----------------------------------------------------------------
-__device__ __forceinline__ float sum8(float v) {
+template <typename T>
+__device__ __forceinline__ T sum8(T v) {
   v += __shfl_xor_sync(0xffffffffu, v, 1);
   v += __shfl_xor_sync(0xffffffffu, v, 2);
   v += __shfl_xor_sync(0xffffffffu, v, 4);
@@ -180,12 +183,13 @@ __device__ __forceinline__ float sum8(float v) {
 
 // coarsest level: kCoarseSweeps weighted Jacobi sweeps from zero by one
 // block of kCoarseMax threads, one node per thread, iterates in buf
-__device__ __forceinline__ void coarsest_solve(const MgLevel &L, const float *__restrict__ A,
-                                               const float *__restrict__ r, float *__restrict__ e,
-                                               float (*buf)[kCoarseMax]) {
+template <typename T>
+__device__ __forceinline__ void coarsest_solve(const MgLevel &L, const T *__restrict__ A,
+                                               const T *__restrict__ r, T *__restrict__ e,
+                                               T (*buf)[kCoarseMax]) {
   const int I = threadIdx.x;
   const bool own = I < L.N;
-  float d = 0.f, ri = 0.f, a[27];
+  T d = 0, ri = 0, a[27];
   int nb[27];
   if (own) {
     int X, Y, Z;
@@ -198,16 +202,16 @@ __device__ __forceinline__ void coarsest_solve(const MgLevel &L, const float *__
       const int jx = wrap(X + q % 3 - 1, L.nx), jy = wrap(Y + (q / 3) % 3 - 1, L.ny), jz = wrap(Z + q / 9 - 1, L.nz);
       nb[q] = jx + L.nx * (jy + L.ny * jz);
     }
-    buf[0][I] = d != 0.f ? kOmega * ri / d : 0.f;
+    buf[0][I] = d != (T)0 ? kOmega * ri / d : (T)0;
   }
   __syncthreads();
   int cur = 0;
   for (int s = 1; s < kCoarseSweeps; ++s) {
     if (own) {
-      float acc = 0.f;
+      T acc = 0;
 #pragma unroll
       for (int q = 0; q < 27; ++q) acc += a[q] * buf[cur][nb[q]];
-      buf[cur ^ 1][I] = d != 0.f ? buf[cur][I] + kOmega * (ri - acc) / d : 0.f;
+      buf[cur ^ 1][I] = d != (T)0 ? buf[cur][I] + kOmega * (ri - acc) / d : (T)0;
     }
     __syncthreads();
     cur ^= 1;
@@ -218,11 +222,12 @@ __device__ __forceinline__ void coarsest_solve(const MgLevel &L, const float *__
 
 // a coarse node's restricted residual rc and pre-smoothed iterate
 // zc = omega rc/diag
-__device__ __forceinline__ void store_coarse(const MgLevel &C, int I, float v, const float *__restrict__ AC,
-                                             float *__restrict__ rc, float *__restrict__ zc) {
-  const float d = AC[13 * C.S + I];
+template <typename T>
+__device__ __forceinline__ void store_coarse(const MgLevel &C, int I, T v, const T *__restrict__ AC,
+                                             T *__restrict__ rc, T *__restrict__ zc) {
+  const T d = AC[13 * C.S + I];
   rc[I] = v;
-  zc[I] = d != 0.f ? kOmega * v / d : 0.f;
+  zc[I] = d != (T)0 ? kOmega * v / d : (T)0;
 }
 
 // --- forms with integer link weights and a stored pre-smoothed iterate -------
@@ -274,38 +279,40 @@ __device__ __forceinline__ float nbsum6(uint32_t m, uint32_t selfmask, const Off
 
 // residual of a 27-point level after pre-smoothing, the pre-smoothed iterate
 // z = omega r/diag being stored: r - A z at (X,Y,Z)
-__device__ __forceinline__ float presmoothed_res_z(const MgLevel &L, const float *__restrict__ A,
-                                                   const float *__restrict__ r, const float *__restrict__ z, int X,
-                                                   int Y, int Z) {
+template <typename T>
+__device__ __forceinline__ T presmoothed_res_z(const MgLevel &L, const T *__restrict__ A,
+                                               const T *__restrict__ r, const T *__restrict__ z, int X,
+                                               int Y, int Z) {
   const int I = X + L.nx * (Y + L.ny * Z);
-  if (A[13 * L.S + I] == 0.f) return 0.f;
-  float s = 0.f;
+  if (A[13 * L.S + I] == (T)0) return (T)0;
+  T s = 0;
 #pragma unroll
   for (int d = 0; d < 27; ++d) {  // a zero coefficient adds nothing; no branch
-    const float a = A[d * L.S + I];
+    const T a = A[d * L.S + I];
     const int jx = wrap(X + d % 3 - 1, L.nx), jy = wrap(Y + (d / 3) % 3 - 1, L.ny), jz = wrap(Z + d / 9 - 1, L.nz);
-    s = fmaf(a, z[jx + L.nx * (jy + L.ny * jz)], s);
+    s = fma(a, z[jx + L.nx * (jy + L.ny * jz)], s);
   }
   return r[I] - s;
 }
 
 // fused prolongation + post-smoothing with the stored iterate:
 // e = z + alpha P e_c, out = e + omega (r - A e)/diag
-__device__ __forceinline__ float post_value_z(const MgLevel &L, const float *__restrict__ A,
-                                             const float *__restrict__ r, const float *__restrict__ z,
-                                             const MgLevel &C, const float *__restrict__ ec, int X, int Y, int Z) {
+template <typename T>
+__device__ __forceinline__ T post_value_z(const MgLevel &L, const T *__restrict__ A,
+                                          const T *__restrict__ r, const T *__restrict__ z,
+                                          const MgLevel &C, const T *__restrict__ ec, int X, int Y, int Z) {
   const int I = X + L.nx * (Y + L.ny * Z);
-  const float d = A[13 * L.S + I];
-  if (d == 0.f) return 0.f;
-  float s = 0.f;
+  const T d = A[13 * L.S + I];
+  if (d == (T)0) return (T)0;
+  T s = 0;
 #pragma unroll
   for (int q = 0; q < 27; ++q) {  // a zero coefficient adds nothing; no branch
-    const float a = A[q * L.S + I];
+    const T a = A[q * L.S + I];
     const int jx = wrap(X + q % 3 - 1, L.nx), jy = wrap(Y + (q / 3) % 3 - 1, L.ny), jz = wrap(Z + q / 9 - 1, L.nz);
-    const float ej = fmaf(kAlpha, ec[agg_index(C, jx, jy, jz)], z[jx + L.nx * (jy + L.ny * jz)]);
-    s = fmaf(a, ej, s);
+    const T ej = fma((T)kAlpha, ec[agg_index(C, jx, jy, jz)], z[jx + L.nx * (jy + L.ny * jz)]);
+    s = fma(a, ej, s);
   }
-  const float e = fmaf(kAlpha, ec[agg_index(C, X, Y, Z)], z[I]);
+  const T e = fma((T)kAlpha, ec[agg_index(C, X, Y, Z)], z[I]);
   return e + kOmega * (r[I] - s) / d;
 }
 

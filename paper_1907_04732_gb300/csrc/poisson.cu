@@ -33,7 +33,11 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "fp32_device.cuh"
+#include "march.cuh"
 
 namespace lbe {
 
@@ -42,32 +46,11 @@ namespace {
 constexpr int kMaxOuter = 24;  // refinement rounds per solve
 constexpr int kChunk = 16;     // fallback: iterations between host polls
 
-enum { S_RU = 0, S_WU = 1, S_MAX = 2 };
+enum { S_RU = 0, S_WU = 1 };
 
-__host__ __device__ constexpr uint32_t nn_bits() {
-  uint32_t b = 0;
-  for (int i = 1; i < kQ; ++i)
-    if (c2_of(i) == 1) b |= 1u << (i - 1);
-  return b;
-}
-constexpr uint32_t kNN = nn_bits();
-constexpr uint32_t kNNN = ((1u << 18) - 1) & ~kNN;
-
-// diagonal of -lap_mod at a fluid node: 1/3 per nearest and 1/6 per
-// next-nearest link, doubled towards solid (not under the first-order rule,
-// kPlainLaplacian); links joining a node to itself (boxes one node wide)
-// cancel and are left out.
-template <typename T>
-__device__ __forceinline__ T diag_t(uint32_t m, uint32_t selfmask) {
-  const uint32_t nself = ~selfmask;
-  const int dbl = (selfmask & kPlainLaplacian) ? 0 : 1;
-  const int nn = __popc(kNN & nself), nns = dbl * __popc(kNN & nself & ~m);
-  const int mm = __popc(kNNN & nself), mms = dbl * __popc(kNNN & nself & ~m);
-  return (T)(2 * (nn + nns) + (mm + mms)) * (T)(1.0 / 6.0);
-}
-
-// 1/diag.  A double division takes a dozen instructions on the narrow FP64
-// pipe; the diagonal is an integer over 6, so its inverses are a table.
+// 1/diag from a node's code (6 diag; 0 on a solid node, as its inverse).  A
+// double division takes a dozen instructions on the narrow FP64 pipe, so the
+// FP64 form reads the inverses from a table.
 struct InvDiag {
   double v[49];
   constexpr InvDiag() : v() {
@@ -76,22 +59,18 @@ struct InvDiag {
 };
 __constant__ InvDiag kInvDiag = InvDiag();
 template <typename T>
-__device__ __forceinline__ T inv_diag(uint32_t m, uint32_t selfmask) {
-  if (sizeof(T) == 4) return (T)1 / diag_t<T>(m, selfmask);
-  const uint32_t nself = ~selfmask;
-  const int dbl = (selfmask & kPlainLaplacian) ? 0 : 1;
-  const int nn = __popc(kNN & nself), nns = dbl * __popc(kNN & nself & ~m);
-  const int mm = __popc(kNNN & nself), mms = dbl * __popc(kNNN & nself & ~m);
-  return (T)kInvDiag.v[2 * (nn + nns) + (mm + mms)];
+__device__ __forceinline__ T inv_diag(int code) {
+  const int d6 = code & kCodeDiag;
+  if (sizeof(T) == 8) return (T)kInvDiag.v[d6];
+  return (T)(d6 ? 1.f / ((float)d6 * (1.f / 6.f)) : 0.f);
 }
 
 // lap_mod(v)(r) at a fluid node, FP64.  With the link weights scaled by 6
 // (2 nearest, 1 next-nearest, doubled towards solid unless dbl is false:
 // the first-order rule) the sum needs one FP64 add per link:
 // 6 lap = sum_i w_i v_i - (sum_i w_i) v0, w_i in {1, 2, 4}.
-__device__ __forceinline__ double lap_at(const Geo &g, int r, int x, int y, int z, uint32_t m,
-                                         const double *__restrict__ v, bool dbl = true) {
-  const Offs o = offsets_of(g, x, y, z);
+__device__ __forceinline__ double lap_at(const Offs &o, int r, uint32_t m, const double *__restrict__ v,
+                                         bool dbl = true) {
   double s1 = 0.0, s2 = 0.0, s4 = 0.0;
   int wsum = 0;
 #pragma unroll
@@ -297,160 +276,172 @@ __global__ void k_solve_reset(PoissonCtl *c) {
   c->solves += 1;
 }
 
-// Residual of the current potential; seeds the inner solve:
-// r = (T)res, u = r/diag, x = p = s = 0.  Partial max |res|/diag.
+// Residual of the current potential; seeds the inner solve: r = (T)res,
+// uj = r/diag (the CG's first update writes x, p and s).  max |res|/diag by
+// atomicMax on its bits; the last block runs the outer test.
 // MODE: R_N64 the FP64 form (FP64 potential and n); R_FX the FP32 form for
 // a 1:1 salt: the fixed-point potential's Laplacian summed exactly in
 // integers, the charge term from the fixed-point solute, both combined in
 // float-float arithmetic; R_FXG the FP32 form for other salts (the exact
 // Laplacian and the charge density in FP64); R_RHS a given rhs (linear
 // solve A x = rhs with an FP64 iterate; its relative test also needs
-// max |rhs|/diag, kept in the otherwise idle (r,u) partial slots); R_RHS_FF
-// the same in float-float arithmetic (rhs values that are floats, x held as
-// two floats).
+// max |rhs|/diag); R_RHS_FF the same in float-float arithmetic (rhs values
+// that are floats, x held as two floats).
+// The potential of R_N64, R_FX and R_FXG is marched plane by plane
+// (march.cuh) where a node's links all join fluid (their weights are then
+// constants and integer sums do not depend on the order); a node next to a
+// wall takes the per-link form.
 enum { R_N64 = 0, R_FXG = 1, R_RHS = 2, R_FX = 3, R_RHS_FF = 4 };
+struct ResArgs {
+  Cols cols;
+  Geo g;
+  Phys P;
+  P32 P3;
+  const uint8_t *code;
+  const uint32_t *mask;
+  const double *n64;
+  const int64_t *nq;
+  const double *rhs;
+  const double *phi;
+  const float *phi_hi, *phi_lo;
+  const int64_t *phifx;
+  float c6_hi, c6_lo;
+  int nblk, maxit, use_cond;
+  PoissonCtl *c;
+  double tol, tol_rel;
+  cudaGraphConditionalHandle hout, hin;
+};
 template <typename T, int MODE>
-__global__ void __launch_bounds__(kBlock) k_res(const Geo g, int zpt, const Phys P, const P32 P3,
-                                                const uint32_t *__restrict__ mask, const double *__restrict__ n64,
-                                                const int64_t *__restrict__ nq, const double *__restrict__ rhs,
-                                                const double *__restrict__ phi, const float *__restrict__ phi_hi,
-                                                const float *__restrict__ phi_lo, const int64_t *__restrict__ phifx,
-                                                float c6_hi, float c6_lo,
-                                                T *__restrict__ r,
-                                                T *__restrict__ u, T *__restrict__ x, T *__restrict__ p,
-                                                T *__restrict__ s, double *__restrict__ part, int nblk,
-                                                PoissonCtl *c, double tol, double tol_rel, int maxit,
-                                                cudaGraphConditionalHandle hout, cudaGraphConditionalHandle hin,
-                                                int use_cond) {
+__global__ void __launch_bounds__(kBlock) k_res(const ResArgs A, T *__restrict__ r, T *__restrict__ uj) {
   constexpr bool RHS = MODE == R_RHS || MODE == R_RHS_FF;
+  constexpr bool MARCH = MODE == R_FX || MODE == R_FXG || MODE == R_N64;
+  using V = typename std::conditional<MODE == R_N64, double, long long>::type;
+  const V *v = MODE == R_N64 ? (const V *)A.phi : (const V *)A.phifx;
   float mx = 0.f, mb = 0.f;
-  for (int kz = 0; kz < zpt; ++kz) {
-    int X, Y, Z;
-    long long i;
-    if (!node_of(g, zpt, kz, X, Y, Z, i)) continue;
-    const uint32_t m = mask[i];
-    if (!(m & kFluidBit)) {
-      r[i] = u[i] = x[i] = p[i] = s[i] = (T)0;
-      continue;
+  Column c;
+  if (column_of(A.cols, c)) {
+    const int plane = A.cols.plane, nz = A.cols.nz;
+    ZMarch<V> m;
+    if (MARCH) m.begin(v, c.o, c.p, plane, nz, c.z0);
+    for (int z = c.z0; z < c.z1; ++z) {
+      V v0 = 0, nsum = 0;
+      int i = c.p + plane * z;
+      if (MARCH) nsum = m.step(v, c.o, c.p, plane, nz, z, z + 1 < c.z1, v0, i);
+      const int code = A.code[i];
+      if (!code) {
+        r[i] = uj[i] = (T)0;
+        continue;
+      }
+      const bool wall = code & kCodeWall;
+      const uint32_t mk = wall || !MARCH ? A.mask[i] : kLinkBits;
+      T rt, dinv;
+      if (MODE == R_FX || MODE == R_RHS_FF) {
+        float S, E, B, Be;
+        if (MODE == R_FX) {
+          // 6 res = 6 lap + 6 (4 pi l_B s) (q+ - q-): 6 lap exact in fixed
+          // point, split into float-float (the nearest float of the integer
+          // sum and the float of its exact remainder), the charge term in
+          // float-float too
+          const long long L6 = wall ? fp32::lap6_fx_<false>(col_offs(c.o, plane, nz, z), i, mk, A.phifx)
+                                    : (long long)(nsum - 24 * v0);
+          const float Lh = fp32::ll2f(L6);
+          const float Ll = fp32::ll2f(L6 - fp32::f2ll_rn(Lh));
+          S = __fmul_rn(Lh, fp32::kPhiUnitF);
+          E = __fmul_rn(Ll, fp32::kPhiUnitF);
+          const long long dq = A.nq[i] - A.nq[A.g.N + i];
+          const float dq_hi = fp32::ll2f(dq);
+          const float dq_lo = fp32::ll2f(dq - fp32::f2ll_rn(dq_hi));  // exact remainder
+          B = A.c6_hi * dq_hi;
+          Be = fmaf(A.c6_hi, dq_hi, -B) + (A.c6_hi * dq_lo + A.c6_lo * dq_hi);  // product error and tails
+        } else {
+          // 6 res = 6 rhs + 6 lap(x), x = hi + lo, in float-float; rhs is a float
+          if ((mk & kLinkBits) == kLinkBits)
+            fp32::lap6_ff_<true>(col_offs(c.o, plane, nz, z), i, mk, A.phi_hi, A.phi_lo, S, E);
+          else
+            fp32::lap6_ff_<false>(col_offs(c.o, plane, nz, z), i, mk, A.phi_hi, A.phi_lo, S, E);
+          const float bf = (float)A.rhs[i];
+          B = 6.f * bf;
+          Be = fmaf(6.f, bf, -B);  // 6 rhs = B + Be exactly
+          mb = fmaxf(mb, finite_or_inf(fabsf(bf) * inv_diag<float>(code)));
+        }
+        float t, te;
+        fp32::two_sum(S, B, t, te);
+        rt = (T)((t + (te + (E + Be))) * (1.f / 6.f));
+        dinv = inv_diag<T>(code);
+      } else {
+        double b;
+        if (MODE == R_RHS) {
+          b = A.rhs[i];
+        } else {
+          double q = 0.0;
+          for (int k = 0; k < A.P.ns; ++k)
+            q += A.P.z[k] * (MODE == R_FXG ? A.P3.rbd[k] + A.P3.sd[k] * (double)A.nq[k * A.g.N + i]
+                                           : A.n64[k * A.g.N + i]);
+          b = A.P.four_pi_lb * q;
+        }
+        double lap;
+        if (MODE == R_FXG)
+          lap = (double)(wall ? fp32::lap6_fx_<false>(col_offs(c.o, plane, nz, z), i, mk, A.phifx)
+                              : (long long)(nsum - 24 * v0)) *
+                (1.0 / 281474976710656.0 / 6.0);
+        else if (MODE == R_N64 && !wall)
+          lap = ((double)nsum - 24.0 * (double)v0) * (1.0 / 6.0);
+        else
+          lap = lap_at(col_offs(c.o, plane, nz, z), i, mk, A.phi, !(A.P.selfmask & kPlainLaplacian));
+        const double rr = b + lap;
+        rt = (T)rr;
+        dinv = inv_diag<T>(code);
+        if (MODE == R_RHS) mb = fmaxf(mb, finite_or_inf(fabsf((float)b) * (float)dinv));
+      }
+      r[i] = rt;
+      uj[i] = rt * dinv;
+      mx = fmaxf(mx, finite_or_inf(fabsf((float)rt) * (float)dinv));  // the stopping test needs no FP64
     }
-    if (MODE == R_FX) {
-      // 6 res = 6 lap + 6 (4 pi l_B s) (q+ - q-): 6 lap exact in fixed
-      // point, split into float-float (the nearest float of the integer sum
-      // and the float of its exact remainder), the charge term in
-      // float-float too
-      const long long L6 = fp32::lap6_fx(g, (int)i, X, Y, Z, m, phifx);
-      const float Lh = fp32::ll2f(L6);
-      const float Ll = fp32::ll2f(L6 - fp32::f2ll_rn(Lh));
-      const float S = __fmul_rn(Lh, fp32::kPhiUnitF), E = __fmul_rn(Ll, fp32::kPhiUnitF);
-      const long long dq = nq[i] - nq[g.N + i];
-      const float dq_hi = fp32::ll2f(dq);
-      const float dq_lo = fp32::ll2f(dq - fp32::f2ll_rn(dq_hi));  // exact remainder
-      const float B = c6_hi * dq_hi;
-      const float Be = fmaf(c6_hi, dq_hi, -B) + (c6_hi * dq_lo + c6_lo * dq_hi);  // product error and tails
-      float t, te;
-      fp32::two_sum(S, B, t, te);
-      const float rt = (t + (te + (E + Be))) * (1.f / 6.f);
-      const float dinv = 1.f / diag_t<float>(m, P.selfmask);
-      r[i] = (T)rt;
-      u[i] = (T)(rt * dinv);
-      x[i] = p[i] = s[i] = (T)0;
-      mx = fmaxf(mx, finite_or_inf(fabsf(rt) * dinv));
-      continue;
-    }
-    if (MODE == R_RHS_FF) {
-      // 6 res = 6 rhs + 6 lap(x), x = hi + lo, in float-float; rhs is a float
-      float S, E;
-      fp32::lap6_ff(g, (int)i, X, Y, Z, m, phi_hi, phi_lo, S, E);
-      const float bf = (float)rhs[i];
-      const float B = 6.f * bf, Be = fmaf(6.f, bf, -B);  // 6 rhs = B + Be exactly
-      float t, te;
-      fp32::two_sum(S, B, t, te);
-      const float rt = (t + (te + (E + Be))) * (1.f / 6.f);
-      const float dinv = 1.f / diag_t<float>(m, P.selfmask);
-      r[i] = (T)rt;
-      u[i] = (T)(rt * dinv);
-      x[i] = p[i] = s[i] = (T)0;
-      mx = fmaxf(mx, finite_or_inf(fabsf(rt) * dinv));
-      mb = fmaxf(mb, finite_or_inf(fabsf(bf) * dinv));
-      continue;
-    }
-    double b;
-    if (MODE == R_RHS) {
-      b = rhs[i];
-    } else {
-      double q = 0.0;
-      for (int k = 0; k < P.ns; ++k)
-        q += P.z[k] * (MODE == R_FXG ? P3.rbd[k] + P3.sd[k] * (double)nq[k * g.N + i] : n64[k * g.N + i]);
-      b = P.four_pi_lb * q;
-    }
-    const double lap = MODE == R_FXG
-                           ? (double)fp32::lap6_fx(g, (int)i, X, Y, Z, m, phifx) * (1.0 / 281474976710656.0 / 6.0)
-                           : lap_at(g, (int)i, X, Y, Z, m, phi, !(P.selfmask & kPlainLaplacian));
-    const double rr = b + lap;
-    const T rt = (T)rr;
-    const T dinv = (T)1 / diag_t<T>(m, P.selfmask);
-    r[i] = rt;
-    u[i] = rt * dinv;
-    x[i] = p[i] = s[i] = (T)0;
-    mx = fmaxf(mx, finite_or_inf(fabsf((float)rr) * (float)dinv));  // the stopping test needs no FP64
-    if (MODE == R_RHS) mb = fmaxf(mb, finite_or_inf(fabsf((float)b) * (float)dinv));
   }
   mx = block_reduce<true, float>(mx);
-  if (flat_tid() == 0) part[S_MAX * nblk + flat_bid()] = (double)mx;
-  if (RHS) {
-    mb = block_reduce<true, float>(mb);
-    if (flat_tid() == 0) part[S_RU * nblk + flat_bid()] = (double)mb;
-  }
-  if (!last_block(c, nblk)) return;
-  double m = 0.0, ref = 0.0;
-  for (int i = flat_tid(); i < nblk; i += kBlock) {
-    m = fmax(m, __ldcg(part + S_MAX * nblk + i));
-    if (RHS) ref = fmax(ref, __ldcg(part + S_RU * nblk + i));
-  }
-  m = block_reduce<true>(m);
-  if (RHS) ref = block_reduce<true>(ref);
+  if (RHS) mb = block_reduce<true, float>(mb);
   if (flat_tid() == 0) {
-    c->arrive = 0;
-    if (RHS) c->ref = ref;
-    outer_check(c, m, RHS ? fmax(tol, tol_rel * ref) : tol, maxit, hout, hin, use_cond);
+    PoissonCtl *ctl = A.c;
+    atomicMax(&ctl->max_bits, (unsigned long long)__double_as_longlong((double)mx));
+    if (RHS) atomicMax(&ctl->ref_bits, (unsigned long long)__double_as_longlong((double)mb));
+    __threadfence();
+    if (atomicAdd(&ctl->arrive, 1) == A.nblk - 1) {
+      const double m = __longlong_as_double((long long)atomicExch(&ctl->max_bits, 0ULL));
+      double ref = 0.0;
+      if (RHS) {
+        ref = __longlong_as_double((long long)atomicExch(&ctl->ref_bits, 0ULL));
+        ctl->ref = ref;
+      }
+      ctl->arrive = 0;
+      outer_check(ctl, m, RHS ? fmax(A.tol, A.tol_rel * ref) : A.tol, A.maxit, A.hout, A.hin, A.use_cond);
+    }
   }
 }
 
 // stencil + dot products: w = A u; partials (r,u), (w,u); the last block
-// runs the scalar recurrence
+// runs the scalar recurrence.  Marched (march.cuh); u is zero on solid nodes
+// and w is set to zero there, so that the update needs no mask.
 template <typename T>
-__global__ void __launch_bounds__(kBlock) k_cg_b(const Geo g, int zpt, uint32_t selfmask,
-                                                 const uint32_t *__restrict__ mask, const T *__restrict__ u,
-                                                 const T *__restrict__ r, T *__restrict__ w,
-                                                 double *__restrict__ part, int nblk, PoissonCtl *c,
-                                                 cudaGraphConditionalHandle hin, int use_cond) {
-  if (c->inner_done) return;
+__global__ void __launch_bounds__(kBlock) k_cg_b(const Cols C, const uint8_t *__restrict__ code,
+                                                 const T *__restrict__ u, const T *__restrict__ r,
+                                                 T *__restrict__ w, double *__restrict__ part, int nblk,
+                                                 PoissonCtl *c, cudaGraphConditionalHandle hin, int use_cond) {
+  if (!use_cond && c->inner_done) return;  // the graph's loop has ended by then
   T ru = 0, wu = 0;
-  for (int kz = 0; kz < zpt; ++kz) {
-    int X, Y, Z;
-    long long i;
-    if (!node_of(g, zpt, kz, X, Y, Z, i)) continue;
-    const uint32_t m = mask[i];
-    if (!(m & kFluidBit)) continue;
-    const T u0 = u[i];
-    const Offs o = offsets_of(g, X, Y, Z);
-    const T *__restrict__ ui = u + i;
-    T sum = 0;
-    if (all_links(m, selfmask)) {  // the same sum without the weight tests
-#pragma unroll
-      for (int l = 1; l < kQ; ++l) sum += (T)lapc_of(l) * ui[o.at(cx_of(l), cy_of(l), cz_of(l))];
-    } else {
-#pragma unroll
-      for (int l = 1; l < kQ; ++l) {  // every neighbour read; a zero weight drops it
-        const uint32_t b = 1u << (l - 1);
-        const T ul = ui[o.at(cx_of(l), cy_of(l), cz_of(l))];
-        sum += ((selfmask & b) || !(m & b) ? (T)0 : (T)lapc_of(l)) * ul;
-      }
+  Column col;
+  if (column_of(C, col)) {
+    ZMarch<T> m;
+    m.begin(u, col.o, col.p, C.plane, C.nz, col.z0);
+    for (int z = col.z0; z < col.z1; ++z) {
+      T u0;
+      int i;
+      const T nsum = m.step(u, col.o, col.p, C.plane, C.nz, z, z + 1 < col.z1, u0, i);
+      const int cd = code[i];
+      const T wv = cd ? ((T)((cd & kCodeDiag) + C.selfw) * u0 - nsum) * (T)(1.0 / 6.0) : (T)0;
+      w[i] = wv;
+      ru += r[i] * u0;
+      wu += wv * u0;
     }
-    const T wv = diag_t<T>(m, selfmask) * u0 - sum;
-    w[i] = wv;
-    ru += r[i] * u0;
-    wu += wv * u0;
   }
   const T a = block_reduce<false, T>(ru);
   const T b = block_reduce<false, T>(wu);
@@ -467,38 +458,63 @@ __global__ void __launch_bounds__(kBlock) k_cg_b(const Geo g, int zpt, uint32_t 
   }
 }
 
+// VEC consecutive values as one load or store (16 bytes; the codes VEC bytes)
+template <typename T, int VEC>
+struct alignas(sizeof(T) * VEC) Pack {
+  T v[VEC];
+};
+
 // vector update: p = u + beta p, s = w + beta s, x += alpha p,
-// r -= alpha s, u = r/diag; the last block runs the stopping test on
+// r -= alpha s, uj = r/diag; the last block runs the stopping test on
 // max |r|/diag, so that the loop ends here.  (With the test in the stencil
 // kernel, the round's last V-cycle and stencil served only to carry it: on
 // the 64x64x256 electro-osmosis lattice, tolerance 1e-13, the solve took
-// 388 us per step instead of 333.)
-template <typename T>
-__global__ void __launch_bounds__(kBlock) k_cg_a(const Geo g, int zpt, uint32_t selfmask,
-                                                 const uint32_t *__restrict__ mask, T *__restrict__ x,
-                                                 T *__restrict__ r, T *__restrict__ u, const T *__restrict__ w,
-                                                 T *__restrict__ p, T *__restrict__ s, int nblk, PoissonCtl *c,
-                                                 double eta, double tol_abs, int maxit,
+// 388 us per step instead of 333.)  A round's first update starts x, p and s
+// instead of reading zeros that the residual kernel would have to write.
+// Every vector is zero on solid nodes, so no node waits for its mask.
+template <typename T, int VEC>
+__global__ void __launch_bounds__(kBlock) k_cg_a(long long N, const uint8_t *__restrict__ code, T *__restrict__ x,
+                                                 T *__restrict__ r, const T *u, T *uj,
+                                                 const T *__restrict__ w, T *__restrict__ p, T *__restrict__ s,
+                                                 int nblk, PoissonCtl *c, double eta, double tol_abs, int maxit,
                                                  cudaGraphConditionalHandle hin, int use_cond) {
-  if (c->inner_done) return;
+  if (c->inner_done) return;  // a breakdown in this iteration
   const T alpha = (T)c->alpha, beta = (T)c->beta;
+  const bool first = c->round_iters == 0;
+  using PT = Pack<T, VEC>;
+  using PC = Pack<uint8_t, VEC>;
   T mx = 0;
-  for (int kz = 0; kz < zpt; ++kz) {
-    int X, Y, Z;
-    long long i;
-    if (!node_of(g, zpt, kz, X, Y, Z, i)) continue;
-    const uint32_t m = mask[i];
-    if (!(m & kFluidBit)) continue;
-    const T pv = u[i] + beta * p[i];
-    const T sv = w[i] + beta * s[i];
-    p[i] = pv;
-    s[i] = sv;
-    x[i] += alpha * pv;
-    const T rv = r[i] - alpha * sv;
-    r[i] = rv;
-    const T dinv = inv_diag<T>(m, selfmask);
-    u[i] = rv * dinv;
-    mx = fmax(mx, finite_or_inf(fabs(rv) * dinv));
+  const long long n = N / VEC;
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
+    const PT uv = ((const PT *)u)[k], wv = ((const PT *)w)[k];
+    PT rv = ((PT *)r)[k];
+    const PC cv = ((const PC *)code)[k];
+    PT pv = uv, sv = wv, xv, jv;
+    if (first) {
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) xv.v[e] = alpha * uv.v[e];
+    } else {
+      const PT p0 = ((PT *)p)[k], s0 = ((PT *)s)[k];
+      xv = ((PT *)x)[k];
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) {
+        pv.v[e] = uv.v[e] + beta * p0.v[e];
+        sv.v[e] = wv.v[e] + beta * s0.v[e];
+        xv.v[e] += alpha * pv.v[e];
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) {
+      rv.v[e] -= alpha * sv.v[e];
+      const T dinv = inv_diag<T>(cv.v[e]);
+      jv.v[e] = rv.v[e] * dinv;
+      mx = fmax(mx, finite_or_inf(fabs(rv.v[e]) * dinv));
+    }
+    ((PT *)p)[k] = pv;
+    ((PT *)s)[k] = sv;
+    ((PT *)x)[k] = xv;
+    ((PT *)r)[k] = rv;
+    ((PT *)uj)[k] = jv;
   }
   // a maximum does not depend on the order: the blocks combine theirs in one
   // word (the bits of a non-negative double order as an integer), and the
@@ -529,26 +545,20 @@ __global__ void k_extrapolate(const Geo g, int zpt, const uint32_t *__restrict__
 }
 
 // FP32 form: the fixed-point potential += e (rounded to the fixed-point
-// unit) on fluid nodes and its float copy; |phi| reaching kPhiMax raises
-// range flag 4
-__global__ void k_correct_fx(const Geo g, int zpt, const uint32_t *__restrict__ mask, const float *__restrict__ e,
-                             int64_t *__restrict__ phifx, float *__restrict__ phi32, int *__restrict__ flag,
-                             const PoissonCtl *__restrict__ c) {
-  if (c->outer_done) return;  // the round's test had already converged
+// unit) and its float copy; |phi| reaching kPhiMax raises range flag 4.  e is
+// zero on solid nodes, which keep their values.
+__global__ void __launch_bounds__(kBlock) k_correct_fx(long long N, const float *__restrict__ e,
+                                                       int64_t *__restrict__ phifx, float *__restrict__ phi32,
+                                                       int *__restrict__ flag, const PoissonCtl *__restrict__ c) {
+  if (c->outer_done || c->round_iters == 0) return;  // converged, or no update in this round
   constexpr float kMaxFx = (float)(kPhiMax * 281474976710656.0);  // kPhiMax 2^kPhiFixBits
   bool over = false;
-  for (int kz = 0; kz < zpt; ++kz) {
-    int X, Y, Z;
-    long long i;
-    if (!node_of(g, zpt, kz, X, Y, Z, i)) continue;
-    if (!(mask[i] & kFluidBit)) continue;
+#pragma unroll 4
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
     const float d = __fmul_rn(e[i], 281474976710656.0f);  // e 2^kPhiFixBits, exact
-    if (!(fabsf(d) < kMaxFx)) {  // also NaN
-      over = true;
-      continue;
-    }
-    const long long v = phifx[i] + fp32::f2ll_rn(d);
-    over |= !(fabsf(fp32::ll2f(v)) < kMaxFx);
+    const bool bad = !(fabsf(d) < kMaxFx);  // also NaN
+    const long long v = phifx[i] + (bad ? 0LL : fp32::f2ll_rn(d));
+    over |= bad || !(fabsf(fp32::ll2f(v)) < kMaxFx);
     phifx[i] = v;
     phi32[i] = fp32::fx_to_f(v);
   }
@@ -567,19 +577,17 @@ __global__ void k_extrapolate_fx(const Geo g, int zpt, const uint32_t *__restric
   }
 }
 
-// phi64 += e on fluid nodes; with phi32 given its float split follows
+// phi64 += e (zero on solid nodes); with phi32 given its float split follows
 // (the FP64 form, and the linear solves' FP64 iterates)
 template <typename T>
-__global__ void k_correct(const Geo g, int zpt, const uint32_t *__restrict__ mask, const T *__restrict__ e,
-                          double *__restrict__ phi, float *__restrict__ phi32, float *__restrict__ phi_lo,
-                          const PoissonCtl *__restrict__ c) {
-  if (c && c->outer_done) return;  // the round's test had already converged
-  for (int kz = 0; kz < zpt; ++kz) {
-    int X, Y, Z;
-    long long i;
-    if (!node_of(g, zpt, kz, X, Y, Z, i)) continue;
+__global__ void __launch_bounds__(kBlock) k_correct(long long N, const T *__restrict__ e, double *__restrict__ phi,
+                                                    float *__restrict__ phi32, float *__restrict__ phi_lo,
+                                                    const PoissonCtl *__restrict__ c) {
+  if (c && (c->outer_done || c->round_iters == 0)) return;  // converged, or no update in this round
+#pragma unroll 4
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
     double v = phi[i];
-    if (e && (mask[i] & kFluidBit)) {
+    if (e) {
       v += (double)e[i];
       phi[i] = v;
     }
@@ -594,25 +602,17 @@ __global__ void k_correct(const Geo g, int zpt, const uint32_t *__restrict__ mas
 // ---------------------------------------------------------------------------
 // kernel argument storage for graph nodes (values are copied at node creation)
 struct Args {
-  Geo g;
-  int zpt, nblk, maxit, use_cond = 1;
-  Phys P;
-  P32 P3;
-  uint32_t selfmask;
-  double tol, tol_rel = 0.0, eta, tol_inner;
-  const uint32_t *mask;
-  const double *n64;
-  const int64_t *nq;
-  const double *rhs = nullptr;
-  double *phi;
+  ResArgs R;  // the residual kernel's arguments, shared values among them
+  int nblk, nblk_a;
+  long long N;
+  double eta, tol_inner;
+  double *phi;               // FP64 iterate (FP64 form, linear solves)
   float *phi32, *phi_lo = nullptr;
-  float c6_hi = 0.f, c6_lo = 0.f;  // 6 * 4 pi l_B * s, as two floats (R_FX)
-  int64_t *phifx = nullptr;        // the FP32 form's fixed-point potential
-  int *flag = nullptr;             // the FP32 form's range flags
-  void *r, *u, *w, *x, *p, *s;
+  int64_t *phifx = nullptr;  // the FP32 form's fixed-point potential
+  int *flag = nullptr;       // the FP32 form's range flags
+  void *r, *u, *uj, *w, *x, *p, *s;
   double *part;
-  PoissonCtl *c;
-  cudaGraphConditionalHandle hout = 0, hin = 0;
+  dim3 flat;                 // grid of the pointwise kernels
 };
 
 cudaError_t add_kernel(cudaGraph_t gr, cudaGraphNode_t *last, void *func, dim3 grid, dim3 block, void **args) {
@@ -651,85 +651,115 @@ void fill_args(lbe_handle *h, Args &A) {
   PoissonWork &w = h->pw;
   const long long N = h->geo.N;
   T *base = (T *)w.vec;
-  A.g = h->geo;
-  A.zpt = w.L.zpt;
-  A.nblk = (int)w.L.nblk();
-  A.maxit = h->prm.poisson_max_iter;
-  A.P = h->phys;
-  A.P3 = h->p32;
-  A.selfmask = h->phys.selfmask;
-  A.tol = h->prm.poisson_tol;
+  const ColLaunch L = make_cols(h->geo, h->phys.selfmask, kSolveBlocks);
+  ResArgs &R = A.R;
+  R = ResArgs{};
+  R.cols = L.c;
+  R.g = h->geo;
+  R.P = h->phys;
+  R.P3 = h->p32;
+  R.code = h->code;
+  R.mask = h->mask;
+  R.n64 = h->n;
+  R.nq = h->q;
+  R.phi = h->phi;
+  R.phi_hi = h->phi32;
+  R.phifx = h->phifx;
+  R.nblk = (int)L.nblk();
+  R.maxit = h->prm.poisson_max_iter;
+  R.use_cond = 1;
+  R.c = w.ctl;
+  R.tol = h->prm.poisson_tol;
+  {
+    const double c6 = 6.0 * h->phys.four_pi_lb * h->p32.sd[0];  // 6 * 4 pi l_B * s, as two floats (R_FX)
+    R.c6_hi = (float)c6;
+    R.c6_lo = (float)(c6 - (double)R.c6_hi);
+  }
+  A.N = N;
+  A.nblk = (int)L.nblk();
+  A.flat = dim3((unsigned)std::min<long long>((N + kBlock - 1) / kBlock, kSolveBlocks));
   A.eta = sizeof(T) == 4 ? 1e-4 : 1e-9;
   // an inner solve need not go below a fraction of the outer tolerance:
   // 0.8 measured 2.15 CG iterations per step on the 64x64x256
   // electro-osmosis lattice against 2.9 at 0.25 and 2.4 at 0.5, with no
   // extra refinement round (the outer test still decides convergence)
-  A.tol_inner = 0.8 * A.tol;
-  A.mask = h->mask;
-  A.n64 = h->n;
-  A.nq = h->q;
+  A.tol_inner = 0.8 * R.tol;
   A.phi = h->phi;
   A.phi32 = h->phi32;
   A.phifx = h->phifx;
   A.flag = h->flag;
-  {
-    const double c6 = 6.0 * h->phys.four_pi_lb * h->p32.sd[0];
-    A.c6_hi = (float)c6;
-    A.c6_lo = (float)(c6 - (double)A.c6_hi);
-  }
   A.r = base;
   A.u = base + N;
   A.w = base + 2 * N;
   A.x = base + 3 * N;
   A.p = base + 4 * N;
   A.s = base + 5 * N;
+  // the Jacobi vector r/diag: the V-cycle's input, or the preconditioned
+  // vector itself without a hierarchy
+  A.uj = h->mg.nlev >= 2 ? h->mg.t0 : A.u;
   A.part = w.partial;
-  A.c = w.ctl;
+}
+
+template <typename T>
+using ResKernel = void (*)(const ResArgs, T *, T *);
+template <typename T>
+ResKernel<T> res_kernel(const lbe_handle *h, const Args &A) {
+  if (A.R.rhs) return A.R.phi_lo ? k_res<T, R_RHS_FF> : k_res<T, R_RHS>;
+  if (h->prm.precision != LBE_FP32) return k_res<T, R_N64>;
+  return h->p32.salt11 ? k_res<T, R_FX> : k_res<T, R_FXG>;
+}
+// The update handles 16 bytes of every vector at a time where the component
+// stride (N values) keeps them aligned, else one value.
+template <typename T>
+using UpdateKernel = void (*)(long long, const uint8_t *, T *, T *, const T *, T *, const T *, T *, T *, int,
+                              PoissonCtl *, double, double, int, cudaGraphConditionalHandle, int);
+template <typename T>
+UpdateKernel<T> update_kernel(long long N, int *vec) {
+  constexpr int V = 16 / sizeof(T);
+  *vec = N % V == 0 ? V : 1;
+  return N % V == 0 ? k_cg_a<T, V> : k_cg_a<T, 1>;
 }
 
 template <typename T>
 cudaError_t build_graph(lbe_handle *h, Args &A, cudaGraphExec_t *exec) {
-  const Launch &L = h->pw.L;
-  const dim3 one(1);
-  const bool fixed = h->prm.precision == LBE_FP32;
-  void *f_res = A.rhs ? (A.phi32 && A.phi_lo ? (void *)k_res<T, R_RHS_FF> : (void *)k_res<T, R_RHS>)
-                      : (fixed ? (h->p32.salt11 ? (void *)k_res<T, R_FX> : (void *)k_res<T, R_FXG>)
-                               : (void *)k_res<T, R_N64>);
+  const ColLaunch L = make_cols(h->geo, h->phys.selfmask, kSolveBlocks);
+  const dim3 one(1), blk(kBlock);
+  ResArgs &R = A.R;
   // the FP32 form's own solve corrects its fixed-point potential; the FP64
   // form and the linear solves correct an FP64 iterate
-  const bool corr_fx = fixed && !A.rhs;
+  const bool corr_fx = h->prm.precision == LBE_FP32 && !R.rhs;
+  int vec = 1;
+  const UpdateKernel<T> f_a = update_kernel<T>(A.N, &vec);
+  const dim3 ga((unsigned)std::min<long long>((A.N / vec + kBlock - 1) / kBlock, kSolveBlocks));
+  A.nblk_a = (int)ga.x;
   cudaGraph_t G = nullptr;
   cudaError_t e = cudaGraphCreate(&G, 0);
   if (e != cudaSuccess) return e;
   cudaGraphNode_t last = nullptr, lo = nullptr, li = nullptr;
   cudaGraph_t body_out = nullptr, body_in = nullptr;
-  void *a_reset[] = {&A.c};
-  void *a_res[] = {&A.g,     &A.zpt,   &A.P,      &A.P3,    &A.mask,    &A.n64,   &A.nq, &A.rhs,
-                   &A.phi,   &A.phi32, &A.phi_lo, &A.phifx, &A.c6_hi,   &A.c6_lo, &A.r,  &A.u,
-                   &A.x,     &A.p,     &A.s,      &A.part,  &A.nblk,    &A.c,     &A.tol, &A.tol_rel,
-                   &A.maxit, &A.hout,  &A.hin,    &A.use_cond};
-  void *a_b[] = {&A.g, &A.zpt, &A.selfmask, &A.mask, &A.u, &A.r, &A.w, &A.part, &A.nblk, &A.c, &A.hin, &A.use_cond};
-  void *a_a[] = {&A.g, &A.zpt,  &A.selfmask, &A.mask, &A.x,   &A.r,         &A.u,     &A.w,   &A.p,
-                 &A.s, &A.nblk, &A.c,        &A.eta,  &A.tol_inner, &A.maxit, &A.hin, &A.use_cond};
-  void *a_cor[] = {&A.g, &A.zpt, &A.mask, &A.x, &A.phi, &A.phi32, &A.phi_lo, &A.c};
-  void *a_corfx[] = {&A.g, &A.zpt, &A.mask, &A.x, &A.phifx, &A.phi32, &A.flag, &A.c};
+  void *a_reset[] = {&R.c};
+  void *a_res[] = {&R, &A.r, &A.uj};
+  void *a_b[] = {&R.cols, &R.code, &A.u, &A.r, &A.w, &A.part, &A.nblk, &R.c, &R.hin, &R.use_cond};
+  void *a_a[] = {&A.N, &R.code,   &A.x, &A.r,   &A.u,         &A.uj,    &A.w,   &A.p,
+                 &A.s, &A.nblk_a, &R.c, &A.eta, &A.tol_inner, &R.maxit, &R.hin, &R.use_cond};
+  void *a_cor[] = {&A.N, &A.x, &A.phi, &A.phi32, &A.phi_lo, &R.c};
+  void *a_corfx[] = {&A.N, &A.x, &A.phifx, &A.phi32, &A.flag, &R.c};
   // reset -> while (not converged) { residual test -> while (CG) { V-cycle ->
   // stencil and dot products -> update and test } -> correct }.  The residual
   // test sets both conditions; in the pass where it converges the CG loop is
   // not entered and the correction returns at once.
-  e = cudaGraphConditionalHandleCreate(&A.hout, G, 1, cudaGraphCondAssignDefault);
+  e = cudaGraphConditionalHandleCreate(&R.hout, G, 1, cudaGraphCondAssignDefault);
   if (e == cudaSuccess) e = add_kernel(G, &last, (void *)k_solve_reset, one, one, a_reset);
-  if (e == cudaSuccess) e = add_while(G, &last, A.hout, &body_out);
-  if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&A.hin, body_out, 0, 0);
-  const bool mg = sizeof(T) == 4 && h->mg.nlev >= 2;
-  if (e == cudaSuccess) e = add_kernel(body_out, &lo, f_res, L.grid, L.block, a_res);
-  if (e == cudaSuccess) e = add_while(body_out, &lo, A.hin, &body_in);
-  if (e == cudaSuccess && mg) e = mg_vcycle(h, (const float *)A.r, (float *)A.u, A.c, body_in, &li, nullptr);
+  if (e == cudaSuccess) e = add_while(G, &last, R.hout, &body_out);
+  if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&R.hin, body_out, 0, 0);
+  if (e == cudaSuccess) e = add_kernel(body_out, &lo, (void *)res_kernel<T>(h, A), L.grid, L.block, a_res);
+  if (e == cudaSuccess) e = add_while(body_out, &lo, R.hin, &body_in);
+  if (e == cudaSuccess && h->mg.nlev >= 2) e = mg_vcycle(h, A.r, A.uj, A.u, nullptr, body_in, &li, nullptr);
   if (e == cudaSuccess) e = add_kernel(body_in, &li, (void *)k_cg_b<T>, L.grid, L.block, a_b);
-  if (e == cudaSuccess) e = add_kernel(body_in, &li, (void *)k_cg_a<T>, L.grid, L.block, a_a);
+  if (e == cudaSuccess) e = add_kernel(body_in, &li, (void *)f_a, ga, blk, a_a);
   if (e == cudaSuccess)
-    e = corr_fx ? add_kernel(body_out, &lo, (void *)k_correct_fx, L.grid, L.block, a_corfx)
-                : add_kernel(body_out, &lo, (void *)k_correct<T>, L.grid, L.block, a_cor);
+    e = corr_fx ? add_kernel(body_out, &lo, (void *)k_correct_fx, A.flat, blk, a_corfx)
+                : add_kernel(body_out, &lo, (void *)k_correct<T>, A.flat, blk, a_cor);
   if (e == cudaSuccess) e = cudaGraphInstantiate(exec, G, 0);
   cudaGraphDestroy(G);
   return e;
@@ -739,15 +769,17 @@ cudaError_t build_graph(lbe_handle *h, Args &A, cudaGraphExec_t *exec) {
 template <typename T>
 int solve_polled(lbe_handle *h, Args &A) {
   PoissonWork &w = h->pw;
-  const Launch &L = w.L;
+  const ColLaunch L = make_cols(h->geo, h->phys.selfmask, kSolveBlocks);
   cudaStream_t st = h->stream;
-  const bool fixed = h->prm.precision == LBE_FP32;
-  A.use_cond = 0;
-  k_solve_reset<<<1, 1, 0, st>>>(A.c);
+  ResArgs &R = A.R;
+  R.use_cond = 0;
+  int vec = 1;
+  const UpdateKernel<T> f_a = update_kernel<T>(A.N, &vec);
+  const dim3 ga((unsigned)std::min<long long>((A.N / vec + kBlock - 1) / kBlock, kSolveBlocks));
+  const ResKernel<T> f_res = res_kernel<T>(h, A);
+  const bool mg = h->mg.nlev >= 2;
+  k_solve_reset<<<1, 1, 0, st>>>(R.c);
   h->launches += 1;
-  const bool mg = sizeof(T) == 4 && h->mg.nlev >= 2;
-  auto kres = A.rhs ? (A.phi32 && A.phi_lo ? k_res<T, R_RHS_FF> : k_res<T, R_RHS>)
-                    : (fixed ? (h->p32.salt11 ? k_res<T, R_FX> : k_res<T, R_FXG>) : k_res<T, R_N64>);
   auto poll = [&]() {
     cudaError_t e = cudaMemcpyAsync(w.ctl_host, w.ctl, sizeof(PoissonCtl), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -755,30 +787,25 @@ int solve_polled(lbe_handle *h, Args &A) {
     return e;
   };
   for (int round = 0; round <= kMaxOuter + 1; ++round) {
-    kres<<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.P, A.P3, A.mask, A.n64, A.nq, A.rhs, A.phi, A.phi32, A.phi_lo,
-                                     A.phifx, A.c6_hi, A.c6_lo, (T *)A.r, (T *)A.u, (T *)A.x, (T *)A.p, (T *)A.s,
-                                     A.part, A.nblk, A.c, A.tol, A.tol_rel, A.maxit, 0, 0, 0);
+    f_res<<<L.grid, L.block, 0, st>>>(R, (T *)A.r, (T *)A.uj);
     h->launches += 1;
     if (poll() != cudaSuccess) return LBE_ERR_CUDA;
     if (w.ctl_host->outer_done) break;
-    const long long max_chunks = (long long)A.maxit / kChunk + 2;
+    const long long max_chunks = (long long)R.maxit / kChunk + 2;
     for (long long ch = 0; ch <= max_chunks && !w.ctl_host->inner_done; ++ch) {
       for (int k = 0; k < kChunk; ++k) {
-        if (mg && mg_vcycle(h, (const float *)A.r, (float *)A.u, A.c, nullptr, nullptr, st) != cudaSuccess)
-          return LBE_ERR_CUDA;
-        k_cg_b<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.selfmask, A.mask, (T *)A.u, (T *)A.r, (T *)A.w, A.part,
-                                               A.nblk, A.c, 0, 0);
-        k_cg_a<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.selfmask, A.mask, (T *)A.x, (T *)A.r, (T *)A.u,
-                                               (T *)A.w, (T *)A.p, (T *)A.s, A.nblk, A.c, A.eta,
-                                               A.tol_inner, A.maxit, 0, 0);
+        if (mg && mg_vcycle(h, A.r, A.uj, A.u, R.c, nullptr, nullptr, st) != cudaSuccess) return LBE_ERR_CUDA;
+        k_cg_b<T><<<L.grid, L.block, 0, st>>>(R.cols, R.code, (T *)A.u, (T *)A.r, (T *)A.w, A.part, A.nblk, R.c, 0, 0);
+        f_a<<<ga, kBlock, 0, st>>>(A.N, R.code, (T *)A.x, (T *)A.r, (T *)A.u, (T *)A.uj, (T *)A.w, (T *)A.p, (T *)A.s,
+                                   (int)ga.x, R.c, A.eta, A.tol_inner, R.maxit, 0, 0);
       }
       h->launches += 2 * kChunk;
       if (poll() != cudaSuccess) return LBE_ERR_CUDA;
     }
-    if (fixed && !A.rhs)
-      k_correct_fx<<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.mask, (const float *)A.x, A.phifx, A.phi32, A.flag, A.c);
+    if (h->prm.precision == LBE_FP32 && !R.rhs)
+      k_correct_fx<<<A.flat, kBlock, 0, st>>>(A.N, (const float *)A.x, A.phifx, A.phi32, A.flag, R.c);
     else
-      k_correct<T><<<L.grid, L.block, 0, st>>>(A.g, A.zpt, A.mask, (const T *)A.x, A.phi, A.phi32, A.phi_lo, A.c);
+      k_correct<T><<<A.flat, kBlock, 0, st>>>(A.N, (const T *)A.x, A.phi, A.phi32, A.phi_lo, R.c);
     h->launches += 1;
   }
   return cudaGetLastError() == cudaSuccess ? LBE_OK : LBE_ERR_CUDA;
@@ -830,7 +857,8 @@ cudaError_t poisson_alloc(lbe_handle *h) {
   const size_t tsz = h->prm.precision == LBE_FP32 ? sizeof(float) : sizeof(double);
   cudaError_t e;
   if ((e = cudaMalloc(&w.vec, tsz * 6 * N)) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&w.partial, sizeof(double) * 3 * w.L.nblk())) != cudaSuccess) return e;
+  const size_t nblk = (size_t)make_cols(h->geo, h->phys.selfmask, kSolveBlocks).nblk();
+  if ((e = cudaMalloc(&w.partial, sizeof(double) * 2 * nblk)) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.phi_prev, sizeof(double) * kHist * N)) != cudaSuccess) return e;
   if ((e = cudaMalloc(&w.ctl, sizeof(PoissonCtl))) != cudaSuccess) return e;
   if ((e = cudaMemset(w.ctl, 0, sizeof(PoissonCtl))) != cudaSuccess) return e;
@@ -876,16 +904,16 @@ int poisson_solve_linear(lbe_handle *h, const double *rhs, double *x, double tol
   PoissonWork &w = h->pw;
   Args A;
   fill_args<float>(h, A);
-  A.rhs = rhs;
-  A.phi = x;
-  A.phi32 = x_hi;
-  A.phi_lo = x_lo;
-  if (x_hi && x_lo) {  // the split of the starting x; the corrections keep it current
-    k_correct<float><<<w.L.grid, w.L.block, 0, h->stream>>>(h->geo, w.L.zpt, h->mask, nullptr, x, x_hi, x_lo, nullptr);
+  A.R.rhs = rhs;
+  A.R.phi = A.phi = x;
+  A.R.phi_hi = A.phi32 = x_hi;
+  A.R.phi_lo = A.phi_lo = x_hi ? x_lo : nullptr;
+  if (A.phi_lo) {  // the split of the starting x; the corrections keep it current
+    k_correct<float><<<A.flat, kBlock, 0, h->stream>>>(A.N, nullptr, x, x_hi, x_lo, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LBE_ERR_CUDA;
   }
-  A.tol = tol_abs;
-  A.tol_rel = tol_rel;
+  A.R.tol = tol_abs;
+  A.R.tol_rel = tol_rel;
   A.tol_inner = 0.25 * tol_abs;
   if (!w.graph_ok) return solve_polled<float>(h, A);
   if (!w.exec_lin || w.lin_key[0] != rhs || w.lin_key[1] != x || w.lin_key[2] != x_hi) {
@@ -951,7 +979,7 @@ int poisson_status(lbe_handle *h, lbe_stats *st, long long *kernels) {
     // kernels of the graph path: per solve the reset; per residual test the
     // test and the correction; per iteration V-cycle (with multigrid),
     // stencil and update
-    const long long vc = h->prm.precision == LBE_FP32 ? mg_kernels_per_cycle(h) : 0;
+    const long long vc = mg_kernels_per_cycle(h);
     *kernels = c.solves + 2 * c.total_rounds + (2 + vc) * c.total_iters;
   }
   if (c.sticky_status == LBE_ERR_NOCONVERGE || c.status == LBE_ERR_NOCONVERGE) {
