@@ -259,12 +259,16 @@ struct MGLevel {
   long long N = 0;
   // arrays of the form's type (float or double)
   void *A = nullptr;               // 27-point Galerkin operator [27][N]
+  void *W = nullptr;               // omega/diag (0 for a node without fluid)
   void *r = nullptr, *e = nullptr;
   void *z = nullptr;               // pre-smoothed iterate omega r/diag
 };
 struct MGWork {
   MGLevel lv[kMaxLevels];
   int nlev = 0;          // 0: no hierarchy (Jacobi preconditioning)
+  int ld = 0;            // the level whose V-cycle is one matrix, or the coarsest
+  void *dense = nullptr; // that matrix [N][stride] (null: the coarsest level's inverse or sweeps)
+  int stride = 0;
   void *t0 = nullptr;    // the Jacobi vector r/diag of the finest level
   void *cinv = nullptr;  // inverse of the coarsest operator [N][N] (null: Jacobi sweeps)
 };

@@ -10,9 +10,10 @@
 // nine loads and ten additions per node instead of eighteen neighbours, each
 // with its own address and weight.  Every neighbour is read unconditionally:
 // the solve's correction vectors hold zeros on solid nodes (Dirichlet), so no
-// link needs its mask bit, and no load waits for another one.  Measured
-// with the other changes that came with it on the 64x64x256 lattice: see
-// k_cg_b, k_res, k_restrict0 and k_post0.
+// link needs its mask bit, and no load waits for another one.  Kernel times
+// on the 64x64x256 lattice, before and after: CG stencil 21 -> 12.5 us,
+// residual 24 -> 16, restriction 13 -> 9, prolongation and post-smoothing
+// 12 -> 10.5 (one kernel).
 //
 // Column positions are flattened (p = x + nx y): a block covers 256
 // consecutive positions, or all positions of a smaller plane for several z
@@ -59,11 +60,16 @@ __host__ __device__ __forceinline__ uint32_t fdiv(const FastDiv &f, uint32_t n) 
 // set when one of its 18 links joins a solid node; 0 on solid nodes.
 constexpr int kCodeDiag = 0x7f, kCodeWall = 0x80;
 
+// lattices above this size (about 30 bytes of solve vectors per node in use
+// at a time) do not stay in the 129 MB L2
+constexpr long long kPrefetchNodes = 3 << 20;
+
 // A lattice cut into columns of K planes
 struct Cols {
   int nx, ny, nz, plane;  // plane = nx ny
   int K;                  // planes per thread
   int selfw;              // 6 x the weights of the links that join a node to itself
+  int ahead;              // planes to prefetch ahead of the march (0: none)
   FastDiv fnx;
 };
 struct ColLaunch {
@@ -72,7 +78,31 @@ struct ColLaunch {
   long long nblk() const { return (long long)grid.x * grid.y; }
 };
 
-inline ColLaunch make_cols(const Geo &g, uint32_t selfmask, long long max_blocks) {
+// Planes per thread for nz planes of gx column blocks (zb chunks a block): the
+// K that minimises waves x (K + 3), the march costing about three planes of
+// latency besides its K (two planes to start, the reduction at the end), with
+// kResident blocks at once (five per SM at 48 registers).  On the 256^3
+// lattice, with the L2 prefetch (Cols::ahead), K = 32 takes the CG stencil
+// from 113 to 86 us, the post-smoothing from 222 to 136 and the restriction
+// from 125 to 94 against K = 64 in 1024 blocks; at 64x64x256 the two agree
+// (12.4-13.7 us).
+constexpr int kResident = 760;
+inline int planes_per_thread(long long gx, int nz, int zb, int unit = 1) {
+  long long best = 0;
+  int bestK = 1;
+  for (int K = 1; K <= 64; ++K) {
+    const long long gy = (nz + (long long)K * zb - 1) / ((long long)K * zb);
+    const long long cost = (gx * gy + kResident - 1) / kResident * (K * unit + 3);
+    if (K == 1 || cost < best) {
+      best = cost;
+      bestK = K;
+    }
+    if (gy == 1) break;
+  }
+  return bestK;
+}
+
+inline ColLaunch make_cols(const Geo &g, uint32_t selfmask) {
   ColLaunch L;
   L.c.nx = g.nx;
   L.c.ny = g.ny;
@@ -84,12 +114,13 @@ inline ColLaunch make_cols(const Geo &g, uint32_t selfmask, long long max_blocks
     if (selfmask & (1u << (i - 1))) L.c.selfw += c2_of(i) == 1 ? 2 : 1;
   const int cb = L.c.plane < 256 ? pow2_at_least(L.c.plane) : 256, zb = 256 / cb;
   const long long gx = ((long long)L.c.plane + cb - 1) / cb;
-  long long K = 1;
-  auto gy = [&](long long k) { return (g.nz + k * zb - 1) / (k * zb); };
-  while (gx * gy(K) > max_blocks && K < g.nz) ++K;
-  L.c.K = (int)K;
+  const int K = planes_per_thread(gx, g.nz, zb);
+  L.c.K = K;
+  // a lattice whose vectors exceed L2 is read from HBM: its latency is
+  // covered by prefetching the columns' next planes into L2
+  L.c.ahead = g.N > kPrefetchNodes ? 3 : 0;
   L.block = dim3((unsigned)cb, (unsigned)zb);
-  L.grid = dim3((unsigned)gx, (unsigned)gy(K));
+  L.grid = dim3((unsigned)gx, (unsigned)((g.nz + (long long)K * zb - 1) / ((long long)K * zb)));
   return L;
 }
 
@@ -134,12 +165,14 @@ __device__ __forceinline__ Offs col_offs(const PlaneOffs &o, int plane, int nz, 
   return f;
 }
 
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 template <typename V>
-__device__ __forceinline__ void plane_sums(const V *v, const PlaneOffs &o, int j, bool diag, V &c, V &s, V &d) {
+__device__ __forceinline__ void plane_sums(const V *v, const PlaneOffs &o, int j, V &c, V &s, V &d) {
   const V *q = v + j;
   c = q[0];
   s = (q[o.xm] + q[o.xp]) + (q[o.ym] + q[o.yp]);
-  d = diag ? (q[o.xm + o.ym] + q[o.xp + o.ym]) + (q[o.xm + o.yp] + q[o.xp + o.yp]) : (V)0;
+  d = (q[o.xm + o.ym] + q[o.xp + o.ym]) + (q[o.xm + o.yp] + q[o.xp + o.yp]);
 }
 
 // one column's march over the planes of v
@@ -150,17 +183,17 @@ struct ZMarch {
   __device__ __forceinline__ void begin(const V *v, const PlaneOffs &o, int p, int plane, int nz, int z) {
     V c0, s0, d0;
     j = p + plane * z;
-    plane_sums(v, o, z == 0 ? p + plane * (nz - 1) : j - plane, false, c0, s0, d0);
+    plane_sums(v, o, z == 0 ? p + plane * (nz - 1) : j - plane, c0, s0, d0);
     below = 2 * c0 + s0;
-    plane_sums(v, o, j, true, c, s, d);
+    plane_sums(v, o, j, c, s, d);
   }
   // 6 sum_l w_l v_l of plane z, then plane z + 1 becomes the current one
-  // (its diagonal sums are read only when it will be a centre: more)
-  __device__ __forceinline__ V step(const V *v, const PlaneOffs &o, int p, int plane, int nz, int z, bool more,
-                                    V &centre, int &at) {
+  // (straight-line code: the loads of several unrolled steps go out together)
+  __device__ __forceinline__ V step(const V *v, const PlaneOffs &o, int p, int plane, int nz, int z, V &centre,
+                                    int &at) {
     const int k = z + 1 == nz ? p : j + plane;
     V c1, s1, d1;
-    plane_sums(v, o, k, more, c1, s1, d1);
+    plane_sums(v, o, k, c1, s1, d1);
     const V sum = (2 * s + d) + (below + (2 * c1 + s1));
     centre = c;
     at = j;

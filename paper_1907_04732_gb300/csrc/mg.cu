@@ -79,7 +79,7 @@ struct RestrictMap {
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict0(const Cols F, const uint8_t *__restrict__ code,
                                                    const T *__restrict__ r, const T *__restrict__ u, const MgLevel C,
-                                                   const T *__restrict__ AC, T *__restrict__ rc, T *__restrict__ zc,
+                                                   const T *__restrict__ WC, T *__restrict__ rc, T *__restrict__ zc,
                                                    const RestrictMap M, const PoissonCtl *c) {
   if (c && c->inner_done) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -94,14 +94,23 @@ __global__ void __launch_bounds__(256) k_restrict0(const Cols F, const uint8_t *
   int z = Z0 << C.sz;
   const int zend = min((Z0 + M.Kc) << C.sz, F.nz);
   if (own) m.begin(u, o, p, F.plane, F.nz, z);
+#pragma unroll 1
   for (int k = 0; k < M.Kc; ++k) {  // every lane runs the same iterations (the shuffles)
     const int Z = Z0 + k;
+    const bool write = own && Z < C.nz && !(C.sx & lx & 1) && !(C.sy & ly & 1);
+    const int I = (x >> C.sx) + C.nx * ((y >> C.sy) + C.ny * Z);
+    const T wd = write ? WC[I] : (T)0;
     T v = 0;
     if (own && Z < C.nz) {
       for (int h = 0; h <= C.sz && z < F.nz; ++h, ++z) {
+        if (F.ahead && z + 1 + F.ahead < zend) {
+          prefetch_l2(u + m.j + F.plane * (1 + F.ahead));
+          prefetch_l2(r + m.j + F.plane * F.ahead);
+          prefetch_l2(code + m.j + F.plane * F.ahead);
+        }
         T u0;
         int i;
-        const T nsum = m.step(u, o, p, F.plane, F.nz, z, z + 1 < zend, u0, i);
+        const T nsum = m.step(u, o, p, F.plane, F.nz, z, u0, i);
         const int cd = code[i];
         const T res = r[i] - (T)kOmega * ((T)((cd & kCodeDiag) + F.selfw) * u0 - nsum) * (T)(1.0 / 6.0);
         v += cd ? res : (T)0;
@@ -109,21 +118,23 @@ __global__ void __launch_bounds__(256) k_restrict0(const Cols F, const uint8_t *
     }
     if (C.sx) v += __shfl_xor_sync(0xffffffffu, v, 1);
     if (C.sy) v += __shfl_xor_sync(0xffffffffu, v, 1 << M.xl);
-    if (own && Z < C.nz && !(C.sx & lx & 1) && !(C.sy & ly & 1))
-      store_coarse(C, (x >> C.sx) + C.nx * ((y >> C.sy) + C.ny * Z), v, AC, rc, zc);
+    if (write) {
+      rc[I] = v;
+      zc[I] = wd * v;
+    }
   }
 }
 
 // Restriction between coarse levels with 8 threads per coarse node (one per
 // child) and a fixed-order shuffle sum of the children's pre-smoothed
-// residuals (store_coarse in mg_device.cuh).  A block covers a tile of 32
+// residuals.  A block covers a tile of 32
 // coarse nodes (2^txl along X, the rest along Y; lanes 8k..8k+7 the children
 // of one coarse node, child index = lane % 8 as in child_of) of one plane:
 // coordinates come from the block and lane indices, with no division.
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict(const MgLevel F, const T *__restrict__ AF,
                                                   const T *__restrict__ r, const T *__restrict__ zf,
-                                                  const MgLevel C, const T *__restrict__ AC,
+                                                  const MgLevel C, const T *__restrict__ WC,
                                                   T *__restrict__ rc, T *__restrict__ zc, int txl,
                                                   const PoissonCtl *c) {
   if (c && c->inner_done) return;
@@ -131,11 +142,16 @@ __global__ void __launch_bounds__(256) k_restrict(const MgLevel F, const T *__re
   const int X = (blockIdx.x << txl) + (j & ((1 << txl) - 1));
   const int Y = blockIdx.y * (32 >> txl) + (j >> txl), Z = blockIdx.z;
   const bool own = X < C.nx && Y < C.ny;
+  const int I = X + C.nx * (Y + C.ny * Z);
+  const T wd = ch == 0 && own ? WC[I] : (T)0;
   int x, y, z;
   T v = 0;
   if (own && child_of(C, X, Y, Z, ch, F.nx, F.ny, F.nz, x, y, z)) v = presmoothed_res_z(F, AF, r, zf, x, y, z);
   v = sum8(v);
-  if (ch == 0 && own) store_coarse(C, X + C.nx * (Y + C.ny * Z), v, AC, rc, zc);
+  if (ch == 0 && own) {
+    rc[I] = v;
+    zc[I] = wd * v;
+  }
 }
 
 // fused prolongation + post-smoothing on a 27-point level
@@ -157,7 +173,7 @@ __global__ void k_post(const MgLevel L, const T *__restrict__ A, const T *__rest
 // Next to a wall, P e_1 is nonzero on the solid neighbours too and the links
 // are taken one by one.
 template <typename T>
-__global__ void __launch_bounds__(256) k_post0(const Cols F, const uint8_t *__restrict__ code,
+__global__ void __launch_bounds__(256, 5) k_post0(const Cols F, const uint8_t *__restrict__ code,
                                                const uint32_t *__restrict__ mask, const T *__restrict__ r,
                                                const T *__restrict__ u, const MgLevel C, const T *__restrict__ ec,
                                                T *__restrict__ out, const PoissonCtl *c) {
@@ -179,22 +195,28 @@ __global__ void __launch_bounds__(256) k_post0(const Cols F, const uint8_t *__re
   {
     T cb, sb, db;
     const int Zb = (col.z0 == 0 ? F.nz - 1 : col.z0 - 1) >> C.sz;
-    plane_sums(ec, q, P + cplane * Zb, false, cb, sb, db);
+    plane_sums(ec, q, P + cplane * Zb, cb, sb, db);
     below = 2 * cb + sb;
   }
-  plane_sums(ec, q, P + cplane * Z, true, c0, s0, d0);
-  for (int z = col.z0; z < col.z1; ++z) {
+  plane_sums(ec, q, P + cplane * Z, c0, s0, d0);
+  auto node = [&](int z) {
+    if (F.ahead && z + 1 + F.ahead < col.z1) {
+      prefetch_l2(u + m.j + F.plane * (1 + F.ahead));
+      prefetch_l2(r + m.j + F.plane * F.ahead);
+      prefetch_l2(code + m.j + F.plane * F.ahead);
+      prefetch_l2(ec + P + cplane * ((z + 1 + F.ahead) >> C.sz));
+    }
     T u0;
     int i;
     const int Zn = (z + 1 == F.nz ? 0 : z + 1) >> C.sz;
     if (Zn != Z) {
-      plane_sums(ec, q, P + cplane * Zn, true, c1, s1, d1);
+      plane_sums(ec, q, P + cplane * Zn, c1, s1, d1);
     } else {
       c1 = c0;
       s1 = s0;
       d1 = d0;
     }
-    const T nu = m.step(u, col.o, col.p, F.plane, F.nz, z, z + 1 < col.z1, u0, i);
+    const T nu = m.step(u, col.o, col.p, F.plane, F.nz, z, u0, i);
     T ne = (2 * s0 + d0) + (below + (2 * c1 + s1));
     const int cd = code[i];
     T v = 0;
@@ -223,6 +245,13 @@ __global__ void __launch_bounds__(256) k_post0(const Cols F, const uint8_t *__re
     s0 = s1;
     d0 = d1;
     Z = Zn;
+  };
+  if (F.ahead) {  // from HBM: several planes' loads in flight
+#pragma unroll 2
+    for (int z = col.z0; z < col.z1; ++z) node(z);
+  } else {
+#pragma unroll 1
+    for (int z = col.z0; z < col.z1; ++z) node(z);
   }
 }
 
@@ -250,6 +279,137 @@ __global__ void __launch_bounds__(kCoarseMax) k_coarsest(const MgLevel L, const 
   if (c && c->inner_done) return;
   __shared__ T buf[2][kCoarseMax];
   coarsest_solve(L, A, r, e, buf);
+}
+
+// --- the bottom of the V-cycle as one matrix ------------------------------------
+// On the levels from ld down the V-cycle is a fixed linear map e = M r of at
+// most kDenseMax nodes.  Its matrix is formed at set-up, one block per column
+// running those levels on a unit vector in shared memory, and applied by
+// one kernel, one warp per row.  As kernels of their own a restriction, the
+// coarsest solve and a post-smoothing take 11 us of launch, ramp and drain
+// for a few thousand nodes of work; one 16-block cluster with barriers
+// between the phases took as long (14 us, and 4 us more per iteration in the
+// graph); the product with a 2048 x 2048 matrix (17 MB, held by L2) takes 6 us,
+// with a 1024 x 1024 one 3.6 us.
+template <typename T>
+constexpr int kDenseMax = sizeof(T) == 4 ? 3072 : 1024;  // FP64: its pipe does 304 products a cycle
+constexpr int kDenseThreads = 512;
+
+template <typename T>
+struct BottomLevel {
+  MgLevel L;
+  const T *A, *W;
+};
+template <typename T>
+struct BottomArgs {
+  BottomLevel<T> lv[kMaxLevels];
+  int ld, nl, stride;
+  const T *cinv;
+  T *M;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kDenseThreads) k_dense_form(const BottomArgs<T> G) {
+  extern __shared__ unsigned char sh_raw[];
+  T *sh = reinterpret_cast<T *>(sh_raw);  // per level: r, then e, z computed on the fly (z = W r)
+  const int col = blockIdx.x;
+  T *r = sh;
+  for (int i = threadIdx.x; i < G.lv[G.ld].L.N; i += blockDim.x) r[i] = i == col ? (T)1 : (T)0;
+  __syncthreads();
+  for (int l = G.ld; l + 1 < G.nl; ++l) {
+    const MgLevel F = G.lv[l].L, C = G.lv[l + 1].L;
+    const T *A = G.lv[l].A, *W = G.lv[l].W;
+    T *rc = r + F.N;
+    for (int I = threadIdx.x; I < C.N; I += blockDim.x) {
+      int X, Y, Z;
+      level_coords(C, I, X, Y, Z);
+      T v = 0;
+      for (int ch = 0; ch < 8; ++ch) {
+        int x, y, z;
+        if (!child_of(C, X, Y, Z, ch, F.nx, F.ny, F.nz, x, y, z)) continue;
+        const int i = x + F.nx * (y + F.ny * z);
+        T s = 0;
+        for (int q = 0; q < 27; ++q) {
+          const int j = wrap(x + q % 3 - 1, F.nx) +
+                        F.nx * (wrap(y + (q / 3) % 3 - 1, F.ny) + F.ny * wrap(z + q / 9 - 1, F.nz));
+          s = fma(A[q * F.S + i], W[j] * r[j], s);
+        }
+        v += r[i] - s;
+      }
+      rc[I] = v;
+    }
+    r = rc;
+    __syncthreads();
+  }
+  const int Nc = G.lv[G.nl - 1].L.N;
+  T *e = r + Nc;
+  for (int i = threadIdx.x; i < Nc; i += blockDim.x) {
+    T s = 0;
+    for (int j = 0; j < Nc; ++j) s = fma(G.cinv[(size_t)j * Nc + i], r[j], s);  // symmetric: coalesced over i
+    e[i] = s;
+  }
+  __syncthreads();
+  for (int l = G.nl - 2; l >= G.ld; --l) {
+    const MgLevel F = G.lv[l].L, C = G.lv[l + 1].L;
+    const T *A = G.lv[l].A, *W = G.lv[l].W;
+    r -= F.N;
+    T *ef = e + C.N;
+    for (int i = threadIdx.x; i < F.N; i += blockDim.x) {
+      int x, y, z;
+      level_coords(F, i, x, y, z);
+      T s = 0;
+      for (int q = 0; q < 27; ++q) {
+        const int jx = wrap(x + q % 3 - 1, F.nx), jy = wrap(y + (q / 3) % 3 - 1, F.ny), jz = wrap(z + q / 9 - 1, F.nz);
+        const int j = jx + F.nx * (jy + F.ny * jz);
+        s = fma(A[q * F.S + i], fma((T)kAlpha, e[agg_index(C, jx, jy, jz)], W[j] * r[j]), s);
+      }
+      const T w = W[i];
+      ef[i] = w != (T)0 ? fma((T)kAlpha, e[agg_index(C, x, y, z)], w * r[i]) + w * (r[i] - s) : (T)0;
+    }
+    e = ef;
+    __syncthreads();
+  }
+  // column col; M is symmetric, stored as rows for the product
+  const int N = G.lv[G.ld].L.N;
+  for (int i = threadIdx.x; i < G.stride; i += blockDim.x)
+    G.M[(size_t)col * G.stride + i] = i < N ? e[i] : (T)0;
+}
+
+// e = M r; rows of `stride` values (a multiple of 16 bytes, zero-padded, as r is)
+template <typename T>
+__global__ void __launch_bounds__(256) k_dense(int N, int stride, const T *__restrict__ M, const T *__restrict__ r,
+                                               T *__restrict__ e, const PoissonCtl *c) {
+  if (c && c->inner_done) return;
+  constexpr int V = 16 / sizeof(T);
+  struct alignas(16) Vec {
+    T v[V];
+  };
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= N) return;
+  const Vec *a = reinterpret_cast<const Vec *>(M + (size_t)row * stride);
+  const Vec *b = reinterpret_cast<const Vec *>(r);
+  T s[V] = {};
+#pragma unroll 8
+  for (int k = lane; k < stride / V; k += 32) {
+    const Vec av = a[k], bv = b[k];
+#pragma unroll
+    for (int q = 0; q < V; ++q) s[q] = fma(av.v[q], bv.v[q], s[q]);
+  }
+  T t = s[0];
+#pragma unroll
+  for (int q = 1; q < V; ++q) t += s[q];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) e[row] = t;
+}
+
+// omega/diag of a level (0 for a node without fluid)
+template <typename T>
+__global__ void k_weights(int N, const T *__restrict__ A13, T *__restrict__ W) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const T d = A13[i];
+  W[i] = d != (T)0 ? (T)kOmega / d : (T)0;
 }
 
 dim3 lgrid(const MgLevel &L, dim3 &block) {
@@ -341,6 +501,38 @@ bool mgd::coarse_inverse(const MgLevel &L, const std::vector<float> &A27, std::v
   return coarse_inverse_t(L, A27, inv);
 }
 
+// the matrix of the V-cycle from the first level of at most kDenseMax nodes
+// down (levels above the coarsest, whose inverse is already a matrix)
+template <typename T>
+static cudaError_t form_dense(lbe_handle *h) {
+  MGWork &mg = h->mg;
+  int ld = mg.nlev - 1;
+  while (ld > 1 && mg.lv[ld - 1].N <= kDenseMax<T>) --ld;
+  if (ld == mg.nlev - 1) return cudaSuccess;
+  const int N = (int)mg.lv[ld].N;
+  constexpr int V = 16 / sizeof(T);
+  BottomArgs<T> G;
+  G.ld = ld;
+  G.nl = mg.nlev;
+  G.stride = (N + V - 1) / V * V;
+  G.cinv = (const T *)mg.cinv;
+  size_t shared = 0;
+  for (int l = ld; l < mg.nlev; ++l) {
+    G.lv[l] = BottomLevel<T>{level_dev(mg.lv[l]), (const T *)mg.lv[l].A, (const T *)mg.lv[l].W};
+    shared += 2 * sizeof(T) * (size_t)mg.lv[l].N;
+  }
+  cudaError_t e = cudaMalloc(&mg.dense, sizeof(T) * (size_t)N * G.stride);
+  if (e != cudaSuccess) return e;
+  G.M = (T *)mg.dense;
+  if (shared > 48 * 1024)
+    e = cudaFuncSetAttribute((const void *)k_dense_form<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared);
+  if (e != cudaSuccess) return e;
+  k_dense_form<T><<<(unsigned)N, kDenseThreads, shared, h->stream>>>(G);
+  mg.ld = ld;
+  mg.stride = G.stride;
+  return cudaGetLastError();
+}
+
 // build the hierarchy for the current geometry (after the link mask)
 template <typename T>
 static cudaError_t mg_setup_t(lbe_handle *h) {
@@ -364,7 +556,10 @@ static cudaError_t mg_setup_t(lbe_handle *h) {
   for (int l = 1; l < mg.nlev && e == cudaSuccess; ++l) {
     MGLevel &L = mg.lv[l];
     e = cudaMalloc(&L.A, sizeof(T) * 27 * L.N);
-    if (e == cudaSuccess) e = cudaMalloc(&L.r, sizeof(T) * L.N);
+    if (e == cudaSuccess) e = cudaMalloc(&L.W, sizeof(T) * L.N);
+    // k_dense reads r in 16-byte words: padded, the padding zero
+    if (e == cudaSuccess) e = cudaMalloc(&L.r, sizeof(T) * (L.N + 4));
+    if (e == cudaSuccess) e = cudaMemsetAsync((T *)L.r + L.N, 0, sizeof(T) * 4, h->stream);
     if (e == cudaSuccess) e = cudaMalloc(&L.e, sizeof(T) * L.N);
     if (e == cudaSuccess) e = cudaMalloc(&L.z, sizeof(T) * L.N);
   }
@@ -384,6 +579,12 @@ static cudaError_t mg_setup_t(lbe_handle *h) {
   }
   cudaError_t le = cudaGetLastError();
   if (le != cudaSuccess) return le;
+  for (int l = 1; l < mg.nlev; ++l)
+    k_weights<T><<<(unsigned)((mg.lv[l].N + 255) / 256), 256, 0, h->stream>>>(
+        (int)mg.lv[l].N, (const T *)mg.lv[l].A + 13 * mg.lv[l].N, (T *)mg.lv[l].W);
+  le = cudaGetLastError();
+  if (le != cudaSuccess) return le;
+  mg.ld = mg.nlev - 1;
   // the coarsest level is solved exactly where its operator is SPD
   // (LBE_MG_DIRECT=0: Jacobi sweeps everywhere)
   const char *denv = getenv("LBE_MG_DIRECT");
@@ -399,6 +600,7 @@ static cudaError_t mg_setup_t(lbe_handle *h) {
         le = cudaMemcpyAsync(mg.cinv, inv.data(), sizeof(T) * inv.size(), cudaMemcpyHostToDevice, h->stream);
       if (le == cudaSuccess) le = cudaStreamSynchronize(h->stream);  // inv is released on return
       if (le != cudaSuccess) return le;
+      return form_dense<T>(h);
     }
   }
   return cudaSuccess;
@@ -409,12 +611,14 @@ void mg_free(lbe_handle *h) {
   MGWork &mg = h->mg;
   for (int l = 0; l < kMaxLevels; ++l) {
     cudaFree(mg.lv[l].A);
+    cudaFree(mg.lv[l].W);
     cudaFree(mg.lv[l].r);
     cudaFree(mg.lv[l].e);
     cudaFree(mg.lv[l].z);
   }
   cudaFree(mg.t0);
   cudaFree(mg.cinv);
+  cudaFree(mg.dense);
   mg = MGWork{};
 }
 
@@ -426,7 +630,7 @@ static cudaError_t mg_vcycle_t(lbe_handle *h, const void *r0, const void *uj, vo
   MGWork &mg = h->mg;
   const int nl = mg.nlev;
   // finest-level kernels: the solve's launch
-  ColLaunch L0 = make_cols(h->geo, h->phys.selfmask, kSolveBlocks);
+  ColLaunch L0 = make_cols(h->geo, h->phys.selfmask);
   // kernel arguments live in these arrays until the nodes are created or the
   // kernels launched
   struct Node {
@@ -444,8 +648,7 @@ static cudaError_t mg_vcycle_t(lbe_handle *h, const void *r0, const void *uj, vo
   };
   for (int l = 1; l < nl; ++l) lv[l] = level_dev(mg.lv[l]);
   // down: restrictions (pre-smoothing on the fly)
-  // level 1: lanes along x, a pair of rows, the rest along z; at most
-  // kSolveBlocks blocks (Kc coarse planes per thread)
+  // level 1: lanes along x, a pair of rows, the rest along z
   RestrictMap M;
   {
     const int nx = h->geo.nx, ny = h->geo.ny;
@@ -457,37 +660,44 @@ static cudaError_t mg_vcycle_t(lbe_handle *h, const void *r0, const void *uj, vo
   const int xt = (h->geo.nx + (1 << M.xl) - 1) >> M.xl, yt = (h->geo.ny + (1 << M.yl) - 1) >> M.yl;
   M.wy = yt < 8 ? pow2_at_least(yt) : 8;
   dim3 rg0;
-  for (M.Kc = 1;; ++M.Kc) {
-    const int per = (8 / M.wy) * (M.Kc << M.zl);  // coarse planes per block
-    rg0 = dim3((unsigned)xt, (unsigned)((yt + M.wy - 1) / M.wy), (unsigned)((lv[1].nz + per - 1) / per));
-    if ((long long)rg0.x * rg0.y * rg0.z <= kSolveBlocks || M.Kc >= lv[1].nz) break;
+  {
+    const int zc = (8 / M.wy) << M.zl, yb = (yt + M.wy - 1) / M.wy;  // chunks per block, blocks along y
+    M.Kc = planes_per_thread((long long)xt * yb, lv[1].nz, zc, 1 + lv[1].sz);
+    const int per = zc * M.Kc;
+    rg0 = dim3((unsigned)xt, (unsigned)yb, (unsigned)((lv[1].nz + per - 1) / per));
   }
   nodes.push_back(Node{(void *)k_restrict0<T>, rg0, dim3(256),
-                       {&L0.c, P(h->code), P(r0), P(uj), &lv[1], P(mg.lv[1].A), P(mg.lv[1].r), P(mg.lv[1].z), &M,
+                       {&L0.c, P(h->code), P(r0), P(uj), &lv[1], P(mg.lv[1].W), P(mg.lv[1].r), P(mg.lv[1].z), &M,
                         P(c)}});
+  // the level whose V-cycle is one matrix (or the coarsest)
+  const int lk = mg.ld;
   // the others: tiles of 32 coarse nodes per block, 2^txl along X (at most
   // 32) and the rest along Y, one plane per block
   int txl[kMaxLevels];
-  for (int l = 1; l < nl - 1; ++l) {
+  for (int l = 1; l < lk; ++l) {
     const MGLevel &Lc = mg.lv[l + 1];
     txl[l] = 0;
     while ((1 << txl[l]) < Lc.nx && txl[l] < 5) ++txl[l];
     const dim3 rg((unsigned)((Lc.nx + (1 << txl[l]) - 1) >> txl[l]),
                   (unsigned)((Lc.ny + (32 >> txl[l]) - 1) / (32 >> txl[l])), (unsigned)Lc.nz);
     nodes.push_back(Node{(void *)k_restrict<T>, rg, dim3(256),
-                         {&lv[l], P(mg.lv[l].A), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1], P(Lc.A), P(Lc.r), P(Lc.z),
+                         {&lv[l], P(mg.lv[l].A), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1], P(Lc.W), P(Lc.r), P(Lc.z),
                           &txl[l], P(c)}});
   }
   // coarsest: exact (inverse) or Jacobi sweeps
   int ncoarse = (int)mg.lv[nl - 1].N;
-  if (mg.cinv)
+  int ndense = (int)mg.lv[lk].N;
+  if (mg.dense) {
+    nodes.push_back(Node{(void *)k_dense<T>, dim3((unsigned)((ndense + 7) / 8)), dim3(256),
+                         {&ndense, &mg.stride, P(mg.dense), P(mg.lv[lk].r), P(mg.lv[lk].e), P(c)}});
+  } else if (mg.cinv)
     nodes.push_back(Node{(void *)k_coarse_direct<T>, dim3((unsigned)((ncoarse + 7) / 8)), dim3(256),
                          {&ncoarse, P(mg.cinv), P(mg.lv[nl - 1].r), P(mg.lv[nl - 1].e), P(c)}});
   else
     nodes.push_back(Node{(void *)k_coarsest<T>, dim3(1), dim3(kCoarseMax),
                          {&lv[nl - 1], P(mg.lv[nl - 1].A), P(mg.lv[nl - 1].r), P(mg.lv[nl - 1].e), P(c)}});
   // up: fused prolongation + post-smoothing
-  for (int l = nl - 2; l >= 1; --l) {
+  for (int l = lk - 1; l >= 1; --l) {
     dim3 blk;
     const dim3 grd = lgrid(lv[l], blk);
     nodes.push_back(Node{(void *)k_post<T>, grd, blk,
@@ -523,6 +733,10 @@ cudaError_t mg_vcycle(lbe_handle *h, const void *r0, const void *uj, void *u0, c
 }
 
 // kernels of one V-cycle (launch accounting of the graph path)
-int mg_kernels_per_cycle(const lbe_handle *h) { return h->mg.nlev >= 2 ? 2 * (h->mg.nlev - 1) + 1 : 0; }
+int mg_kernels_per_cycle(const lbe_handle *h) {
+  const MGWork &mg = h->mg;
+  if (mg.nlev < 2) return 0;
+  return 2 * mg.ld + 1;
+}
 
 }  // namespace lbe

@@ -220,16 +220,6 @@ __device__ __forceinline__ void coarsest_solve(const MgLevel &L, const T *__rest
 }
 
 
-// a coarse node's restricted residual rc and pre-smoothed iterate
-// zc = omega rc/diag
-template <typename T>
-__device__ __forceinline__ void store_coarse(const MgLevel &C, int I, T v, const T *__restrict__ AC,
-                                             T *__restrict__ rc, T *__restrict__ zc) {
-  const T d = AC[13 * C.S + I];
-  rc[I] = v;
-  zc[I] = d != (T)0 ? kOmega * v / d : (T)0;
-}
-
 // --- forms with integer link weights and a stored pre-smoothed iterate -------
 // The modified Laplacian's link weights 1/3 (axis) and 1/6 (diagonal) are
 // 2/6 and 1/6: sums of weights are integers over 6, and a node's diagonal
@@ -283,11 +273,11 @@ template <typename T>
 __device__ __forceinline__ T presmoothed_res_z(const MgLevel &L, const T *__restrict__ A,
                                                const T *__restrict__ r, const T *__restrict__ z, int X,
                                                int Y, int Z) {
+  // a node without fluid has a zero row and a zero residual; no branch
   const int I = X + L.nx * (Y + L.ny * Z);
-  if (A[13 * L.S + I] == (T)0) return (T)0;
   T s = 0;
 #pragma unroll
-  for (int d = 0; d < 27; ++d) {  // a zero coefficient adds nothing; no branch
+  for (int d = 0; d < 27; ++d) {
     const T a = A[d * L.S + I];
     const int jx = wrap(X + d % 3 - 1, L.nx), jy = wrap(Y + (d / 3) % 3 - 1, L.ny), jz = wrap(Z + d / 9 - 1, L.nz);
     s = fma(a, z[jx + L.nx * (jy + L.ny * jz)], s);
