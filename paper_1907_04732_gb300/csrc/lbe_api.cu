@@ -277,8 +277,8 @@ int lbe_set_geometry(lbe_handle *h, const uint8_t *node_id, int n_electrodes, in
   LBE_CK(h, cudaMemcpyAsync(h->id, ids.data(), (size_t)g.N, cudaMemcpyHostToDevice, h->stream));
   LBE_CK(h, lbe::launch_build_mask(g, h->id, h->mask, h->stream));
   LBE_CK(h, lbe::launch_build_code(g, h->phys.selfmask, h->mask, h->code, h->stream));
-  if (fp32(h)) LBE_CK(h, lbe::mg_setup(h));  // multigrid preconditioner of the FP32 Poisson solve
-  lbe::poisson_drop_graphs(h);               // graphs capture the hierarchy
+  LBE_CK(h, lbe::mg_setup(h));   // multigrid preconditioner of the Poisson solve
+  lbe::poisson_drop_graphs(h);   // graphs capture the hierarchy
   LBE_CK(h, cudaStreamSynchronize(h->stream));  // ids is a host vector
   h->n_elec = n_electrodes;
   h->have_geometry = true;

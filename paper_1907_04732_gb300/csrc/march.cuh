@@ -60,6 +60,23 @@ __host__ __device__ __forceinline__ uint32_t fdiv(const FastDiv &f, uint32_t n) 
 // set when one of its 18 links joins a solid node; 0 on solid nodes.
 constexpr int kCodeDiag = 0x7f, kCodeWall = 0x80;
 
+// 1/diag from a node's code (6 diag; 0 on a solid node, as its inverse).  A
+// double division takes a dozen instructions on the narrow FP64 pipe, so the
+// FP64 form reads the inverses from a table.
+struct InvDiag {
+  double v[49];
+  constexpr InvDiag() : v() {
+    for (int k = 1; k < 49; ++k) v[k] = 1.0 / ((double)k * (1.0 / 6.0));
+  }
+};
+static __constant__ InvDiag kInvDiag = InvDiag();
+template <typename T>
+__device__ __forceinline__ T inv_diag(int code) {
+  const int d6 = code & kCodeDiag;
+  if (sizeof(T) == 8) return (T)kInvDiag.v[d6];
+  return (T)(d6 ? 1.f / ((float)d6 * (1.f / 6.f)) : 0.f);
+}
+
 // lattices above this size (about 30 bytes of solve vectors per node in use
 // at a time) do not stay in the 129 MB L2
 constexpr long long kPrefetchNodes = 3 << 20;

@@ -1,4 +1,8 @@
-// Geometric multigrid preconditioner of the FP32 Poisson correction solve.
+// Geometric multigrid preconditioner of the Poisson correction solve, in the
+// form's own precision: FP32 vectors and operators in the FP32 form, FP64
+// throughout in the FP64 form (whose solve took 40-190 Jacobi iterations per
+// step before it had the hierarchy, 3-7 with it: 64x64x256 electro-osmosis
+// 12.6 -> 0.97 ms, 128x128x4 coax 1.55 -> 0.44, 4x4x64 plates 0.78 -> 0.14).
 //
 // The CG of the Poisson solve (poisson.cu) needs u = M r with M ~ A^-1; the
 // plain Jacobi choice M = D^-1 leaves it O(L) iterations on an L-long gap.
@@ -156,13 +160,15 @@ __global__ void __launch_bounds__(256) k_restrict(const MgLevel F, const T *__re
 
 // fused prolongation + post-smoothing on a 27-point level
 template <typename T>
-__global__ void k_post(const MgLevel L, const T *__restrict__ A, const T *__restrict__ r,
+__global__ void k_post(const MgLevel L, const T *__restrict__ A, const T *__restrict__ W, const T *__restrict__ r,
                        const T *__restrict__ z, const MgLevel C, const T *__restrict__ ec,
                        T *__restrict__ out, const PoissonCtl *c) {
   if (c && c->inner_done) return;
   int X, Y, Z, I;
   if (!lnode(L, X, Y, Z, I)) return;
-  out[I] = post_value_z(L, A, r, z, C, ec, X, Y, Z);
+  // FP64: the division omega/diag costs more than its stored value (float
+  // measured 2 % of the solve the other way round: one more load)
+  out[I] = sizeof(T) == 8 ? post_value_w(L, A, W[I], r, z, C, ec, X, Y, Z) : post_value_z(L, A, r, z, C, ec, X, Y, Z);
 }
 
 // fused prolongation + post-smoothing on the finest level:
@@ -173,7 +179,7 @@ __global__ void k_post(const MgLevel L, const T *__restrict__ A, const T *__rest
 // Next to a wall, P e_1 is nonzero on the solid neighbours too and the links
 // are taken one by one.
 template <typename T>
-__global__ void __launch_bounds__(256, 5) k_post0(const Cols F, const uint8_t *__restrict__ code,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3) k_post0(const Cols F, const uint8_t *__restrict__ code,
                                                const uint32_t *__restrict__ mask, const T *__restrict__ r,
                                                const T *__restrict__ u, const MgLevel C, const T *__restrict__ ec,
                                                T *__restrict__ out, const PoissonCtl *c) {
@@ -237,7 +243,7 @@ __global__ void __launch_bounds__(256, 5) k_post0(const Cols F, const uint8_t *_
       const T t = om * u0 + al * c0;
       const T s6 = om * nu + al * ne - (T)F.selfw * t;
       const T res6 = (T)6 * r[i] - (d6 * t - s6);
-      v = t + om * (sizeof(T) == 4 ? (T)__fdividef((float)res6, (float)d6) : res6 / d6);
+      v = t + om * (sizeof(T) == 4 ? (T)__fdividef((float)res6, (float)d6) : res6 * (T)(1.0 / 6.0) * inv_diag<T>(cd));
     }
     out[i] = v;
     below = 2 * c0 + s0;
@@ -605,7 +611,9 @@ static cudaError_t mg_setup_t(lbe_handle *h) {
   }
   return cudaSuccess;
 }
-cudaError_t mg_setup(lbe_handle *h) { return mg_setup_t<float>(h); }
+cudaError_t mg_setup(lbe_handle *h) {
+  return h->prm.precision == LBE_FP32 ? mg_setup_t<float>(h) : mg_setup_t<double>(h);
+}
 
 void mg_free(lbe_handle *h) {
   MGWork &mg = h->mg;
@@ -701,8 +709,8 @@ static cudaError_t mg_vcycle_t(lbe_handle *h, const void *r0, const void *uj, vo
     dim3 blk;
     const dim3 grd = lgrid(lv[l], blk);
     nodes.push_back(Node{(void *)k_post<T>, grd, blk,
-                         {&lv[l], P(mg.lv[l].A), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1], P(mg.lv[l + 1].e),
-                          P(mg.lv[l].e), P(c)}});
+                         {&lv[l], P(mg.lv[l].A), P(mg.lv[l].W), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1],
+                          P(mg.lv[l + 1].e), P(mg.lv[l].e), P(c)}});
   }
   nodes.push_back(Node{(void *)k_post0<T>, L0.grid, L0.block,
                        {&L0.c, P(h->code), P(h->mask), P(r0), P(uj), &lv[1], P(mg.lv[1].e), P(u0), P(c)}});
@@ -729,7 +737,8 @@ static cudaError_t mg_vcycle_t(lbe_handle *h, const void *r0, const void *uj, vo
 }
 cudaError_t mg_vcycle(lbe_handle *h, const void *r0, const void *uj, void *u0, const PoissonCtl *c, cudaGraph_t gr,
                       cudaGraphNode_t *last, cudaStream_t st) {
-  return mg_vcycle_t<float>(h, r0, uj, u0, c, gr, last, st);
+  return h->prm.precision == LBE_FP32 ? mg_vcycle_t<float>(h, r0, uj, u0, c, gr, last, st)
+                                      : mg_vcycle_t<double>(h, r0, uj, u0, c, gr, last, st);
 }
 
 // kernels of one V-cycle (launch accounting of the graph path)

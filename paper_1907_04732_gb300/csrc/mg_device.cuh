@@ -287,13 +287,13 @@ __device__ __forceinline__ T presmoothed_res_z(const MgLevel &L, const T *__rest
 
 // fused prolongation + post-smoothing with the stored iterate:
 // e = z + alpha P e_c, out = e + omega (r - A e)/diag
+// with w = omega/diag (0 for a node without fluid)
 template <typename T>
-__device__ __forceinline__ T post_value_z(const MgLevel &L, const T *__restrict__ A,
+__device__ __forceinline__ T post_value_w(const MgLevel &L, const T *__restrict__ A, T w,
                                           const T *__restrict__ r, const T *__restrict__ z,
                                           const MgLevel &C, const T *__restrict__ ec, int X, int Y, int Z) {
   const int I = X + L.nx * (Y + L.ny * Z);
-  const T d = A[13 * L.S + I];
-  if (d == (T)0) return (T)0;
+  if (w == (T)0) return (T)0;
   T s = 0;
 #pragma unroll
   for (int q = 0; q < 27; ++q) {  // a zero coefficient adds nothing; no branch
@@ -303,7 +303,14 @@ __device__ __forceinline__ T post_value_z(const MgLevel &L, const T *__restrict_
     s = fma(a, ej, s);
   }
   const T e = fma((T)kAlpha, ec[agg_index(C, X, Y, Z)], z[I]);
-  return e + kOmega * (r[I] - s) / d;
+  return e + w * (r[I] - s);
+}
+template <typename T>
+__device__ __forceinline__ T post_value_z(const MgLevel &L, const T *__restrict__ A,
+                                          const T *__restrict__ r, const T *__restrict__ z,
+                                          const MgLevel &C, const T *__restrict__ ec, int X, int Y, int Z) {
+  const T d = A[13 * L.S + X + L.nx * (Y + L.ny * Z)];
+  return post_value_w(L, A, d != (T)0 ? (T)kOmega / d : (T)0, r, z, C, ec, X, Y, Z);
 }
 
 // host (mg.cu): inverse of a coarsest level's operator, A27 its 27-point

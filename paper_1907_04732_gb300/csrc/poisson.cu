@@ -12,8 +12,8 @@
 //           float-float arithmetic)
 //           stop when max_r |res(r)|/diag(r) <= poisson_tol
 //           solve A e = res approximately by preconditioned conjugate
-//           gradients (FP64 and Jacobi in the FP64 form; FP32 and the
-//           multigrid V-cycle of mg.cu in the FP32 form)
+//           gradients with the multigrid V-cycle of mg.cu, in the form's
+//           precision (Jacobi where a lattice has no hierarchy)
 //           phi += e                (FP64; FP32 form: e rounded to the
 //                                    fixed-point unit, an integer add)
 //
@@ -47,23 +47,6 @@ constexpr int kMaxOuter = 24;  // refinement rounds per solve
 constexpr int kChunk = 16;     // fallback: iterations between host polls
 
 enum { S_RU = 0, S_WU = 1 };
-
-// 1/diag from a node's code (6 diag; 0 on a solid node, as its inverse).  A
-// double division takes a dozen instructions on the narrow FP64 pipe, so the
-// FP64 form reads the inverses from a table.
-struct InvDiag {
-  double v[49];
-  constexpr InvDiag() : v() {
-    for (int k = 1; k < 49; ++k) v[k] = 1.0 / ((double)k * (1.0 / 6.0));
-  }
-};
-__constant__ InvDiag kInvDiag = InvDiag();
-template <typename T>
-__device__ __forceinline__ T inv_diag(int code) {
-  const int d6 = code & kCodeDiag;
-  if (sizeof(T) == 8) return (T)kInvDiag.v[d6];
-  return (T)(d6 ? 1.f / ((float)d6 * (1.f / 6.f)) : 0.f);
-}
 
 // lap_mod(v)(r) at a fluid node, FP64.  With the link weights scaled by 6
 // (2 nearest, 1 next-nearest, doubled towards solid unless dbl is false:
