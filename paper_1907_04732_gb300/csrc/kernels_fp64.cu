@@ -88,99 +88,214 @@ __global__ void k_set_solid_phi(const Geo g, const uint8_t *__restrict__ id, con
   if (id[r]) phi[r] = psi[id[r]];
 }
 
-// Link fluxes of Eq. LF2 in the relative form
-//   j = -d/|c| * (1 + e^{-dmu})/2 * (n' e^{dmu} - n),
-// dmu = z (phi' - phi - E.c); the solute update n* = n - sum_i j; the link
-// excess flux g = j/d + (n' - n)/|c| summed into the solvent force
-// F = (1/(2 A0)) sum_i c_i sum_k g.
-__device__ __forceinline__ void ion_fluxes(const Geo &g, const Phys &P, long long r, int x, int y, int z,
-                                           uint32_t m, const double *__restrict__ n,
-                                           const double *__restrict__ phi, double *nstar_r, double F[3]) {
-  const double phi0 = phi[r];
-  double n0[LBE_MAX_SPECIES];
-  for (int k = 0; k < P.ns; ++k) {
-    n0[k] = n[k * g.N + r];
-    nstar_r[k] = n0[k];
+// sinh x and cosh x - 1, odd and even in x exactly: Taylor series to x^7 and
+// x^8 for |x| < 1/64 (most links: a kT/e over the Debye length), to x^11 and
+// x^12 for |x| < 1/4, each truncated below 2e-17 relative; beyond that from
+// expm1, out of line.  The ranges are tested on the high word, without the
+// FP64 pipe.
+static __device__ __noinline__ double2 shch_wide(double x) {
+  const double ep = expm1(x), em = expm1(-x);
+  return make_double2(0.5 * (ep - em), 0.5 * (ep + em));
+}
+__device__ __forceinline__ void shch(double x, double &sh, double &ch) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  if (hi < 0x3fd00000) {
+    const double x2 = x * x;
+    double p = 1.0 / 5040.0, q = 1.0 / 40320.0;
+    if (hi >= 0x3f900000) {
+      p = fma(fma(1.0 / 39916800.0, x2, 1.0 / 362880.0), x2, p);
+      q = fma(fma(1.0 / 479001600.0, x2, 1.0 / 3628800.0), x2, q);
+    }
+    p = fma(p, x2, 1.0 / 120.0);
+    q = fma(q, x2, 1.0 / 720.0);
+    p = fma(p, x2, 1.0 / 6.0);
+    q = fma(q, x2, 1.0 / 24.0);
+    p = fma(p, x2, 1.0);
+    q = fma(q, x2, 0.5);
+    sh = p * x;
+    ch = q * x2;
+  } else {
+    const double2 w = shch_wide(x);
+    sh = w.x;
+    ch = w.y;
   }
-  F[0] = F[1] = F[2] = 0.0;
+}
+
+// Link fluxes of Eq. LF2 and the solvent force.  With dmu = z (phi' - phi -
+// E.c), S = n + n' and D = n' - n,
+//   A = n' (e^{dmu} - 1) - n (e^{-dmu} - 1) = S sinh(dmu) + D (cosh(dmu) - 1)
+//   J = n' (1 + e^{dmu}) - n (1 + e^{-dmu}) = 2 D + A
+// the flux is j = -d J/(2|c|) and the link excess flux g = j/d + D/|c| =
+// -A/(2|c|) (D/|c| for an immobile species), summed into the force
+// F = (1/(2 A0)) sum_i c_i sum_k g.  n* = n - sum_i j.  Every term is odd
+// under reversal of the link, so its two ends move exactly opposite amounts.
+// One series serves the species of valence +1 and -1.  Bound by the FP64
+// pipe (1/64 of the FP32 rate): about 30 FP64 instructions per link of a 1:1
+// salt against 80 with an exponential and two divisions per species, and
+// no cancellation between n' e^{dmu} and n.  Axis and diagonal links are
+// summed apart, so that 1/|c| multiplies once.
+__device__ __forceinline__ void ion_fluxes(const Geo &g, const Phys &P, int r, const Offs &o, uint32_t m,
+                                           const double *__restrict__ n, const double *__restrict__ phi,
+                                           double *nstar_r, double F[3]) {
+  const double phi0 = phi[r];
+  double n0[LBE_MAX_SPECIES], acc1[LBE_MAX_SPECIES], acc2[LBE_MAX_SPECIES];
+  // per species: valence +1, -1 or another, and immobile (whole-word tests of
+  // the constants: a double comparison per link would run on the FP64 pipe)
+  int kind[LBE_MAX_SPECIES];
+  bool immobile[LBE_MAX_SPECIES];
+#pragma unroll
+  for (int k = 0; k < LBE_MAX_SPECIES; ++k) {
+    n0[k] = k < P.ns ? n[k * g.N + r] : 0.0;
+    acc1[k] = acc2[k] = 0.0;
+    const int zh = __double2hiint(P.z[k]);
+    kind[k] = zh == 0x3ff00000 ? 1 : (zh == (int)0xbff00000 ? -1 : 0);  // |z| is an integer below 5
+    immobile[k] = __double_as_longlong(P.inv_d[k]) == 0;
+  }
+  double Fa[3] = {0.0, 0.0, 0.0}, Fd[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int i = 1; i < kQ; ++i) {
     if (!(m & (1u << (i - 1)))) continue;
-    const long long r2 = nbr_i(g, x, y, z, i);
-    const double dphi = phi[r2] - phi0 - P.e_dot_c[i];
-    double gsum = 0.0;
-    for (int k = 0; k < P.ns; ++k) {
+    const int r2 = r + o.at(cx_of(i), cy_of(i), cz_of(i));
+    const double x = phi[r2] - phi0 - P.e_dot_c[i];
+    double sh, ch;
+    shch(x, sh, ch);
+    double gsum = 0.0;  // sum over species of -2 |c| g
+#pragma unroll
+    for (int k = 0; k < LBE_MAX_SPECIES; ++k) {
+      if (k >= P.ns) break;
       const double n1 = n[k * g.N + r2];
-      const double dmu = P.z[k] * dphi;
-      const double e = exp(dmu);
-      const double j = -P.d[k] * invlen_of(i) * 0.5 * (1.0 + 1.0 / e) * (n1 * e - n0[k]);
-      nstar_r[k] -= j;
-      gsum += j * P.inv_d[k] + (n1 - n0[k]) * invlen_of(i);
+      const double D = n1 - n0[k], S = n1 + n0[k];
+      double A;
+      if (kind[k] > 0) {
+        A = fma(S, sh, D * ch);
+      } else if (kind[k] < 0) {
+        A = fma(-S, sh, D * ch);
+      } else {
+        double s, c;
+        shch(P.z[k] * x, s, c);
+        A = fma(S, s, D * c);
+      }
+      const double J = fma(2.0, D, A);
+      if (c2_of(i) == 1) acc1[k] += J;
+      else acc2[k] += J;
+      if (immobile[k]) A = -2.0 * D;
+      gsum += A;
     }
-    F[0] += cx_of(i) * gsum;
-    F[1] += cy_of(i) * gsum;
-    F[2] += cz_of(i) * gsum;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int ca = a == 0 ? cx_of(i) : (a == 1 ? cy_of(i) : cz_of(i));
+      if (ca == 0) continue;
+      double &f = c2_of(i) == 1 ? Fa[a] : Fd[a];
+      f = ca > 0 ? f - gsum : f + gsum;
+    }
   }
-  F[0] *= P.inv_2a0;
-  F[1] *= P.inv_2a0;
-  F[2] *= P.inv_2a0;
+  constexpr double il = 0.70710678118654752440;  // 1/|c| of a diagonal link
+#pragma unroll
+  for (int k = 0; k < LBE_MAX_SPECIES; ++k)
+    if (k < P.ns) nstar_r[k] = fma(0.5 * P.d[k], fma(il, acc2[k], acc1[k]), n0[k]);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) F[a] = (0.5 * P.inv_2a0) * fma(il, Fd[a], Fa[a]);
 }
 
 // Pull streaming: population i at r comes from r - c_i = r + c_opp(i) if that
 // node is fluid, else it is the population opp(i) that left r towards the
 // wall and was bounced back (halfway bounce-back).
-__device__ __forceinline__ void gather(const Geo &g, long long r, int x, int y, int z, uint32_t m,
+__device__ __forceinline__ void gather(const Geo &g, int r, const Offs &o, uint32_t m,
                                        const double *__restrict__ fin, double f[kQ]) {
   f[0] = fin[r];
 #pragma unroll
   for (int i = 1; i < kQ; ++i) {
     const int io = opp_of(i);
     if (m & (1u << (io - 1)))
-      f[i] = fin[i * g.N + nbr_i(g, x, y, z, io)];
+      f[i] = fin[i * g.N + (r + o.at(cx_of(io), cy_of(io), cz_of(io)))];
     else
       f[i] = fin[io * g.N + r];
   }
 }
 
+// Nodes of the FP64 sweep and advection: flattened, in blocks so small that
+// even a lattice of a thousand nodes spreads over the SMs (their FP64 pipes
+// bound both kernels: 4x4x64 in four blocks of 256 took 71 and 21 us).
+struct FlatGeo {
+  Geo g;
+  FastDiv fx, fxy;
+};
+inline FlatGeo flat_geo(const Geo &g) {
+  return FlatGeo{g, make_fastdiv((uint32_t)g.nx), make_fastdiv((uint32_t)((long long)g.nx * g.ny))};
+}
+inline unsigned flat_block(const Geo &g) { return g.N < 32768 ? 32 : 128; }
+inline unsigned flat_grid(const Geo &g) { return (unsigned)((g.N + flat_block(g) - 1) / flat_block(g)); }
+__device__ __forceinline__ bool flat_node(const FlatGeo &G, int &x, int &y, int &z, int &r) {
+  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= G.g.N) return false;
+  r = (int)i;
+  z = (int)fdiv(G.fxy, i);
+  const int rem = r - z * (int)G.fxy.d;
+  y = (int)fdiv(G.fx, (uint32_t)rem);
+  x = rem - y * G.g.nx;
+  return true;
+}
+
+// Fused step at a fluid node.  The collision takes the pairs c_i, -c_i
+// together (even and odd parts of equilibrium and Guo source):
+//   f'_i = (1 - omega) f_i + E_even +- E_odd,
+//   E_even = w [omega rho (1 + 4.5 cu^2 - 1.5 uu) + guo (9 cu cF - 3 uF)]
+//   E_odd  = w [3 omega rho cu + 3 guo cF]
+// The kernel is bound by the FP64 pipe: on the 64x64x256 lattice 1.57 ms,
+// against 3.14 ms with an exponential and divisions per link and species and
+// one population at a time (4x4x64: 42 against 125 us).
 template <bool FLOW>
-__global__ void __launch_bounds__(kBlock) k_sweep(const Geo g, const Phys P, const uint32_t *__restrict__ mask,
-                                                  const double *__restrict__ fin, double *__restrict__ fout,
-                                                  const double *__restrict__ n, double *__restrict__ nstar,
-                                                  const double *__restrict__ phi, double *__restrict__ u) {
-  int x, y, z;
-  long long r;
-  if (!node_of(g, 1, 0, x, y, z, r)) return;
+__global__ void __launch_bounds__(128) k_sweep(const FlatGeo G, const Phys P, const uint32_t *__restrict__ mask,
+                                               const double *__restrict__ fin, double *__restrict__ fout,
+                                               const double *__restrict__ n, double *__restrict__ nstar,
+                                               const double *__restrict__ phi, double *__restrict__ u) {
+  const Geo &g = G.g;
+  int x, y, z, r;
+  if (!flat_node(G, x, y, z, r)) return;
   const uint32_t m = mask[r];
   if (!(m & kFluidBit)) return;
+  const Offs o = offsets_of(g, x, y, z);
   double ns_r[LBE_MAX_SPECIES];
   double F[3];
-  ion_fluxes(g, P, r, x, y, z, m, n, phi, ns_r, F);
-  for (int k = 0; k < P.ns; ++k) nstar[k * g.N + r] = ns_r[k];
+  ion_fluxes(g, P, r, o, m, n, phi, ns_r, F);
+#pragma unroll
+  for (int k = 0; k < LBE_MAX_SPECIES; ++k)
+    if (k < P.ns) nstar[k * g.N + r] = ns_r[k];
   if (!FLOW) return;
 
   double f[kQ];
-  gather(g, r, x, y, z, m, fin, f);
-  double rho = 0.0, mx = 0.0, my = 0.0, mz = 0.0;
+  gather(g, r, o, m, fin, f);
+  double rho = f[0], mx = 0.0, my = 0.0, mz = 0.0;
 #pragma unroll
-  for (int i = 0; i < kQ; ++i) {
-    rho += f[i];
-    mx += cx_of(i) * f[i];
-    my += cy_of(i) * f[i];
-    mz += cz_of(i) * f[i];
+  for (int i = 1; i <= 9; ++i) {
+    const double d = f[i] - f[i + 9];
+    rho += f[i] + f[i + 9];
+    if (cx_of(i)) mx += d;  // c_1..c_9 have c_x >= 0
+    if (cy_of(i)) my = cy_of(i) > 0 ? my + d : my - d;
+    if (cz_of(i)) mz = cz_of(i) > 0 ? mz + d : mz - d;
   }
-  const double ux = (mx + 0.5 * F[0]) / rho, uy = (my + 0.5 * F[1]) / rho, uz = (mz + 0.5 * F[2]) / rho;
+  const double inv_rho = 1.0 / rho;
+  const double ux = fma(0.5, F[0], mx) * inv_rho, uy = fma(0.5, F[1], my) * inv_rho,
+               uz = fma(0.5, F[2], mz) * inv_rho;
   u[r] = ux;
   u[g.N + r] = uy;
   u[2 * g.N + r] = uz;
   const double uu = ux * ux + uy * uy + uz * uz;
+  const double uF = ux * F[0] + uy * F[1] + uz * F[2];
+  const double om = P.omega, gu = P.guo, keep = 1.0 - om;
+  const double omr = om * rho;
+  const double base = fma(omr, fma(-1.5, uu, 1.0), -3.0 * gu * uF);  // E_even / w at cu = cF = 0
+  const double b2 = 4.5 * omr, d2 = 3.0 * omr, g3 = 3.0 * gu, g9 = 9.0 * gu;
+  fout[r] = fma(keep, f[0], w_of(0) * base);
 #pragma unroll
-  for (int i = 0; i < kQ; ++i) {
+  for (int i = 1; i <= 9; ++i) {
     const double cu = cx_of(i) * ux + cy_of(i) * uy + cz_of(i) * uz;
-    const double feq = w_of(i) * rho * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
     const double cF = cx_of(i) * F[0] + cy_of(i) * F[1] + cz_of(i) * F[2];
-    const double uF = ux * F[0] + uy * F[1] + uz * F[2];
-    const double src = P.guo * w_of(i) * (3.0 * (cF - uF) + 9.0 * cu * cF);
-    fout[i * g.N + r] = f[i] - P.omega * (f[i] - feq) + src;
+    const double ee = w_of(i) * fma(cu, fma(b2, cu, g9 * cF), base);
+    const double eo = w_of(i) * fma(d2, cu, g3 * cF);
+    const int io = i + 9;
+    fout[i * g.N + r] = fma(keep, f[i], ee + eo);
+    fout[io * g.N + r] = fma(keep, f[io], ee - eo);
   }
 }
 
@@ -192,47 +307,65 @@ __device__ __forceinline__ double ov(int s, double u) {
   return s == 0 ? 1.0 - fabs(u) : (s > 0 ? fmax(u, 0.0) : fmax(-u, 0.0));
 }
 
-__device__ __forceinline__ int dir_bit(int dx, int dy, int dz) {
+__host__ __device__ constexpr int dir_bit(int dx, int dy, int dz) {
   // bit of the mask for the neighbour at offset (dx,dy,dz) != 0
   if (dx != 0 && dy != 0 && dz != 0) return corner_bit(dx, dy, dz);
-#pragma unroll
   for (int i = 1; i < kQ; ++i)
     if (cx_of(i) == dx && cy_of(i) == dy && cz_of(i) == dz) return i - 1;
   return -1;
 }
 
-__global__ void __launch_bounds__(kBlock) k_advect(const Geo g, int ns, const uint32_t *__restrict__ mask,
-                                                   const double *__restrict__ nin, const double *__restrict__ u,
-                                                   double *__restrict__ nout) {
-  int x, y, z;
-  long long r;
-  if (!node_of(g, 1, 0, x, y, z, r)) return;
+// the overlap at offset s can be nonzero: u has the sign of s (or s = 0); from
+// the bits, without the FP64 pipe
+__device__ __forceinline__ bool reaches(int s, double u) {
+  return s == 0 || (s > 0 ? __double_as_longlong(u) > 0 : __double2hiint(u) < 0);
+}
+
+// A displaced cell only reaches the octant its velocity points to, so most
+// sources are dismissed by the signs of their velocity before any FP64
+// arithmetic (64x64x256: 0.32 ms, 0.49 when every overlap was evaluated).
+__global__ void __launch_bounds__(128) k_advect(const FlatGeo G, int ns, const uint32_t *__restrict__ mask,
+                                                const double *__restrict__ nin, const double *__restrict__ u,
+                                                double *__restrict__ nout) {
+  const Geo &g = G.g;
+  int x, y, z, r;
+  if (!flat_node(G, x, y, z, r)) return;
   const uint32_t m = mask[r];
   if (!(m & kFluidBit)) {
     for (int k = 0; k < ns; ++k) nout[k * g.N + r] = 0.0;
     return;
   }
+  const Offs o = offsets_of(g, x, y, z);
   double acc[LBE_MAX_SPECIES] = {0.0, 0.0, 0.0, 0.0};
   const double ux = u[r], uy = u[g.N + r], uz = u[2 * g.N + r];
   double keep = 0.0;  // own shares bound for solid neighbours
-  for (int dz = -1; dz <= 1; ++dz)
-    for (int dy = -1; dy <= 1; ++dy)
-      for (int dx = -1; dx <= 1; ++dx) {
-        if (dx == 0 && dy == 0 && dz == 0) {
-          const double w = ov(0, ux) * ov(0, uy) * ov(0, uz);
-          for (int k = 0; k < ns; ++k) acc[k] += w * nin[k * g.N + r];
-          continue;
-        }
-        // source q = r - s exists as fluid iff the neighbour at -s is fluid
-        if (m & (1u << dir_bit(-dx, -dy, -dz))) {
-          const long long q = nbr(g, x, y, z, -dx, -dy, -dz);
-          const double w = ov(dx, u[q]) * ov(dy, u[g.N + q]) * ov(dz, u[2 * g.N + q]);
-          if (w != 0.0)
-            for (int k = 0; k < ns; ++k) acc[k] += w * nin[k * g.N + q];
-        }
-        if (!(m & (1u << dir_bit(dx, dy, dz)))) keep += ov(dx, ux) * ov(dy, uy) * ov(dz, uz);
+#pragma unroll
+  for (int d = 0; d < 27; ++d) {
+    const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
+    if (d == 13) {
+      const double w = ov(0, ux) * ov(0, uy) * ov(0, uz);
+#pragma unroll
+      for (int k = 0; k < LBE_MAX_SPECIES; ++k)
+        if (k < ns) acc[k] += w * nin[k * g.N + r];
+      continue;
+    }
+    // source q = r - s exists as fluid iff the neighbour at -s is fluid
+    if (m & (1u << dir_bit(-dx, -dy, -dz))) {
+      const int q = r + o.at(-dx, -dy, -dz);
+      const double vx = u[q], vy = u[g.N + q], vz = u[2 * g.N + q];
+      if (reaches(dx, vx) && reaches(dy, vy) && reaches(dz, vz)) {
+        const double w = ov(dx, vx) * ov(dy, vy) * ov(dz, vz);
+#pragma unroll
+        for (int k = 0; k < LBE_MAX_SPECIES; ++k)
+          if (k < ns) acc[k] += w * nin[k * g.N + q];
       }
-  for (int k = 0; k < ns; ++k) nout[k * g.N + r] = acc[k] + keep * nin[k * g.N + r];
+    }
+    if (!(m & (1u << dir_bit(dx, dy, dz))) && reaches(dx, ux) && reaches(dy, uy) && reaches(dz, uz))
+      keep += ov(dx, ux) * ov(dy, uy) * ov(dz, uz);
+  }
+#pragma unroll
+  for (int k = 0; k < LBE_MAX_SPECIES; ++k)
+    if (k < ns) nout[k * g.N + r] = acc[k] + keep * nin[k * g.N + r];
 }
 
 // Velocity and density of the current state, (sum f c + F/2)/rho with F from
@@ -250,10 +383,11 @@ __global__ void k_moments(const Geo g, const Phys P, int flow, const uint32_t *_
     if (u_out) u_out[r] = u_out[g.N + r] = u_out[2 * g.N + r] = 0.0;
     return;
   }
+  const Offs o = offsets_of(g, x, y, z);
   double ns_r[LBE_MAX_SPECIES], F[3];
-  ion_fluxes(g, P, r, x, y, z, m, n, phi, ns_r, F);
+  ion_fluxes(g, P, (int)r, o, m, n, phi, ns_r, F);
   double f[kQ];
-  gather(g, r, x, y, z, m, fin, f);
+  gather(g, (int)r, o, m, fin, f);
   double rho = 0.0, mx = 0.0, my = 0.0, mz = 0.0;
   for (int i = 0; i < kQ; ++i) {
     rho += f[i];
@@ -280,7 +414,7 @@ __global__ void k_gather_f(const Geo g, const uint32_t *__restrict__ mask, const
     return;
   }
   double f[kQ];
-  gather(g, r, x, y, z, m, fin, f);
+  gather(g, (int)r, offsets_of(g, x, y, z), m, fin, f);
   for (int i = 0; i < kQ; ++i) out[i * g.N + r] = f[i];
 }
 
@@ -404,18 +538,16 @@ cudaError_t launch_set_solid_phi(lbe_handle *h) {
 
 cudaError_t launch_sweep(lbe_handle *h) {
   const int nxt = h->cur ^ 1;
-  if (h->prm.flow)
-    k_sweep<true><<<LAUNCH3(h), 0, h->stream>>>(h->geo, h->phys, h->mask, h->f[h->cur],
-                                                                 h->f[nxt], h->n, h->nstar, h->phi, h->u);
-  else
-    k_sweep<false><<<LAUNCH3(h), 0, h->stream>>>(h->geo, h->phys, h->mask, h->f[h->cur],
-                                                                  h->f[nxt], h->n, h->nstar, h->phi, h->u);
+  const FlatGeo G = flat_geo(h->geo);
+  (h->prm.flow ? k_sweep<true> : k_sweep<false>)<<<flat_grid(h->geo), flat_block(h->geo), 0, h->stream>>>(
+      G, h->phys, h->mask, h->f[h->cur], h->f[nxt], h->n, h->nstar, h->phi, h->u);
   if (h->prm.flow) h->cur = nxt;
   return cudaGetLastError();
 }
 
 cudaError_t launch_advect(lbe_handle *h) {
-  k_advect<<<LAUNCH3(h), 0, h->stream>>>(h->geo, h->prm.nspecies, h->mask, h->nstar, h->u, h->n);
+  k_advect<<<flat_grid(h->geo), flat_block(h->geo), 0, h->stream>>>(flat_geo(h->geo), h->prm.nspecies, h->mask,
+                                                                   h->nstar, h->u, h->n);
   return cudaGetLastError();
 }
 
