@@ -223,6 +223,9 @@ struct PoissonWork {
   cudaGraphExec_t exec_lin = nullptr;  // linear solve A x = rhs (adjoint)
   const void *lin_key[3] = {nullptr, nullptr, nullptr};
   bool graph_ok = false;
+  bool one_ok = false;         // small lattice: the solve as one cooperative kernel
+  double *one_part = nullptr;  // its block partials
+  void *one_bar = nullptr;     // its grid barrier
   double *phi_prev = nullptr;  // [kHist][N]: phi of the previous kHist steps (warm start;
                                // the FP32 form keeps fixed-point values, int64, in it)
   int history = 0;             // how many of them hold a solution (0..kHist)

@@ -159,15 +159,20 @@ struct Column {
   int p, x, y, z0, z1;
   PlaneOffs o;
 };
-__device__ __forceinline__ bool column_of(const Cols &C, Column &c) {
-  c.p = blockIdx.x * blockDim.x + threadIdx.x;
-  c.z0 = (int)(blockIdx.y * blockDim.y + threadIdx.y) * C.K;
+// (p: the column, chunk: which K planes of it)
+__device__ __forceinline__ bool column_at(const Cols &C, int p, int chunk, Column &c) {
+  c.p = p;
+  c.z0 = chunk * C.K;
   if (c.p >= C.plane || c.z0 >= C.nz) return false;
   c.z1 = min(c.z0 + C.K, C.nz);
   c.y = (int)fdiv(C.fnx, (uint32_t)c.p);
   c.x = c.p - c.y * C.nx;
   c.o = plane_offs(C.nx, C.ny, c.x, c.y);
   return true;
+}
+
+__device__ __forceinline__ bool column_of(const Cols &C, Column &c) {
+  return column_at(C, (int)(blockIdx.x * blockDim.x + threadIdx.x), (int)(blockIdx.y * blockDim.y + threadIdx.y), c);
 }
 
 // neighbour offsets of node (column, z) for the per-link forms

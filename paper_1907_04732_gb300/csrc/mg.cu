@@ -26,8 +26,7 @@
 #include <cmath>
 #include <vector>
 
-#include "march.cuh"
-#include "mg_device.cuh"
+#include "vcycle.cuh"
 
 namespace lbe {
 
@@ -68,73 +67,16 @@ __global__ void k_galerkin(const MgLevel F, const T *__restrict__ AF, const MgLe
   for (int d = 0; d < 27; ++d) A[d * C.S + I] = a[d];
 }
 
-// --- V-cycle kernels ---------------------------------------------------------
-// Level 1: a fluid child's pre-smoothed residual is r - omega A u, u = r/diag
-// being the Jacobi vector the CG formed.  A thread marches (march.cuh) a fine
-// column over the planes of Kc coarse ones; a warp covers 2^xl x 2^yl columns
-// (aligned pairs along every halved axis) of 2^zl chunks, so that the
-// children of a coarse node meet in the thread (z) and in two shuffles (x, y),
-// a fixed order.
-struct RestrictMap {
-  int xl, yl, zl;  // lanes 2^xl x 2^yl x 2^zl
-  int wy;          // warps of a block along y (the rest along z)
-  int Kc;          // coarse planes per thread
-};
+// --- V-cycle kernels (bodies in vcycle.cuh) ------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict0(const Cols F, const uint8_t *__restrict__ code,
                                                    const T *__restrict__ r, const T *__restrict__ u, const MgLevel C,
                                                    const T *__restrict__ WC, T *__restrict__ rc, T *__restrict__ zc,
                                                    const RestrictMap M, const PoissonCtl *c) {
   if (c && c->inner_done) return;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int lx = lane & ((1 << M.xl) - 1), ly = (lane >> M.xl) & ((1 << M.yl) - 1), lz = lane >> (M.xl + M.yl);
-  const int x = (blockIdx.x << M.xl) + lx;
-  const int y = ((blockIdx.y * M.wy + w % M.wy) << M.yl) + ly;
-  const int Z0 = ((((blockIdx.z * (8 / M.wy) + w / M.wy) << M.zl) + lz)) * M.Kc;
-  const bool own = x < F.nx && y < F.ny && Z0 < C.nz;
-  const int p = x + F.nx * y;
-  const PlaneOffs o = plane_offs(F.nx, F.ny, x, y);
-  ZMarch<T> m;
-  int z = Z0 << C.sz;
-  const int zend = min((Z0 + M.Kc) << C.sz, F.nz);
-  if (own) m.begin(u, o, p, F.plane, F.nz, z);
-#pragma unroll 1
-  for (int k = 0; k < M.Kc; ++k) {  // every lane runs the same iterations (the shuffles)
-    const int Z = Z0 + k;
-    const bool write = own && Z < C.nz && !(C.sx & lx & 1) && !(C.sy & ly & 1);
-    const int I = (x >> C.sx) + C.nx * ((y >> C.sy) + C.ny * Z);
-    const T wd = write ? WC[I] : (T)0;
-    T v = 0;
-    if (own && Z < C.nz) {
-      for (int h = 0; h <= C.sz && z < F.nz; ++h, ++z) {
-        if (F.ahead && z + 1 + F.ahead < zend) {
-          prefetch_l2(u + m.j + F.plane * (1 + F.ahead));
-          prefetch_l2(r + m.j + F.plane * F.ahead);
-          prefetch_l2(code + m.j + F.plane * F.ahead);
-        }
-        T u0;
-        int i;
-        const T nsum = m.step(u, o, p, F.plane, F.nz, z, u0, i);
-        const int cd = code[i];
-        const T res = r[i] - (T)kOmega * ((T)((cd & kCodeDiag) + F.selfw) * u0 - nsum) * (T)(1.0 / 6.0);
-        v += cd ? res : (T)0;
-      }
-    }
-    if (C.sx) v += __shfl_xor_sync(0xffffffffu, v, 1);
-    if (C.sy) v += __shfl_xor_sync(0xffffffffu, v, 1 << M.xl);
-    if (write) {
-      rc[I] = v;
-      zc[I] = wd * v;
-    }
-  }
+  restrict0_block(F, code, r, u, C, WC, rc, zc, M, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z);
 }
 
-// Restriction between coarse levels with 8 threads per coarse node (one per
-// child) and a fixed-order shuffle sum of the children's pre-smoothed
-// residuals.  A block covers a tile of 32
-// coarse nodes (2^txl along X, the rest along Y; lanes 8k..8k+7 the children
-// of one coarse node, child index = lane % 8 as in child_of) of one plane:
-// coordinates come from the block and lane indices, with no division.
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict(const MgLevel F, const T *__restrict__ AF,
                                                   const T *__restrict__ r, const T *__restrict__ zf,
@@ -142,20 +84,7 @@ __global__ void __launch_bounds__(256) k_restrict(const MgLevel F, const T *__re
                                                   T *__restrict__ rc, T *__restrict__ zc, int txl,
                                                   const PoissonCtl *c) {
   if (c && c->inner_done) return;
-  const int ch = threadIdx.x & 7, j = threadIdx.x >> 3;
-  const int X = (blockIdx.x << txl) + (j & ((1 << txl) - 1));
-  const int Y = blockIdx.y * (32 >> txl) + (j >> txl), Z = blockIdx.z;
-  const bool own = X < C.nx && Y < C.ny;
-  const int I = X + C.nx * (Y + C.ny * Z);
-  const T wd = ch == 0 && own ? WC[I] : (T)0;
-  int x, y, z;
-  T v = 0;
-  if (own && child_of(C, X, Y, Z, ch, F.nx, F.ny, F.nz, x, y, z)) v = presmoothed_res_z(F, AF, r, zf, x, y, z);
-  v = sum8(v);
-  if (ch == 0 && own) {
-    rc[I] = v;
-    zc[I] = wd * v;
-  }
+  restrict_block(F, AF, r, zf, C, WC, rc, zc, txl, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z);
 }
 
 // fused prolongation + post-smoothing on a 27-point level
@@ -171,13 +100,6 @@ __global__ void k_post(const MgLevel L, const T *__restrict__ A, const T *__rest
   out[I] = sizeof(T) == 8 ? post_value_w(L, A, W[I], r, z, C, ec, X, Y, Z) : post_value_z(L, A, r, z, C, ec, X, Y, Z);
 }
 
-// fused prolongation + post-smoothing on the finest level:
-// t = omega u + alpha P e_1 (fluid nodes), out = t + omega (r - A t)/diag.
-// The neighbour sum of u is marched; that of P e_1 likewise, with the coarse
-// array's offsets (a column's neighbours lie in its own aggregate or the next
-// one) and each coarse plane's sums kept while the fine planes stay in it.
-// Next to a wall, P e_1 is nonzero on the solid neighbours too and the links
-// are taken one by one.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3) k_post0(const Cols F, const uint8_t *__restrict__ code,
                                                const uint32_t *__restrict__ mask, const T *__restrict__ r,
@@ -185,80 +107,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3) k_post0(const Col
                                                T *__restrict__ out, const PoissonCtl *c) {
   if (c && c->inner_done) return;
   Column col;
-  if (!column_of(F, col)) return;
-  const int X = col.x >> C.sx, Y = col.y >> C.sy, cplane = C.nx * C.ny;
-  PlaneOffs q;  // coarse offsets of the in-plane neighbours' aggregates
-  q.xm = ((col.x + col.o.xm) >> C.sx) - X;
-  q.xp = ((col.x + col.o.xp) >> C.sx) - X;
-  q.ym = C.nx * (((col.y == 0 ? F.ny - 1 : col.y - 1) >> C.sy) - Y);
-  q.yp = C.nx * (((col.y == F.ny - 1 ? 0 : col.y + 1) >> C.sy) - Y);
-  const int P = X + C.nx * Y;
-  const T om = (T)kOmega, al = (T)kAlpha;
-  ZMarch<T> m;
-  m.begin(u, col.o, col.p, F.plane, F.nz, col.z0);
-  int Z = col.z0 >> C.sz;
-  T c0, s0, d0, c1, s1, d1, below;
-  {
-    T cb, sb, db;
-    const int Zb = (col.z0 == 0 ? F.nz - 1 : col.z0 - 1) >> C.sz;
-    plane_sums(ec, q, P + cplane * Zb, cb, sb, db);
-    below = 2 * cb + sb;
-  }
-  plane_sums(ec, q, P + cplane * Z, c0, s0, d0);
-  auto node = [&](int z) {
-    if (F.ahead && z + 1 + F.ahead < col.z1) {
-      prefetch_l2(u + m.j + F.plane * (1 + F.ahead));
-      prefetch_l2(r + m.j + F.plane * F.ahead);
-      prefetch_l2(code + m.j + F.plane * F.ahead);
-      prefetch_l2(ec + P + cplane * ((z + 1 + F.ahead) >> C.sz));
-    }
-    T u0;
-    int i;
-    const int Zn = (z + 1 == F.nz ? 0 : z + 1) >> C.sz;
-    if (Zn != Z) {
-      plane_sums(ec, q, P + cplane * Zn, c1, s1, d1);
-    } else {
-      c1 = c0;
-      s1 = s0;
-      d1 = d0;
-    }
-    const T nu = m.step(u, col.o, col.p, F.plane, F.nz, z, u0, i);
-    T ne = (2 * s0 + d0) + (below + (2 * c1 + s1));
-    const int cd = code[i];
-    T v = 0;
-    if (cd) {
-      if (cd & kCodeWall) {
-        const uint32_t mk = mask[i];
-        const int Zm = (z == 0 ? F.nz - 1 : z - 1) >> C.sz;
-        ne = 0;
-#pragma unroll
-        for (int l = 1; l < kQ; ++l) {
-          const int dx = cx_of(l), dy = cy_of(l), dz = cz_of(l);
-          const int a = P + (dx < 0 ? q.xm : (dx > 0 ? q.xp : 0)) + (dy < 0 ? q.ym : (dy > 0 ? q.yp : 0)) +
-                        cplane * (dz < 0 ? Zm : (dz > 0 ? Zn : Z));
-          if (mk & (1u << (l - 1))) ne += (T)(c2_of(l) == 1 ? 2 : 1) * ec[a];
-        }
-      }
-      const T d6 = (T)(cd & kCodeDiag);
-      const T t = om * u0 + al * c0;
-      const T s6 = om * nu + al * ne - (T)F.selfw * t;
-      const T res6 = (T)6 * r[i] - (d6 * t - s6);
-      v = t + om * (sizeof(T) == 4 ? (T)__fdividef((float)res6, (float)d6) : res6 * (T)(1.0 / 6.0) * inv_diag<T>(cd));
-    }
-    out[i] = v;
-    below = 2 * c0 + s0;
-    c0 = c1;
-    s0 = s1;
-    d0 = d1;
-    Z = Zn;
-  };
-  if (F.ahead) {  // from HBM: several planes' loads in flight
-#pragma unroll 2
-    for (int z = col.z0; z < col.z1; ++z) node(z);
-  } else {
-#pragma unroll 1
-    for (int z = col.z0; z < col.z1; ++z) node(z);
-  }
+  if (column_of(F, col)) post0_column(F, col, code, mask, r, u, C, ec, out);
 }
 
 // coarsest level solved exactly: e = A^-1 r with the inverse formed at
@@ -267,14 +116,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_coarse_direct(int N, const T *__restrict__ Ainv, const T *__restrict__ r,
                                                        T *__restrict__ e, const PoissonCtl *c) {
   if (c && c->inner_done) return;
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= N) return;
-  const T *a = Ainv + (size_t)row * N;
-  T s = 0;
-  for (int j = lane; j < N; j += 32) s = fma(a[j], r[j], s);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) e[row] = s;
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (row < N) inverse_row(row, N, Ainv, r, e);
 }
 
 // coarsest level in one block
@@ -381,32 +224,13 @@ __global__ void __launch_bounds__(kDenseThreads) k_dense_form(const BottomArgs<T
     G.M[(size_t)col * G.stride + i] = i < N ? e[i] : (T)0;
 }
 
-// e = M r; rows of `stride` values (a multiple of 16 bytes, zero-padded, as r is)
+// e = M r
 template <typename T>
 __global__ void __launch_bounds__(256) k_dense(int N, int stride, const T *__restrict__ M, const T *__restrict__ r,
                                                T *__restrict__ e, const PoissonCtl *c) {
   if (c && c->inner_done) return;
-  constexpr int V = 16 / sizeof(T);
-  struct alignas(16) Vec {
-    T v[V];
-  };
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= N) return;
-  const Vec *a = reinterpret_cast<const Vec *>(M + (size_t)row * stride);
-  const Vec *b = reinterpret_cast<const Vec *>(r);
-  T s[V] = {};
-#pragma unroll 8
-  for (int k = lane; k < stride / V; k += 32) {
-    const Vec av = a[k], bv = b[k];
-#pragma unroll
-    for (int q = 0; q < V; ++q) s[q] = fma(av.v[q], bv.v[q], s[q]);
-  }
-  T t = s[0];
-#pragma unroll
-  for (int q = 1; q < V; ++q) t += s[q];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if (lane == 0) e[row] = t;
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (row < N) dense_row(row, stride, M, r, e);
 }
 
 // omega/diag of a level (0 for a node without fluid)
@@ -656,38 +480,17 @@ static cudaError_t mg_vcycle_t(lbe_handle *h, const void *r0, const void *uj, vo
   };
   for (int l = 1; l < nl; ++l) lv[l] = level_dev(mg.lv[l]);
   // down: restrictions (pre-smoothing on the fly)
-  // level 1: lanes along x, a pair of rows, the rest along z
   RestrictMap M;
-  {
-    const int nx = h->geo.nx, ny = h->geo.ny;
-    M.yl = lv[1].sy;
-    M.xl = 0;
-    while ((1 << M.xl) < nx && M.xl < 5 - M.yl) ++M.xl;
-    M.zl = 5 - M.xl - M.yl;
-  }
-  const int xt = (h->geo.nx + (1 << M.xl) - 1) >> M.xl, yt = (h->geo.ny + (1 << M.yl) - 1) >> M.yl;
-  M.wy = yt < 8 ? pow2_at_least(yt) : 8;
-  dim3 rg0;
-  {
-    const int zc = (8 / M.wy) << M.zl, yb = (yt + M.wy - 1) / M.wy;  // chunks per block, blocks along y
-    M.Kc = planes_per_thread((long long)xt * yb, lv[1].nz, zc, 1 + lv[1].sz);
-    const int per = zc * M.Kc;
-    rg0 = dim3((unsigned)xt, (unsigned)yb, (unsigned)((lv[1].nz + per - 1) / per));
-  }
+  const dim3 rg0 = make_restrict_map(h->geo, lv[1], M);
   nodes.push_back(Node{(void *)k_restrict0<T>, rg0, dim3(256),
                        {&L0.c, P(h->code), P(r0), P(uj), &lv[1], P(mg.lv[1].W), P(mg.lv[1].r), P(mg.lv[1].z), &M,
                         P(c)}});
   // the level whose V-cycle is one matrix (or the coarsest)
   const int lk = mg.ld;
-  // the others: tiles of 32 coarse nodes per block, 2^txl along X (at most
-  // 32) and the rest along Y, one plane per block
   int txl[kMaxLevels];
   for (int l = 1; l < lk; ++l) {
     const MGLevel &Lc = mg.lv[l + 1];
-    txl[l] = 0;
-    while ((1 << txl[l]) < Lc.nx && txl[l] < 5) ++txl[l];
-    const dim3 rg((unsigned)((Lc.nx + (1 << txl[l]) - 1) >> txl[l]),
-                  (unsigned)((Lc.ny + (32 >> txl[l]) - 1) / (32 >> txl[l])), (unsigned)Lc.nz);
+    const dim3 rg = restrict_tiles(lv[l + 1], txl[l]);
     nodes.push_back(Node{(void *)k_restrict<T>, rg, dim3(256),
                          {&lv[l], P(mg.lv[l].A), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1], P(Lc.W), P(Lc.r), P(Lc.z),
                           &txl[l], P(c)}});
@@ -740,6 +543,39 @@ cudaError_t mg_vcycle(lbe_handle *h, const void *r0, const void *uj, void *u0, c
   return h->prm.precision == LBE_FP32 ? mg_vcycle_t<float>(h, r0, uj, u0, c, gr, last, st)
                                       : mg_vcycle_t<double>(h, r0, uj, u0, c, gr, last, st);
 }
+
+template <typename T>
+static bool one_args(lbe_handle *h, VCycleArgs<T> *V) {
+  const MGWork &mg = h->mg;
+  if (mg.nlev < 2 || !(mg.dense || mg.cinv)) return false;
+  *V = VCycleArgs<T>{};
+  V->ld = mg.ld;
+  V->ndense = (int)mg.lv[mg.ld].N;
+  V->stride = mg.dense ? mg.stride : 0;
+  V->mat = (const T *)(mg.dense ? mg.dense : mg.cinv);
+  for (int l = 1; l <= mg.ld; ++l) {
+    const MGLevel &L = mg.lv[l];
+    V->lv[l] = level_dev(L);
+    V->A[l] = (const T *)L.A;
+    V->W[l] = (const T *)L.W;
+    V->r[l] = (T *)L.r;
+    V->z[l] = (T *)L.z;
+    V->e[l] = (T *)L.e;
+    if (l > 1) {
+      const dim3 t = restrict_tiles(V->lv[l], V->txl[l - 1]);
+      V->rx[l - 1] = (int)t.x;
+      V->ry[l - 1] = (int)t.y;
+      V->rz[l - 1] = (int)t.z;
+    }
+  }
+  const dim3 g = make_restrict_map(h->geo, V->lv[1], V->M);
+  V->g0x = (int)g.x;
+  V->g0y = (int)g.y;
+  V->g0z = (int)g.z;
+  return true;
+}
+bool mg_one_args(lbe_handle *h, VCycleArgs<float> *V) { return one_args(h, V); }
+bool mg_one_args(lbe_handle *h, VCycleArgs<double> *V) { return one_args(h, V); }
 
 // kernels of one V-cycle (launch accounting of the graph path)
 int mg_kernels_per_cycle(const lbe_handle *h) {

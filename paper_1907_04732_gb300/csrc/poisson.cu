@@ -37,7 +37,7 @@
 #include <type_traits>
 
 #include "fp32_device.cuh"
-#include "march.cuh"
+#include "vcycle.cuh"
 
 namespace lbe {
 
@@ -249,7 +249,7 @@ __device__ void cg_test(PoissonCtl *c, double mx, double eta, double tol_abs, in
 
 // ---------------------------------------------------------------------------
 // start of a solve: fold the previous solve into the sticky fields, reset
-__global__ void k_solve_reset(PoissonCtl *c) {
+__device__ __forceinline__ void solve_reset(PoissonCtl *c) {
   if (c->status && !c->sticky_status) c->sticky_status = c->status;
   if (c->solve_iters > c->max_solve_iters) c->max_solve_iters = c->solve_iters;
   c->outer_done = 0;
@@ -259,6 +259,7 @@ __global__ void k_solve_reset(PoissonCtl *c) {
   c->solve_iters = 0;
   c->solves += 1;
 }
+__global__ void k_solve_reset(PoissonCtl *c) { solve_reset(c); }
 
 // Residual of the current potential; seeds the inner solve: r = (T)res,
 // uj = r/diag (the CG's first update writes x, p and s).  max |res|/diag by
@@ -295,102 +296,106 @@ struct ResArgs {
   double tol, tol_rel;
   cudaGraphConditionalHandle hout, hin;
 };
+template <int MODE>
+constexpr bool kRhs = MODE == R_RHS || MODE == R_RHS_FF;
 template <typename T, int MODE>
-__global__ void __launch_bounds__(kBlock) k_res(const ResArgs A, T *__restrict__ r, T *__restrict__ uj) {
-  constexpr bool RHS = MODE == R_RHS || MODE == R_RHS_FF;
+__device__ __forceinline__ void res_column(const ResArgs &A, const Column &c, T *r, T *uj, float &mx, float &mb) {
   constexpr bool MARCH = MODE == R_FX || MODE == R_FXG || MODE == R_N64;
   using V = typename std::conditional<MODE == R_N64, double, long long>::type;
   const V *v = MODE == R_N64 ? (const V *)A.phi : (const V *)A.phifx;
+  const int plane = A.cols.plane, nz = A.cols.nz;
+  ZMarch<V> m;
+  if (MARCH) m.begin(v, c.o, c.p, plane, nz, c.z0);
+#pragma unroll 1
+  for (int z = c.z0; z < c.z1; ++z) {
+    V v0 = 0, nsum = 0;
+    int i = c.p + plane * z;
+    if (A.cols.ahead && z + 1 + A.cols.ahead < c.z1) {
+      const int j = i + plane * (1 + A.cols.ahead);
+      if (MARCH) prefetch_l2(v + j);
+      if (MODE == R_FX) {
+        prefetch_l2(A.nq + j);
+        prefetch_l2(A.nq + A.g.N + j);
+      }
+    }
+    if (MARCH) nsum = m.step(v, c.o, c.p, plane, nz, z, v0, i);
+    const int code = A.code[i];
+    if (!code) {
+      r[i] = uj[i] = (T)0;
+      continue;
+    }
+    const bool wall = code & kCodeWall;
+    const uint32_t mk = wall || !MARCH ? A.mask[i] : kLinkBits;
+    T rt, dinv;
+    if (MODE == R_FX || MODE == R_RHS_FF) {
+      float S, E, B, Be;
+      if (MODE == R_FX) {
+        // 6 res = 6 lap + 6 (4 pi l_B s) (q+ - q-): 6 lap exact in fixed
+        // point, split into float-float (the nearest float of the integer
+        // sum and the float of its exact remainder), the charge term in
+        // float-float too
+        const long long L6 = wall ? fp32::lap6_fx_<false>(col_offs(c.o, plane, nz, z), i, mk, A.phifx)
+                                  : (long long)(nsum - 24 * v0);
+        const float Lh = fp32::ll2f(L6);
+        const float Ll = fp32::ll2f(L6 - fp32::f2ll_rn(Lh));
+        S = __fmul_rn(Lh, fp32::kPhiUnitF);
+        E = __fmul_rn(Ll, fp32::kPhiUnitF);
+        const long long dq = A.nq[i] - A.nq[A.g.N + i];
+        const float dq_hi = fp32::ll2f(dq);
+        const float dq_lo = fp32::ll2f(dq - fp32::f2ll_rn(dq_hi));  // exact remainder
+        B = A.c6_hi * dq_hi;
+        Be = fmaf(A.c6_hi, dq_hi, -B) + (A.c6_hi * dq_lo + A.c6_lo * dq_hi);  // product error and tails
+      } else {
+        // 6 res = 6 rhs + 6 lap(x), x = hi + lo, in float-float; rhs is a float
+        if ((mk & kLinkBits) == kLinkBits)
+          fp32::lap6_ff_<true>(col_offs(c.o, plane, nz, z), i, mk, A.phi_hi, A.phi_lo, S, E);
+        else
+          fp32::lap6_ff_<false>(col_offs(c.o, plane, nz, z), i, mk, A.phi_hi, A.phi_lo, S, E);
+        const float bf = (float)A.rhs[i];
+        B = 6.f * bf;
+        Be = fmaf(6.f, bf, -B);  // 6 rhs = B + Be exactly
+        mb = fmaxf(mb, finite_or_inf(fabsf(bf) * inv_diag<float>(code)));
+      }
+      float t, te;
+      fp32::two_sum(S, B, t, te);
+      rt = (T)((t + (te + (E + Be))) * (1.f / 6.f));
+      dinv = inv_diag<T>(code);
+    } else {
+      double b;
+      if (MODE == R_RHS) {
+        b = A.rhs[i];
+      } else {
+        double q = 0.0;
+        for (int k = 0; k < A.P.ns; ++k)
+          q += A.P.z[k] * (MODE == R_FXG ? A.P3.rbd[k] + A.P3.sd[k] * (double)A.nq[k * A.g.N + i]
+                                         : A.n64[k * A.g.N + i]);
+        b = A.P.four_pi_lb * q;
+      }
+      double lap;
+      if (MODE == R_FXG)
+        lap = (double)(wall ? fp32::lap6_fx_<false>(col_offs(c.o, plane, nz, z), i, mk, A.phifx)
+                            : (long long)(nsum - 24 * v0)) *
+              (1.0 / 281474976710656.0 / 6.0);
+      else if (MODE == R_N64 && !wall)
+        lap = ((double)nsum - 24.0 * (double)v0) * (1.0 / 6.0);
+      else
+        lap = lap_at(col_offs(c.o, plane, nz, z), i, mk, A.phi, !(A.P.selfmask & kPlainLaplacian));
+      const double rr = b + lap;
+      rt = (T)rr;
+      dinv = inv_diag<T>(code);
+      if (MODE == R_RHS) mb = fmaxf(mb, finite_or_inf(fabsf((float)b) * (float)dinv));
+    }
+    r[i] = rt;
+    uj[i] = rt * dinv;
+    mx = fmaxf(mx, finite_or_inf(fabsf((float)rt) * (float)dinv));  // the stopping test needs no FP64
+  }
+}
+template <typename T, int MODE>
+__global__ void __launch_bounds__(kBlock) k_res(const ResArgs A, T *__restrict__ r, T *__restrict__ uj) {
+  constexpr bool RHS = kRhs<MODE>;
   float mx = 0.f, mb = 0.f;
   Column c;
-  if (column_of(A.cols, c)) {
-    const int plane = A.cols.plane, nz = A.cols.nz;
-    ZMarch<V> m;
-    if (MARCH) m.begin(v, c.o, c.p, plane, nz, c.z0);
-#pragma unroll 1
-    for (int z = c.z0; z < c.z1; ++z) {
-      V v0 = 0, nsum = 0;
-      int i = c.p + plane * z;
-      if (A.cols.ahead && z + 1 + A.cols.ahead < c.z1) {
-        const int j = i + plane * (1 + A.cols.ahead);
-        if (MARCH) prefetch_l2(v + j);
-        if (MODE == R_FX) {
-          prefetch_l2(A.nq + j);
-          prefetch_l2(A.nq + A.g.N + j);
-        }
-      }
-      if (MARCH) nsum = m.step(v, c.o, c.p, plane, nz, z, v0, i);
-      const int code = A.code[i];
-      if (!code) {
-        r[i] = uj[i] = (T)0;
-        continue;
-      }
-      const bool wall = code & kCodeWall;
-      const uint32_t mk = wall || !MARCH ? A.mask[i] : kLinkBits;
-      T rt, dinv;
-      if (MODE == R_FX || MODE == R_RHS_FF) {
-        float S, E, B, Be;
-        if (MODE == R_FX) {
-          // 6 res = 6 lap + 6 (4 pi l_B s) (q+ - q-): 6 lap exact in fixed
-          // point, split into float-float (the nearest float of the integer
-          // sum and the float of its exact remainder), the charge term in
-          // float-float too
-          const long long L6 = wall ? fp32::lap6_fx_<false>(col_offs(c.o, plane, nz, z), i, mk, A.phifx)
-                                    : (long long)(nsum - 24 * v0);
-          const float Lh = fp32::ll2f(L6);
-          const float Ll = fp32::ll2f(L6 - fp32::f2ll_rn(Lh));
-          S = __fmul_rn(Lh, fp32::kPhiUnitF);
-          E = __fmul_rn(Ll, fp32::kPhiUnitF);
-          const long long dq = A.nq[i] - A.nq[A.g.N + i];
-          const float dq_hi = fp32::ll2f(dq);
-          const float dq_lo = fp32::ll2f(dq - fp32::f2ll_rn(dq_hi));  // exact remainder
-          B = A.c6_hi * dq_hi;
-          Be = fmaf(A.c6_hi, dq_hi, -B) + (A.c6_hi * dq_lo + A.c6_lo * dq_hi);  // product error and tails
-        } else {
-          // 6 res = 6 rhs + 6 lap(x), x = hi + lo, in float-float; rhs is a float
-          if ((mk & kLinkBits) == kLinkBits)
-            fp32::lap6_ff_<true>(col_offs(c.o, plane, nz, z), i, mk, A.phi_hi, A.phi_lo, S, E);
-          else
-            fp32::lap6_ff_<false>(col_offs(c.o, plane, nz, z), i, mk, A.phi_hi, A.phi_lo, S, E);
-          const float bf = (float)A.rhs[i];
-          B = 6.f * bf;
-          Be = fmaf(6.f, bf, -B);  // 6 rhs = B + Be exactly
-          mb = fmaxf(mb, finite_or_inf(fabsf(bf) * inv_diag<float>(code)));
-        }
-        float t, te;
-        fp32::two_sum(S, B, t, te);
-        rt = (T)((t + (te + (E + Be))) * (1.f / 6.f));
-        dinv = inv_diag<T>(code);
-      } else {
-        double b;
-        if (MODE == R_RHS) {
-          b = A.rhs[i];
-        } else {
-          double q = 0.0;
-          for (int k = 0; k < A.P.ns; ++k)
-            q += A.P.z[k] * (MODE == R_FXG ? A.P3.rbd[k] + A.P3.sd[k] * (double)A.nq[k * A.g.N + i]
-                                           : A.n64[k * A.g.N + i]);
-          b = A.P.four_pi_lb * q;
-        }
-        double lap;
-        if (MODE == R_FXG)
-          lap = (double)(wall ? fp32::lap6_fx_<false>(col_offs(c.o, plane, nz, z), i, mk, A.phifx)
-                              : (long long)(nsum - 24 * v0)) *
-                (1.0 / 281474976710656.0 / 6.0);
-        else if (MODE == R_N64 && !wall)
-          lap = ((double)nsum - 24.0 * (double)v0) * (1.0 / 6.0);
-        else
-          lap = lap_at(col_offs(c.o, plane, nz, z), i, mk, A.phi, !(A.P.selfmask & kPlainLaplacian));
-        const double rr = b + lap;
-        rt = (T)rr;
-        dinv = inv_diag<T>(code);
-        if (MODE == R_RHS) mb = fmaxf(mb, finite_or_inf(fabsf((float)b) * (float)dinv));
-      }
-      r[i] = rt;
-      uj[i] = rt * dinv;
-      mx = fmaxf(mx, finite_or_inf(fabsf((float)rt) * (float)dinv));  // the stopping test needs no FP64
-    }
-  }
+  if (column_of(A.cols, c)) res_column<T, MODE>(A, c, r, uj, mx, mb);
   mx = block_reduce<true, float>(mx);
   if (RHS) mb = block_reduce<true, float>(mb);
   if (flat_tid() == 0) {
@@ -415,6 +420,39 @@ __global__ void __launch_bounds__(kBlock) k_res(const ResArgs A, T *__restrict__
 // runs the scalar recurrence.  Marched (march.cuh); u is zero on solid nodes
 // and w is set to zero there, so that the update needs no mask.
 template <typename T>
+__device__ __forceinline__ void cg_b_column(const Cols &C, const Column &col, const uint8_t *code, const T *u, const T *r,
+                                            T *w, T &ru, T &wu) {
+  ZMarch<T> m;
+  m.begin(u, col.o, col.p, C.plane, C.nz, col.z0);
+  auto node = [&](int z) {
+    T u0;
+    int i;
+    const T nsum = m.step(u, col.o, col.p, C.plane, C.nz, z, u0, i);
+    const int cd = code[i];
+    const T wv = cd ? ((T)((cd & kCodeDiag) + C.selfw) * u0 - nsum) * (T)(1.0 / 6.0) : (T)0;
+    w[i] = wv;
+    ru += r[i] * u0;
+    wu += wv * u0;
+  };
+  // from HBM: prefetch, and several planes' loads in flight; from L2 a
+  // short loop (on small lattices fetching unrolled code takes longer than
+  // running it: FP64 solve of 4x4x64 0.78 against 0.94 ms per step)
+  if (C.ahead) {
+#pragma unroll 3
+    for (int z = col.z0; z < col.z1; ++z) {
+      if (z + 1 + C.ahead < col.z1) {
+        prefetch_l2(u + m.j + C.plane * (1 + C.ahead));
+        prefetch_l2(r + m.j + C.plane * C.ahead);
+        prefetch_l2(code + m.j + C.plane * C.ahead);
+      }
+      node(z);
+    }
+  } else {
+#pragma unroll 1
+    for (int z = col.z0; z < col.z1; ++z) node(z);
+  }
+}
+template <typename T>
 __global__ void __launch_bounds__(kBlock) k_cg_b(const Cols C, const uint8_t *__restrict__ code,
                                                  const T *__restrict__ u, const T *__restrict__ r,
                                                  T *__restrict__ w, double *__restrict__ part, int nblk,
@@ -422,37 +460,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_b(const Cols C, const uint8_t *__
   if (!use_cond && c->inner_done) return;  // the graph's loop has ended by then
   T ru = 0, wu = 0;
   Column col;
-  if (column_of(C, col)) {
-    ZMarch<T> m;
-    m.begin(u, col.o, col.p, C.plane, C.nz, col.z0);
-    auto node = [&](int z) {
-      T u0;
-      int i;
-      const T nsum = m.step(u, col.o, col.p, C.plane, C.nz, z, u0, i);
-      const int cd = code[i];
-      const T wv = cd ? ((T)((cd & kCodeDiag) + C.selfw) * u0 - nsum) * (T)(1.0 / 6.0) : (T)0;
-      w[i] = wv;
-      ru += r[i] * u0;
-      wu += wv * u0;
-    };
-    // from HBM: prefetch, and several planes' loads in flight; from L2 a
-    // short loop (on small lattices fetching unrolled code takes longer than
-    // running it: FP64 solve of 4x4x64 0.78 against 0.94 ms per step)
-    if (C.ahead) {
-#pragma unroll 3
-      for (int z = col.z0; z < col.z1; ++z) {
-        if (z + 1 + C.ahead < col.z1) {
-          prefetch_l2(u + m.j + C.plane * (1 + C.ahead));
-          prefetch_l2(r + m.j + C.plane * C.ahead);
-          prefetch_l2(code + m.j + C.plane * C.ahead);
-        }
-        node(z);
-      }
-    } else {
-#pragma unroll 1
-      for (int z = col.z0; z < col.z1; ++z) node(z);
-    }
-  }
+  if (column_of(C, col)) cg_b_column(C, col, code, u, r, w, ru, wu);
   block_reduce2(ru, wu);
   if (flat_tid() == 0) {
     part[S_RU * nblk + flat_bid()] = (double)ru;
@@ -482,19 +490,13 @@ struct alignas(sizeof(T) * VEC) Pack {
 // instead of reading zeros that the residual kernel would have to write.
 // Every vector is zero on solid nodes, so no node waits for its mask.
 template <typename T, int VEC>
-__global__ void __launch_bounds__(kBlock) k_cg_a(long long N, const uint8_t *__restrict__ code, T *__restrict__ x,
-                                                 T *__restrict__ r, const T *u, T *uj,
-                                                 const T *__restrict__ w, T *__restrict__ p, T *__restrict__ s,
-                                                 int nblk, PoissonCtl *c, double eta, double tol_abs, int maxit,
-                                                 cudaGraphConditionalHandle hin, int use_cond) {
-  if (c->inner_done) return;  // a breakdown in this iteration
-  const T alpha = (T)c->alpha, beta = (T)c->beta;
-  const bool first = c->round_iters == 0;
+__device__ __forceinline__ T cg_a_nodes(long long N, long long k0, long long dk, const uint8_t *code, T *x, T *r,
+                                        const T *u, T *uj, const T *w, T *p, T *s, T alpha, T beta, bool first) {
   using PT = Pack<T, VEC>;
   using PC = Pack<uint8_t, VEC>;
   T mx = 0;
   const long long n = N / VEC;
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
+  for (long long k = k0; k < n; k += dk) {
     const PT uv = ((const PT *)u)[k], wv = ((const PT *)w)[k];
     PT rv = ((PT *)r)[k];
     const PC cv = ((const PC *)code)[k];
@@ -525,6 +527,17 @@ __global__ void __launch_bounds__(kBlock) k_cg_a(long long N, const uint8_t *__r
     ((PT *)r)[k] = rv;
     ((PT *)uj)[k] = jv;
   }
+  return mx;
+}
+template <typename T, int VEC>
+__global__ void __launch_bounds__(kBlock) k_cg_a(long long N, const uint8_t *__restrict__ code, T *__restrict__ x,
+                                                 T *__restrict__ r, const T *u, T *uj,
+                                                 const T *__restrict__ w, T *__restrict__ p, T *__restrict__ s,
+                                                 int nblk, PoissonCtl *c, double eta, double tol_abs, int maxit,
+                                                 cudaGraphConditionalHandle hin, int use_cond) {
+  if (c->inner_done) return;  // a breakdown in this iteration
+  const T mx = cg_a_nodes<T, VEC>(N, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x,
+                                  code, x, r, u, uj, w, p, s, (T)c->alpha, (T)c->beta, c->round_iters == 0);
   // a maximum does not depend on the order: the blocks combine theirs in one
   // word (the bits of a non-negative double order as an integer), and the
   // last ticket's thread has no partials to read
@@ -556,14 +569,12 @@ __global__ void k_extrapolate(const Geo g, int zpt, const uint32_t *__restrict__
 // FP32 form: the fixed-point potential += e (rounded to the fixed-point
 // unit) and its float copy; |phi| reaching kPhiMax raises range flag 4.  e is
 // zero on solid nodes, which keep their values.
-__global__ void __launch_bounds__(kBlock) k_correct_fx(long long N, const float *__restrict__ e,
-                                                       int64_t *__restrict__ phifx, float *__restrict__ phi32,
-                                                       int *__restrict__ flag, const PoissonCtl *__restrict__ c) {
-  if (c->outer_done || c->round_iters == 0) return;  // converged, or no update in this round
+__device__ __forceinline__ void correct_fx_nodes(long long N, long long k0, long long dk, const float *e, int64_t *phifx,
+                                                 float *phi32, int *flag) {
   constexpr float kMaxFx = (float)(kPhiMax * 281474976710656.0);  // kPhiMax 2^kPhiFixBits
   bool over = false;
 #pragma unroll 4
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+  for (long long i = k0; i < N; i += dk) {
     const float d = __fmul_rn(e[i], 281474976710656.0f);  // e 2^kPhiFixBits, exact
     const bool bad = !(fabsf(d) < kMaxFx);  // also NaN
     const long long v = phifx[i] + (bad ? 0LL : fp32::f2ll_rn(d));
@@ -572,6 +583,13 @@ __global__ void __launch_bounds__(kBlock) k_correct_fx(long long N, const float 
     phi32[i] = fp32::fx_to_f(v);
   }
   if (over) atomicOr(flag, 4);
+}
+__global__ void __launch_bounds__(kBlock) k_correct_fx(long long N, const float *__restrict__ e,
+                                                       int64_t *__restrict__ phifx, float *__restrict__ phi32,
+                                                       int *__restrict__ flag, const PoissonCtl *__restrict__ c) {
+  if (c->outer_done || c->round_iters == 0) return;  // converged, or no update in this round
+  correct_fx_nodes(N, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x, e, phifx,
+                   phi32, flag);
 }
 
 // FP32 form without flow (no advection kernel to carry it): the warm start
@@ -589,12 +607,10 @@ __global__ void k_extrapolate_fx(const Geo g, int zpt, const uint32_t *__restric
 // phi64 += e (zero on solid nodes); with phi32 given its float split follows
 // (the FP64 form, and the linear solves' FP64 iterates)
 template <typename T>
-__global__ void __launch_bounds__(kBlock) k_correct(long long N, const T *__restrict__ e, double *__restrict__ phi,
-                                                    float *__restrict__ phi32, float *__restrict__ phi_lo,
-                                                    const PoissonCtl *__restrict__ c) {
-  if (c && (c->outer_done || c->round_iters == 0)) return;  // converged, or no update in this round
+__device__ __forceinline__ void correct_nodes(long long N, long long k0, long long dk, const T *e, double *phi, float *phi32,
+                                              float *phi_lo) {
 #pragma unroll 4
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+  for (long long i = k0; i < N; i += dk) {
     double v = phi[i];
     if (e) {
       v += (double)e[i];
@@ -604,6 +620,276 @@ __global__ void __launch_bounds__(kBlock) k_correct(long long N, const T *__rest
       const float hi = (float)v;
       phi32[i] = hi;
       if (phi_lo) phi_lo[i] = (float)(v - (double)hi);
+    }
+  }
+}
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_correct(long long N, const T *__restrict__ e, double *__restrict__ phi,
+                                                    float *__restrict__ phi32, float *__restrict__ phi_lo,
+                                                    const PoissonCtl *__restrict__ c) {
+  if (c && (c->outer_done || c->round_iters == 0)) return;  // converged, or no update in this round
+  correct_nodes(N, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x, e, phi, phi32,
+                phi_lo);
+}
+
+// ---------------------------------------------------------------------------
+// The whole solve as one cooperative kernel, for lattices whose kernels are
+// too short to fill the GPU.  There an iteration of the graph (five to nine
+// kernels and a conditional node) is launch, ramp and drain: 35-40 us per
+// iteration on a 32x32x16 or a 128x128x4 lattice, 23-26 us here.  The same
+// bodies run as phases of resident blocks with a barrier of the grid between
+// them; each block keeps the control block in shared memory and runs the
+// scalar recurrence and the tests itself on the same partials, in the same
+// order.  What is left of a small lattice's phase is the latency of the
+// barrier (a release, a poll, L1 refilled) and of two dependent L2 reads.
+struct GridBar {
+  unsigned count, exits;
+  int dead;
+};
+constexpr int kSpinLimit = 1 << 23;  // some seconds: a wait that long never ends
+
+// All blocks of the (cooperative, hence co-resident) grid have arrived and
+// their writes are visible; false when the wait ran out, in every thread of
+// the block (the caller returns, other blocks see `dead` and do the same).
+__device__ __forceinline__ bool grid_sync(GridBar *b, unsigned &target) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    target += gridDim.x;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&b->count) : "memory");
+    unsigned v;
+    int spins = 0, good = 1;
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&b->count) : "memory");
+      if ((int)(v - target) >= 0) break;
+      if ((++spins & 1023) == 0 && (spins >= kSpinLimit || *(volatile int *)&b->dead)) {
+        b->dead = 1;
+        good = 0;
+        break;
+      }
+    }
+    ok = good;
+  }
+  __syncthreads();
+  return ok;
+}
+
+template <typename T>
+struct OneArgs {
+  ResArgs R;
+  mgd::VCycleArgs<T> V;
+  T *r, *u, *uj, *w, *x, *p, *s;
+  double *phi;
+  float *phi32, *phi_lo;
+  int64_t *phifx;
+  int *flag;
+  double *part;  // [3][blocks]: (r,u), (w,u), maxima
+  GridBar *bar;
+  long long N;
+  double eta, tol_inner;
+  int cbl;         // log2 of the columns of a block
+  int gx, blocks;  // column blocks, and all (column, chunk) blocks
+  int vec;         // the update takes 16 bytes at a time
+};
+
+// Lattices up to this size take the single-kernel solve.  Both paths, ms per
+// solve (one kernel / graph): FP32 16x16x64 0.046 / 0.082, 128x128x4 driven
+// coax 0.316 / 0.454, 61x47x53 electrodes 0.278 / 0.351, 64x64x256 0.244 /
+// 0.276, porous 128x128x64 0.452 / 0.487; 128x128x128 0.395 / 0.380 and
+// 128x128x256 0.751 / 0.671, where a kernel of its own keeps more warps in
+// flight.  FP64 4x4x64 0.064 / 0.105, 128x128x4 coax 0.368 / 0.462, 64x64x256
+// 0.915 / 0.980.
+constexpr long long kOneNodes = 3 << 19;
+// Resident blocks: at most so many per SM (FP32 at 64x64x256 with 1, 2, 3:
+// 0.382, 0.274, 0.251 ms; FP64 at 128x128x4 0.368 with one, 0.456 with two,
+// every block repeating the FP64 reductions), as many as the stencils have
+// blocks of columns, and one per SM where only the matrix's rows are more.
+template <typename T>
+constexpr int kOnePerSM = sizeof(T) == 4 ? 3 : 1;
+constexpr int kOneBlocks = 608;  // room for the partials
+enum { ONE_RU = 0, ONE_WU = 1, ONE_MAX = 2, ONE_REF = 1 };
+
+// Two values of every block combined in block order; valid in thread 0.  All
+// threads fetch them (one L2 latency), one warp adds each (an FP64
+// instruction holds the narrow pipe for 16 cycles).
+__device__ __forceinline__ void grid_sums(const double *a_, const double *b_, double &a, double &b) {
+  __shared__ double sv[2][kOneBlocks], sum_b;
+  const int G = gridDim.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < (kOneBlocks + kBlock - 1) / kBlock; ++k) {
+    const int i = threadIdx.x + k * kBlock;
+    if (i < G) {
+      sv[0][i] = __ldcg(a_ + i);
+      sv[1][i] = __ldcg(b_ + i);
+    }
+  }
+  __syncthreads();
+  double v = 0.0;
+  if (w < 2) {
+    for (int i = lane; i < G; i += 32) v += sv[w][i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (w == 1 && lane == 0) sum_b = v;
+  }
+  __syncthreads();
+  a = v;
+  b = sum_b;
+}
+// maxima of the blocks' (non-negative) values, whose bits order as integers
+__device__ __forceinline__ double grid_max(const double *a_) {
+  const long long *a = reinterpret_cast<const long long *>(a_);
+  __shared__ long long sm[kBlock / 32];
+  const int G = gridDim.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  long long v = 0;
+#pragma unroll
+  for (int k = 0; k < (kOneBlocks + kBlock - 1) / kBlock; ++k) {
+    const int i = threadIdx.x + k * kBlock;
+    if (i < G) v = max(v, __ldcg(a + i));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_down_sync(0xffffffffu, v, o));
+  if (lane == 0) sm[w] = v;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int k = 1; k < kBlock / 32; ++k) v = max(v, sm[k]);
+  return __longlong_as_double(v);
+}
+
+// u = M r; every phase but the last ends in a barrier.  false: a wait ran out
+template <typename T>
+__device__ __forceinline__ bool one_vcycle(const OneArgs<T> &S, unsigned &target) {
+  using namespace mgd;
+  const VCycleArgs<T> &V = S.V;
+  const int G = gridDim.x, b0 = blockIdx.x, warp = threadIdx.x >> 5;
+  for (int b = b0; b < V.g0x * V.g0y * V.g0z; b += G) {
+    const int bx = b % V.g0x, t = b / V.g0x;
+    restrict0_block(S.R.cols, S.R.code, S.r, S.uj, V.lv[1], V.W[1], V.r[1], V.z[1], V.M, bx, t % V.g0y, t / V.g0y);
+  }
+  if (!grid_sync(S.bar, target)) return false;
+  for (int l = 1; l < V.ld; ++l) {
+    for (int b = b0; b < V.rx[l] * V.ry[l] * V.rz[l]; b += G) {
+      const int bx = b % V.rx[l], t = b / V.rx[l];
+      restrict_block(V.lv[l], V.A[l], V.r[l], V.z[l], V.lv[l + 1], V.W[l + 1], V.r[l + 1], V.z[l + 1], V.txl[l], bx,
+                     t % V.ry[l], t / V.ry[l]);
+    }
+    if (!grid_sync(S.bar, target)) return false;
+  }
+  for (int row = b0 * (kBlock / 32) + warp; row < V.ndense; row += G * (kBlock / 32)) {
+    if (V.stride) dense_row(row, V.stride, V.mat, V.r[V.ld], V.e[V.ld]);
+    else inverse_row(row, V.ndense, V.mat, V.r[V.ld], V.e[V.ld]);
+  }
+  if (!grid_sync(S.bar, target)) return false;
+  for (int l = V.ld - 1; l >= 1; --l) {
+    for (int i = b0 * kBlock + threadIdx.x; i < V.lv[l].N; i += G * kBlock) {
+      int X, Y, Z;
+      level_coords(V.lv[l], i, X, Y, Z);
+      V.e[l][i] = post_value_w<T>(V.lv[l], V.A[l], V.W[l][i], V.r[l], V.z[l], V.lv[l + 1], V.e[l + 1], X, Y, Z);
+    }
+    if (!grid_sync(S.bar, target)) return false;
+  }
+  for (int b = b0; b < S.blocks; b += G) {
+    Column c;
+    const int tx = threadIdx.x & ((1 << S.cbl) - 1), ty = threadIdx.x >> S.cbl;
+    if (column_at(S.R.cols, ((b % S.gx) << S.cbl) + tx, (b / S.gx) * (kBlock >> S.cbl) + ty, c))
+      post0_column(S.R.cols, c, S.R.code, S.R.mask, S.r, S.uj, V.lv[1], V.e[1], S.u);
+  }
+  return true;
+}
+
+// false: a wait ran out
+template <typename T, int MODE>
+__device__ __forceinline__ bool one_solve(const OneArgs<T> &S, PoissonCtl *sc, unsigned &target) {
+  const int G = gridDim.x, b0 = blockIdx.x, t = threadIdx.x;
+  const int tx = t & ((1 << S.cbl) - 1), ty = t >> S.cbl, zb = kBlock >> S.cbl;
+  const long long k0 = (long long)b0 * kBlock + t, dk = (long long)G * kBlock;
+  double m0, m1;
+  for (;;) {
+    float mx = 0.f, mb = 0.f;
+    for (int b = b0; b < S.blocks; b += G) {
+      Column c;
+      if (column_at(S.R.cols, ((b % S.gx) << S.cbl) + tx, (b / S.gx) * zb + ty, c))
+        res_column<T, MODE>(S.R, c, S.r, S.uj, mx, mb);
+    }
+    mx = block_reduce<true, float>(mx);
+    if (kRhs<MODE>) mb = block_reduce<true, float>(mb);
+    if (t == 0) {
+      S.part[ONE_MAX * G + b0] = (double)mx;
+      if (kRhs<MODE>) S.part[ONE_REF * G + b0] = (double)mb;
+    }
+    if (!grid_sync(S.bar, target)) return false;
+    m0 = grid_max(S.part + ONE_MAX * G);
+    m1 = 0.0;
+    if (kRhs<MODE>) {
+      __syncthreads();  // grid_max's shared words
+      m1 = grid_max(S.part + ONE_REF * G);
+    }
+    if (t == 0) {
+      if (kRhs<MODE>) sc->ref = m1;
+      outer_check(sc, m0, kRhs<MODE> ? fmax(S.R.tol, S.R.tol_rel * m1) : S.R.tol, S.R.maxit, 0, 0, 0);
+    }
+    __syncthreads();
+    if (sc->outer_done) return true;
+    while (!sc->inner_done) {
+      if (!one_vcycle(S, target) || !grid_sync(S.bar, target)) return false;
+      T ru = 0, wu = 0;
+      for (int b = b0; b < S.blocks; b += G) {
+        Column c;
+        if (column_at(S.R.cols, ((b % S.gx) << S.cbl) + tx, (b / S.gx) * zb + ty, c))
+          cg_b_column(S.R.cols, c, S.R.code, S.u, S.r, S.w, ru, wu);
+      }
+      block_reduce2(ru, wu);
+      if (t == 0) {
+        S.part[ONE_RU * G + b0] = (double)ru;
+        S.part[ONE_WU * G + b0] = (double)wu;
+      }
+      if (!grid_sync(S.bar, target)) return false;
+      grid_sums(S.part + ONE_RU * G, S.part + ONE_WU * G, m0, m1);
+      if (t == 0) cg_scalars(sc, m0, m1, 0, 0);
+      __syncthreads();
+      if (sc->inner_done) break;  // a breakdown: no update
+      const T alpha = (T)sc->alpha, beta = (T)sc->beta;
+      const bool first = sc->round_iters == 0;
+      T v;
+      if (S.vec)
+        v = cg_a_nodes<T, 16 / sizeof(T)>(S.N, k0, dk, S.R.code, S.x, S.r, S.u, S.uj, S.w, S.p, S.s, alpha, beta, first);
+      else
+        v = cg_a_nodes<T, 1>(S.N, k0, dk, S.R.code, S.x, S.r, S.u, S.uj, S.w, S.p, S.s, alpha, beta, first);
+      v = block_reduce<true, T>(v);
+      if (t == 0) S.part[ONE_MAX * G + b0] = (double)v;
+      if (!grid_sync(S.bar, target)) return false;
+      m0 = grid_max(S.part + ONE_MAX * G);
+      if (t == 0) cg_test(sc, m0, S.eta, S.tol_inner, S.R.maxit, 0, 0);
+      __syncthreads();
+    }
+    if (sc->round_iters) {
+      if (MODE == R_FX || MODE == R_FXG) correct_fx_nodes(S.N, k0, dk, (const float *)S.x, S.phifx, S.phi32, S.flag);
+      else correct_nodes<T>(S.N, k0, dk, S.x, S.phi, S.phi32, S.phi_lo);
+    }
+    if (!grid_sync(S.bar, target)) return false;
+  }
+}
+
+template <typename T, int MODE>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 3 : 1) k_solve_one(const __grid_constant__ OneArgs<T> S) {
+  __shared__ PoissonCtl sc;
+  PoissonCtl *ctl = S.R.c;
+  if (threadIdx.x == 0) {  // block 0 writes it back behind a barrier
+    sc = *ctl;
+    solve_reset(&sc);
+  }
+  __syncthreads();
+  unsigned target = 0;
+  const bool ok = one_solve<T, MODE>(S, &sc, target);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (!ok) ctl->sticky_status = LBE_ERR_CUDA;
+    else if (blockIdx.x == 0) *ctl = sc;
+    // the block that leaves last (none waits any more) clears the barrier
+    __threadfence();
+    if (atomicAdd(&S.bar->exits, 1u) == gridDim.x - 1) {
+      S.bar->count = 0;
+      S.bar->exits = 0;
+      S.bar->dead = 0;
     }
   }
 }
@@ -820,9 +1106,76 @@ int solve_polled(lbe_handle *h, Args &A) {
   return cudaGetLastError() == cudaSuccess ? LBE_OK : LBE_ERR_CUDA;
 }
 
+// The solve as one cooperative launch; false where the lattice, its hierarchy
+// or the device does not take it (the graph or the polled loop does).
+template <typename T>
+bool solve_one(lbe_handle *h, const Args &A, int *rc) {
+  PoissonWork &w = h->pw;
+  if (!w.one_ok || A.N > kOneNodes) return false;
+  OneArgs<T> S;
+  if (!mg_one_args(h, &S.V)) return false;
+  const void *f;
+  if (sizeof(T) == 8)
+    f = (const void *)k_solve_one<double, R_N64>;
+  else if (A.R.rhs) {
+    if (!A.phi_lo) return false;
+    f = (const void *)k_solve_one<float, R_RHS_FF>;
+  } else
+    f = h->p32.salt11 ? (const void *)k_solve_one<float, R_FX> : (const void *)k_solve_one<float, R_FXG>;
+  const ColLaunch L = make_cols(h->geo, h->phys.selfmask);
+  S.R = A.R;
+  S.R.use_cond = 0;
+  S.r = (T *)A.r;
+  S.u = (T *)A.u;
+  S.uj = (T *)A.uj;
+  S.w = (T *)A.w;
+  S.x = (T *)A.x;
+  S.p = (T *)A.p;
+  S.s = (T *)A.s;
+  S.phi = A.phi;
+  S.phi32 = A.phi32;
+  S.phi_lo = A.phi_lo;
+  S.phifx = A.phifx;
+  S.flag = A.flag;
+  S.part = w.one_part;
+  S.bar = (GridBar *)w.one_bar;
+  S.N = A.N;
+  S.eta = A.eta;
+  S.tol_inner = A.tol_inner;
+  S.cbl = 0;
+  while ((1u << S.cbl) < L.block.x) ++S.cbl;
+  S.gx = (int)L.grid.x;
+  S.blocks = (int)L.nblk();
+  S.vec = A.N % (16 / sizeof(T)) == 0;
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kBlock, 0);
+  if (e == cudaSuccess && per_sm > 0) {
+    per_sm = std::min(per_sm, kOnePerSM<T>);
+    const int G = std::min(std::min(std::max(S.blocks, std::min((S.V.ndense + 7) / 8, sms)), per_sm * sms), kOneBlocks);
+    void *args[] = {&S};
+    e = cudaLaunchCooperativeKernel(f, dim3((unsigned)G), dim3(kBlock), args, 0, h->stream);
+    if (e == cudaSuccess) {
+      h->launches += 1;
+      *rc = LBE_OK;
+      return true;
+    }
+  }
+  cudaGetLastError();  // not on this device: the other paths
+  w.one_ok = false;
+  return false;
+}
+
 template <typename T>
 int solve_t(lbe_handle *h) {
   PoissonWork &w = h->pw;
+  {
+    Args A;
+    int rc;
+    fill_args<T>(h, A);
+    if (solve_one<T>(h, A, &rc)) return rc;
+  }
   // one graph per solute buffer (flow-off steps swap the two buffers)
   const void *key = h->prm.precision == LBE_FP32 ? (const void *)h->q : (const void *)h->n;
   int slot = -1;
@@ -876,6 +1229,15 @@ cudaError_t poisson_alloc(lbe_handle *h) {
   // e.g. for profilers that do not follow conditional graph nodes
   const char *env = getenv("LBE_POISSON_GRAPH");
   w.graph_ok = !(env && env[0] == '0');
+  int dev = 0, coop = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) != cudaSuccess) return e;
+  w.one_ok = coop && w.graph_ok && N <= kOneNodes;
+  if (w.one_ok) {
+    if ((e = cudaMalloc(&w.one_part, sizeof(double) * 3 * kOneBlocks)) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&w.one_bar, sizeof(GridBar))) != cudaSuccess) return e;
+    if ((e = cudaMemset(w.one_bar, 0, sizeof(GridBar))) != cudaSuccess) return e;
+  }
   return cudaSuccess;
 }
 
@@ -887,6 +1249,8 @@ void poisson_free(lbe_handle *h) {
   cudaFree(w.vec);
   cudaFree(w.partial);
   cudaFree(w.phi_prev);
+  cudaFree(w.one_part);
+  cudaFree(w.one_bar);
   cudaFree(w.ctl);
   if (w.ctl_host) cudaFreeHost(w.ctl_host);
   w = PoissonWork{};
@@ -924,6 +1288,8 @@ int poisson_solve_linear(lbe_handle *h, const double *rhs, double *x, double tol
   A.R.tol = tol_abs;
   A.R.tol_rel = tol_rel;
   A.tol_inner = 0.25 * tol_abs;
+  int rc;
+  if (solve_one<float>(h, A, &rc)) return rc;
   if (!w.graph_ok) return solve_polled<float>(h, A);
   if (!w.exec_lin || w.lin_key[0] != rhs || w.lin_key[1] != x || w.lin_key[2] != x_hi) {
     if (w.exec_lin) cudaGraphExecDestroy(w.exec_lin);
@@ -984,12 +1350,16 @@ int poisson_status(lbe_handle *h, lbe_stats *st, long long *kernels) {
     st->poisson_max_iters = (int)(c.solve_iters > c.max_solve_iters ? c.solve_iters : c.max_solve_iters);
     st->poisson_residual = c.res;
   }
-  if (kernels && w.graph_ok) {
+  if (kernels && w.graph_ok && !w.one_ok) {  // the single-kernel solves are counted as they are launched
     // kernels of the graph path: per solve the reset; per residual test the
     // test and the correction; per iteration V-cycle (with multigrid),
     // stencil and update
     const long long vc = mg_kernels_per_cycle(h);
     *kernels = c.solves + 2 * c.total_rounds + (2 + vc) * c.total_iters;
+  }
+  if (c.sticky_status == LBE_ERR_CUDA) {
+    h->err = "poisson: a wait between the solve's blocks ran out";
+    return LBE_ERR_CUDA;
   }
   if (c.sticky_status == LBE_ERR_NOCONVERGE || c.status == LBE_ERR_NOCONVERGE) {
     h->err = "poisson: no convergence within poisson_max_iter";
