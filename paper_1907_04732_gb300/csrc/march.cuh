@@ -21,7 +21,7 @@
 // rounds nx up to a power of two).
 #pragma once
 
-#include "lbe_internal.cuh"
+#include "mg_device.cuh"
 
 namespace lbe {
 
@@ -87,6 +87,7 @@ struct Cols {
   int K;                  // planes per thread
   int selfw;              // 6 x the weights of the links that join a node to itself
   int ahead;              // planes to prefetch ahead of the march (0: none)
+  float omega;            // the V-cycle's Jacobi weight (jacobi_weight)
   FastDiv fnx;
 };
 struct ColLaunch {
@@ -119,6 +120,14 @@ inline int planes_per_thread(long long gx, int nz, int zb, int unit = 1) {
   return bestK;
 }
 
+// The V-cycle's Jacobi weight.  A lattice with one axis longer than one node
+// is a chain: its Jacobi-scaled operator reaches 2, where the weight 1 that
+// suits wider lattices (at most 1.6) does not damp the alternating mode at
+// all, and 2/3 is the best for the upper half of its modes.
+inline float jacobi_weight(const Geo &g, float omega) {
+  return (g.nx > 1) + (g.ny > 1) + (g.nz > 1) == 1 ? omega * (2.f / 3.f) : omega;
+}
+
 inline ColLaunch make_cols(const Geo &g, uint32_t selfmask) {
   ColLaunch L;
   L.c.nx = g.nx;
@@ -136,6 +145,7 @@ inline ColLaunch make_cols(const Geo &g, uint32_t selfmask) {
   // a lattice whose vectors exceed L2 is read from HBM: its latency is
   // covered by prefetching the columns' next planes into L2
   L.c.ahead = g.N > kPrefetchNodes ? 3 : 0;
+  L.c.omega = jacobi_weight(g, mgd::kOmega);
   L.block = dim3((unsigned)cb, (unsigned)zb);
   L.grid = dim3((unsigned)gx, (unsigned)((g.nz + (long long)K * zb - 1) / ((long long)K * zb)));
   return L;

@@ -95,9 +95,10 @@ __global__ void k_post(const MgLevel L, const T *__restrict__ A, const T *__rest
   if (c && c->inner_done) return;
   int X, Y, Z, I;
   if (!lnode(L, X, Y, Z, I)) return;
-  // FP64: the division omega/diag costs more than its stored value (float
-  // measured 2 % of the solve the other way round: one more load)
-  out[I] = sizeof(T) == 8 ? post_value_w(L, A, W[I], r, z, C, ec, X, Y, Z) : post_value_z(L, A, r, z, C, ec, X, Y, Z);
+  // W null: omega/diag by division.  FP64: the division costs more than its
+  // stored value (float measured 2 % of the solve the other way round: one
+  // more load, so it reads W only where the weight is not kOmega)
+  out[I] = W ? post_value_w(L, A, W[I], r, z, C, ec, X, Y, Z) : post_value_z(L, A, r, z, C, ec, X, Y, Z);
 }
 
 template <typename T>
@@ -235,11 +236,11 @@ __global__ void __launch_bounds__(256) k_dense(int N, int stride, const T *__res
 
 // omega/diag of a level (0 for a node without fluid)
 template <typename T>
-__global__ void k_weights(int N, const T *__restrict__ A13, T *__restrict__ W) {
+__global__ void k_weights(int N, float omega, const T *__restrict__ A13, T *__restrict__ W) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   const T d = A13[i];
-  W[i] = d != (T)0 ? (T)kOmega / d : (T)0;
+  W[i] = d != (T)0 ? (T)omega / d : (T)0;
 }
 
 dim3 lgrid(const MgLevel &L, dim3 &block) {
@@ -411,7 +412,7 @@ static cudaError_t mg_setup_t(lbe_handle *h) {
   if (le != cudaSuccess) return le;
   for (int l = 1; l < mg.nlev; ++l)
     k_weights<T><<<(unsigned)((mg.lv[l].N + 255) / 256), 256, 0, h->stream>>>(
-        (int)mg.lv[l].N, (const T *)mg.lv[l].A + 13 * mg.lv[l].N, (T *)mg.lv[l].W);
+        (int)mg.lv[l].N, jacobi_weight(g, kOmega), (const T *)mg.lv[l].A + 13 * mg.lv[l].N, (T *)mg.lv[l].W);
   le = cudaGetLastError();
   if (le != cudaSuccess) return le;
   mg.ld = mg.nlev - 1;
@@ -508,11 +509,12 @@ static cudaError_t mg_vcycle_t(lbe_handle *h, const void *r0, const void *uj, vo
     nodes.push_back(Node{(void *)k_coarsest<T>, dim3(1), dim3(kCoarseMax),
                          {&lv[nl - 1], P(mg.lv[nl - 1].A), P(mg.lv[nl - 1].r), P(mg.lv[nl - 1].e), P(c)}});
   // up: fused prolongation + post-smoothing
+  const bool use_w = sizeof(T) == 8 || jacobi_weight(h->geo, kOmega) != kOmega;
   for (int l = lk - 1; l >= 1; --l) {
     dim3 blk;
     const dim3 grd = lgrid(lv[l], blk);
     nodes.push_back(Node{(void *)k_post<T>, grd, blk,
-                         {&lv[l], P(mg.lv[l].A), P(mg.lv[l].W), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1],
+                         {&lv[l], P(mg.lv[l].A), P(use_w ? mg.lv[l].W : nullptr), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1],
                           P(mg.lv[l + 1].e), P(mg.lv[l].e), P(c)}});
   }
   nodes.push_back(Node{(void *)k_post0<T>, L0.grid, L0.block,

@@ -55,7 +55,7 @@ __device__ __forceinline__ void restrict0_block(const Cols &F, const uint8_t *co
         int i;
         const T nsum = m.step(u, o, p, F.plane, F.nz, z, u0, i);
         const int cd = code[i];
-        const T res = r[i] - (T)kOmega * ((T)((cd & kCodeDiag) + F.selfw) * u0 - nsum) * (T)(1.0 / 6.0);
+        const T res = r[i] - (T)F.omega * ((T)((cd & kCodeDiag) + F.selfw) * u0 - nsum) * (T)(1.0 / 6.0);
         v += cd ? res : (T)0;
       }
     }
@@ -134,7 +134,7 @@ __device__ __forceinline__ void post0_column(const Cols &F, const Column &col, c
   q.ym = C.nx * (((col.y == 0 ? F.ny - 1 : col.y - 1) >> C.sy) - Y);
   q.yp = C.nx * (((col.y == F.ny - 1 ? 0 : col.y + 1) >> C.sy) - Y);
   const int P = X + C.nx * Y;
-  const T om = (T)kOmega, al = (T)kAlpha;
+  const T om = (T)F.omega, al = (T)kAlpha;
   ZMarch<T> m;
   m.begin(u, col.o, col.p, F.plane, F.nz, col.z0);
   int Z = col.z0 >> C.sz;
