@@ -297,34 +297,45 @@ static bool coarse_inverse_t(const mgd::MgLevel &L, const std::vector<T> &A27, s
     }
   }
   if (!(dmax > 0.0) || asym > 1e-5 * amax) return false;
-  // Cholesky, lower triangle in place
+  // Cholesky A = U^T U by rows of U, then the inverse's lower triangle X from
+  // U^T Y = I and U X = Y.  Every inner loop runs along contiguous rows, with
+  // independent elements: the compiler vectorises it, and none waits for the
+  // sum before it (dot products down the columns of a 256-node level took 9 ms,
+  // as long as forty steps of the lattice that needs it).
   for (int j = 0; j < n; ++j) {
-    double d = M[(size_t)j * n + j];
-    for (int k = 0; k < j; ++k) d -= M[(size_t)j * n + k] * M[(size_t)j * n + k];
-    if (!(d > 1e-10 * dmax)) return false;
-    const double ljj = std::sqrt(d);
-    M[(size_t)j * n + j] = ljj;
-    for (int i = j + 1; i < n; ++i) {
-      double s = M[(size_t)i * n + j];
-      for (int k = 0; k < j; ++k) s -= M[(size_t)i * n + k] * M[(size_t)j * n + k];
-      M[(size_t)i * n + j] = s / ljj;
+    double *u = &M[(size_t)j * n];
+    for (int k = 0; k < j; ++k) {
+      const double *uk = &M[(size_t)k * n];
+      const double f = uk[j];
+      for (int i = j; i < n; ++i) u[i] -= f * uk[i];
     }
+    if (!(u[j] > 1e-10 * dmax)) return false;
+    const double ujj = std::sqrt(u[j]), s = 1.0 / ujj;
+    u[j] = ujj;
+    for (int i = j + 1; i < n; ++i) u[i] *= s;
   }
-  // columns of A^-1: solve L y = e_c, L^T x = y
-  std::vector<double> x(n);
-  for (int cidx = 0; cidx < n; ++cidx) {
-    for (int i = 0; i < cidx; ++i) x[i] = 0.0;  // y vanishes above the unit entry
-    for (int i = cidx; i < n; ++i) {
-      double s = i == cidx ? 1.0 : 0.0;
-      for (int k = cidx; k < i; ++k) s -= M[(size_t)i * n + k] * x[k];
-      x[i] = s / M[(size_t)i * n + i];
+  std::vector<double> X((size_t)n * n, 0.0);
+  for (int i = 0; i < n; ++i) {
+    double *x = &X[(size_t)i * n];
+    x[i] = 1.0;
+    for (int k = 0; k < i; ++k) {
+      const double f = M[(size_t)k * n + i], *xk = &X[(size_t)k * n];
+      for (int c = 0; c <= k; ++c) x[c] -= f * xk[c];
     }
-    for (int i = n - 1; i >= 0; --i) {
-      double s = x[i];
-      for (int k = i + 1; k < n; ++k) s -= M[(size_t)k * n + i] * x[k];
-      x[i] = s / M[(size_t)i * n + i];
+    const double s = 1.0 / M[(size_t)i * n + i];
+    for (int c = 0; c <= i; ++c) x[c] *= s;
+  }
+  for (int i = n - 1; i >= 0; --i) {
+    double *x = &X[(size_t)i * n];
+    for (int k = i + 1; k < n; ++k) {
+      const double f = M[(size_t)i * n + k], *xk = &X[(size_t)k * n];
+      for (int c = 0; c <= i; ++c) x[c] -= f * xk[c];
     }
-    for (int i = 0; i < n; ++i) inv[(size_t)act[i] * N + act[cidx]] = (T)x[i];
+    const double s = 1.0 / M[(size_t)i * n + i];
+    for (int c = 0; c <= i; ++c) {
+      x[c] *= s;
+      inv[(size_t)act[i] * N + act[c]] = inv[(size_t)act[c] * N + act[i]] = (T)x[c];
+    }
   }
   return true;
 }
