@@ -28,9 +28,8 @@
 #include <thread>
 #include <vector>
 
-#include "fp32_device.cuh"
-#include "march.cuh"
-#include "mg_device.cuh"
+#include "solve_device.cuh"
+#include "vcycle.cuh"
 
 constexpr int kBE = LBE_BATCH_MAX_ELECTRODES;  // electrodes per instance
 
@@ -67,6 +66,16 @@ struct InstDev {
   P32 P;
 };
 
+// The column march (march.cuh) of one instance's finest-level solve kernels:
+// its blocks of 256 columns' chunks, first entry in the partials, and the
+// blocks of the restriction into level 1.
+struct InstMarch {
+  Cols c;
+  int cbl, gx, blocks, part0;
+  mgd::RestrictMap M;
+  int g0x, g0y;
+};
+
 // one multigrid level of one instance: its shape (component stride = the
 // level's total node count), first node in the level arrays, first tile in
 // the level's tile list, tile count
@@ -99,6 +108,7 @@ struct BatchCtl {
 // CG vectors (each Ntot floats)
 struct CgVec {
   float *r, *u, *w, *x, *p, *s;
+  float *uj;  // r/diag of instances with a hierarchy (the others keep it in u)
 };
 
 }  // namespace lbe
@@ -125,6 +135,10 @@ struct lbe_batch {
   int *tile_inst = nullptr;
   uint8_t *id = nullptr;
   uint32_t *mask = nullptr;
+  uint8_t *code = nullptr;            // node codes of the solve's kernels (march.cuh)
+  lbe::InstMarch *im = nullptr;       // [n]
+  int *mpref = nullptr;               // [n + 1] prefix sums of InstMarch::blocks
+  int MT = 0;                         // their sum
   float *f[2] = {nullptr, nullptr};  // populations: f[0], updated in place
   bool aa_odd = false;                // the next step is an odd one of the AA pattern
   int64_t *q = nullptr, *qstar = nullptr;
@@ -136,7 +150,7 @@ struct lbe_batch {
   float4 *u = nullptr;            // velocity records (fp32::octant_code)
   float4 *lf = nullptr;     // link records, one per node (fp32::link_record)
   float *vec = nullptr;     // CG vectors [6][Ntot]
-  double *part = nullptr;   // per-tile partials [3][T]
+  double *part = nullptr;   // partials (r,u) and (w,u) [2][MT], maxima [max(T, MT)]
   double *psi_d = nullptr;  // [n][kBE + 1]
   lbe::InstCtl *ictl = nullptr;
   lbe::BatchCtl *bctl = nullptr, *bctl_h = nullptr;
@@ -155,7 +169,8 @@ struct lbe_batch {
   int *mg_tiles = nullptr;               // tile -> instance, levels 1.. concatenated
   lbe::LvSeg *mg_seg = nullptr;          // [kMaxLevels][n]
   lbe::LvPtrs mg_p{};
-  float *mg_t0 = nullptr;
+  float *mg_t0 = nullptr;                // the Jacobi vector r/diag of instances with a hierarchy
+  float *mg_w1 = nullptr;                // omega/diag of level 1
   float *mg_cinv = nullptr;          // inverses of the coarsest operators, concatenated
   long long *mg_cinv_off = nullptr;  // device [n]: an instance's inverse (-1: Jacobi sweeps)
   // step graphs keyed by (in-place step kind, solute read); [4] = solve
@@ -172,7 +187,7 @@ struct lbe_batch {
 
   lbe::CgVec cg() const {
     const long long N = Ntot;
-    return lbe::CgVec{vec, vec + N, vec + 2 * N, vec + 3 * N, vec + 4 * N, vec + 5 * N};
+    return lbe::CgVec{vec, vec + N, vec + 2 * N, vec + 3 * N, vec + 4 * N, vec + 5 * N, mg_t0};
   }
 };
 
@@ -187,6 +202,17 @@ constexpr int kMaxOuterB = 24;
 //   f = nlev + l    level-l tiles of instances that have level l+1
 __host__ __device__ constexpr int famA(int l) { return l; }
 __host__ __device__ constexpr int famB(int nlev, int l) { return nlev + l; }
+//   f = 2 nlev - 1  column blocks of the march, 2 nlev those of instances
+//   with a hierarchy, 2 nlev + 1 blocks of the restriction into level 1
+__host__ __device__ constexpr int famM(int nlev) { return 2 * nlev - 1; }
+__host__ __device__ constexpr int famP(int nlev) { return 2 * nlev; }
+__host__ __device__ constexpr int famR(int nlev) { return 2 * nlev + 1; }
+
+// this thread's column chunk of block b of an instance
+__device__ __forceinline__ bool march_column(const InstMarch &I, int b, Column &c) {
+  const int tx = threadIdx.x & ((1 << I.cbl) - 1), ty = threadIdx.x >> I.cbl;
+  return column_at(I.c, ((b % I.gx) << I.cbl) + tx, (b / I.gx) * (kBlock >> I.cbl) + ty, c);
+}
 
 // instance-local coordinates of node lo (false past the instance's end)
 __device__ __forceinline__ bool node_xyz(const InstDev &I, int lo, int &x, int &y, int &z) {
@@ -458,66 +484,52 @@ __global__ void kb_solve_reset(int n, InstCtl *c, BatchCtl *b, int *hist, int se
   if (i == 0) b->solves += 1;
 }
 
-// Residual (float-float, phi = hi + lo) of the instances still solving;
-// seeds their CG (r, u = r/diag, x = p = s = 0); per-tile max |r|/diag
-__global__ void __launch_bounds__(kBlock) kb_res(const InstDev *__restrict__ inst, const int *__restrict__ tile_inst,
-                                                 int T, int Ntot, const uint32_t *__restrict__ mask,
+// Residual (res_column, R_FX) of the instances still solving; seeds their CG
+// (r and the Jacobi vector r/diag); max |r|/diag per column block.  The
+// stencil kernels march columns as the single lattice's do: reading 18
+// neighbours with an address, a mask bit and a weight each, the solve of 64
+// capacitors (33 M nodes) took 17.5 ms per step, 13.4 marched.
+__global__ void __launch_bounds__(kBlock) kb_res(const InstDev *__restrict__ inst, const InstMarch *__restrict__ im,
+                                                 int n, const int *__restrict__ mpref, int Ntot,
+                                                 const uint32_t *__restrict__ mask, const uint8_t *__restrict__ code,
                                                  const int64_t *__restrict__ qn, const int64_t *__restrict__ phifx,
-                                                 const CgVec v,
-                                                 double *__restrict__ part, const InstCtl *__restrict__ c) {
-  for (int t = blockIdx.x; t < T; t += gridDim.x) {
-    const int ii = tile_inst[t];
+                                                 const CgVec v, double *__restrict__ part,
+                                                 const InstCtl *__restrict__ c) {
+  const int MT = mpref[n];
+  for (int t = blockIdx.x; t < MT; t += gridDim.x) {
+    const int ii = find_inst(mpref, n, t);
     if (c[ii].outer_done) continue;  // block-uniform
     const InstDev &I = inst[ii];
-    float mx = 0.f;
-#pragma unroll
-    for (int k = 0; k < kSub; ++k) {
-      int x, y, z;
-      const int lo = (t - I.tile0) * kTile + k * kBlock + threadIdx.x;
-      if (!node_xyz(I, lo, x, y, z)) continue;
-      const int r = I.off + lo;
-      const uint32_t m = mask[r];
-      if (!(m & kFluidBit)) {
-        v.r[r] = v.u[r] = v.x[r] = v.p[r] = v.s[r] = 0.f;
-        continue;
-      }
-      // 6 res = 6 lap(phi) + 6 (4 pi l_B s)(q+ - q-): 6 lap exact in fixed
-      // point, split into float-float and added to the charge term in
-      // float-float (as the single lattice's residual)
-      const long long L6 = fp32::lap6_fx(I.g, r, x, y, z, m, phifx);
-      const float Lh = ll2f(L6);
-      const float S = __fmul_rn(Lh, fp32::kPhiUnitF), E = __fmul_rn(ll2f(L6 - f2ll_rn(Lh)), fp32::kPhiUnitF);
-      const long long dq = qn[r] - qn[Ntot + r];  // 1:1 salt, one bulk value
-      const float dq_hi = ll2f(dq), dq_lo = ll2f(dq - f2ll_rn(dq_hi));
-      const float Bv = I.c6_hi * dq_hi;
-      const float Be = fmaf(I.c6_hi, dq_hi, -Bv) + (I.c6_hi * dq_lo + I.c6_lo * dq_hi);
-      float t6, te6;
-      fp32::two_sum(S, Bv, t6, te6);
-      const float rf = (t6 + (te6 + (E + Be))) * (1.f / 6.f);
-      const float dinv = __fdividef(6.f, (float)mgd::diag6(m, I.selfmask));
-      v.r[r] = rf;
-      v.u[r] = rf * dinv;
-      v.x[r] = v.p[r] = v.s[r] = 0.f;
-      mx = fmaxf(mx, finite_or_inf(fabsf(rf) * dinv));
-    }
+    ResArgs A;
+    A.cols = im[ii].c;
+    A.g.N = Ntot;  // the solute's component stride
+    A.code = code + I.off;
+    A.mask = mask + I.off;
+    A.nq = qn + I.off;
+    A.phifx = phifx + I.off;
+    A.c6_hi = I.c6_hi;
+    A.c6_lo = I.c6_lo;
+    float mx = 0.f, mb = 0.f;
+    Column col;
+    if (march_column(im[ii], t - mpref[ii], col))
+      res_column<float, R_FX>(A, col, v.r + I.off, (I.mg_levels >= 2 ? v.uj : v.u) + I.off, mx, mb);
     mx = breducef<true>(mx);
-    if (threadIdx.x == 0) part[2LL * T + t] = (double)mx;
+    if (threadIdx.x == 0) part[2LL * MT + t] = (double)mx;
   }
 }
 
 // per-instance outer test (one block per instance); the last block sets the
 // refinement loop's condition (any instance still solving) and rebuilds the
 // active-tile lists
-__global__ void __launch_bounds__(kBlock) kb_outer(const InstDev *__restrict__ inst, int n, int T,
+__global__ void __launch_bounds__(kBlock) kb_outer(const InstMarch *__restrict__ im, int n, int MT,
                                                    const double *__restrict__ part, InstCtl *c, BatchCtl *b,
                                                    double tol, int maxit, int nfam, const int *__restrict__ fam_cnt,
                                                    int *__restrict__ fam_pref, cudaGraphConditionalHandle hout,
                                                    cudaGraphConditionalHandle hin, int use_cond) {
   const int ii = blockIdx.x;
   if (!c[ii].outer_done) {
-    const InstDev &I = inst[ii];
     double m = 0.0;
-    for (int k = threadIdx.x; k < I.ntiles; k += kBlock) m = fmax(m, __ldcg(part + 2LL * T + I.tile0 + k));
+    for (int k = threadIdx.x; k < im[ii].blocks; k += kBlock) m = fmax(m, __ldcg(part + 2LL * MT + im[ii].part0 + k));
     m = breduce<true>(m);
     if (threadIdx.x == 0) {
       InstCtl &C = c[ii];
@@ -555,38 +567,26 @@ __global__ void __launch_bounds__(kBlock) kb_outer(const InstDev *__restrict__ i
   build_active(c, n, nfam, fam_cnt, fam_pref);
 }
 
-// w = A u (fluid operator) on the active tiles; per-tile partials (r,u), (w,u)
-__global__ void __launch_bounds__(kBlock) kb_cg_b(const InstDev *__restrict__ inst, int n, const int *__restrict__ pref,
-                                                  int T, const uint32_t *__restrict__ mask,
-                                                  const float *__restrict__ r_, const float *__restrict__ u_,
-                                                  float *__restrict__ w_, double *__restrict__ part) {
-  const int Tact = pref[n];
-  for (int tp = blockIdx.x; tp < Tact; tp += gridDim.x) {
-    const int ii = find_inst(pref, n, tp);
-    const InstDev &I = inst[ii];
-    const int j = tp - pref[ii];
+// w = A u (fluid operator) on the active column blocks; their (r,u), (w,u)
+__global__ void __launch_bounds__(kBlock) kb_cg_b(const InstDev *__restrict__ inst, const InstMarch *__restrict__ im,
+                                                  int n, const int *__restrict__ pref, int MT,
+                                                  const uint8_t *__restrict__ code, const float *__restrict__ r_,
+                                                  const float *__restrict__ u_, float *__restrict__ w_,
+                                                  double *__restrict__ part) {
+  const int act = pref[n];
+  for (int t = blockIdx.x; t < act; t += gridDim.x) {
+    const int ii = find_inst(pref, n, t);
+    const int j = t - pref[ii], off = inst[ii].off;
+    const Cols C = im[ii].c;
     float ru = 0.f, wu = 0.f;
-#pragma unroll
-    for (int k = 0; k < kSub; ++k) {
-      int x, y, z;
-      const int lo = j * kTile + k * kBlock + threadIdx.x;
-      if (!node_xyz(I, lo, x, y, z)) continue;
-      const int r = I.off + lo;
-      const uint32_t m = mask[r];
-      if (!(m & kFluidBit)) continue;
-      const float u0 = u_[r];
-      const float s6 = mgd::nbsum6(m, I.selfmask, offsets_of(I.g, x, y, z), r, u_);
-      const float wv = ((float)mgd::diag6(m, I.selfmask) * u0 - s6) * (1.f / 6.f);
-      w_[r] = wv;
-      ru += r_[r] * u0;
-      wu += wv * u0;
-    }
+    Column col;
+    if (march_column(im[ii], j, col)) cg_b_column(C, col, code + off, u_ + off, r_ + off, w_ + off, ru, wu);
     ru = breducef<false>(ru);
     wu = breducef<false>(wu);
     if (threadIdx.x == 0) {
-      const int t = I.tile0 + j;
-      part[t] = (double)ru;
-      part[(long long)T + t] = (double)wu;
+      const int at = im[ii].part0 + j;
+      part[at] = (double)ru;
+      part[(long long)MT + at] = (double)wu;
     }
   }
 }
@@ -595,15 +595,14 @@ __global__ void __launch_bounds__(kBlock) kb_cg_b(const InstDev *__restrict__ in
 // of the update that follows.  A breakdown (the correction is converged to
 // rounding, or a zero residual) ends the instance's inner solve without an
 // update.
-__global__ void __launch_bounds__(kBlock) kb_scal(const InstDev *__restrict__ inst, int T,
+__global__ void __launch_bounds__(kBlock) kb_scal(const InstMarch *__restrict__ im, int MT,
                                                   const double *__restrict__ part, InstCtl *c) {
   const int ii = blockIdx.x;
   if (c[ii].inner_done) return;
-  const InstDev &I = inst[ii];
   double g = 0.0, d = 0.0;
-  for (int k = threadIdx.x; k < I.ntiles; k += kBlock) {
-    g += __ldcg(part + I.tile0 + k);
-    d += __ldcg(part + (long long)T + I.tile0 + k);
+  for (int k = threadIdx.x; k < im[ii].blocks; k += kBlock) {
+    g += __ldcg(part + im[ii].part0 + k);
+    d += __ldcg(part + (long long)MT + im[ii].part0 + k);
   }
   g = breduce<false>(g);
   d = breduce<false>(d);
@@ -630,7 +629,7 @@ __global__ void __launch_bounds__(kBlock) kb_scal(const InstDev *__restrict__ in
 // instance); the last block sets the CG loop's condition (any instance still
 // iterating) and rebuilds the active-tile lists.  The loop ends here, before
 // the V-cycle and the stencil that the next update would need.
-__global__ void __launch_bounds__(kBlock) kb_test(const InstDev *__restrict__ inst, int n, int T,
+__global__ void __launch_bounds__(kBlock) kb_test(const InstDev *__restrict__ inst, int n, int MT,
                                                   const double *__restrict__ part, InstCtl *c, BatchCtl *b,
                                                   double eta, double tol_abs, int maxit, int nfam,
                                                   const int *__restrict__ fam_cnt, int *__restrict__ fam_pref,
@@ -639,7 +638,7 @@ __global__ void __launch_bounds__(kBlock) kb_test(const InstDev *__restrict__ in
   if (!c[ii].inner_done) {
     const InstDev &I = inst[ii];
     double m = 0.0;
-    for (int k = threadIdx.x; k < I.ntiles; k += kBlock) m = fmax(m, __ldcg(part + 2LL * T + I.tile0 + k));
+    for (int k = threadIdx.x; k < I.ntiles; k += kBlock) m = fmax(m, __ldcg(part + 2LL * MT + I.tile0 + k));
     m = breduce<true>(m);
     if (threadIdx.x == 0) {
       InstCtl &C = c[ii];
@@ -664,13 +663,14 @@ __global__ void __launch_bounds__(kBlock) kb_test(const InstDev *__restrict__ in
   build_active(c, n, nfam, fam_cnt, fam_pref);
 }
 
-// p = u + beta p, s = w + beta s, x += alpha p, r -= alpha s, u = r/diag on
-// the active tiles; per-tile max |r|/diag
+// p = u + beta p, s = w + beta s, x += alpha p, r -= alpha s, uj = r/diag on
+// the active tiles (a round's first update starts x, p and s; every vector is
+// zero on solid nodes); per-tile max |r|/diag
 __global__ void __launch_bounds__(kBlock) kb_cg_a(const InstDev *__restrict__ inst, int n, const int *__restrict__ pref,
-                                                  int T, const uint32_t *__restrict__ mask, const CgVec v,
+                                                  int MT, const uint8_t *__restrict__ code, const CgVec v,
                                                   double *__restrict__ part, const InstCtl *__restrict__ c) {
   float *__restrict__ r_ = v.r;
-  float *__restrict__ u_ = v.u;
+  const float *u_ = v.u;
   const float *__restrict__ w_ = v.w;
   float *__restrict__ x_ = v.x;
   float *__restrict__ p_ = v.p;
@@ -682,27 +682,37 @@ __global__ void __launch_bounds__(kBlock) kb_cg_a(const InstDev *__restrict__ in
     const InstDev &I = inst[ii];
     const int j = tp - pref[ii];
     const float alpha = (float)c[ii].alpha, beta = (float)c[ii].beta;
-    float mx = 0.f;
+    const bool first = c[ii].round_iters == 0;
+    float *uj = I.mg_levels >= 2 ? v.uj : v.u;
+    float uv[kSub], wv[kSub], rv[kSub], dv[kSub], mx = 0.f;
+#pragma unroll
+    for (int k = 0; k < kSub; ++k) {  // the loads of the thread's nodes go out together
+      const int lo = j * kTile + k * kBlock + threadIdx.x;
+      const bool in = lo < I.g.N;
+      const int r = I.off + lo;
+      uv[k] = in ? u_[r] : 0.f;
+      wv[k] = in ? w_[r] : 0.f;
+      rv[k] = in ? r_[r] : 0.f;
+      dv[k] = in ? inv_diag<float>(code[r]) : 0.f;
+    }
 #pragma unroll
     for (int k = 0; k < kSub; ++k) {
       const int lo = j * kTile + k * kBlock + threadIdx.x;
       if (lo >= I.g.N) continue;
       const int r = I.off + lo;
-      const uint32_t m = mask[r];
-      if (!(m & kFluidBit)) continue;
-      const float pv = u_[r] + beta * p_[r];
-      const float sv = w_[r] + beta * s_[r];
+      const float pv = first ? uv[k] : uv[k] + beta * p_[r];
+      const float sv = first ? wv[k] : wv[k] + beta * s_[r];
+      const float xv = first ? alpha * pv : x_[r] + alpha * pv;
+      const float rn = rv[k] - alpha * sv;
       p_[r] = pv;
       s_[r] = sv;
-      x_[r] += alpha * pv;
-      const float rv = r_[r] - alpha * sv;
-      r_[r] = rv;
-      const float dinv = __fdividef(6.f, (float)mgd::diag6(m, I.selfmask));
-      u_[r] = rv * dinv;
-      mx = fmaxf(mx, finite_or_inf(fabsf(rv) * dinv));
+      x_[r] = xv;
+      r_[r] = rn;
+      uj[r] = rn * dv[k];
+      mx = fmaxf(mx, finite_or_inf(fabsf(rn) * dv[k]));
     }
     mx = breducef<true>(mx);
-    if (threadIdx.x == 0) part[2LL * T + I.tile0 + j] = (double)mx;
+    if (threadIdx.x == 0) part[2LL * MT + I.tile0 + j] = (double)mx;
   }
 }
 
@@ -717,7 +727,7 @@ __global__ void kb_correct(const InstDev *__restrict__ inst, const int *__restri
   bool over = false;
   for (int t = blockIdx.x; t < T; t += gridDim.x) {
     const int ii = tile_inst[t];
-    if (!c[ii].solving) continue;
+    if (!c[ii].solving || c[ii].round_iters == 0) continue;  // done, or no update in this round
     const InstDev &I = inst[ii];
     for (int k = 0; k < kSub; ++k) {
       const int lo = (t - I.tile0) * kTile + k * kBlock + threadIdx.x;
@@ -844,38 +854,22 @@ __device__ __forceinline__ void store_coarse(const LvSeg &C, int I, float v, con
   zc[C.off + I] = d != 0.f ? mgd::kOmega * v / d : 0.f;
 }
 
-// Restriction into level 1 over the active level-1 tiles.  Work item: 32
-// coarse nodes, 8 threads each (one per child, fixed-order shuffle sum).  A
-// fluid child's pre-smoothed residual is r - omega A u: u = r/diag is the
-// Jacobi vector the CG just formed.
-__global__ void __launch_bounds__(kBlock) kbm_restrict0(const InstDev *__restrict__ inst, int n,
+// restriction into level 1 over the active blocks (restrict0_block)
+__global__ void __launch_bounds__(kBlock) kbm_restrict0(const InstDev *__restrict__ inst,
+                                                        const InstMarch *__restrict__ im, int n,
                                                         const int *__restrict__ pref, const LvSeg *__restrict__ seg1,
-                                                        const uint32_t *__restrict__ mask, const float *__restrict__ r,
-                                                        const float *__restrict__ u, const float *__restrict__ A1,
+                                                        const uint8_t *__restrict__ code, const float *__restrict__ r,
+                                                        const float *__restrict__ u, const float *__restrict__ W1,
                                                         float *__restrict__ rc, float *__restrict__ zc) {
-  const int items = pref[n] * (kTile / 32);
-  const int ch = threadIdx.x & 7;
-  for (int ip = blockIdx.x; ip < items; ip += gridDim.x) {
-    const int tp = ip / (kTile / 32);
-    const int ii = find_inst(pref, n, tp);
-    const LvSeg C = seg1[ii];
-    const InstDev &In = inst[ii];
-    const int I = (tp - pref[ii]) * kTile + (ip % (kTile / 32)) * 32 + (threadIdx.x >> 3);
-    float v = 0.f;
-    int X, Y, Z, x, y, z;
-    if (I < C.L.N) {
-      lv_xyz(C, I, X, Y, Z);
-      if (mgd::child_of(C.L, X, Y, Z, ch, In.g.nx, In.g.ny, In.g.nz, x, y, z)) {
-        const int i = In.off + x + In.g.nx * (y + In.g.ny * z);
-        const uint32_t m = mask[i];
-        if (m & kFluidBit) {
-          const float s6 = mgd::nbsum6(m, In.selfmask, offsets_of(In.g, x, y, z), i, u);
-          v = r[i] - mgd::kOmega * ((float)mgd::diag6(m, In.selfmask) * u[i] - s6) * (1.f / 6.f);
-        }
-      }
-    }
-    v = mgd::sum8(v);
-    if (ch == 0 && I < C.L.N) store_coarse(C, I, v, A1, rc, zc);
+  const int act = pref[n];
+  for (int t = blockIdx.x; t < act; t += gridDim.x) {
+    const int ii = find_inst(pref, n, t);
+    const int j = t - pref[ii], off = inst[ii].off, co = seg1[ii].off;
+    const InstMarch I = im[ii];
+    const MgLevel C = seg1[ii].L;
+    const int bx = j % I.g0x, q = j / I.g0x;
+    mgd::restrict0_block(I.c, code + off, r + off, u + off, C, W1 + co, rc + co, zc + co, I.M, bx, q % I.g0y,
+                         q / I.g0y);
   }
 }
 
@@ -954,56 +948,31 @@ __global__ void __launch_bounds__(kBlock) kbm_post(int n, const int *__restrict_
   }
 }
 
-// level 0 over the active tiles of instances with a hierarchy:
-// t = omega u + alpha P e_1 (u = r/diag, the Jacobi vector)
-__global__ void __launch_bounds__(kBlock) kbm_prolong0(const InstDev *__restrict__ inst, int n,
+// fused prolongation and post-smoothing of level 0 over the active column
+// blocks of instances with a hierarchy (post0_column)
+__global__ void __launch_bounds__(kBlock, 4) kbm_post0(const InstDev *__restrict__ inst,
+                                                       const InstMarch *__restrict__ im, int n,
                                                        const int *__restrict__ pref, const LvSeg *__restrict__ seg1,
-                                                       const uint32_t *__restrict__ mask, const float *__restrict__ u,
-                                                       const float *__restrict__ e1, float *__restrict__ t0) {
-  const int Tact = pref[n];
-  for (int tp = blockIdx.x; tp < Tact; tp += gridDim.x) {
-    const int ii = find_inst(pref, n, tp);
-    const InstDev &I = inst[ii];
-    const LvSeg C = seg1[ii];
-    const int j = tp - pref[ii];
-#pragma unroll
-    for (int k = 0; k < kSub; ++k) {
-      int x, y, z;
-      const int lo = j * kTile + k * kBlock + threadIdx.x;
-      if (!node_xyz(I, lo, x, y, z)) continue;
-      const int rr = I.off + lo;
-      t0[rr] = (mask[rr] & kFluidBit) ? fmaf(mgd::kAlpha, e1[C.off + mgd::agg_index(C.L, x, y, z)], mgd::kOmega * u[rr])
-                                      : 0.f;
-    }
+                                                       const uint8_t *__restrict__ code,
+                                                       const uint32_t *__restrict__ mask, const float *__restrict__ r,
+                                                       const float *__restrict__ uj, const float *__restrict__ e1,
+                                                       float *__restrict__ u) {
+  const int act = pref[n];
+  for (int t = blockIdx.x; t < act; t += gridDim.x) {
+    const int ii = find_inst(pref, n, t);
+    const int off = inst[ii].off;
+    const Cols C = im[ii].c;
+    Column col;
+    if (march_column(im[ii], t - pref[ii], col))
+      mgd::post0_column(C, col, code + off, mask + off, r + off, uj + off, seg1[ii].L, e1 + seg1[ii].off, u + off);
   }
 }
 
-// then u = t + omega (r - A t)/diag
-__global__ void __launch_bounds__(kBlock) kbm_post0(const InstDev *__restrict__ inst, int n,
-                                                    const int *__restrict__ pref, const uint32_t *__restrict__ mask,
-                                                    const float *__restrict__ r, const float *__restrict__ t0,
-                                                    float *__restrict__ u) {
-  const int Tact = pref[n];
-  for (int tp = blockIdx.x; tp < Tact; tp += gridDim.x) {
-    const int ii = find_inst(pref, n, tp);
-    const InstDev &I = inst[ii];
-    const int j = tp - pref[ii];
-#pragma unroll
-    for (int k = 0; k < kSub; ++k) {
-      int x, y, z;
-      const int lo = j * kTile + k * kBlock + threadIdx.x;
-      if (!node_xyz(I, lo, x, y, z)) continue;
-      const int i = I.off + lo;
-      const uint32_t m = mask[i];
-      if (!(m & kFluidBit)) {
-        u[i] = 0.f;
-        continue;
-      }
-      const float d6 = (float)mgd::diag6(m, I.selfmask);
-      const float s6 = mgd::nbsum6(m, I.selfmask, offsets_of(I.g, x, y, z), i, t0);
-      const float ti = t0[i];
-      u[i] = ti + mgd::kOmega * __fdividef(6.f * r[i] - (d6 * ti - s6), d6);
-    }
+// omega/diag of a level's nodes
+__global__ void kbm_weights(long long M, const float *__restrict__ A13, float *__restrict__ W) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (long long)gridDim.x * blockDim.x) {
+    const float d = A13[i];
+    W[i] = d != 0.f ? mgd::kOmega / d : 0.f;
   }
 }
 
@@ -1029,6 +998,7 @@ void mg_release(lbe_batch *b) {
   cudaFree(b->mg_tiles);
   cudaFree(b->mg_seg);
   cudaFree(b->mg_t0);
+  cudaFree(b->mg_w1);
   cudaFree(b->mg_cinv);
   cudaFree(b->mg_cinv_off);
   cudaFree(b->fam_cnt);
@@ -1041,7 +1011,7 @@ void mg_release(lbe_batch *b) {
   }
   b->mg_tiles = nullptr;
   b->mg_seg = nullptr;
-  b->mg_t0 = nullptr;
+  b->mg_t0 = b->mg_w1 = nullptr;
   b->mg_cinv = nullptr;
   b->mg_cinv_off = nullptr;
   b->fam_cnt = b->fam_pref = nullptr;
@@ -1054,7 +1024,7 @@ void bfree(lbe_batch *b) {
   void *ptrs[] = {b->inst_d, b->tile_inst, b->id,   b->mask, b->f[0],  b->f[1], b->q,    b->qstar, b->phi,
                   b->phi_prev, b->phi32,  b->phifx, b->u, b->vec, b->part, b->psi_d, b->ictl, b->bctl, b->qpart,
                   b->qout,
-                  b->flag,     b->hist,   b->lf};
+                  b->flag,     b->hist,   b->lf,   b->code, b->im,   b->mpref};
   for (void *p : ptrs) cudaFree(p);
   mg_release(b);
   if (b->bctl_h) cudaFreeHost(b->bctl_h);
@@ -1170,6 +1140,25 @@ int coarse_inverses(lbe_batch *b, const std::vector<lbe::LvSeg> &seg) {
   return LBE_OK;
 }
 
+// Planes per thread of the batch's column march: long chunks (the march's two
+// planes of start-up, the block's reduction), as long as a kernel still has
+// several blocks for each resident one when half of the instances are done.
+int march_planes(long long Ntot) {
+  return (int)std::min<long long>(32, std::max<long long>(1, Ntot / (256LL * lbe::kResident * 4)));
+}
+lbe::InstMarch march_of(const lbe::InstDev &I, int K, long long Ntot, int &part0) {
+  const lbe::ColLaunch L = lbe::make_cols(I.g, I.selfmask, K, Ntot);
+  lbe::InstMarch m{};
+  m.c = L.c;
+  m.c.omega = lbe::mgd::kOmega;  // every instance's levels keep the one weight
+  while ((1u << m.cbl) < L.block.x) ++m.cbl;
+  m.gx = (int)L.grid.x;
+  m.blocks = (int)L.nblk();
+  m.part0 = part0;
+  part0 += m.blocks;
+  return m;
+}
+
 // tile families, then the inverse fine diagonal and the Galerkin operators on
 // the GPU.  Uploads the instance table (it carries each instance's level
 // count).
@@ -1212,16 +1201,32 @@ int mg_setup(lbe_batch *b) {
     b->mg_M[l] = M;
     b->mg_T[l] = T;
   }
+  std::vector<InstMarch> march(n);
+  {
+    const int K = march_planes(b->Ntot);
+    int at = 0;
+    for (int i = 0; i < n; ++i) march[i] = march_of(b->inst[i], K, b->Ntot, at);
+  }
   // active-tile families
   const int FL = fam_levels(b);
-  b->nfam = 2 * FL - 1;
+  b->nfam = 2 * FL + 2;
   std::vector<int> cnt((size_t)b->nfam * n, 0);
   for (int i = 0; i < n; ++i) {
     const int ml = b->inst[i].mg_levels;
     auto tiles_at = [&](int l) { return l == 0 ? b->inst[i].ntiles : seg[(size_t)l * n + i].ntiles; };
     for (int l = 0; l < FL; ++l) cnt[(size_t)famA(l) * n + i] = (l == 0 || ml > l) ? tiles_at(l) : 0;
     for (int l = 0; l + 1 < FL; ++l) cnt[(size_t)famB(FL, l) * n + i] = ml > l + 1 ? tiles_at(l) : 0;
+    InstMarch &I = march[i];
+    cnt[(size_t)famM(FL) * n + i] = I.blocks;
+    if (ml >= 2) {
+      const dim3 g0 = mgd::make_restrict_map(b->inst[i].g, seg[(size_t)n + i].L, I.M, std::max(1, I.c.K / 2));
+      I.g0x = (int)g0.x;
+      I.g0y = (int)g0.y;
+      cnt[(size_t)famP(FL) * n + i] = I.blocks;
+      cnt[(size_t)famR(FL) * n + i] = (int)(g0.x * g0.y * g0.z);
+    }
   }
+  BCK(b, cudaMemcpyAsync(b->im, march.data(), sizeof(InstMarch) * n, cudaMemcpyHostToDevice, b->stream));
   cudaError_t e = cudaMalloc(&b->fam_cnt, sizeof(int) * cnt.size());
   if (e == cudaSuccess) e = cudaMalloc(&b->fam_pref, sizeof(int) * (size_t)b->nfam * (n + 1));
   if (e == cudaSuccess)
@@ -1242,6 +1247,7 @@ int mg_setup(lbe_batch *b) {
     e = cudaMemcpyAsync(b->mg_tiles, tiles.data(), sizeof(int) * tiles.size(), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->mg_seg, seg.data(), sizeof(LvSeg) * seg.size(), cudaMemcpyHostToDevice, b->stream);
+  if (e == cudaSuccess) e = cudaMalloc(&b->mg_w1, sizeof(float) * b->mg_M[1]);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->mg_t0, 0, sizeof(float) * b->Ntot, b->stream);
   BCK(b, e);
   const int G = b->grid;
@@ -1252,6 +1258,7 @@ int mg_setup(lbe_batch *b) {
     kbm_galerkin<<<std::min(G, b->mg_T[l + 1]), kBlock, 0, b->stream>>>(
         b->mg_tiles + b->mg_tbase[l + 1], b->mg_T[l + 1], b->mg_seg + (size_t)l * n, b->mg_seg + (size_t)(l + 1) * n,
         b->mg_p.A[l], b->mg_p.A[l + 1]);
+  kbm_weights<<<G, kBlock, 0, b->stream>>>(b->mg_M[1], b->mg_p.A[1] + 13 * b->mg_M[1], b->mg_w1);
   BCK(b, cudaGetLastError());
   return coarse_inverses(b, seg);
 }
@@ -1286,19 +1293,21 @@ cudaError_t add_vcycle(lbe_batch *b, cudaGraph_t gr, cudaGraphNode_t *last) {
   const InstDev *inst = b->inst_d;
   const InstCtl *c = b->ictl;
   const uint32_t *mask = b->mask;
+  const uint8_t *code = b->code;
+  const InstMarch *im = b->im;
   const CgVec v = b->cg();
-  const float *r0 = v.r, *uj = v.u;
-  float *u0 = v.u, *t0 = b->mg_t0;
+  const float *r0 = v.r, *uj = v.uj;
+  float *u0 = v.u;
   const LvSeg *seg_all = b->mg_seg;
   LvPtrs P = b->mg_p;
   const dim3 G(b->grid), B(kBlock);
   cudaError_t e;
   {
-    const int *pref = fam(b, famA(1));
+    const int *pref = fam(b, famR(L));
     const LvSeg *seg1 = seg_all + n;
-    const float *A1 = P.A[1];
+    const float *W1 = b->mg_w1;
     float *rc = P.r[1], *zc = P.z[1];
-    void *a[] = {&inst, &n, &pref, &seg1, &mask, &r0, &uj, &A1, &rc, &zc};
+    void *a[] = {&inst, &im, &n, &pref, &seg1, &code, &r0, &uj, &W1, &rc, &zc};
     e = add_node(gr, last, (void *)kbm_restrict0, dim3(resident_grid(b, (void *)kbm_restrict0)), B, a);
     if (e != cudaSuccess) return e;
   }
@@ -1327,31 +1336,24 @@ cudaError_t add_vcycle(lbe_batch *b, cudaGraph_t gr, cudaGraphNode_t *last) {
     e = add_node(gr, last, (void *)kbm_post, dim3(resident_grid(b, (void *)kbm_post)), B, a);
     if (e != cudaSuccess) return e;
   }
-  const int *prefB0 = fam(b, famB(L, 0));
-  {
-    const LvSeg *seg1 = seg_all + n;
-    const float *e1 = P.e[1];
-    void *a[] = {&inst, &n, &prefB0, &seg1, &mask, &uj, &e1, &t0};
-    e = add_node(gr, last, (void *)kbm_prolong0, dim3(resident_grid(b, (void *)kbm_prolong0)), B, a);
-    if (e != cudaSuccess) return e;
-  }
-  {
-    const float *tc = t0;
-    void *a[] = {&inst, &n, &prefB0, &mask, &r0, &tc, &u0};
-    e = add_node(gr, last, (void *)kbm_post0, dim3(resident_grid(b, (void *)kbm_post0)), B, a);
-  }
-  return e;
+  const int *prefP = fam(b, famP(L));
+  const LvSeg *seg1 = seg_all + n;
+  const float *e1 = P.e[1];
+  void *a[] = {&inst, &im, &n, &prefP, &seg1, &code, &mask, &r0, &uj, &e1, &u0};
+  return add_node(gr, last, (void *)kbm_post0, dim3(resident_grid(b, (void *)kbm_post0)), B, a);
 }
 
 // kernels of one V-cycle
-int vcycle_kernels(const lbe_batch *b) { return b->mg_nlev >= 2 ? 2 * (b->mg_nlev - 1) + 2 : 0; }
+int vcycle_kernels(const lbe_batch *b) { return b->mg_nlev >= 2 ? 2 * (b->mg_nlev - 1) + 1 : 0; }
 
 // Arguments of the solve kernels (kept alive while nodes are created or
 // kernels launched)
 struct SolveArgs {
   const lbe::InstDev *inst;
-  const int *tile_inst, *pref0, *fam_cnt;
-  int T, Ntot, n, maxit, nfam, use = 1, set_hist;
+  const lbe::InstMarch *im;
+  const int *tile_inst, *pref0, *prefM, *mpref, *fam_cnt;
+  const uint8_t *code;
+  int T, MT, Ntot, n, maxit, nfam, use = 1, set_hist;
   const uint32_t *mask;
   const float *fin;
   float *fout;
@@ -1374,6 +1376,11 @@ void solve_args(lbe_batch *b, bool step, const float *fin, float *fout, int64_t 
   A.inst = b->inst_d;
   A.tile_inst = b->tile_inst;
   A.pref0 = fam(b, lbe::famA(0));
+  A.prefM = fam(b, lbe::famM(fam_levels(b)));
+  A.mpref = b->mpref;
+  A.im = b->im;
+  A.code = b->code;
+  A.MT = b->MT;
   A.fam_cnt = b->fam_cnt;
   A.fam_pref = b->fam_pref;
   A.T = b->T;
@@ -1437,14 +1444,15 @@ cudaError_t build_graph(lbe_batch *b, bool step, const float *fin, float *fout, 
                    &A.u,    &A.qin,       &A.phifx, &A.phi_prev, &A.phi32, &A.hist};
   void *a_ext[] = {&A.inst, &A.tile_inst, &A.T, &A.Ntot, &A.mask, &A.phifx, &A.phi_prev, &A.phi32, &A.hist};
   void *a_reset[] = {&A.n, &A.c, &A.bc, &A.hist, &A.set_hist};
-  void *a_res[] = {&A.inst, &A.tile_inst, &A.T, &A.Ntot, &A.mask, &A.qsolve, &A.phifx, &A.v, &A.part, &A.c};
-  void *a_out[] = {&A.inst, &A.n,    &A.T,       &A.part,     &A.c,    &A.bc,  &A.tol,
+  void *a_res[] = {&A.inst, &A.im,     &A.n,     &A.mpref, &A.Ntot, &A.mask,
+                   &A.code, &A.qsolve, &A.phifx, &A.v,     &A.part, &A.c};
+  void *a_out[] = {&A.im,   &A.n,    &A.MT,      &A.part,     &A.c,    &A.bc,  &A.tol,
                    &A.maxit, &A.nfam, &A.fam_cnt, &A.fam_pref, &A.hout, &A.hin, &A.use};
-  void *a_b[] = {&A.inst, &A.n, &A.pref0, &A.T, &A.mask, &A.vr, &A.vu, &A.vw, &A.part};
-  void *a_sc[] = {&A.inst, &A.T, &A.part, &A.c};
-  void *a_te[] = {&A.inst, &A.n,    &A.T,       &A.part,     &A.c,   &A.bc, &A.eta, &A.tol_abs,
+  void *a_b[] = {&A.inst, &A.im, &A.n, &A.prefM, &A.MT, &A.code, &A.vr, &A.vu, &A.vw, &A.part};
+  void *a_sc[] = {&A.im, &A.MT, &A.part, &A.c};
+  void *a_te[] = {&A.inst, &A.n,    &A.MT,      &A.part,     &A.c,   &A.bc, &A.eta, &A.tol_abs,
                   &A.maxit, &A.nfam, &A.fam_cnt, &A.fam_pref, &A.hin, &A.use};
-  void *a_a[] = {&A.inst, &A.n, &A.pref0, &A.T, &A.mask, &A.v, &A.part, &A.c};
+  void *a_a[] = {&A.inst, &A.n, &A.pref0, &A.MT, &A.code, &A.v, &A.part, &A.c};
   void *a_cor[] = {&A.inst, &A.tile_inst, &A.T, &A.mask, &A.vx, &A.phifx, &A.phi32, &A.flag, &A.c};
   if (step) {
     void *sweep = (void *)sweep_kernel(b->flow, b->Ntot, b->aa_odd);
@@ -1541,8 +1549,9 @@ int run_polled(lbe_batch *b, bool step, const float *fin, float *fout, int64_t *
   const cudaGraphConditionalHandle h0 = 0;
   int any_outer = 1;
   while (any_outer && err == cudaSuccess) {
-    kb_res<<<Gres, kBlock, 0, st>>>(A.inst, A.tile_inst, A.T, A.Ntot, A.mask, A.qsolve, A.phifx, A.v, A.part, A.c);
-    kb_outer<<<n, kBlock, 0, st>>>(A.inst, n, A.T, A.part, A.c, A.bc, A.tol, A.maxit, A.nfam, A.fam_cnt, A.fam_pref,
+    kb_res<<<Gres, kBlock, 0, st>>>(A.inst, A.im, n, A.mpref, A.Ntot, A.mask, A.code, A.qsolve, A.phifx, A.v, A.part,
+                                    A.c);
+    kb_outer<<<n, kBlock, 0, st>>>(A.im, n, A.MT, A.part, A.c, A.bc, A.tol, A.maxit, A.nfam, A.fam_cnt, A.fam_pref,
                                    h0, h0, 0);
     nl += 2;
     flags(&any_outer, nullptr);
@@ -1550,10 +1559,10 @@ int run_polled(lbe_batch *b, bool step, const float *fin, float *fout, int64_t *
     int any_inner = 1;
     while (any_inner && err == cudaSuccess) {
       if (vc) err = cudaGraphLaunch(vc, st), nl += vck;
-      kb_cg_b<<<Gb, kBlock, 0, st>>>(A.inst, n, A.pref0, A.T, A.mask, A.vr, A.vu, A.vw, A.part);
-      kb_scal<<<n, kBlock, 0, st>>>(A.inst, A.T, A.part, A.c);
-      kb_cg_a<<<Ga, kBlock, 0, st>>>(A.inst, n, A.pref0, A.T, A.mask, A.v, A.part, A.c);
-      kb_test<<<n, kBlock, 0, st>>>(A.inst, n, A.T, A.part, A.c, A.bc, A.eta, A.tol_abs, A.maxit, A.nfam, A.fam_cnt,
+      kb_cg_b<<<Gb, kBlock, 0, st>>>(A.inst, A.im, n, A.prefM, A.MT, A.code, A.vr, A.vu, A.vw, A.part);
+      kb_scal<<<n, kBlock, 0, st>>>(A.im, A.MT, A.part, A.c);
+      kb_cg_a<<<Ga, kBlock, 0, st>>>(A.inst, n, A.pref0, A.MT, A.code, A.v, A.part, A.c);
+      kb_test<<<n, kBlock, 0, st>>>(A.inst, n, A.MT, A.part, A.c, A.bc, A.eta, A.tol_abs, A.maxit, A.nfam, A.fam_cnt,
                                     A.fam_pref, h0, 0);
       nl += 4;
       flags(nullptr, &any_inner);
@@ -1813,7 +1822,19 @@ int lbe_batch_create(const lbe_params *params, int n, void *cuda_stream, lbe_bat
   alloc((void **)&b->phifx, 8 * N);
   alloc((void **)&b->u, sizeof(float4) * N);
   alloc((void **)&b->vec, 4 * N * 6);
-  alloc((void **)&b->part, sizeof(double) * 3 * T);
+  std::vector<int> mpref(n + 1, 0);
+  {
+    const int K = march_planes(Ntot);
+    for (int i = 0; i < n; ++i) {
+      mpref[i + 1] = mpref[i];
+      march_of(b->inst[i], K, Ntot, mpref[i + 1]);
+    }
+    b->MT = mpref[n];
+  }
+  alloc((void **)&b->code, N);
+  alloc((void **)&b->im, sizeof(lbe::InstMarch) * n);
+  alloc((void **)&b->mpref, sizeof(int) * (n + 1));
+  alloc((void **)&b->part, sizeof(double) * (2 * (size_t)b->MT + std::max<size_t>(T, b->MT)));
   alloc((void **)&b->psi_d, sizeof(double) * n * (kBE + 1));
   alloc((void **)&b->ictl, sizeof(lbe::InstCtl) * n);
   alloc((void **)&b->bctl, sizeof(lbe::BatchCtl));
@@ -1824,6 +1845,7 @@ int lbe_batch_create(const lbe_params *params, int n, void *cuda_stream, lbe_bat
   if (e == cudaSuccess) e = cudaMallocHost((void **)&b->bctl_h, sizeof(lbe::BatchCtl));
   if (e == cudaSuccess) e = cudaMallocHost((void **)&b->qhost, sizeof(double) * kBE * n);
   if (e == cudaSuccess) e = cudaMemcpy(b->tile_inst, tile_inst.data(), sizeof(int) * T, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(b->mpref, mpref.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(b->ictl, 0, sizeof(lbe::InstCtl) * n);
   if (e == cudaSuccess) e = cudaMemset(b->bctl, 0, sizeof(lbe::BatchCtl));
   if (e == cudaSuccess) e = cudaMemset(b->flag, 0, sizeof(int));
@@ -1900,6 +1922,7 @@ int lbe_batch_init(lbe_batch *b) {
     const InstDev &I = b->inst[i];
     BCK(b, cudaMemcpyAsync(b->id + I.off, b->ids[i].data(), I.g.N, cudaMemcpyHostToDevice, b->stream));
     BCK(b, launch_build_mask(I.g, b->id + I.off, b->mask + I.off, b->stream));
+    BCK(b, launch_build_code(I.g, I.selfmask, b->mask + I.off, b->code + I.off, b->stream));
   }
   int rc = mg_setup(b);  // also uploads the instance table
   if (rc != LBE_OK) return rc;

@@ -683,10 +683,5 @@ __device__ __forceinline__ long long lap6_fx_(const Offs &o, int r, uint32_t m, 
   }
   return s;
 }
-__device__ __forceinline__ long long lap6_fx(const Geo &g, int r, int x, int y, int z, uint32_t m,
-                                             const int64_t *__restrict__ v) {
-  const Offs o = offsets_of(g, x, y, z);
-  return (m & kLinkBits) == kLinkBits ? lap6_fx_<true>(o, r, m, v) : lap6_fx_<false>(o, r, m, v);
-}
 }  // namespace fp32
 }  // namespace lbe

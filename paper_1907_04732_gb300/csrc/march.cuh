@@ -128,7 +128,9 @@ inline float jacobi_weight(const Geo &g, float omega) {
   return (g.nx > 1) + (g.ny > 1) + (g.nz > 1) == 1 ? omega * (2.f / 3.f) : omega;
 }
 
-inline ColLaunch make_cols(const Geo &g, uint32_t selfmask) {
+// K: planes per thread (0: chosen for this lattice alone); nodes: of all the
+// lattices that a kernel works on (0: this one alone)
+inline ColLaunch make_cols(const Geo &g, uint32_t selfmask, int K = 0, long long nodes = 0) {
   ColLaunch L;
   L.c.nx = g.nx;
   L.c.ny = g.ny;
@@ -140,11 +142,11 @@ inline ColLaunch make_cols(const Geo &g, uint32_t selfmask) {
     if (selfmask & (1u << (i - 1))) L.c.selfw += c2_of(i) == 1 ? 2 : 1;
   const int cb = L.c.plane < 256 ? pow2_at_least(L.c.plane) : 256, zb = 256 / cb;
   const long long gx = ((long long)L.c.plane + cb - 1) / cb;
-  const int K = planes_per_thread(gx, g.nz, zb);
+  if (K == 0) K = planes_per_thread(gx, g.nz, zb);
   L.c.K = K;
   // a lattice whose vectors exceed L2 is read from HBM: its latency is
   // covered by prefetching the columns' next planes into L2
-  L.c.ahead = g.N > kPrefetchNodes ? 3 : 0;
+  L.c.ahead = (nodes ? nodes : g.N) > kPrefetchNodes ? 3 : 0;
   L.c.omega = jacobi_weight(g, mgd::kOmega);
   L.block = dim3((unsigned)cb, (unsigned)zb);
   L.grid = dim3((unsigned)gx, (unsigned)((g.nz + (long long)K * zb - 1) / ((long long)K * zb)));

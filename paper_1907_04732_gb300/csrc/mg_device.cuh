@@ -220,53 +220,7 @@ __device__ __forceinline__ void coarsest_solve(const MgLevel &L, const T *__rest
 }
 
 
-// --- forms with integer link weights and a stored pre-smoothed iterate -------
-// The modified Laplacian's link weights 1/3 (axis) and 1/6 (diagonal) are
-// 2/6 and 1/6: sums of weights are integers over 6, and a node's diagonal
-// 6 * diag = sum over non-self links of (2 - fluid) * (2 axis, 1 diagonal)
-// follows from two population counts of its link mask.
-__host__ __device__ constexpr uint32_t axis_links() {
-  uint32_t m = 0;
-  for (int l = 1; l < kQ; ++l)
-    if (c2_of(l) == 1) m |= 1u << (l - 1);
-  return m;
-}
-__host__ __device__ constexpr uint32_t diag_links() {
-  uint32_t m = 0;
-  for (int l = 1; l < kQ; ++l)
-    if (c2_of(l) == 2) m |= 1u << (l - 1);
-  return m;
-}
-
-// 6 * diagonal of a fluid node's row
-__device__ __forceinline__ int diag6(uint32_t m, uint32_t selfmask) {
-  const uint32_t ax = axis_links() & ~selfmask, dg = diag_links() & ~selfmask;
-  return 2 * (2 * __popc(ax) + __popc(dg)) - (2 * __popc(m & ax) + __popc(m & dg));
-}
-
-// 6 * sum over fluid links of weight * v[neighbour]; every neighbour is
-// read (a zero weight drops it) so that the loads do not wait for the mask.
-// A node with all links fluid takes the same fmaf sequence without the
-// per-link weight tests.
-__device__ __forceinline__ float nbsum6(uint32_t m, uint32_t selfmask, const Offs &o, int i,
-                                        const float *__restrict__ v) {
-  const float *__restrict__ vi = v + i;
-  float s = 0.f;
-  if (all_links(m, selfmask)) {
-#pragma unroll
-    for (int l = 1; l < kQ; ++l) s = fmaf(c2_of(l) == 1 ? 2.f : 1.f, vi[o.at(cx_of(l), cy_of(l), cz_of(l))], s);
-    return s;
-  }
-#pragma unroll
-  for (int l = 1; l < kQ; ++l) {
-    const uint32_t b = 1u << (l - 1);
-    const float vj = vi[o.at(cx_of(l), cy_of(l), cz_of(l))];
-    const float wl = ((m & b) && !(selfmask & b)) ? (c2_of(l) == 1 ? 2.f : 1.f) : 0.f;
-    s = fmaf(wl, vj, s);
-  }
-  return s;
-}
-
+// --- forms with a stored pre-smoothed iterate ---------------------------------
 // residual of a 27-point level after pre-smoothing, the pre-smoothed iterate
 // z = omega r/diag being stored: r - A z at (X,Y,Z)
 template <typename T>

@@ -70,7 +70,7 @@ __device__ __forceinline__ void restrict0_block(const Cols &F, const uint8_t *co
 
 // lanes along x, a pair of rows, the rest along z; returns the grid of
 // 256-thread blocks
-inline dim3 make_restrict_map(const Geo &g, const MgLevel &L1, RestrictMap &M) {
+inline dim3 make_restrict_map(const Geo &g, const MgLevel &L1, RestrictMap &M, int Kc = 0) {
   M.yl = L1.sy;
   M.xl = 0;
   while ((1 << M.xl) < g.nx && M.xl < 5 - M.yl) ++M.xl;
@@ -78,7 +78,7 @@ inline dim3 make_restrict_map(const Geo &g, const MgLevel &L1, RestrictMap &M) {
   const int xt = (g.nx + (1 << M.xl) - 1) >> M.xl, yt = (g.ny + (1 << M.yl) - 1) >> M.yl;
   M.wy = yt < 8 ? pow2_at_least(yt) : 8;
   const int zc = (8 / M.wy) << M.zl, yb = (yt + M.wy - 1) / M.wy;  // chunks per block, blocks along y
-  M.Kc = planes_per_thread((long long)xt * yb, L1.nz, zc, 1 + L1.sz);
+  M.Kc = Kc ? Kc : planes_per_thread((long long)xt * yb, L1.nz, zc, 1 + L1.sz);
   const int per = zc * M.Kc;
   return dim3((unsigned)xt, (unsigned)yb, (unsigned)((L1.nz + per - 1) / per));
 }
