@@ -178,30 +178,81 @@ __global__ void k_n_from_double(const Geo g, const P32 P, const double *__restri
   }
 }
 
-// density, velocity (current state) or populations, as FP64
-template <int LAYOUT>
+// A sum of floats kept as three (two-sums of the value and of its error:
+// Knuth, Ogita, Rump and Oishi 2005), exact to below 2^-70 of the terms'
+// magnitude, so that FP64 additions come only at the end.
+struct Sum3 {
+  float s = 0.f, e = 0.f, e2 = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    float t, d, q, d2;
+    two_sum(s, v, t, d);
+    two_sum(e, d, q, d2);
+    s = t;
+    e = q;
+    e2 += d2;
+  }
+  __device__ __forceinline__ double value() const;
+};
+
+// float -> double in integer instructions (the conversion instruction runs on
+// the narrow FP64 pipe); zero, subnormal and non-finite values by conversion
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu;
+  if (a == 0u) return 0.0;
+  if (a < 0x00800000u || a >= 0x7f800000u) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
+}
+// (an infinite or NaN sum has no error terms)
+__device__ __forceinline__ double Sum3::value() const {
+  return fabsf(s) < __int_as_float(0x7f800000) ? widen(s) + (widen(e) + widen(e2)) : (double)s;
+}
+
+// density, velocity (current state) or populations, as FP64.  The sums of 19
+// populations and their momenta in FP64 (a conversion and two or three
+// additions each on a pipe at 1/64 of the FP32 rate) bounded it, and every
+// field paid for every other's: all fields of a 64x64x256 state 807 -> 537 us
+// (with the copies and reductions around them), a 256^3 run's outputs 1 ms less.
+enum { M_RHO = 0, M_U = 1, M_F = 2 };
+template <int LAYOUT, int WHAT>
 __global__ void k_moments32(const Geo g, const P32 P, int flow, const uint32_t *__restrict__ mask,
                             const float *__restrict__ fin, const int64_t *__restrict__ q,
-                            const float *__restrict__ phi, double *__restrict__ rho_out,
-                            double *__restrict__ u_out, double *__restrict__ f_out) {
+                            const float *__restrict__ phi, double *__restrict__ out) {
   int x, y, z;
   long long rl;
   if (!node_of(g, 1, 0, x, y, z, rl)) return;
   const int r = (int)rl, N = (int)g.N;
   const uint32_t m = mask[r];
   if (!(m & kFluidBit)) {
-    if (rho_out) rho_out[r] = 0.0;
-    if (u_out) u_out[r] = u_out[N + r] = u_out[2 * N + r] = 0.0;
-    if (f_out)
-      for (int i = 0; i < kQ; ++i) f_out[(long long)i * N + r] = 0.0;
+    constexpr int kOut = WHAT == M_RHO ? 1 : (WHAT == M_U ? 3 : kQ);
+    for (int i = 0; i < kOut; ++i) out[(long long)i * N + r] = 0.0;
     return;
   }
   const Offs o = offsets_of(g, x, y, z);
   float f[kQ];
   gather32<2, false, LAYOUT>(N, r, o, m, fin, f);  // what the next step's collision reads
-  if (f_out) {
-    for (int i = 0; i < kQ; ++i) f_out[(long long)i * N + r] = w_of(i) + (double)f[i];
+  if (WHAT == M_F) {
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) out[(long long)i * N + r] = w_of(i) + widen(f[i]);
     return;
+  }
+  Sum3 drho;
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) drho.add(f[i]);
+  const double rho = 1.0 + drho.value();
+  if (WHAT == M_RHO) {
+    out[r] = rho;
+    return;
+  }
+  if (!flow) {
+    out[r] = out[N + r] = out[2 * N + r] = 0.0;
+    return;
+  }
+  Sum3 jx, jy, jz;
+#pragma unroll
+  for (int i = 1; i < kQ; ++i) {
+    if (cx_of(i)) jx.add(cx_of(i) * f[i]);
+    if (cy_of(i)) jy.add(cy_of(i) * f[i]);
+    if (cz_of(i)) jz.add(cz_of(i) * f[i]);
   }
   long long q0[LBE_MAX_SPECIES], dq[LBE_MAX_SPECIES];
   float q0f[LBE_MAX_SPECIES];
@@ -213,20 +264,9 @@ __global__ void k_moments32(const Geo g, const P32 P, int flow, const uint32_t *
   float F[3];
   bool over = false;
   ion_links<false>(P, N, r, o, m, q, phi, q0, q0f, dq, F, over);
-  double drho = 0.0, jx = 0.0, jy = 0.0, jz = 0.0;
-  for (int i = 0; i < kQ; ++i) {
-    drho += f[i];
-    jx += cx_of(i) * (double)f[i];
-    jy += cy_of(i) * (double)f[i];
-    jz += cz_of(i) * (double)f[i];
-  }
-  const double rho = 1.0 + drho;
-  if (rho_out) rho_out[r] = rho;
-  if (u_out) {
-    u_out[r] = flow ? (jx + 0.5 * F[0]) / rho : 0.0;
-    u_out[N + r] = flow ? (jy + 0.5 * F[1]) / rho : 0.0;
-    u_out[2 * N + r] = flow ? (jz + 0.5 * F[2]) / rho : 0.0;
-  }
+  out[r] = (jx.value() + 0.5 * widen(F[0])) / rho;
+  out[N + r] = (jy.value() + 0.5 * widen(F[1])) / rho;
+  out[2 * N + r] = (jz.value() + 0.5 * widen(F[2])) / rho;
 }
 
 inline unsigned grid_for(long long N) { return (unsigned)((N + kBlock - 1) / kBlock); }
@@ -315,8 +355,16 @@ cudaError_t launch_n_from_double(lbe_handle *h, const double *n) {
 }
 
 cudaError_t launch_moments32(lbe_handle *h, double *rho_out, double *u_out, double *f_out) {
-  (h->aa_odd ? k_moments32<POP_AA_ODD> : k_moments32<POP_AA_EVEN>)<<<LAUNCH3(h), 0, h->stream>>>(
-      h->geo, h->p32, h->prm.flow, h->mask, h->f32[0], h->q, h->phi32, rho_out, u_out, f_out);
+  using Kern = void (*)(const Geo, const P32, int, const uint32_t *, const float *, const int64_t *, const float *,
+                        double *);
+  const Kern k[2][3] = {
+      {k_moments32<POP_AA_EVEN, M_RHO>, k_moments32<POP_AA_EVEN, M_U>, k_moments32<POP_AA_EVEN, M_F>},
+      {k_moments32<POP_AA_ODD, M_RHO>, k_moments32<POP_AA_ODD, M_U>, k_moments32<POP_AA_ODD, M_F>}};
+  double *const out[3] = {rho_out, u_out, f_out};
+  for (int w = 0; w < 3; ++w)
+    if (out[w])
+      k[h->aa_odd][w]<<<LAUNCH3(h), 0, h->stream>>>(h->geo, h->p32, h->prm.flow, h->mask, h->f32[0], h->q, h->phi32,
+                                                    out[w]);
   return cudaGetLastError();
 }
 
