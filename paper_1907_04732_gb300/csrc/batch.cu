@@ -298,33 +298,30 @@ __device__ __forceinline__ bool last_block(int *arrive, int nblk) {
 
 // Prefix sums of the active instances' tile counts for every family; all
 // threads of one block (the last block of a convergence-test kernel, after
-// every instance's inner_done is final)
+// every instance's inner_done is final).  A warp scans a family: one
+// family after another by the whole block waits on a dozen barriers each (the
+// test kernel took 29 us for 64 instances, the solve 13.4 -> 13.2 ms per step
+// without).
 __device__ void build_active(const InstCtl *__restrict__ c, int n, int nfam, const int *__restrict__ cnt,
                              int *__restrict__ pref) {
-  __shared__ int sc[kBlock];
-  const int t = threadIdx.x;
-  const int per = (n + kBlock - 1) / kBlock;
-  const int i0 = t * per, i1 = min(i0 + per, n);
-  for (int f = 0; f < nfam; ++f) {
+  const int lane = threadIdx.x & 31;
+  for (int f = threadIdx.x >> 5; f < nfam; f += kBlock / 32) {
     const int *cf = cnt + (long long)f * n;
     int *pf = pref + (long long)f * (n + 1);
-    int s = 0;
-    for (int i = i0; i < i1; ++i) s += __ldcg(&c[i].inner_done) ? 0 : cf[i];
-    sc[t] = s;
-    __syncthreads();
-    for (int o = 1; o < kBlock; o <<= 1) {  // inclusive scan
-      const int v = t >= o ? sc[t - o] : 0;
-      __syncthreads();
-      sc[t] += v;
-      __syncthreads();
+    int run = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + lane;
+      const int own = i < n && !__ldcg(&c[i].inner_done) ? cf[i] : 0;
+      int s = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += v;
+      }
+      if (i < n) pf[i] = run + s - own;
+      run += __shfl_sync(0xffffffffu, s, 31);
     }
-    int run = t ? sc[t - 1] : 0;
-    for (int i = i0; i < i1; ++i) {
-      pf[i] = run;
-      run += __ldcg(&c[i].inner_done) ? 0 : cf[i];
-    }
-    if (t == kBlock - 1) pf[n] = sc[t];
-    __syncthreads();
+    if (lane == 0) pf[n] = run;
   }
 }
 
@@ -1142,9 +1139,10 @@ int coarse_inverses(lbe_batch *b, const std::vector<lbe::LvSeg> &seg) {
 
 // Planes per thread of the batch's column march: long chunks (the march's two
 // planes of start-up, the block's reduction), as long as a kernel still has
-// several blocks for each resident one when half of the instances are done.
+// several blocks for each resident one when half of the instances are done
+// (64 capacitors: 12.9 ms per step with up to 16, 13.2 with up to 32).
 int march_planes(long long Ntot) {
-  return (int)std::min<long long>(32, std::max<long long>(1, Ntot / (256LL * lbe::kResident * 4)));
+  return (int)std::min<long long>(16, std::max<long long>(1, Ntot / (256LL * lbe::kResident * 4)));
 }
 lbe::InstMarch march_of(const lbe::InstDev &I, int K, long long Ntot, int &part0) {
   const lbe::ColLaunch L = lbe::make_cols(I.g, I.selfmask, K, Ntot);
@@ -1263,14 +1261,14 @@ int mg_setup(lbe_batch *b) {
   return coarse_inverses(b, seg);
 }
 
-// Blocks of a persistent kernel other than the sweep: the tuned grid, but at
-// most as many as the GPU holds at once at the kernel's own occupancy.  A
-// block beyond that would start only when a resident one had finished its
-// whole share of the tiles, and the kernel would take up to twice as long
-// (the coarse levels' post-smoothing, at 64 registers, holds four blocks per
-// SM; the tuned grid can have eight).  On the 256-instance sweep: solve 49.7
-// -> 47.3 ms per step.  The advection (48 registers) measured no better
-// capped (9.29 against 9.14 ms) and keeps the tuned grid, as the sweep.
+// Blocks of a persistent kernel other than the sweep: as many as the GPU holds
+// at once at the kernel's own occupancy.  A block beyond that would start only
+// when a resident one had finished its whole share of the tiles, and the
+// kernel would take up to twice as long; fewer (the sweep's tuned grid can be
+// half of it, its candidates lying within a few per cent) leave it waiting on
+// memory: solve of 64 capacitors 15.0 ms per step with the tuner at 608 blocks,
+// 13.4 with it at 1216.  The advection takes the tuned grid where that is
+// larger (no better capped: 9.29 against 9.14 ms on 256 instances).
 int resident_grid(const lbe_batch *b, const void *kernel) {
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -1280,7 +1278,7 @@ int resident_grid(const lbe_batch *b, const void *kernel) {
     cudaGetLastError();  // clear; the tuned grid
     return b->grid;
   }
-  return std::min(b->grid, per_sm * sms);
+  return per_sm * sms;
 }
 
 // u = M r (one V-cycle over every active instance with a hierarchy) as graph
@@ -1426,9 +1424,9 @@ cudaError_t build_graph(lbe_batch *b, bool step, const float *fin, float *fout, 
   SolveArgs A;
   solve_args(b, step, fin, fout, qin, qmid, A);
   const dim3 G(b->grid), B(kBlock), NB(b->n), rb((b->n + 255) / 256);
-  // the sweep and the advection take the tuned grid, the other persistent
-  // kernels at most one resident wave each (resident_grid)
-  const dim3 Gprep(resident_grid(b, (void *)prep_kernel(b->Ntot))), Gadv(b->grid),
+  // the sweep takes the tuned grid, the other persistent kernels one resident
+  // wave each (resident_grid)
+  const dim3 Gprep(resident_grid(b, (void *)prep_kernel(b->Ntot))), Gadv(std::max(b->grid, resident_grid(b, (void *)kb_advect))),
       Gext(resident_grid(b, (void *)kb_extrapolate)), Gres(resident_grid(b, (void *)kb_res)),
       Gb(resident_grid(b, (void *)kb_cg_b)), Ga(resident_grid(b, (void *)kb_cg_a)),
       Gcor(resident_grid(b, (void *)kb_correct));
@@ -1504,7 +1502,7 @@ int run_polled(lbe_batch *b, bool step, const float *fin, float *fout, int64_t *
   solve_args(b, step, fin, fout, qin, qmid, A);
   cudaStream_t st = b->stream;
   const int G = b->grid, n = b->n;
-  const int Gprep = resident_grid(b, (void *)prep_kernel(b->Ntot)), Gadv = G,
+  const int Gprep = resident_grid(b, (void *)prep_kernel(b->Ntot)), Gadv = std::max(G, resident_grid(b, (void *)kb_advect)),
             Gext = resident_grid(b, (void *)kb_extrapolate), Gres = resident_grid(b, (void *)kb_res),
             Gb = resident_grid(b, (void *)kb_cg_b), Ga = resident_grid(b, (void *)kb_cg_a),
             Gcor = resident_grid(b, (void *)kb_correct);
