@@ -98,3 +98,29 @@ def test_chain_takes_few_iterations(lbe, nz):
         g.init()
         g.step(2)
         assert g.stats().poisson_max_iters <= 30
+
+
+def test_single_kernel_solves_of_two_threads(lbe):
+    """Two lattices, each on its own stream and host thread, both solving with
+    as many blocks as the GPU holds: each grid is resident as a whole before
+    it starts, and the results are bitwise those of one after the other."""
+    import threading
+    ws = [lattice(64, 64, 64), lattice(96, 48, 60)]
+
+    def run(w, out, k):
+        g = lbe.Lattice.from_workload(w, precision=lbe.LBE_FP32, tol=1e-12)
+        g.init()
+        g.step(40)
+        out[k] = (g.phi(), g.charge())
+
+    alone, together = [None, None], [None, None]
+    for k, w in enumerate(ws):
+        run(w, alone, k)
+    th = [threading.Thread(target=run, args=(w, together, k)) for k, w in enumerate(ws)]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    for a, b in zip(alone, together):
+        np.testing.assert_array_equal(a[0], b[0])
+        np.testing.assert_array_equal(a[1], b[1])
