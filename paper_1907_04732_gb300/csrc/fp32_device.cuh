@@ -637,10 +637,12 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
 // float-float on the FP32 pipes: per link the difference of the high parts
 // is split exactly (two_sum), the low parts and the rounding errors go to the
 // error word.  Returns S + E ~ 6 lap to ~2^-46 of the terms; the FP64 form
-// of lap_at needs 18 FP64 adds, which are slow on this GPU.
+// of lap_at needs 18 FP64 adds, which are slow on this GPU.  (No __restrict__
+// here and in lap6_fx_: the single-kernel solve writes these potentials between
+// the grid's barriers.)
 template <bool ALL>
-__device__ __forceinline__ void lap6_ff_(const Offs &o, int r, uint32_t m, const float *__restrict__ hi,
-                                         const float *__restrict__ lo, float &S, float &E) {
+__device__ __forceinline__ void lap6_ff_(const Offs &o, int r, uint32_t m, const float *hi, const float *lo, float &S,
+                                         float &E) {
   const float h0 = hi[r], l0 = lo[r];
   S = 0.f;
   E = 0.f;
@@ -671,9 +673,9 @@ __device__ __forceinline__ void lap6_ff(const Geo &g, int r, int x, int y, int z
 // differences (weights 2 axis, 1 diagonal, doubled towards solid) summed in
 // 64-bit integers.  |phi| < kPhiMax keeps the sum far below 2^63.
 template <bool ALL>
-__device__ __forceinline__ long long lap6_fx_(const Offs &o, int r, uint32_t m, const int64_t *__restrict__ v) {
+__device__ __forceinline__ long long lap6_fx_(const Offs &o, int r, uint32_t m, const int64_t *v) {
   const long long v0 = v[r];
-  const int64_t *__restrict__ vr = v + r;
+  const int64_t *vr = v + r;
   long long s = 0;
 #pragma unroll
   for (int i = 1; i < kQ; ++i) {

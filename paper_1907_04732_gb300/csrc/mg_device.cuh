@@ -221,12 +221,15 @@ __device__ __forceinline__ void coarsest_solve(const MgLevel &L, const T *__rest
 
 
 // --- forms with a stored pre-smoothed iterate ---------------------------------
+// (r, z and ec carry no __restrict__: in the single-kernel solve other blocks
+// write them between the grid's barriers, and a qualified load could be
+// served by the read-only cache, which those barriers do not refresh)
+//
 // residual of a 27-point level after pre-smoothing, the pre-smoothed iterate
 // z = omega r/diag being stored: r - A z at (X,Y,Z)
 template <typename T>
-__device__ __forceinline__ T presmoothed_res_z(const MgLevel &L, const T *__restrict__ A,
-                                               const T *__restrict__ r, const T *__restrict__ z, int X,
-                                               int Y, int Z) {
+__device__ __forceinline__ T presmoothed_res_z(const MgLevel &L, const T *__restrict__ A, const T *r, const T *z,
+                                               int X, int Y, int Z) {
   // a node without fluid has a zero row and a zero residual; no branch
   const int I = X + L.nx * (Y + L.ny * Z);
   T s = 0;
@@ -243,9 +246,8 @@ __device__ __forceinline__ T presmoothed_res_z(const MgLevel &L, const T *__rest
 // e = z + alpha P e_c, out = e + omega (r - A e)/diag
 // with w = omega/diag (0 for a node without fluid)
 template <typename T>
-__device__ __forceinline__ T post_value_w(const MgLevel &L, const T *__restrict__ A, T w,
-                                          const T *__restrict__ r, const T *__restrict__ z,
-                                          const MgLevel &C, const T *__restrict__ ec, int X, int Y, int Z) {
+__device__ __forceinline__ T post_value_w(const MgLevel &L, const T *__restrict__ A, T w, const T *r, const T *z,
+                                          const MgLevel &C, const T *ec, int X, int Y, int Z) {
   const int I = X + L.nx * (Y + L.ny * Z);
   if (w == (T)0) return (T)0;
   T s = 0;
@@ -260,9 +262,8 @@ __device__ __forceinline__ T post_value_w(const MgLevel &L, const T *__restrict_
   return e + w * (r[I] - s);
 }
 template <typename T>
-__device__ __forceinline__ T post_value_z(const MgLevel &L, const T *__restrict__ A,
-                                          const T *__restrict__ r, const T *__restrict__ z,
-                                          const MgLevel &C, const T *__restrict__ ec, int X, int Y, int Z) {
+__device__ __forceinline__ T post_value_z(const MgLevel &L, const T *__restrict__ A, const T *r, const T *z,
+                                          const MgLevel &C, const T *ec, int X, int Y, int Z) {
   const T d = A[13 * L.S + X + L.nx * (Y + L.ny * Z)];
   return post_value_w(L, A, d != (T)0 ? (T)kOmega / d : (T)0, r, z, C, ec, X, Y, Z);
 }

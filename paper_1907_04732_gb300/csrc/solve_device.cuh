@@ -1,5 +1,8 @@
 // Thread bodies of the Poisson solve's stencil kernels, shared by the single
-// lattice (poisson.cu) and the batched form (batch.cu).
+// lattice (poisson.cu) and the batched form (batch.cu).  Pointers to values
+// that another phase of the single-kernel solve writes (the vectors, the
+// potential) carry no __restrict__: those must not become read-only-cache
+// loads.
 #pragma once
 
 #include <type_traits>
@@ -13,8 +16,7 @@ namespace lbe {
 // (2 nearest, 1 next-nearest, doubled towards solid unless dbl is false:
 // the first-order rule) the sum needs one FP64 add per link:
 // 6 lap = sum_i w_i v_i - (sum_i w_i) v0, w_i in {1, 2, 4}.
-__device__ __forceinline__ double lap_at(const Offs &o, int r, uint32_t m, const double *__restrict__ v,
-                                         bool dbl = true) {
+__device__ __forceinline__ double lap_at(const Offs &o, int r, uint32_t m, const double *v, bool dbl = true) {
   double s1 = 0.0, s2 = 0.0, s4 = 0.0;
   int wsum = 0;
 #pragma unroll
