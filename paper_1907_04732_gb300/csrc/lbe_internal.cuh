@@ -219,6 +219,7 @@ struct PoissonWork {
   bool one_ok = false;         // small lattice: the solve as one cooperative kernel
   double *one_part = nullptr;  // its block partials
   void *one_bar = nullptr;     // its grid barrier
+  int one_spins = 0;           // polls after which a wait there gives up
   double *phi_prev = nullptr;  // [kHist][N]: phi of the previous kHist steps (warm start;
                                // the FP32 form keeps fixed-point values, int64, in it)
   int history = 0;             // how many of them hold a solution (0..kHist)

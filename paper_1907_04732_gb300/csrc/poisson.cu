@@ -464,24 +464,26 @@ struct GridBar {
   unsigned count, exits;
   int dead;
 };
-constexpr int kSpinLimit = 1 << 23;  // some seconds: a wait that long never ends
+// polls of a wait, some seconds: one that long never ends.  LBE_SOLVE_SPINS sets
+// another limit (0: a wait that is not over at its first poll runs out).
+constexpr int kSpinLimit = 1 << 23;
 
 // All blocks of the (cooperative, hence co-resident) grid have arrived and
 // their writes are visible; false when the wait ran out, in every thread of
 // the block (the caller returns, other blocks see `dead` and do the same).
-__device__ __forceinline__ bool grid_sync(GridBar *b, unsigned &target) {
+__device__ __forceinline__ bool grid_sync(GridBar *b, int limit, unsigned &target) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     target += gridDim.x;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&b->count) : "memory");
     unsigned v;
-    int spins = 0, good = 1;
-    for (;;) {
+    int good = 1;
+    for (int spins = 0;; ++spins) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&b->count) : "memory");
       if ((int)(v - target) >= 0) break;
-      if ((++spins & 1023) == 0 && (spins >= kSpinLimit || *(volatile int *)&b->dead)) {
-        b->dead = 1;
+      if (spins >= limit || ((spins & 1023) == 1023 && *(volatile int *)&b->dead)) {
+        *(volatile int *)&b->dead = 1;
         good = 0;
         break;
       }
@@ -503,6 +505,7 @@ struct OneArgs {
   int *flag;
   double *part;  // [3][blocks]: (r,u), (w,u), maxima
   GridBar *bar;
+  int spins;     // limit of a wait
   long long N;
   double eta, tol_inner;
   int cbl;         // log2 of the columns of a block
@@ -583,27 +586,27 @@ __device__ __forceinline__ bool one_vcycle(const OneArgs<T> &S, unsigned &target
     const int bx = b % V.g0x, t = b / V.g0x;
     restrict0_block(S.R.cols, S.R.code, S.r, S.uj, V.lv[1], V.W[1], V.r[1], V.z[1], V.M, bx, t % V.g0y, t / V.g0y);
   }
-  if (!grid_sync(S.bar, target)) return false;
+  if (!grid_sync(S.bar, S.spins, target)) return false;
   for (int l = 1; l < V.ld; ++l) {
     for (int b = b0; b < V.rx[l] * V.ry[l] * V.rz[l]; b += G) {
       const int bx = b % V.rx[l], t = b / V.rx[l];
       restrict_block(V.lv[l], V.A[l], V.r[l], V.z[l], V.lv[l + 1], V.W[l + 1], V.r[l + 1], V.z[l + 1], V.txl[l], bx,
                      t % V.ry[l], t / V.ry[l]);
     }
-    if (!grid_sync(S.bar, target)) return false;
+    if (!grid_sync(S.bar, S.spins, target)) return false;
   }
   for (int row = b0 * (kBlock / 32) + warp; row < V.ndense; row += G * (kBlock / 32)) {
     if (V.stride) dense_row(row, V.stride, V.mat, V.r[V.ld], V.e[V.ld]);
     else inverse_row(row, V.ndense, V.mat, V.r[V.ld], V.e[V.ld]);
   }
-  if (!grid_sync(S.bar, target)) return false;
+  if (!grid_sync(S.bar, S.spins, target)) return false;
   for (int l = V.ld - 1; l >= 1; --l) {
     for (int i = b0 * kBlock + threadIdx.x; i < V.lv[l].N; i += G * kBlock) {
       int X, Y, Z;
       level_coords(V.lv[l], i, X, Y, Z);
       V.e[l][i] = post_value_w<T>(V.lv[l], V.A[l], V.W[l][i], V.r[l], V.z[l], V.lv[l + 1], V.e[l + 1], X, Y, Z);
     }
-    if (!grid_sync(S.bar, target)) return false;
+    if (!grid_sync(S.bar, S.spins, target)) return false;
   }
   for (int b = b0; b < S.blocks; b += G) {
     Column c;
@@ -634,7 +637,7 @@ __device__ __forceinline__ bool one_solve(const OneArgs<T> &S, PoissonCtl *sc, u
       S.part[ONE_MAX * G + b0] = (double)mx;
       if (kRhs<MODE>) S.part[ONE_REF * G + b0] = (double)mb;
     }
-    if (!grid_sync(S.bar, target)) return false;
+    if (!grid_sync(S.bar, S.spins, target)) return false;
     m0 = grid_max(S.part + ONE_MAX * G);
     m1 = 0.0;
     if (kRhs<MODE>) {
@@ -648,7 +651,7 @@ __device__ __forceinline__ bool one_solve(const OneArgs<T> &S, PoissonCtl *sc, u
     __syncthreads();
     if (sc->outer_done) return true;
     while (!sc->inner_done) {
-      if (!one_vcycle(S, target) || !grid_sync(S.bar, target)) return false;
+      if (!one_vcycle(S, target) || !grid_sync(S.bar, S.spins, target)) return false;
       T ru = 0, wu = 0;
       for (int b = b0; b < S.blocks; b += G) {
         Column c;
@@ -660,7 +663,7 @@ __device__ __forceinline__ bool one_solve(const OneArgs<T> &S, PoissonCtl *sc, u
         S.part[ONE_RU * G + b0] = (double)ru;
         S.part[ONE_WU * G + b0] = (double)wu;
       }
-      if (!grid_sync(S.bar, target)) return false;
+      if (!grid_sync(S.bar, S.spins, target)) return false;
       grid_sums(S.part + ONE_RU * G, S.part + ONE_WU * G, m0, m1);
       if (t == 0) cg_scalars(sc, m0, m1, 0, 0);
       __syncthreads();
@@ -674,7 +677,7 @@ __device__ __forceinline__ bool one_solve(const OneArgs<T> &S, PoissonCtl *sc, u
         v = cg_a_nodes<T, 1>(S.N, k0, dk, S.R.code, S.x, S.r, S.u, S.uj, S.w, S.p, S.s, alpha, beta, first);
       v = block_reduce<true, T>(v);
       if (t == 0) S.part[ONE_MAX * G + b0] = (double)v;
-      if (!grid_sync(S.bar, target)) return false;
+      if (!grid_sync(S.bar, S.spins, target)) return false;
       m0 = grid_max(S.part + ONE_MAX * G);
       if (t == 0) cg_test(sc, m0, S.eta, S.tol_inner, S.R.maxit, 0, 0);
       __syncthreads();
@@ -683,7 +686,7 @@ __device__ __forceinline__ bool one_solve(const OneArgs<T> &S, PoissonCtl *sc, u
       if (MODE == R_FX || MODE == R_FXG) correct_fx_nodes(S.N, k0, dk, (const float *)S.x, S.phifx, S.phi32, S.flag);
       else correct_nodes<T>(S.N, k0, dk, S.x, S.phi, S.phi32, S.phi_lo);
     }
-    if (!grid_sync(S.bar, target)) return false;
+    if (!grid_sync(S.bar, S.spins, target)) return false;
   }
 }
 
@@ -700,11 +703,14 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 3 : 1) k_solve_one(co
   const bool ok = one_solve<T, MODE>(S, &sc, target);
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (!ok) ctl->sticky_status = LBE_ERR_CUDA;
-    else if (blockIdx.x == 0) *ctl = sc;
-    // the block that leaves last (none waits any more) clears the barrier
+    if (ok && blockIdx.x == 0) *ctl = sc;
+    // the block that leaves last (none waits any more) reports a wait that ran
+    // out, after block 0 may have written the control block, and clears the
+    // barrier
     __threadfence();
     if (atomicAdd(&S.bar->exits, 1u) == gridDim.x - 1) {
+      __threadfence();
+      if (*(volatile int *)&S.bar->dead) ctl->sticky_status = LBE_ERR_CUDA;
       S.bar->count = 0;
       S.bar->exits = 0;
       S.bar->dead = 0;
@@ -957,6 +963,7 @@ bool solve_one(lbe_handle *h, const Args &A, int *rc) {
   S.flag = A.flag;
   S.part = w.one_part;
   S.bar = (GridBar *)w.one_bar;
+  S.spins = w.one_spins;
   S.N = A.N;
   S.eta = A.eta;
   S.tol_inner = A.tol_inner;
@@ -1051,6 +1058,8 @@ cudaError_t poisson_alloc(lbe_handle *h) {
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) != cudaSuccess) return e;
   w.one_ok = coop && w.graph_ok && N <= kOneNodes;
+  const char *spins = getenv("LBE_SOLVE_SPINS");
+  w.one_spins = spins ? std::max(0, atoi(spins)) : kSpinLimit;
   if (w.one_ok) {
     if ((e = cudaMalloc(&w.one_part, sizeof(double) * 3 * kOneBlocks)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&w.one_bar, sizeof(GridBar))) != cudaSuccess) return e;
