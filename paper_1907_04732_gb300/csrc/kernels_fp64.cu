@@ -88,18 +88,22 @@ __global__ void k_set_solid_phi(const Geo g, const uint8_t *__restrict__ id, con
   if (id[r]) phi[r] = psi[id[r]];
 }
 
-// sinh x and cosh x - 1, odd and even in x exactly: Taylor series to x^7 and
-// x^8 for |x| < 1/64 (most links: a kT/e over the Debye length), to x^11 and
-// x^12 for |x| < 1/4, each truncated below 2e-17 relative; beyond that from
-// expm1, out of line.  The ranges are tested on the high word, without the
-// FP64 pipe.
-static __device__ __noinline__ double2 shch_wide(double x) {
-  const double ep = expm1(x), em = expm1(-x);
-  return make_double2(0.5 * (ep - em), 0.5 * (ep + em));
-}
-__device__ __forceinline__ void shch(double x, double &sh, double &ch) {
+// The two numbers of a link's potential step x from which its flux is formed.
+// |x| < 1/4: sinh x and cosh x - 1, odd and even in x exactly, by Taylor series
+// to x^7 and x^8 for |x| < 1/64 (most links: a kT/e over the Debye length), to
+// x^11 and x^12 beyond, each truncated below 2e-17 relative.  Wide steps:
+// expm1(x) and expm1(-x), out of line.  The ranges are tested on the high word,
+// without the FP64 pipe.
+struct LinkStep {
+  double a, b;
+  bool wide;
+};
+static __device__ __noinline__ double2 expm1_pm(double x) { return make_double2(expm1(x), expm1(-x)); }
+__device__ __forceinline__ LinkStep link_step(double x) {
+  LinkStep t;
   const int hi = __double2hiint(x) & 0x7fffffff;
-  if (hi < 0x3fd00000) {
+  t.wide = hi >= 0x3fd00000;
+  if (!t.wide) {
     const double x2 = x * x;
     double p = 1.0 / 5040.0, q = 1.0 / 40320.0;
     if (hi >= 0x3f900000) {
@@ -112,18 +116,32 @@ __device__ __forceinline__ void shch(double x, double &sh, double &ch) {
     q = fma(q, x2, 1.0 / 24.0);
     p = fma(p, x2, 1.0);
     q = fma(q, x2, 0.5);
-    sh = p * x;
-    ch = q * x2;
+    t.a = p * x;
+    t.b = q * x2;
   } else {
-    const double2 w = shch_wide(x);
-    sh = w.x;
-    ch = w.y;
+    const double2 w = expm1_pm(x);
+    t.a = w.x;
+    t.b = w.y;
   }
+  return t;
+}
+// A = n' (e^x - 1) - n (e^-x - 1) at dmu = x, or at dmu = -x (neg).  A small
+// step takes S sinh + D (cosh - 1), S = n + n', D = n' - n, whose terms do not
+// cancel there; near equilibrium (n' = n e^-x) those two terms are e^|x| times
+// as large as A, so that a wide step takes the exponentials.  Its products are
+// rounded before they are subtracted: the two ends of a link then get
+// opposite values exactly, which a fused multiply-add would not give.
+__device__ __forceinline__ double link_flux(const LinkStep &t, bool neg, double n1, double n0, double S, double D) {
+  if (t.wide) {
+    const double p = neg ? t.b : t.a, m = neg ? t.a : t.b;
+    return __dsub_rn(__dmul_rn(n1, p), __dmul_rn(n0, m));
+  }
+  return fma(neg ? -S : S, t.a, D * t.b);
 }
 
 // Link fluxes of Eq. LF2 and the solvent force.  With dmu = z (phi' - phi -
-// E.c), S = n + n' and D = n' - n,
-//   A = n' (e^{dmu} - 1) - n (e^{-dmu} - 1) = S sinh(dmu) + D (cosh(dmu) - 1)
+// E.c) and D = n' - n,
+//   A = n' (e^{dmu} - 1) - n (e^{-dmu} - 1)     (link_flux)
 //   J = n' (1 + e^{dmu}) - n (1 + e^{-dmu}) = 2 D + A
 // the flux is j = -d J/(2|c|) and the link excess flux g = j/d + D/|c| =
 // -A/(2|c|) (D/|c| for an immobile species), summed into the force
@@ -131,9 +149,10 @@ __device__ __forceinline__ void shch(double x, double &sh, double &ch) {
 // under reversal of the link, so its two ends move exactly opposite amounts.
 // One series serves the species of valence +1 and -1.  Bound by the FP64
 // pipe (1/64 of the FP32 rate): about 30 FP64 instructions per link of a 1:1
-// salt against 80 with an exponential and two divisions per species, and
-// no cancellation between n' e^{dmu} and n.  Axis and diagonal links are
-// summed apart, so that 1/|c| multiplies once.
+// salt with |dmu| < 1/4 against 80 with an exponential and two divisions per
+// species.  J is exact to a few roundings of max(n, n') at any |dmu| near
+// equilibrium (test_gpu_steep_links.py).  Axis and diagonal links are summed
+// apart, so that 1/|c| multiplies once.
 __device__ __forceinline__ void ion_fluxes(const Geo &g, const Phys &P, int r, const Offs &o, uint32_t m,
                                            const double *__restrict__ n, const double *__restrict__ phi,
                                            double *nstar_r, double F[3]) {
@@ -157,8 +176,7 @@ __device__ __forceinline__ void ion_fluxes(const Geo &g, const Phys &P, int r, c
     if (!(m & (1u << (i - 1)))) continue;
     const int r2 = r + o.at(cx_of(i), cy_of(i), cz_of(i));
     const double x = phi[r2] - phi0 - P.e_dot_c[i];
-    double sh, ch;
-    shch(x, sh, ch);
+    const LinkStep t = link_step(x);
     double gsum = 0.0;  // sum over species of -2 |c| g
 #pragma unroll
     for (int k = 0; k < LBE_MAX_SPECIES; ++k) {
@@ -166,15 +184,8 @@ __device__ __forceinline__ void ion_fluxes(const Geo &g, const Phys &P, int r, c
       const double n1 = n[k * g.N + r2];
       const double D = n1 - n0[k], S = n1 + n0[k];
       double A;
-      if (kind[k] > 0) {
-        A = fma(S, sh, D * ch);
-      } else if (kind[k] < 0) {
-        A = fma(-S, sh, D * ch);
-      } else {
-        double s, c;
-        shch(P.z[k] * x, s, c);
-        A = fma(S, s, D * c);
-      }
+      if (kind[k] != 0) A = link_flux(t, kind[k] < 0, n1, n0[k], S, D);
+      else A = link_flux(link_step(P.z[k] * x), false, n1, n0[k], S, D);
       const double J = fma(2.0, D, A);
       if (c2_of(i) == 1) acc1[k] += J;
       else acc2[k] += J;
