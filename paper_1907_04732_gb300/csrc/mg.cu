@@ -84,7 +84,8 @@ __global__ void __launch_bounds__(256) k_restrict(const MgLevel F, const T *__re
                                                   T *__restrict__ rc, T *__restrict__ zc, int txl,
                                                   const PoissonCtl *c) {
   if (c && c->inner_done) return;
-  restrict_block(F, AF, r, zf, C, WC, rc, zc, txl, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z);
+  for (int Z = (int)blockIdx.z; Z < C.nz; Z += (int)gridDim.z)
+    restrict_block(F, AF, r, zf, C, WC, rc, zc, txl, (int)blockIdx.x, (int)blockIdx.y, Z);
 }
 
 // fused prolongation + post-smoothing on a 27-point level
@@ -502,7 +503,8 @@ static cudaError_t mg_vcycle_t(lbe_handle *h, const void *r0, const void *uj, vo
   int txl[kMaxLevels];
   for (int l = 1; l < lk; ++l) {
     const MGLevel &Lc = mg.lv[l + 1];
-    const dim3 rg = restrict_tiles(lv[l + 1], txl[l]);
+    dim3 rg = restrict_tiles(lv[l + 1], txl[l]);
+    rg.z = std::min(rg.z, 65535u);  // the grid's limit; the kernel strides over the other planes
     nodes.push_back(Node{(void *)k_restrict<T>, rg, dim3(256),
                          {&lv[l], P(mg.lv[l].A), P(mg.lv[l].r), P(mg.lv[l].z), &lv[l + 1], P(Lc.W), P(Lc.r), P(Lc.z),
                           &txl[l], P(c)}});
