@@ -201,6 +201,7 @@ struct PoissonCtl {
   unsigned long long max_bits;  // max |r|/diag of a residual or an update, as the bits of a double
   unsigned long long ref_bits;  // linear solves: max |rhs|/diag likewise
   long long solve_iters, total_iters, total_rounds, solves, max_solve_iters;
+  long long one_iters, one_rounds, one_solves;  // those of single-kernel solves
   double res, alpha, beta, gamma;
   double ref;  // linear solves: max |rhs|/diag, the scale of the relative test
 };

@@ -703,7 +703,12 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 3 : 1) k_solve_one(co
   const bool ok = one_solve<T, MODE>(S, &sc, target);
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (ok && blockIdx.x == 0) *ctl = sc;
+    if (ok && blockIdx.x == 0) {
+      sc.one_iters += sc.solve_iters;
+      sc.one_rounds += sc.rounds;
+      sc.one_solves += 1;
+      *ctl = sc;
+    }
     // the block that leaves last (none waits any more) reports a wait that ran
     // out, after block 0 may have written the control block, and clears the
     // barrier
@@ -1177,12 +1182,13 @@ int poisson_status(lbe_handle *h, lbe_stats *st, long long *kernels) {
     st->poisson_max_iters = (int)(c.solve_iters > c.max_solve_iters ? c.solve_iters : c.max_solve_iters);
     st->poisson_residual = c.res;
   }
-  if (kernels && w.graph_ok && !w.one_ok) {  // the single-kernel solves are counted as they are launched
+  if (kernels && w.graph_ok) {  // the polled and the single-kernel solves are counted as they are launched
     // kernels of the graph path: per solve the reset; per residual test the
     // test and the correction; per iteration V-cycle (with multigrid),
     // stencil and update
     const long long vc = mg_kernels_per_cycle(h);
-    *kernels = c.solves + 2 * c.total_rounds + (2 + vc) * c.total_iters;
+    *kernels = (c.solves - c.one_solves) + 2 * (c.total_rounds - c.one_rounds) +
+               (2 + vc) * (c.total_iters - c.one_iters);
   }
   if (c.sticky_status == LBE_ERR_CUDA) {
     h->err = "poisson: a wait between the solve's blocks ran out";
