@@ -265,15 +265,20 @@ int lbe_set_geometry(lbe_handle *h, const uint8_t *node_id, int n_electrodes, in
     memcpy(ids.data(), node_id, (size_t)g.N);
   }
   // validate: ids in range; fluid nodes keep all 26 neighbours inside the box
+  bool solid = false;
   for (long long r = 0; r < g.N; ++r) {
     if (ids[r] > n_electrodes) return fail(h, LBE_ERR_GEOMETRY, "set_geometry: node id exceeds n_electrodes");
-    if (ids[r]) continue;
+    if (ids[r]) {
+      solid = true;
+      continue;
+    }
     int x, y, z;
     lbe::coords(g, r, x, y, z);
     if ((!g.px && (x == 0 || x == g.nx - 1)) || (!g.py && (y == 0 || y == g.ny - 1)) ||
         (!g.pz && (z == 0 || z == g.nz - 1)))
       return fail(h, LBE_ERR_GEOMETRY, "set_geometry: fluid node on a non-periodic face");
   }
+  h->no_solid = !solid;
   LBE_CK(h, cudaMemcpyAsync(h->id, ids.data(), (size_t)g.N, cudaMemcpyHostToDevice, h->stream));
   LBE_CK(h, lbe::launch_build_mask(g, h->id, h->mask, h->stream));
   LBE_CK(h, lbe::launch_build_code(g, h->phys.selfmask, h->mask, h->code, h->stream));

@@ -284,6 +284,7 @@ struct lbe_handle {
   bool owns_stream = false;           // stream created by the library
   int n_elec = 0;
   bool have_geometry = false;
+  bool no_solid = false;              // the potential is defined up to a constant
   bool initialised = false;
   double psi[LBE_MAX_ELECTRODES] = {};
   std::string err;

@@ -14,8 +14,8 @@
 // is evaluated on the fly where it is needed (restriction, prolongation), so
 // a cycle over levels 0..L is L restrictions, the coarsest solve and L fused
 // prolongation+post-smoothing kernels.  The
-// coarsest level is solved exactly (its inverse, formed once on the host)
-// where its operator is positive definite: a weak coarse solve costs CG
+// coarsest level is solved exactly (its inverse, formed once on the host; a
+// lattice without solid nodes takes the pseudo-inverse): a weak coarse solve costs CG
 // iterations (on the 64x64x256 electro-osmosis lattice 3.2 per step with 32
 // Jacobi sweeps, 2.6 with 64 or 128 sweeps or the exact solve).
 #include <math.h>
@@ -261,10 +261,16 @@ MgLevel level_dev(const MGLevel &L) { return MgLevel{L.nx, L.ny, L.nz, L.sx, L.s
 // (aggregates holding fluid) is assembled densely, factored A = L L^T
 // (Cholesky) and inverted; rows and columns of the other nodes are zero,
 // as the Jacobi sweeps leave them.  False when the operator is not
-// symmetric positive definite to working accuracy (e.g. a periodic lattice
-// without electrodes, whose operator is singular): the sweeps are used then.
+// symmetric positive definite to working accuracy: the sweeps are used then.
+//
+// singular: a lattice without solid nodes, whose operator annihilates
+// constants.  The rounding of the FP32 form's rows decides whether its last
+// pivot is positive, and an inverse that passed would answer a constant with
+// 1e7 times what it answers anything else (of 20 such lattices, half failed to
+// converge in some of their solves).  The pseudo-inverse is formed instead,
+//   A+ = (A + (c/n) 1 1^T)^-1 - 1/(c n) 1 1^T   for any c > 0.
 template <typename T>
-static bool coarse_inverse_t(const mgd::MgLevel &L, const std::vector<T> &A27, std::vector<T> &inv) {
+static bool coarse_inverse_t(const mgd::MgLevel &L, const std::vector<T> &A27, std::vector<T> &inv, bool singular) {
   const int N = L.N;
   std::vector<int> act;  // active node -> level index
   std::vector<int> pos(N, -1);
@@ -275,7 +281,7 @@ static bool coarse_inverse_t(const mgd::MgLevel &L, const std::vector<T> &A27, s
     }
   const int n = (int)act.size();
   inv.assign((size_t)N * N, (T)0);
-  if (n == 0) return true;
+  if (n == 0 || (singular && n == 1)) return true;
   std::vector<double> M((size_t)n * n, 0.0);
   for (int a = 0; a < n; ++a) {
     const int I = act[a];
@@ -298,6 +304,8 @@ static bool coarse_inverse_t(const mgd::MgLevel &L, const std::vector<T> &A27, s
     }
   }
   if (!(dmax > 0.0) || asym > 1e-5 * amax) return false;
+  if (singular)
+    for (double &m : M) m += dmax / n;
   // Cholesky A = U^T U by rows of U, then the inverse's lower triangle X from
   // U^T Y = I and U X = Y.  Every inner loop runs along contiguous rows, with
   // independent elements: the compiler vectorises it, and none waits for the
@@ -335,13 +343,14 @@ static bool coarse_inverse_t(const mgd::MgLevel &L, const std::vector<T> &A27, s
     const double s = 1.0 / M[(size_t)i * n + i];
     for (int c = 0; c <= i; ++c) {
       x[c] *= s;
-      inv[(size_t)act[i] * N + act[c]] = inv[(size_t)act[c] * N + act[i]] = (T)x[c];
+      const double v = singular ? x[c] - 1.0 / (dmax * n) : x[c];
+      inv[(size_t)act[i] * N + act[c]] = inv[(size_t)act[c] * N + act[i]] = (T)v;
     }
   }
   return true;
 }
-bool mgd::coarse_inverse(const MgLevel &L, const std::vector<float> &A27, std::vector<float> &inv) {
-  return coarse_inverse_t(L, A27, inv);
+bool mgd::coarse_inverse(const MgLevel &L, const std::vector<float> &A27, std::vector<float> &inv, bool singular) {
+  return coarse_inverse_t(L, A27, inv, singular);
 }
 
 // the matrix of the V-cycle from the first level of at most kDenseMax nodes
@@ -437,7 +446,7 @@ static cudaError_t mg_setup_t(lbe_handle *h) {
     le = cudaMemcpyAsync(a27.data(), Lc.A, sizeof(T) * a27.size(), cudaMemcpyDeviceToHost, h->stream);
     if (le == cudaSuccess) le = cudaStreamSynchronize(h->stream);
     if (le != cudaSuccess) return le;
-    if (coarse_inverse_t(level_dev(Lc), a27, inv)) {
+    if (coarse_inverse_t(level_dev(Lc), a27, inv, h->no_solid)) {
       le = cudaMalloc(&mg.cinv, sizeof(T) * inv.size());
       if (le == cudaSuccess)
         le = cudaMemcpyAsync(mg.cinv, inv.data(), sizeof(T) * inv.size(), cudaMemcpyHostToDevice, h->stream);

@@ -271,8 +271,9 @@ __device__ __forceinline__ T post_value_z(const MgLevel &L, const T *__restrict_
 // host (mg.cu): inverse of a coarsest level's operator, A27 its 27-point
 // rows [27][L.N]; inv [L.N][L.N] with zero rows and columns for the nodes
 // with a zero diagonal; false when the operator is not symmetric positive
-// definite to working accuracy
-bool coarse_inverse(const MgLevel &L, const std::vector<float> &A27, std::vector<float> &inv);
+// definite to working accuracy.  singular: of a lattice without solid nodes,
+// the pseudo-inverse
+bool coarse_inverse(const MgLevel &L, const std::vector<float> &A27, std::vector<float> &inv, bool singular = false);
 
 }  // namespace mgd
 }  // namespace lbe
