@@ -1915,6 +1915,9 @@ int lbe_batch_init(lbe_batch *b) {
   if (!b) return LBE_ERR_ARG;
   for (int i = 0; i < b->n; ++i)
     if (!b->have_geometry[i]) return bfail(b, LBE_ERR_STATE, "batch init: an instance has no geometry");
+  for (int i = 0; i < b->n; ++i)
+    if (lone_fluid_node(b->inst[i].g, b->ids[i][0] == 0))
+      return bfail(b, LBE_ERR_NONFINITE, "batch poisson: non-finite residual");
   // geometry: ids, link masks (per instance, set-up only)
   for (int i = 0; i < b->n; ++i) {
     const InstDev &I = b->inst[i];

@@ -75,6 +75,10 @@ __host__ __device__ inline long long nbr(const Geo &g, int x, int y, int z, int 
   return (long long)X + (long long)g.nx * ((long long)Y + (long long)g.ny * Z);
 }
 
+// A lattice of one fluid node: all of its links join it to itself, the
+// operator's diagonal is zero and its residual over the diagonal is undefined
+inline bool lone_fluid_node(const Geo &g, bool no_solid) { return g.N == 1 && no_solid; }
+
 // 3-D launch geometry: 256-thread blocks tiled over (x, y, z), x fastest, so
 // that node coordinates come from the thread indices (no divisions).  Each
 // thread visits zpt z-planes (zpt > 1 bounds the block count of kernels that

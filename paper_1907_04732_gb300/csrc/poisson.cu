@@ -1146,6 +1146,10 @@ int poisson_solve_linear(lbe_handle *h, const double *rhs, double *x, double tol
 
 int poisson_enqueue(lbe_handle *h, bool extrapolate, bool extrapolated) {
   PoissonWork &w = h->pw;
+  if (lone_fluid_node(h->geo, h->no_solid)) {
+    h->err = "poisson: non-finite residual";
+    return LBE_ERR_NONFINITE;
+  }
   if (extrapolate) {
     if (!extrapolated) {
       if (h->prm.precision == LBE_FP32)
