@@ -210,8 +210,7 @@ __host__ __device__ constexpr int famR(int nlev) { return 2 * nlev + 1; }
 
 // this thread's column chunk of block b of an instance
 __device__ __forceinline__ bool march_column(const InstMarch &I, int b, Column &c) {
-  const int tx = threadIdx.x & ((1 << I.cbl) - 1), ty = threadIdx.x >> I.cbl;
-  return column_at(I.c, ((b % I.gx) << I.cbl) + tx, (b / I.gx) * (kBlock >> I.cbl) + ty, c);
+  return block_column(I.c, I.cbl, I.gx, b, (int)threadIdx.x, c);
 }
 
 // instance-local coordinates of node lo (false past the instance's end)

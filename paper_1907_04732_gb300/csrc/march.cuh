@@ -157,7 +157,7 @@ inline ColLaunch make_cols(const Geo &g, uint32_t selfmask, int K = 0, long long
 struct PlaneOffs {
   int xm, xp, ym, yp;
 };
-__device__ __forceinline__ PlaneOffs plane_offs(int nx, int ny, int x, int y) {
+__host__ __device__ __forceinline__ PlaneOffs plane_offs(int nx, int ny, int x, int y) {
   PlaneOffs o;
   o.xm = x == 0 ? nx - 1 : -1;
   o.xp = x == nx - 1 ? 1 - nx : 1;
@@ -172,15 +172,21 @@ struct Column {
   PlaneOffs o;
 };
 // (p: the column, chunk: which K planes of it)
-__device__ __forceinline__ bool column_at(const Cols &C, int p, int chunk, Column &c) {
+__host__ __device__ __forceinline__ bool column_at(const Cols &C, int p, int chunk, Column &c) {
   c.p = p;
   c.z0 = chunk * C.K;
   if (c.p >= C.plane || c.z0 >= C.nz) return false;
-  c.z1 = min(c.z0 + C.K, C.nz);
+  c.z1 = c.z0 + C.K < C.nz ? c.z0 + C.K : C.nz;
   c.y = (int)fdiv(C.fnx, (uint32_t)c.p);
   c.x = c.p - c.y * C.nx;
   c.o = plane_offs(C.nx, C.ny, c.x, c.y);
   return true;
+}
+
+// thread t of block b, the blocks numbered in one dimension: gx across the
+// columns (2^cbl of them each), then up the chunks
+__host__ __device__ __forceinline__ bool block_column(const Cols &C, int cbl, int gx, int b, int t, Column &c) {
+  return column_at(C, ((b % gx) << cbl) + (t & ((1 << cbl) - 1)), (b / gx) * (256 >> cbl) + (t >> cbl), c);
 }
 
 __device__ __forceinline__ bool column_of(const Cols &C, Column &c) {

@@ -610,8 +610,7 @@ __device__ __forceinline__ bool one_vcycle(const OneArgs<T> &S, unsigned &target
   }
   for (int b = b0; b < S.blocks; b += G) {
     Column c;
-    const int tx = threadIdx.x & ((1 << S.cbl) - 1), ty = threadIdx.x >> S.cbl;
-    if (column_at(S.R.cols, ((b % S.gx) << S.cbl) + tx, (b / S.gx) * (kBlock >> S.cbl) + ty, c))
+    if (block_column(S.R.cols, S.cbl, S.gx, b, (int)threadIdx.x, c))
       post0_column(S.R.cols, c, S.R.code, S.R.mask, S.r, S.uj, V.lv[1], V.e[1], S.u);
   }
   return true;
@@ -621,14 +620,13 @@ __device__ __forceinline__ bool one_vcycle(const OneArgs<T> &S, unsigned &target
 template <typename T, int MODE>
 __device__ __forceinline__ bool one_solve(const OneArgs<T> &S, PoissonCtl *sc, unsigned &target) {
   const int G = gridDim.x, b0 = blockIdx.x, t = threadIdx.x;
-  const int tx = t & ((1 << S.cbl) - 1), ty = t >> S.cbl, zb = kBlock >> S.cbl;
   const long long k0 = (long long)b0 * kBlock + t, dk = (long long)G * kBlock;
   double m0, m1;
   for (;;) {
     float mx = 0.f, mb = 0.f;
     for (int b = b0; b < S.blocks; b += G) {
       Column c;
-      if (column_at(S.R.cols, ((b % S.gx) << S.cbl) + tx, (b / S.gx) * zb + ty, c))
+      if (block_column(S.R.cols, S.cbl, S.gx, b, t, c))
         res_column<T, MODE>(S.R, c, S.r, S.uj, mx, mb);
     }
     mx = block_reduce<true, float>(mx);
@@ -655,7 +653,7 @@ __device__ __forceinline__ bool one_solve(const OneArgs<T> &S, PoissonCtl *sc, u
       T ru = 0, wu = 0;
       for (int b = b0; b < S.blocks; b += G) {
         Column c;
-        if (column_at(S.R.cols, ((b % S.gx) << S.cbl) + tx, (b / S.gx) * zb + ty, c))
+        if (block_column(S.R.cols, S.cbl, S.gx, b, t, c))
           cg_b_column(S.R.cols, c, S.R.code, S.u, S.r, S.w, ru, wu);
       }
       block_reduce2(ru, wu);

@@ -21,15 +21,27 @@ struct RestrictMap {
   int wy;          // warps of a block along y (the rest along z)
   int Kc;          // coarse planes per thread
 };
+// where thread t of block (bx, by, bz) works: its fine column and first coarse
+// plane, and its place in the warp along x and y
+struct RestrictLane {
+  int lx, ly, x, y, Z0;
+};
+__host__ __device__ __forceinline__ RestrictLane restrict_lane(const RestrictMap &M, int t, int bx, int by, int bz) {
+  const int lane = t & 31, w = t >> 5;
+  RestrictLane l;
+  l.lx = lane & ((1 << M.xl) - 1);
+  l.ly = (lane >> M.xl) & ((1 << M.yl) - 1);
+  l.x = (bx << M.xl) + l.lx;
+  l.y = ((by * M.wy + w % M.wy) << M.yl) + l.ly;
+  l.Z0 = (((bz * (8 / M.wy) + w / M.wy) << M.zl) + (lane >> (M.xl + M.yl))) * M.Kc;
+  return l;
+}
 template <typename T>
 __device__ __forceinline__ void restrict0_block(const Cols &F, const uint8_t *code, const T *r, const T *u,
                                                 const MgLevel &C, const T *WC, T *rc, T *zc, const RestrictMap &M,
                                                 int bx, int by, int bz) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int lx = lane & ((1 << M.xl) - 1), ly = (lane >> M.xl) & ((1 << M.yl) - 1), lz = lane >> (M.xl + M.yl);
-  const int x = (bx << M.xl) + lx;
-  const int y = ((by * M.wy + w % M.wy) << M.yl) + ly;
-  const int Z0 = ((((bz * (8 / M.wy) + w / M.wy) << M.zl) + lz)) * M.Kc;
+  const RestrictLane l = restrict_lane(M, (int)threadIdx.x, bx, by, bz);
+  const int lx = l.lx, ly = l.ly, x = l.x, y = l.y, Z0 = l.Z0;
   const bool own = x < F.nx && y < F.ny && Z0 < C.nz;
   const int p = x + F.nx * y;
   const PlaneOffs o = plane_offs(F.nx, F.ny, x, y);
