@@ -1917,6 +1917,11 @@ int lbe_batch_init(lbe_batch *b) {
   for (int i = 0; i < b->n; ++i)
     if (lone_fluid_node(b->inst[i].g, b->ids[i][0] == 0))
       return bfail(b, LBE_ERR_NONFINITE, "batch poisson: non-finite residual");
+  // should a call below fail (out of memory), nothing may run with graphs that
+  // hold the freed hierarchy
+  drop_graphs(b);
+  const bool was_initialised = b->initialised;
+  b->initialised = false;
   // geometry: ids, link masks (per instance, set-up only)
   for (int i = 0; i < b->n; ++i) {
     const InstDev &I = b->inst[i];
@@ -1926,6 +1931,7 @@ int lbe_batch_init(lbe_batch *b) {
   }
   int rc = mg_setup(b);  // also uploads the instance table
   if (rc != LBE_OK) return rc;
+  b->initialised = was_initialised;
   BCK(b, cudaMemcpyAsync(b->psi_d, b->psi.data(), sizeof(double) * b->psi.size(), cudaMemcpyHostToDevice, b->stream));
   b->aa_odd = false;
   kb_init<<<b->grid, kBlock, 0, b->stream>>>(b->inst_d, b->tile_inst, b->T, b->Ntot, b->id, b->psi_d, b->f[0], b->q,
@@ -1933,7 +1939,6 @@ int lbe_batch_init(lbe_batch *b) {
   BCK(b, cudaGetLastError());
   BCK(b, cudaMemsetAsync(b->hist, 0, sizeof(int), b->stream));
   BCK(b, cudaStreamSynchronize(b->stream));
-  drop_graphs(b);
   rc = autotune(b);
   if (rc != LBE_OK) return rc;
   BCK(b, cudaMemsetAsync(b->flag, 0, sizeof(int), b->stream));

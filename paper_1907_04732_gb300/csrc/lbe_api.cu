@@ -278,16 +278,18 @@ int lbe_set_geometry(lbe_handle *h, const uint8_t *node_id, int n_electrodes, in
         (!g.pz && (z == 0 || z == g.nz - 1)))
       return fail(h, LBE_ERR_GEOMETRY, "set_geometry: fluid node on a non-periodic face");
   }
+  // from here on the old geometry is gone: should a call below fail (out of
+  // memory), nothing may run with graphs that hold the freed hierarchy
+  lbe::poisson_drop_graphs(h);
+  h->have_geometry = h->initialised = false;
   h->no_solid = !solid;
   LBE_CK(h, cudaMemcpyAsync(h->id, ids.data(), (size_t)g.N, cudaMemcpyHostToDevice, h->stream));
   LBE_CK(h, lbe::launch_build_mask(g, h->id, h->mask, h->stream));
   LBE_CK(h, lbe::launch_build_code(g, h->phys.selfmask, h->mask, h->code, h->stream));
   LBE_CK(h, lbe::mg_setup(h));   // multigrid preconditioner of the Poisson solve
-  lbe::poisson_drop_graphs(h);   // graphs capture the hierarchy
   LBE_CK(h, cudaStreamSynchronize(h->stream));  // ids is a host vector
   h->n_elec = n_electrodes;
   h->have_geometry = true;
-  h->initialised = false;
   return LBE_OK;
 }
 
