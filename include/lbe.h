@@ -121,7 +121,11 @@ const char *lbe_last_error(const lbe_handle *h);
  * node_id lives.  Fails with LBE_ERR_GEOMETRY if an id exceeds n_electrodes
  * or a fluid node lies on a non-periodic face.  It also builds the multigrid
  * hierarchy of the Poisson preconditioner, in the form's precision, and
- * inverts its coarsest operator on the host (synchronising the stream). */
+ * inverts its coarsest operator on the host (synchronising the stream).  The
+ * hierarchy takes about 22 B per node in the FP32 form and 43 B in the FP64
+ * form (three long axes), and the matrix of its small levels up to 38 MB in
+ * the FP32 form, 8 MB in the FP64 form, per lattice.  A call that fails after
+ * its arguments were checked leaves the handle without a geometry. */
 int lbe_set_geometry(lbe_handle *h, const uint8_t *node_id, int n_electrodes, int on_device);
 
 /* Electrode potentials psi_e (reduced, host array of n_electrodes doubles).

@@ -637,7 +637,8 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
 // float-float on the FP32 pipes: per link the difference of the high parts
 // is split exactly (two_sum), the low parts and the rounding errors go to the
 // error word.  Returns S + E ~ 6 lap to ~2^-46 of the terms; the FP64 form
-// of lap_at needs 18 FP64 adds, which are slow on this GPU.  (No __restrict__
+// of lap_at needs 18 FP64 adds, which are slow on this GPU.  ALL: a node whose
+// links all join fluid, with constant weights.  (No __restrict__
 // here and in lap6_fx_: the single-kernel solve writes these potentials between
 // the grid's barriers.)
 template <bool ALL>
@@ -657,16 +658,6 @@ __device__ __forceinline__ void lap6_ff_(const Offs &o, int r, uint32_t m, const
     S = t;
     E += te + w * (de + (lo[j] - l0));
   }
-}
-// (a node whose links all join fluid takes constant weights)
-__device__ __forceinline__ void lap6_ff(const Geo &g, int r, int x, int y, int z, uint32_t m,
-                                        const float *__restrict__ hi, const float *__restrict__ lo, float &S,
-                                        float &E) {
-  const Offs o = offsets_of(g, x, y, z);
-  if ((m & kLinkBits) == kLinkBits)
-    lap6_ff_<true>(o, r, m, hi, lo, S, E);
-  else
-    lap6_ff_<false>(o, r, m, hi, lo, S, E);
 }
 
 // 6 lap_mod(phi)(r) of the fixed-point potential, exactly: the weighted link

@@ -212,10 +212,10 @@ struct PoissonCtl {
 
 struct PoissonWork {
   void *vec = nullptr;        // CG vectors r, u, w, x, p, s ([6][N], FP32 or FP64)
-  double *partial = nullptr;  // block partials [3][nblk]
+  double *partial = nullptr;  // block partials (r,u) and (w,u) [2][nblk]
   PoissonCtl *ctl = nullptr;  // device
   PoissonCtl *ctl_host = nullptr;  // pinned
-  Launch L{};                 // launch of the CG kernels (<= kMaxPartials blocks)
+  Launch L{};                 // launch of the warm start (<= kSolveBlocks blocks)
   cudaGraphExec_t exec[2] = {nullptr, nullptr};
   const void *exec_key[2] = {nullptr, nullptr};
   cudaGraphExec_t exec_lin = nullptr;  // linear solve A x = rhs (adjoint)
@@ -229,7 +229,6 @@ struct PoissonWork {
                                // the FP32 form keeps fixed-point values, int64, in it)
   int history = 0;             // how many of them hold a solution (0..kHist)
 };
-constexpr int kMaxPartials = 2048;
 // Order of the warm start's extrapolation in time = the number of earlier
 // solutions kept (fp32::extrapolate_node).
 #ifndef LBE_EXTRAP_ORDER
@@ -272,7 +271,7 @@ struct MGWork {
   void *dense = nullptr; // that matrix [N][stride] (null: the coarsest level's inverse or sweeps)
   int stride = 0;
   void *t0 = nullptr;    // the Jacobi vector r/diag of the finest level
-  void *cinv = nullptr;  // inverse of the coarsest operator [N][N] (null: Jacobi sweeps)
+  void *cinv = nullptr;  // (pseudo-)inverse of the coarsest operator [N][N] (null: Jacobi sweeps)
 };
 
 struct AdjWork;  // adjoint.cu
@@ -323,7 +322,6 @@ struct lbe_handle {
   float4 *u32 = nullptr;               // velocity of the last collision (fp32::octant_code records)
   int *flag = nullptr;                 // device error flags (fixed-point range)
   float4 *lf = nullptr;                // 1:1 salt link records, one per node (fp32::link_record)
-  float *pw32 = nullptr;               // FP32 Poisson work: res, p, q, e [4][N]
 
   // profiling (lbe_profile_begin/end): events [sweep start, sweep end,
   // advect end, poisson end] per step

@@ -368,7 +368,7 @@ static cudaError_t form_dense(lbe_handle *h) {
   G.nl = mg.nlev;
   G.stride = (N + V - 1) / V * V;
   G.cinv = (const T *)mg.cinv;
-  size_t shared = 0;
+  size_t shared = 0;  // at most 47.6 KB (a chain: 3072 + 1536 + ... + 192 nodes)
   for (int l = ld; l < mg.nlev; ++l) {
     G.lv[l] = BottomLevel<T>{level_dev(mg.lv[l]), (const T *)mg.lv[l].A, (const T *)mg.lv[l].W};
     shared += 2 * sizeof(T) * (size_t)mg.lv[l].N;
@@ -376,9 +376,6 @@ static cudaError_t form_dense(lbe_handle *h) {
   cudaError_t e = cudaMalloc(&mg.dense, sizeof(T) * (size_t)N * G.stride);
   if (e != cudaSuccess) return e;
   G.M = (T *)mg.dense;
-  if (shared > 48 * 1024)
-    e = cudaFuncSetAttribute((const void *)k_dense_form<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared);
-  if (e != cudaSuccess) return e;
   k_dense_form<T><<<(unsigned)N, kDenseThreads, shared, h->stream>>>(G);
   mg.ld = ld;
   mg.stride = G.stride;

@@ -22,11 +22,13 @@
 // inner products of an iteration come from one reduction phase, so an
 // iteration is the preconditioner, the stencil with the dot products (k_cg_b,
 // whose last block runs the scalar recurrence) and the vector update with the
-// stopping test (k_cg_a).  The whole solve is one CUDA graph: a device-side `while`
-// over refinement rounds containing a `while` over CG iterations; kernels set
-// the loop conditions, bounded by the round limit and poisson_max_iter.
-// Where conditional graph nodes are not available the same kernels run from
-// a host loop that polls the device.
+// stopping test (k_cg_a).  Up to kOneNodes nodes the whole solve is one
+// cooperative kernel (k_solve_one).  Beyond, or with Jacobi sweeps on the
+// coarsest level, it is one CUDA graph: a device-side `while` over refinement
+// rounds containing a `while` over CG iterations; kernels set the loop
+// conditions, bounded by the round limit and poisson_max_iter.  Where
+// conditional graph nodes are not available the same kernels run from a host
+// loop that polls the device.
 //
 // Reductions are deterministic: each block reduces in a fixed tree order and
 // writes one partial; a single block sums the partials in block order.
@@ -118,10 +120,12 @@ __device__ __forceinline__ void block_reduce2(V &a, V &b) {
 }
 
 // sums of the partials in block order (every thread of the block calls).
-// All of a thread's partials are loaded before any is added (one L2 latency
-// instead of one per stride of the block), then summed in the same order.
+// A thread's partials of the first kSolveBlocks blocks are loaded before any is
+// added (one L2 latency instead of one per stride of the block), then summed in
+// the same order; those of further blocks (the stencil has 2048 on the 256^3
+// lattice) follow one stride after another.
 __device__ __forceinline__ void reduce_partials(const double *part, int nblk, double *ru, double *wu) {
-  constexpr int kPer = (kSolveBlocks + kBlock - 1) / kBlock;  // the solve launches at most kSolveBlocks blocks
+  constexpr int kPer = (kSolveBlocks + kBlock - 1) / kBlock;
   double pa[kPer], pb[kPer];
   const int t = flat_tid();
 #pragma unroll
@@ -139,7 +143,7 @@ __device__ __forceinline__ void reduce_partials(const double *part, int nblk, do
       b += pb[k];
     }
   }
-  for (int i = t + kPer * kBlock; i < nblk; i += kBlock) {  // a larger launch (not used by the solve)
+  for (int i = t + kPer * kBlock; i < nblk; i += kBlock) {
     a += __ldcg(part + S_RU * nblk + i);
     b += __ldcg(part + S_WU * nblk + i);
   }
