@@ -465,9 +465,11 @@ __global__ void __launch_bounds__(kBlock) k_correct(long long N, const T *__rest
 // order.  What is left of a small lattice's phase is the latency of the
 // barrier (a release, a poll, L1 refilled) and of two dependent L2 reads.
 struct GridBar {
-  unsigned count, exits;
+  unsigned count;
+  unsigned exits;  // blocks that left; kDeadExit more for each whose wait ran out
   int dead;
 };
+constexpr unsigned kDeadExit = 1u << 16;
 // polls of a wait, some seconds: one that long never ends.  LBE_SOLVE_SPINS sets
 // another limit (0: a wait that is not over at its first poll runs out).
 constexpr int kSpinLimit = 1 << 23;
@@ -532,6 +534,7 @@ constexpr long long kOneNodes = 3 << 19;
 template <typename T>
 constexpr int kOnePerSM = sizeof(T) == 4 ? 3 : 1;
 constexpr int kOneBlocks = 608;  // room for the partials
+static_assert(kOneBlocks < (int)kDeadExit, "exits are counted in the low half of the word");
 enum { ONE_RU = 0, ONE_WU = 1, ONE_MAX = 2, ONE_REF = 1 };
 
 // Two values of every block combined in block order; valid in thread 0.  All
@@ -713,11 +716,14 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 3 : 1) k_solve_one(co
     }
     // the block that leaves last (none waits any more) reports a wait that ran
     // out, after block 0 may have written the control block, and clears the
-    // barrier
+    // barrier (the ticket itself tells: a read of `dead` here is 1 us per solve)
     __threadfence();
-    if (atomicAdd(&S.bar->exits, 1u) == gridDim.x - 1) {
-      __threadfence();
-      if (*(volatile int *)&S.bar->dead) ctl->sticky_status = LBE_ERR_CUDA;
+    const unsigned ticket = atomicAdd(&S.bar->exits, ok ? 1u : 1u + kDeadExit);
+    if (ticket % kDeadExit == gridDim.x - 1) {
+      if (!ok || ticket >= kDeadExit) {
+        __threadfence();
+        ctl->sticky_status = LBE_ERR_CUDA;
+      }
       S.bar->count = 0;
       S.bar->exits = 0;
       S.bar->dead = 0;
