@@ -92,17 +92,18 @@ __global__ void k_set_solid_phi(const Geo g, const uint8_t *__restrict__ id, con
 // |x| < 1/4: sinh x and cosh x - 1, odd and even in x exactly, by Taylor series
 // to x^7 and x^8 for |x| < 1/64 (most links: a kT/e over the Debye length), to
 // x^11 and x^12 beyond, each truncated below 2e-17 relative.  Wide steps:
-// expm1(x) and expm1(-x), out of line.  The ranges are tested on the high word,
-// without the FP64 pipe.
+// expm1(-|x|) and expm1(|x|), out of line.  The ranges are tested on the high
+// word, without the FP64 pipe.
 struct LinkStep {
   double a, b;
-  bool wide;
+  bool wide, up;
 };
-static __device__ __noinline__ double2 expm1_pm(double x) { return make_double2(expm1(x), expm1(-x)); }
+static __device__ __noinline__ double2 expm1_pm(double x) { return make_double2(expm1(-x), expm1(x)); }
 __device__ __forceinline__ LinkStep link_step(double x) {
   LinkStep t;
   const int hi = __double2hiint(x) & 0x7fffffff;
   t.wide = hi >= 0x3fd00000;
+  t.up = __double2hiint(x) >= 0;
   if (!t.wide) {
     const double x2 = x * x;
     double p = 1.0 / 5040.0, q = 1.0 / 40320.0;
@@ -119,22 +120,34 @@ __device__ __forceinline__ LinkStep link_step(double x) {
     t.a = p * x;
     t.b = q * x2;
   } else {
-    const double2 w = expm1_pm(x);
+    const double2 w = expm1_pm(fabs(x));
     t.a = w.x;
     t.b = w.y;
   }
   return t;
 }
-// A = n' (e^dmu - 1) - n (e^-dmu - 1), p and m the two exponentials less 1.  A
-// small step takes S sinh + D (cosh - 1) instead, S = n + n', D = n' - n, whose
-// terms do not cancel there; near equilibrium (n' = n e^-dmu) those two are
-// e^|dmu| times as large as A.  The products are rounded before they are
-// subtracted: the two ends of a link then get opposite values exactly, which a
-// fused multiply-add would not give.  Out of line, and called from each branch
-// on the valence: in line, or with one call for both signs, the compiler adds
-// FP64 instructions to the small steps (64x64x256: 1.57 ms, against 1.64-1.67).
-static __device__ __noinline__ double wide_flux(double p, double m, double n1, double n0) {
-  return __dsub_rn(__dmul_rn(n1, p), __dmul_rn(n0, m));
+// sign change on the integer pipe
+__device__ __forceinline__ double flip(double v) {
+  return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
+}
+// A = n' (e^dmu - 1) - n (e^-dmu - 1) of a species with dmu = x.  A small step
+// takes S sinh + D (cosh - 1), S = n + n', D = n' - n, whose terms do not cancel
+// there; near equilibrium (n' = n e^-dmu) those two are e^|dmu| times as large
+// as A, so that a wide step takes the exponentials themselves.  Both are one
+// rounded product and one fused multiply-add, with the operands selected: no
+// branch, and no FP64 instruction more for the small steps (sweep of 64x64x256
+// 1.57 ms, as with sinh and cosh at every step; 1.64-1.67 with branches in line).
+// Wide steps: 2.98 ms, 3.09 with sinh and cosh formed from the exponentials.
+// The rounded product is that of the growing exponential at either end of a
+// link, so that its two ends get opposite values exactly.  (m0 = -n)
+__device__ __forceinline__ double link_flux(const LinkStep &t, double n1, double m0, double S, double D) {
+  const double U = t.wide ? (t.up ? m0 : n1) : S, V = t.wide ? (t.up ? n1 : m0) : D;
+  return fma(U, t.a, V * t.b);
+}
+// the same of a species with dmu = -x
+__device__ __forceinline__ double link_flux_neg(const LinkStep &t, double n1, double n0, double m0, double S, double D) {
+  const double U = t.wide ? (t.up ? flip(n1) : n0) : S, V = t.wide ? (t.up ? m0 : n1) : D;
+  return fma(-U, t.a, V * t.b);
 }
 
 // Link fluxes of Eq. LF2 and the solvent force.  With dmu = z (phi' - phi -
@@ -182,17 +195,10 @@ __device__ __forceinline__ void ion_fluxes(const Geo &g, const Phys &P, int r, c
       const double n1 = n[k * g.N + r2];
       const double D = n1 - n0[k], S = n1 + n0[k];
       double A;
-      if (kind[k] > 0) {
-        A = fma(S, t.a, D * t.b);
-        if (t.wide) A = wide_flux(t.a, t.b, n1, n0[k]);
-      } else if (kind[k] < 0) {
-        A = fma(-S, t.a, D * t.b);
-        if (t.wide) A = wide_flux(t.b, t.a, n1, n0[k]);
-      } else {
-        const LinkStep w = link_step(P.z[k] * x);
-        A = fma(S, w.a, D * w.b);
-        if (w.wide) A = wide_flux(w.a, w.b, n1, n0[k]);
-      }
+      const double m0 = flip(n0[k]);
+      if (kind[k] > 0) A = link_flux(t, n1, m0, S, D);
+      else if (kind[k] < 0) A = link_flux_neg(t, n1, n0[k], m0, S, D);
+      else A = link_flux(link_step(P.z[k] * x), n1, m0, S, D);
       const double J = fma(2.0, D, A);
       if (c2_of(i) == 1) acc1[k] += J;
       else acc2[k] += J;
