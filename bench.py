@@ -135,9 +135,10 @@ IMPL_BYTES = {
 # for the kernel source it was taken from (a hash of the sweep's sources)
 SWEEP_TRAFFIC = {
     # k_prep32 + k_sweep32 (odd in-place step), one launch each, from an ncu
-    # capture of these sources on GB300: 20.975616 + 116.610560 MB read,
-    # 51.737088 MB written
-    ("fp32", "eof_64x64x256", "f77fe34b5fd6f73b"): 189323264,
+    # capture of these sources on GB300 (summary in
+    # profiles/fp32_eof64x64x256_k_sweep32_ncu_full.md): 20.974592 + 116.609536 MB
+    # read, 53.459712 MB written
+    ("fp32", "eof_64x64x256", "eefb9e069b27da22"): 191043840,
 }
 
 
@@ -576,12 +577,12 @@ def main():
                     "gbs": pois_bytes / (phases["poisson"] * 1e-3) / 1e9,
                     "hbm_frac": pois_bytes / (phases["poisson"] * 1e-3) / 1e9 / peak,
                     "note": ("refinement on the fixed-point potential (exact integer Laplacian, float-float "
-                             "charge term), multigrid-preconditioned FP32 CG, cubic warm start in time; one CUDA "
-                             "graph launch per solve (conditional while nodes for the refinement and CG loops); "
+                             "charge term), multigrid-preconditioned FP32 CG, cubic warm start in time; one launch "
+                             "per solve (a cooperative kernel up to 1.5 M nodes, a CUDA graph beyond); "
                              "its vectors stay in L2, so the fraction is of effective bandwidth")
                             if args.precision == "fp32" else
-                            ("FP64 Jacobi-preconditioned CG in one CUDA graph launch per solve, cubic warm start "
-                             "in time")},
+                            ("multigrid-preconditioned FP64 CG, one launch per solve (a cooperative kernel up to "
+                             "1.5 M nodes, a CUDA graph beyond), cubic warm start in time")},
         "step": {"bytes_per_node": step_bytes / fluid, "gbs": step_bytes / (step_ms * 1e-3) / 1e9,
                  "hbm_frac": step_bytes / (step_ms * 1e-3) / 1e9 / peak,
                  "parts": "fused sweep + advection + Poisson CG iterations (algorithmic bytes)"},
