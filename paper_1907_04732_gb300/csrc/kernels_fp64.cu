@@ -96,14 +96,15 @@ __global__ void k_set_solid_phi(const Geo g, const uint8_t *__restrict__ id, con
 // word, without the FP64 pipe.
 struct LinkStep {
   double a, b;
-  bool wide, up;
+  bool wide;
+  int hi;  // high word of x
 };
 static __device__ __noinline__ double2 expm1_pm(double x) { return make_double2(expm1(-x), expm1(x)); }
 __device__ __forceinline__ LinkStep link_step(double x) {
   LinkStep t;
   const int hi = __double2hiint(x) & 0x7fffffff;
   t.wide = hi >= 0x3fd00000;
-  t.up = __double2hiint(x) >= 0;
+  t.hi = __double2hiint(x);
   if (!t.wide) {
     const double x2 = x * x;
     double p = 1.0 / 5040.0, q = 1.0 / 40320.0;
@@ -126,28 +127,28 @@ __device__ __forceinline__ LinkStep link_step(double x) {
   }
   return t;
 }
-// sign change on the integer pipe
-__device__ __forceinline__ double flip(double v) {
-  return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
+// v with its sign bit flipped where `sign` has it set, on the integer pipe
+constexpr int kSign = (int)0x80000000;
+__device__ __forceinline__ double flip(double v, int sign) {
+  return __hiloint2double(__double2hiint(v) ^ sign, __double2loint(v));
 }
-// A = n' (e^dmu - 1) - n (e^-dmu - 1) of a species with dmu = x.  A small step
+// A = n' (e^dmu - 1) - n (e^-dmu - 1) at dmu = x, or -x (neg: the sign bit).  A small step
 // takes S sinh + D (cosh - 1), S = n + n', D = n' - n, whose terms do not cancel
 // there; near equilibrium (n' = n e^-dmu) those two are e^|dmu| times as large
 // as A, so that a wide step takes the exponentials themselves.  Both are one
 // rounded product and one fused multiply-add, with the operands selected: no
 // branch, and no FP64 instruction more for the small steps (sweep of 64x64x256
-// 1.57 ms, as with sinh and cosh at every step; 1.64-1.67 with branches in line).
+// 1.57 ms, as with sinh and cosh at every step; 1.64-1.67 with branches in
+// line).  One expression for both signs: a copy for each made the code of a
+// one-warp block so much longer to fetch that 4x4x64 took 42.8 us, 40.9 here.
 // Wide steps: 2.98 ms, 3.09 with sinh and cosh formed from the exponentials.
 // The rounded product is that of the growing exponential at either end of a
 // link, so that its two ends get opposite values exactly.  (m0 = -n)
-__device__ __forceinline__ double link_flux(const LinkStep &t, double n1, double m0, double S, double D) {
-  const double U = t.wide ? (t.up ? m0 : n1) : S, V = t.wide ? (t.up ? n1 : m0) : D;
+__device__ __forceinline__ double link_flux(const LinkStep &t, int neg, double n1, double m0, double S, double D) {
+  const bool up = (t.hi ^ neg) >= 0;
+  const double Sn = flip(S, neg);
+  const double U = t.wide ? (up ? m0 : n1) : Sn, V = t.wide ? (up ? n1 : m0) : D;
   return fma(U, t.a, V * t.b);
-}
-// the same of a species with dmu = -x
-__device__ __forceinline__ double link_flux_neg(const LinkStep &t, double n1, double n0, double m0, double S, double D) {
-  const double U = t.wide ? (t.up ? flip(n1) : n0) : S, V = t.wide ? (t.up ? m0 : n1) : D;
-  return fma(-U, t.a, V * t.b);
 }
 
 // Link fluxes of Eq. LF2 and the solvent force.  With dmu = z (phi' - phi -
@@ -195,10 +196,9 @@ __device__ __forceinline__ void ion_fluxes(const Geo &g, const Phys &P, int r, c
       const double n1 = n[k * g.N + r2];
       const double D = n1 - n0[k], S = n1 + n0[k];
       double A;
-      const double m0 = flip(n0[k]);
-      if (kind[k] > 0) A = link_flux(t, n1, m0, S, D);
-      else if (kind[k] < 0) A = link_flux_neg(t, n1, n0[k], m0, S, D);
-      else A = link_flux(link_step(P.z[k] * x), n1, m0, S, D);
+      const double m0 = flip(n0[k], kSign);
+      if (kind[k] != 0) A = link_flux(t, kind[k] & kSign, n1, m0, S, D);
+      else A = link_flux(link_step(P.z[k] * x), 0, n1, m0, S, D);
       const double J = fma(2.0, D, A);
       if (c2_of(i) == 1) acc1[k] += J;
       else acc2[k] += J;
